@@ -157,7 +157,6 @@ struct lya_handle {
   // rank-1 tiles of the distortion-matrix kernel (lya_set_dmat_tiles)
   int dm_tensor_tiles = 0;
   // tuning and diagnostics
-  int tuned_warps = 8;
   int tuned_grab = 4;
   int tuned_for_npar = -1;
   XiLaunch last{};
@@ -473,9 +472,8 @@ int run_xi(lya_handle* h, const lya_catalog* cats, int ncat, const lya_bins* b, 
     return fail(h, LYA_ERR_TOO_LARGE, "the FP64 path supports n_par <= 256");
   if (prec == LYA_PREC_MIXED) {
     XiLaunch L;
-    const int warps = (h->tuned_for_npar == b->n_par) ? h->tuned_warps : 8;
     const int grab = (h->tuned_for_npar == b->n_par) ? h->tuned_grab : 4;
-    CK(plan_xi_mixed(h->dev, b->n_par, h->max_len, warps, grab, &L), "plan xi");
+    CK(plan_xi_mixed(h->dev, b->n_par, h->max_len, grab, &L), "plan xi");
     stage_begin(h, 0, s);
     CK(launch_xi_mixed(A, L, s), "xi kernel");
     stage_end(h, 0, s);
@@ -827,8 +825,8 @@ int lya_autotune(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, in
   if (st) return st;
   st = ensure_pairs(h, cat, 1, bins, s);
   if (st) return st;
-  // candidate (warps per block, pairs per work grab)
-  static const int cand[][2] = {{8, 1}, {8, 4}, {8, 16}, {4, 4}, {16, 4}, {12, 4}, {13, 4}, {14, 4}, {13, 2}};
+  // candidate pairs per work grab
+  static const int cand[] = {1, 2, 4, 8, 16};
   const int nc = sizeof(cand) / sizeof(cand[0]);
   const int nb = bins->n_par * bins->n_perp;
   cudaError_t e = grow(&h->outbuf, &h->out_cap, static_cast<size_t>(nb) * 16);
@@ -839,10 +837,10 @@ int lya_autotune(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, in
   CK(cudaEventCreate(&e0), "event");
   CK(cudaEventCreate(&e1), "event");
   float best = 1e30f;
-  int besti = 1;
+  int besti = 2;
   for (int c = 0; c < nc; ++c) {
     XiLaunch L;
-    if (plan_xi_mixed(h->dev, bins->n_par, h->max_len, cand[c][0], cand[c][1], &L) != cudaSuccess) {
+    if (plan_xi_mixed(h->dev, bins->n_par, h->max_len, cand[c], &L) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -876,8 +874,7 @@ int lya_autotune(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, in
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  h->tuned_warps = cand[besti][0];
-  h->tuned_grab = cand[besti][1];
+  h->tuned_grab = cand[besti];
   h->tuned_for_npar = bins->n_par;
   if (choice) *choice = besti;
   return LYA_OK;

@@ -176,8 +176,7 @@ struct XiArgs {
 };
 // largest n_par the mixed pair kernel's shared-memory layout holds
 int xi_mixed_max_npar();
-cudaError_t plan_xi_mixed(const DevInfo& dev, int n_par, int max_len, int warps, int grab,
-                          XiLaunch* L);
+cudaError_t plan_xi_mixed(const DevInfo& dev, int n_par, int max_len, int grab, XiLaunch* L);
 cudaError_t launch_xi_mixed(const XiArgs& a, const XiLaunch& L, cudaStream_t s);
 cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats, const DevInfo& dev,
                            int max_len, double r_par_max, double r_perp_max, XiLaunch* used,

@@ -162,7 +162,7 @@ extern "C" int lya_xi_pairs_static(const lya_catalog* cat, const lya_bins* bins,
   XiLaunch L{};
   // staging buffers sized for forests of up to 1024 pixels; longer forests
   // are processed in 1024-pixel segments by the same kernel
-  if (plan_xi_mixed(info, bins->n_par, 1024, 8, 4, &L) != cudaSuccess) return LYA_ERR_CUDA;
+  if (plan_xi_mixed(info, bins->n_par, 1024, 4, &L) != cudaSuccess) return LYA_ERR_CUDA;
   if (launch_xi_mixed(A, L, s) != cudaSuccess) return LYA_ERR_CUDA;
   if (xi && launch_finalize(N, W, xi, nb, s) != cudaSuccess) return LYA_ERR_CUDA;
   unsigned flags = 0;

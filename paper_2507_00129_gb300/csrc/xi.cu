@@ -36,6 +36,7 @@
 namespace lya {
 namespace {
 
+constexpr int kTeam = 64;         // threads of a team (one block): two warps on one forest pair
 constexpr int kHcap = 440;       // words per chunk-histogram array per warp: bins (K+1) x (n_par+1)
                                  // below kHcap - 32, then one dummy word per lane
 constexpr uint32_t kM15Bits = 0x4B400000u;   // bits of 1.5 * 2^23
@@ -60,37 +61,65 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
 // are kept in separate 32-bit words (no carries between them), which shared
 // memory adds natively; FP32 shared-memory reductions are emulated on this
 // part and far slower.
-__device__ __forceinline__ void split_fixed(float v, float sc16, uint32_t& hi, uint32_t& lo) {
-  // q = v * sc16 is exact (sc16 is a power of two) and |q| < 2^21
-  const float hm = __fmaf_rd(v, sc16, kM15);      // 1.5 * 2^23 + floor(q)
-  const float fr = fmaf(v, sc16, kM15 - hm);      // q - floor(q), exact
-  const float lm = fmaf(fr, 65536.f, kM15);       // 1.5 * 2^23 + round(fr * 2^16)
-  hi = __float_as_uint(hm) - kM15Bits;
-  lo = __float_as_uint(lm) - kM15Bits;
+// Two FP32 values in one 64-bit register: one instruction does both lanes'
+// fused multiply-adds, each rounded exactly as the scalar one.
+using F2 = uint64_t;
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unf2(F2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ F2 fma2_rd(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
 // A lane's ended run, held in registers until the warp adds the held runs to
 // the chunk histogram.
 struct Held {
   uint32_t key;
-  float n, w;
+  F2 nw;
   bool on;
+};
+
+// Constants of a walk (see chunk_runs).
+struct Walk {
+  F2 cpsp;           // (-c/D_par, s/D_perp)
+  F2 sc;             // fixed-point scales of N and W
+  float pmax, tmax;  // clamps of the two floors (guard column and row)
+  uint32_t stride, base, guard, twin, tspan, dummy;
 };
 
 // Adds every lane's held run to the chunk histogram (four 32-bit reductions
 // per lane; a lane without a held run adds to its own dummy word).
-__device__ __forceinline__ void add_held(Held& h, uint32_t base, float scN, float scW, uint32_t dummy) {
-  uint32_t nh, nl, wh, wl;
-  split_fixed(h.n, scN, nh, nl);
-  split_fixed(h.w, scW, wh, wl);
-  const uint32_t addr = h.on ? base + (h.key << 2) : dummy;
+__device__ __forceinline__ void add_held(Held& h, const Walk& k) {
+  const F2 m15 = f2(kM15, kM15);
+  // q = v * sc16 is exact (sc16 is a power of two) and |q| < 2^21
+  const F2 hm = fma2_rd(h.nw, k.sc, m15);                         // 1.5 * 2^23 + floor(q)
+  const F2 fr = fma2(h.nw, k.sc, fma2(hm, f2(-1.f, -1.f), m15));  // q - floor(q), exact
+  const F2 lm = fma2(fr, f2(65536.f, 65536.f), m15);              // 1.5 * 2^23 + round(fr * 2^16)
+  const float2 hi = unf2(hm), lo = unf2(lm);
+  const uint32_t addr = h.on ? k.base + (h.key << 2) : k.dummy;
   asm volatile(
       "{\n\t"
       "red.shared.add.u32 [%0], %1;\n\t"
       "red.shared.add.u32 [%0+%5], %2;\n\t"
       "red.shared.add.u32 [%0+%6], %3;\n\t"
       "red.shared.add.u32 [%0+%7], %4;\n\t}"
-      ::"r"(addr), "r"(nh), "r"(nl), "r"(wh), "r"(wl), "n"(kHcap * 4), "n"(kHcap * 8), "n"(kHcap * 12));
+      ::"r"(addr), "r"(__float_as_uint(hi.x) - kM15Bits), "r"(__float_as_uint(lo.x) - kM15Bits),
+        "r"(__float_as_uint(hi.y) - kM15Bits), "r"(__float_as_uint(lo.y) - kM15Bits), "n"(kHcap * 4),
+        "n"(kHcap * 8), "n"(kHcap * 12));
   h.on = false;
 }
 
@@ -100,26 +129,20 @@ __device__ __forceinline__ void add_held(Held& h, uint32_t base, float scN, floa
 // grid a run is about seven pixels long, so the reductions come once per ~6
 // steps instead of every step.
 template <bool WINDOW>
-__device__ __forceinline__ void run_step(const Pix& q, float cp, float sp, float uc, float us, float wdi,
-                                         float wi, float pmax, float tmax, uint32_t stride, uint32_t base,
-                                         float scN, float scW, uint32_t guard, uint32_t twin,
-                                         uint32_t tspan, uint32_t dummy, uint32_t& cur, float& aN, float& aW,
+__device__ __forceinline__ void run_step(const ulonglong2& q, const Walk& k, F2 ucus, F2 wdw, uint32_t& cur, F2& acc,
                                          Held& held) {
-  const float rp = fabsf(fmaf(-q.x, cp, uc));
-  const float rt = fmaf(q.x, sp, us);
-  const float pf = fminf(__fadd_rd(rp, kMagic), pmax);
-  const float tf = fminf(__fadd_rd(rt, kMagic), tmax);
-  uint32_t key = __float_as_uint(tf) * stride + __float_as_uint(pf);
-  if (WINDOW) key = ((__float_as_uint(tf) - kMagicBits - twin) <= tspan) ? key : guard;
+  const float2 r = unf2(fma2(q.x, k.cpsp, ucus));
+  const float pf = fminf(__fadd_rd(fabsf(r.x), kMagic), k.pmax);
+  const float tf = fminf(__fadd_rd(r.y, kMagic), k.tmax);
+  uint32_t key = __float_as_uint(tf) * k.stride + __float_as_uint(pf);
+  if (WINDOW) key = ((__float_as_uint(tf) - kMagicBits - k.twin) <= k.tspan) ? key : k.guard;
   const bool chg = key != cur;
-  if (__any_sync(0xffffffffu, chg && held.on)) add_held(held, base, scN, scW, dummy);
+  if (__any_sync(0xffffffffu, chg && held.on)) add_held(held, k);
   held.key = chg ? cur : held.key;
-  held.n = chg ? aN : held.n;
-  held.w = chg ? aW : held.w;
+  held.nw = chg ? acc : held.nw;
   held.on = held.on || chg;
   cur = key;
-  aN = fmaf(wdi, q.z, chg ? 0.f : aN);
-  aW = fmaf(wi, q.y, chg ? 0.f : aW);
+  acc = fma2(wdw, q.y, chg ? 0ull : acc);
 }
 
 // One 32-pixel chunk of forest a against pixels [jlo, jhi) of the staged
@@ -128,34 +151,27 @@ __device__ __forceinline__ void run_step(const Pix& q, float cp, float sp, float
 // run_step) and later added to the shared chunk histogram.  Out-of-grid pairs
 // land in the guard row / column (floor clamped with fminf); WINDOW
 // additionally sends rows outside [twin, twin + tspan] to the guard.  Pixels
-// are read eight at a time before the eight steps: the reductions write
-// shared memory, so a later load cannot be hoisted above them.
+// are read kUnroll at a time before the steps: the reductions write shared
+// memory, so a later load cannot be hoisted above them.
 template <bool WINDOW>
-__device__ __forceinline__ void chunk_runs(const Pix* __restrict__ buf, int jlo, int jhi, float cp,
-                                           float sp, float uc, float us, float wdi, float wi,
-                                           float pmax, float tmax, uint32_t stride, uint32_t base,
-                                           float scN, float scW, uint32_t guard, uint32_t twin,
-                                           uint32_t tspan, uint32_t dummy) {
-  uint32_t cur = guard;
-  float aN = 0.f, aW = 0.f;
-  Held held{guard, 0.f, 0.f, false};
+__device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int jhi, const Walk& k, F2 ucus, F2 wdw) {
+  constexpr int kUnroll = 4;
+  uint32_t cur = k.guard;
+  F2 acc = 0ull;
+  Held held{k.guard, 0ull, false};
   int j = jlo;
-  for (; j + 8 <= jhi; j += 8) {
-    Pix q[8];
+  for (; j + kUnroll <= jhi; j += kUnroll) {
+    ulonglong2 q[kUnroll];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) q[u] = buf[j + u];
+    for (int u = 0; u < kUnroll; ++u) q[u] = buf[j + u];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      run_step<WINDOW>(q[u], cp, sp, uc, us, wdi, wi, pmax, tmax, stride, base, scN, scW, guard, twin, tspan,
-                       dummy, cur, aN, aW, held);
+    for (int u = 0; u < kUnroll; ++u) run_step<WINDOW>(q[u], k, ucus, wdw, cur, acc, held);
   }
-  for (; j < jhi; ++j)
-    run_step<WINDOW>(buf[j], cp, sp, uc, us, wdi, wi, pmax, tmax, stride, base, scN, scW, guard, twin, tspan,
-                     dummy, cur, aN, aW, held);
+  for (; j < jhi; ++j) run_step<WINDOW>(buf[j], k, ucus, wdw, cur, acc, held);
   // the held runs, then the last run of every lane
-  if (__any_sync(0xffffffffu, held.on)) add_held(held, base, scN, scW, dummy);
-  held = Held{cur, aN, aW, true};
-  add_held(held, base, scN, scW, dummy);
+  if (__any_sync(0xffffffffu, held.on)) add_held(held, k);
+  held = Held{cur, acc, true};
+  add_held(held, k);
 }
 
 // Per-pair scale sc16 = 2^(20 - e) with 2^e <= B < 2^(e+1): every |v| < B
@@ -167,19 +183,18 @@ __device__ __forceinline__ float fixed_scale(float B) {
   return __uint_as_float(static_cast<uint32_t>(min(max(ex, 1), 254)) << 23);
 }
 
-struct WarpSm {
+struct TeamSm {
   uint32_t* h;      // chunk histogram: N hi, N lo, W hi, W lo (kHcap words each)
   float* acc;       // accumulator: N hi, N lo, W hi, W lo (kAcap each)
-  Pix* buf;         // staged pixels of forest b
-  uint32_t sN;      // shared address of hN
+  ulonglong2* buf;  // staged pixels of forest b: {x, x}, {w delta, w}
+  uint32_t sN;      // shared address of h
 };
 
-// chunk rows [0, nrows) x columns [0, npar) -> accumulator rows [r0, r0+nrows)
+// chunk rows [0, nrows) x columns [0, npar) -> accumulator rows [0, nrows)
 // (fixed point -> FP32 with the pair's scales); clears the whole chunk
-// histogram including the guard row and column
-__device__ __forceinline__ void fold_chunk(const WarpSm& w, int nrows, int npar, int r0, float inv_scN,
-                                           float inv_scW, int lane) {
-  __syncwarp();
+// histogram including the guard row and column.  All threads of the team.
+__device__ __forceinline__ void fold_chunk(const TeamSm& w, int nrows, int npar, float inv_scN, float inv_scW) {
+  __syncthreads();
   const int stride = npar + 1;
   uint32_t* nh = w.h;
   uint32_t* nl = w.h + kHcap;
@@ -190,12 +205,12 @@ __device__ __forceinline__ void fold_chunk(const WarpSm& w, int nrows, int npar,
   float* whi = w.acc + 2 * kAcap;
   float* wlo = w.acc + 3 * kAcap;
   for (int r = 0; r <= nrows; ++r) {
-    for (int p = lane; p < stride; p += 32) {
+    for (int p = threadIdx.x; p < stride; p += kTeam) {
       const int k = r * stride + p;
       const uint32_t a1 = nh[k], a2 = nl[k], b1 = wh[k], b2 = wl[k];
       if ((a1 | a2 | b1 | b2) != 0u) {
         if (r < nrows && p < npar) {
-          const int a = (r0 + r) * npar + p;
+          const int a = r * npar + p;
           const float vn = fmaf(static_cast<float>(a2), 1.f / 65536.f, static_cast<float>(static_cast<int32_t>(a1))) * inv_scN;
           const float vw = fmaf(static_cast<float>(b2), 1.f / 65536.f, static_cast<float>(static_cast<int32_t>(b1))) * inv_scW;
           two_sum(nhi[a], nlo[a], vn);
@@ -208,20 +223,19 @@ __device__ __forceinline__ void fold_chunk(const WarpSm& w, int nrows, int npar,
       }
     }
   }
-  __syncwarp();
+  __syncthreads();
 }
 
 // accumulator rows [0, rows) with origin t0 -> FP64 bin sums in global memory
-__device__ __forceinline__ void flush_acc(const WarpSm& w, const XiArgs& A, int rows, int t0,
-                                          int64_t out_off, int lane) {
-  __syncwarp();
+__device__ __forceinline__ void flush_acc(const TeamSm& w, const XiArgs& A, int rows, int t0, int64_t out_off) {
+  __syncthreads();
   const int npar = A.n_par;
   float* nhi = w.acc;
   float* nlo = w.acc + kAcap;
   float* whi = w.acc + 2 * kAcap;
   float* wlo = w.acc + 3 * kAcap;
   for (int r = 0; r < rows; ++r) {
-    for (int p = lane; p < npar; p += 32) {
+    for (int p = threadIdx.x; p < npar; p += kTeam) {
       const int a = r * npar + p;
       const float h1 = nhi[a], h2 = whi[a];
       if (h1 != 0.f || h2 != 0.f) {
@@ -235,93 +249,115 @@ __device__ __forceinline__ void flush_acc(const WarpSm& w, const XiArgs& A, int 
       }
     }
   }
-  __syncwarp();
+  __syncthreads();
+}
+
+// Number of staged pixels with distance strictly below v (v NaN -> n).
+__device__ __forceinline__ int staged_below(const ulonglong2* buf, int n, float v) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (*reinterpret_cast<const float*>(buf + mid) < v) lo = mid + 1; else hi = mid;
+  }
+  return lo;
 }
 
 // Bin rows t0 .. t0 + K - 1 of forest pair (a, b) into the chunk histogram
-// (origin t0) and fold them into accumulator rows r0 ..; WINDOW restricts to
+// (origin t0) and fold them into accumulator rows 0 ..; WINDOW restricts to
 // rows [t0, t0 + K) of a wider band whose top is t_hi.
 template <bool WINDOW>
-__device__ void pair_rows(const XiArgs& A, const WarpSm& w, int aidx, int bidx, const Pix* __restrict__ pa,
-                          const Pix* __restrict__ pb, int na, int nb, float cp, float sp, float Dc,
-                          float Ds, int t0, int K, int t_hi, int r0, int seg, int lane) {
+__device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, const Pix* __restrict__ pa,
+                          const Pix* __restrict__ pb, int na, int nb, float cp, float sp, float Dc, float Ds, int t0,
+                          int K, int t_hi, int seg) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int npar = A.n_par;
   const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(A.n_perp);
-  const uint32_t stride = static_cast<uint32_t>(npar + 1);
-  // key (M+t)*(npar+1) + (M+p) -> local index (t - t0)*(npar+1) + p
-  const uint32_t C = kMagicBits * (stride + 1u) + static_cast<uint32_t>(t0) * stride;
-  const uint32_t base = w.sN - 4u * C;
   // fixed-point scales: a run of in-grid pairs (fixed i, one bin) spans less
   // than 2 / cp in distance, so it holds at most 2 / (cp hmin_b) + 1 pixels of b
   const float nrun = 2.f / (cp * A.F.hmin[bidx]) + 1.f;
   const float scN = fixed_scale(A.F.wdmax[aidx] * A.F.wdmax[bidx] * nrun);
   const float scW = fixed_scale(A.F.wmax[aidx] * A.F.wmax[bidx] * nrun);
   const float inv_scN = 1.f / scN, inv_scW = 1.f / scW;
-  const uint32_t guard = C + static_cast<uint32_t>(npar);   // row 0, guard column
-  const float pmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(npar));
-  const float tmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(t_hi + 1));
-  int pending = 0;
+  Walk k;
+  k.cpsp = f2(-cp, sp);
+  k.sc = f2(scN, scW);
+  k.stride = static_cast<uint32_t>(npar + 1);
+  // key (M+t)*(npar+1) + (M+p) -> local index (t - t0)*(npar+1) + p
+  const uint32_t C = kMagicBits * (k.stride + 1u) + static_cast<uint32_t>(t0) * k.stride;
+  k.base = w.sN - 4u * C;
+  k.guard = C + static_cast<uint32_t>(npar);   // row 0, guard column
+  k.pmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(npar));
+  k.tmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(t_hi + 1));
+  k.twin = static_cast<uint32_t>(t0);
+  k.tspan = static_cast<uint32_t>(K - 1);
+  k.dummy = w.sN + 4u * static_cast<uint32_t>(kHcap - 32 + lane);
+  const int nchunk = (na + 31) >> 5;
   for (int j0 = 0; j0 < nb; j0 += seg) {
     const int segn = min(seg, nb - j0);
-    __syncwarp();
-    for (int k = lane; k < segn; k += 32) w.buf[k] = pb[j0 + k];
-    __syncwarp();
-    for (int i0 = 0; i0 < na; i0 += 32) {
-      const int i = i0 + lane;
-      // lanes past the end carry a NaN distance: they only ever hit the guard
-      const Pix pi = (i < na) ? pa[i] : make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
-      const float uc = fmaf(pi.x, cp, Dc);
-      const float us = fmaf(pi.x, sp, Ds);
-      const int last = min(31, na - 1 - i0);
-      const float uc_first = __shfl_sync(0xffffffffu, uc, 0);
-      const float us_first = __shfl_sync(0xffffffffu, us, 0);
-      const float uc_last = __shfl_sync(0xffffffffu, uc, last);
-      float dlo = (uc_first - fnpar) / cp;
-      float dhi = (uc_last + fnpar) / cp;
-      if (sp > 0.f) dhi = fminf(dhi, (fnperp - us_first) / sp);
-      dlo -= fabsf(dlo) * 1e-5f + 1e-2f;
-      dhi += fabsf(dhi) * 1e-5f + 1e-2f;
-      const int jlo = count_below(w.buf, segn, dlo);
-      const int jhi = count_below(w.buf, segn, dhi);
-      if (jlo >= jhi) continue;
-      chunk_runs<WINDOW>(w.buf, jlo, jhi, cp, sp, uc, us, pi.z, pi.y, pmax, tmax, stride, base, scN, scW,
-                         guard, static_cast<uint32_t>(t0), static_cast<uint32_t>(K - 1),
-                         w.sN + 4u * static_cast<uint32_t>(kHcap - 32 + lane));
-      if (++pending == 2) {
-        fold_chunk(w, K, npar, r0, inv_scN, inv_scW, lane);
-        pending = 0;
+    for (int q = threadIdx.x; q < segn; q += kTeam) {
+      const Pix p = pb[j0 + q];
+      w.buf[q] = make_ulonglong2(f2(p.x, p.x), f2(p.z, p.y));
+    }
+    __syncthreads();
+    for (int cb = 0; cb < nchunk; cb += 32) {
+      // lane c: the range of b that chunk cb + c can reach (distances are sorted; two binary searches)
+      const int i0 = (cb + lane) << 5;
+      int jlo = 0, jhi = 0;
+      if (i0 < na) {
+        const float xf = pa[i0].x, xl = pa[min(i0 + 31, na - 1)].x;
+        float dlo = (fmaf(xf, cp, Dc) - fnpar) / cp;
+        float dhi = (fmaf(xl, cp, Dc) + fnpar) / cp;
+        if (sp > 0.f) dhi = fminf(dhi, (fnperp - fmaf(xf, sp, Ds)) / sp);
+        dlo -= fabsf(dlo) * 1e-5f + 1e-2f;
+        dhi += fabsf(dhi) * 1e-5f + 1e-2f;
+        jlo = staged_below(w.buf, segn, dlo);
+        jhi = staged_below(w.buf, segn, dhi);
+      }
+      // two chunks with work at a time, one per warp, then a fold
+      unsigned todo = __ballot_sync(0xffffffffu, jlo < jhi);
+      while (todo) {
+        const unsigned rest = todo & (todo - 1u);
+        const unsigned mine = (wid == 0) ? todo : rest;
+        todo = rest & (rest - 1u);
+        if (mine) {
+          const int c = __ffs(mine) - 1;
+          const int i = ((cb + c) << 5) + lane;
+          // lanes past the end carry a NaN distance: they only ever hit the guard
+          const Pix pi = (i < na) ? pa[i] : make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
+          chunk_runs<WINDOW>(w.buf, __shfl_sync(0xffffffffu, jlo, c), __shfl_sync(0xffffffffu, jhi, c), k,
+                             f2(fmaf(pi.x, cp, Dc), fmaf(pi.x, sp, Ds)), f2(pi.z, pi.y));
+        }
+        fold_chunk(w, K, npar, inv_scN, inv_scW);
       }
     }
+    __syncthreads();
   }
-  if (pending) fold_chunk(w, K, npar, r0, inv_scN, inv_scW, lane);
 }
 
-__global__ void __launch_bounds__(512, 1) xi_mixed_kernel(XiArgs A, int seg, int kmax, int grab) {
+__global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int kmax, int grab) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // per warp: accumulator (4 x kAcap floats), chunk histogram (4 x kHcap
-  // words), pixel buffer (seg float4)
-  const int per_warp = kAcap * 16 + kHcap * 16 + seg * 16;
-  unsigned char* wb = smem + wid * per_warp;
-  WarpSm w;
-  w.acc = reinterpret_cast<float*>(wb);
-  w.h = reinterpret_cast<uint32_t*>(wb + kAcap * 16);
-  w.buf = reinterpret_cast<Pix*>(wb + kAcap * 16 + kHcap * 16);
+  __shared__ unsigned long long s_it;
+  // accumulator (4 x kAcap floats), chunk histogram (4 x kHcap words), pixel buffer (seg x 16 bytes)
+  TeamSm w;
+  w.acc = reinterpret_cast<float*>(smem);
+  w.h = reinterpret_cast<uint32_t*>(smem + kAcap * 16);
+  w.buf = reinterpret_cast<ulonglong2*>(smem + kAcap * 16 + kHcap * 16);
   w.sN = smem_addr(w.h);
-  for (int k = lane; k < 4 * kAcap; k += 32) w.acc[k] = 0.f;
-  for (int k = lane; k < 4 * kHcap; k += 32) w.h[k] = 0u;
-  __syncwarp();
-  const int npar = A.n_par, nperp = A.n_perp;
+  for (int k = threadIdx.x; k < 4 * kAcap; k += kTeam) w.acc[k] = 0.f;
+  for (int k = threadIdx.x; k < 4 * kHcap; k += kTeam) w.h[k] = 0u;
+  const int nperp = A.n_perp;
   const float fnperp = static_cast<float>(nperp);
   // the accumulator holds rows [acc_t0, acc_t0 + kmax) of catalogue acc_off
   int acc_t0 = -1;
   int64_t acc_off = -1;
   for (;;) {
-    unsigned long long it0 = 0;
-    if (lane == 0) it0 = atomicAdd(A.counter, static_cast<unsigned long long>(grab));
-    it0 = __shfl_sync(0xffffffffu, it0, 0);
+    __syncthreads();
+    if (threadIdx.x == 0) s_it = atomicAdd(A.counter, static_cast<unsigned long long>(grab));
+    __syncthreads();
+    const unsigned long long it0 = s_it;
     if (it0 >= static_cast<unsigned long long>(A.n_pairs)) break;
     const int64_t it1 = min(static_cast<int64_t>(it0) + grab, A.n_pairs);
+    // everything below is uniform over the team
     for (int64_t it = static_cast<int64_t>(it0); it < it1; ++it) {
       const int2 ab = A.pairs[it];
       if (ab.x < 0) continue;   // rejected pair
@@ -345,24 +381,24 @@ __global__ void __launch_bounds__(512, 1) xi_mixed_kernel(XiArgs A, int seg, int
       const int64_t out_off = static_cast<int64_t>(A.F.mock[a]) * A.nb;
       if (K <= kmax) {
         if (t_lo != acc_t0 || out_off != acc_off) {
-          if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off, lane);
+          if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
           acc_t0 = t_lo;
           acc_off = out_off;
         }
-        pair_rows<false>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, t_lo, K, t_hi, 0, seg, lane);
+        pair_rows<false>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, t_lo, K, t_hi, seg);
       } else {
         // wide band: windows of kmax rows, each flushed on its own
-        if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off, lane);
+        if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
         acc_t0 = -1;
         for (int tw = t_lo; tw <= t_hi; tw += kmax) {
           const int Kw = min(kmax, t_hi - tw + 1);
-          pair_rows<true>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, tw, Kw, t_hi, 0, seg, lane);
-          flush_acc(w, A, Kw, tw, out_off, lane);
+          pair_rows<true>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, tw, Kw, t_hi, seg);
+          flush_acc(w, A, Kw, tw, out_off);
         }
       }
     }
   }
-  if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off, lane);
+  if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
 }
 
 // ----------------------------------------------------------------------------
@@ -618,23 +654,20 @@ int xi_mixed_max_npar() {
   return std::min((kHcap - 32) / 2 - 1, kAcap);
 }
 
-cudaError_t plan_xi_mixed(const DevInfo& dev, int n_par, int max_len, int warps, int grab,
-                          XiLaunch* L) {
+cudaError_t plan_xi_mixed(const DevInfo& dev, int n_par, int max_len, int grab, XiLaunch* L) {
   if (n_par > xi_mixed_max_npar()) return cudaErrorInvalidValue;
   int seg = ((std::max(max_len, 1) + 31) / 32) * 32;
-  if (seg > kMaxSeg) seg = kMaxSeg;
-  // longer forests are staged in segments: shrink the segment until the block fits
-  while (seg > 32 && warps * (kAcap * 16 + kHcap * 16 + seg * 16) > dev.smem_optin) seg -= 32;
-  L->warps = warps;
+  if (seg > kMaxSeg) seg = kMaxSeg;   // longer forests are staged in segments
+  L->warps = kTeam / 32;
   L->hcap = kHcap;
   L->seg = seg;
   L->grab = grab;
-  L->smem = warps * (kAcap * 16 + kHcap * 16 + seg * 16);
+  L->smem = kAcap * 16 + kHcap * 16 + seg * 16;
   if (L->smem > dev.smem_optin) return cudaErrorInvalidValue;
   cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_mixed_kernel), L->smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_mixed_kernel, warps * 32, L->smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_mixed_kernel, kTeam, L->smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidValue;
   L->blocks = per_sm * dev.sms;
@@ -648,7 +681,7 @@ cudaError_t launch_xi_mixed(const XiArgs& a, const XiLaunch& L, cudaStream_t s) 
   // band rows per window: the chunk histogram needs (kmax + 1) x (n_par + 1)
   // entries (guard row and column), the accumulator kmax x n_par
   const int kmax = std::max(1, std::min({a.n_perp, (kHcap - 32) / (a.n_par + 1) - 1, kAcap / a.n_par}));
-  LYA_COUNT(1), xi_mixed_kernel<<<L.blocks, L.warps * 32, L.smem, s>>>(a, L.seg, kmax, L.grab);
+  LYA_COUNT(1), xi_mixed_kernel<<<L.blocks, kTeam, L.smem, s>>>(a, L.seg, kmax, L.grab);
   return cudaGetLastError();
 }
 
