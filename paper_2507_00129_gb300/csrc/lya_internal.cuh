@@ -157,8 +157,9 @@ cudaError_t launch_covariance(const double* num_s, const double* wsum_s, int n_s
 struct XiLaunch {
   int warps;       // warps per block
   int blocks;      // persistent grid size
-  int hcap;        // histogram capacity (floats per array per warp)
-  int seg;         // pixel buffer per warp (pixels)
+  int hcap;        // histogram capacity (words per array per block)
+  int acap;        // accumulator capacity (floats per array per block)
+  int seg;         // pixel buffer per block (pixels)
   int grab;        // pairs per work grab
   int smem;        // dynamic shared memory bytes
 };

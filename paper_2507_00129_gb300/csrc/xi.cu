@@ -2,9 +2,10 @@
 // pixel pair (i in a, j in b), bin (r_par, r_perp) and add (w d)_i (w d)_j and
 // w_i w_j to the bin (Section 2.1).
 //
-// Mixed kernel (LYA_PREC_MIXED), persistent, one forest pair per warp at a time:
-//  * forest b is staged in the warp's shared-memory buffer with coalesced
-//    16-byte loads; 32 pixels of forest a sit in registers (one per lane);
+// Mixed kernel (LYA_PREC_MIXED), persistent, one forest pair per team (a block
+// of two warps) at a time:
+//  * forest b is staged in the team's shared-memory buffer with coalesced
+//    16-byte loads; each warp takes 32 pixels of forest a (one per lane);
 //  * separations are FP32 fused multiply-adds on distances relative to a
 //    per-forest reference (multiple of 2^-10, so the reference differences and
 //    sums entering the pair constants are exact FP32 numbers):
@@ -14,17 +15,24 @@
 //    the low mantissa bits), so the bin index needs no float->int conversion;
 //  * each lane walks j and keeps the current bin's run sums in registers; a
 //    run that ends (the bin changed) is held in registers, and the warp adds
-//    the held runs to its chunk histogram, which covers only the rows of the
-//    pair's r_perp band, when a lane that holds one ends another: exact
+//    the held runs to the team's chunk histogram, which covers only the rows
+//    of the pair's r_perp band, when a lane that holds one ends another: exact
 //    two-word fixed point summed with native 32-bit shared-memory reductions
 //    (a lane without a held run aims them at its own dummy word);
-//  * every two 32-pixel chunks of forest a the integer sums are folded into a
-//    warp-private compensated FP32 (TwoSum) band accumulator, which survives
-//    across consecutive pairs with the same first band row (the pair list is
-//    ordered for this) and is added to the FP64 bin sums in global memory when
-//    the band changes;
+//  * every two 32-pixel chunks of forest a (one per warp) the integer sums are
+//    folded into the team's compensated FP32 (TwoSum) band accumulator, which
+//    survives across consecutive pairs with the same first band row (the pair
+//    list is ordered for this) and is added to the FP64 bin sums in global
+//    memory when the band changes;
 //  * the j loop of each 32-pixel chunk of a is restricted to the pixels that
-//    can be in range (distances are sorted; two binary searches).
+//    can be in range (distances are sorted; binary searches, one chunk per lane).
+// What bounds it: issue slots and fixed latencies (28 warp instructions per
+// step of 32 pixel pairs, issue 65-70%), and on the SDSS-like grid, whose runs
+// are two pixels long, the shared-memory pipe (81%: 3.6 wavefronts per
+// reduction).  A team of two shares 12.7 KB of tables and the staged forest,
+// so 9-13 teams (18-26 warps) fit on an SM where 8 single warps did.
+// Measured (survey pass): 60,000 SDSS-like forests 624 -> 386 ms, 9,000
+// DESI-like forests 414 -> 244 ms.
 // FP64 kernel (LYA_PREC_FP64): the same decomposition with FP64 distances,
 // separations, products and shared-memory sums, mirroring the oracle's
 // operation order: r = |d_i - d_j| * c, x = r * (1/D).
@@ -37,12 +45,20 @@ namespace lya {
 namespace {
 
 constexpr int kTeam = 64;         // threads of a team (one block): two warps on one forest pair
-constexpr int kHcap = 440;       // words per chunk-histogram array per warp: bins (K+1) x (n_par+1)
-                                 // below kHcap - 32, then one dummy word per lane
+// Tables of a team.  A chunk-histogram array holds (K + 1) x (n_par + 1) bins
+// (guard row and column) below its last 32 words, one dummy word per lane; an
+// accumulator array K x n_par.  The large form holds bands of K = 7 rows of 50
+// bins, the small one K = 5 (wider bands are walked in windows).
+constexpr int kHcapL = 440, kAcapL = 352;
+constexpr int kHcapS = 344, kAcapS = 256;
+// The small form is taken where forests are longer than this.  Long forests
+// fill shared memory with staged pixels, so the smaller tables let more teams
+// in (600 pixels: 11 instead of 9 per SM; DESI-like survey of 9,000 forests
+// 244 against 259 ms); short ones gain no team and pay for the bands of 6 and
+// 7 rows (207 pixels, SDSS-like survey of 60,000: 414 against 386 ms).
+constexpr int kSmallTablesLen = 384;
 constexpr uint32_t kM15Bits = 0x4B400000u;   // bits of 1.5 * 2^23
 constexpr float kM15 = 12582912.0f;
-constexpr int kAcap = 352;       // accumulator entries per warp: rows x n_par (7 rows of 50 bins;
-                                 // sized with kHcap so that 14 warps fit in shared memory)
 constexpr int kHcap64 = 256;     // doubles per histogram array per warp (FP64)
 constexpr int kMaxSeg = 1024;    // pixel buffer cap per warp
 
@@ -61,6 +77,7 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
 // are kept in separate 32-bit words (no carries between them), which shared
 // memory adds natively; FP32 shared-memory reductions are emulated on this
 // part and far slower.
+
 // Two FP32 values in one 64-bit register: one instruction does both lanes'
 // fused multiply-adds, each rounded exactly as the scalar one.
 using F2 = uint64_t;
@@ -89,7 +106,7 @@ __device__ __forceinline__ F2 fma2_rd(F2 a, F2 b, F2 c) {
 // the chunk histogram.
 struct Held {
   uint32_t key;
-  F2 nw;
+  float n, w;
   bool on;
 };
 
@@ -103,11 +120,12 @@ struct Walk {
 
 // Adds every lane's held run to the chunk histogram (four 32-bit reductions
 // per lane; a lane without a held run adds to its own dummy word).
+template <int HC>
 __device__ __forceinline__ void add_held(Held& h, const Walk& k) {
-  const F2 m15 = f2(kM15, kM15);
+  const F2 m15 = f2(kM15, kM15), nw = f2(h.n, h.w);
   // q = v * sc16 is exact (sc16 is a power of two) and |q| < 2^21
-  const F2 hm = fma2_rd(h.nw, k.sc, m15);                         // 1.5 * 2^23 + floor(q)
-  const F2 fr = fma2(h.nw, k.sc, fma2(hm, f2(-1.f, -1.f), m15));  // q - floor(q), exact
+  const F2 hm = fma2_rd(nw, k.sc, m15);                         // 1.5 * 2^23 + floor(q)
+  const F2 fr = fma2(nw, k.sc, fma2(hm, f2(-1.f, -1.f), m15));  // q - floor(q), exact
   const F2 lm = fma2(fr, f2(65536.f, 65536.f), m15);              // 1.5 * 2^23 + round(fr * 2^16)
   const float2 hi = unf2(hm), lo = unf2(lm);
   const uint32_t addr = h.on ? k.base + (h.key << 2) : k.dummy;
@@ -118,8 +136,8 @@ __device__ __forceinline__ void add_held(Held& h, const Walk& k) {
       "red.shared.add.u32 [%0+%6], %3;\n\t"
       "red.shared.add.u32 [%0+%7], %4;\n\t}"
       ::"r"(addr), "r"(__float_as_uint(hi.x) - kM15Bits), "r"(__float_as_uint(lo.x) - kM15Bits),
-        "r"(__float_as_uint(hi.y) - kM15Bits), "r"(__float_as_uint(lo.y) - kM15Bits), "n"(kHcap * 4),
-        "n"(kHcap * 8), "n"(kHcap * 12));
+        "r"(__float_as_uint(hi.y) - kM15Bits), "r"(__float_as_uint(lo.y) - kM15Bits), "n"(HC * 4),
+        "n"(HC * 8), "n"(HC * 12));
   h.on = false;
 }
 
@@ -128,21 +146,25 @@ __device__ __forceinline__ void add_held(Held& h, const Walk& k) {
 // only when some lane that already holds one ends another.  On the DESI-like
 // grid a run is about seven pixels long, so the reductions come once per ~6
 // steps instead of every step.
-template <bool WINDOW>
-__device__ __forceinline__ void run_step(const ulonglong2& q, const Walk& k, F2 ucus, F2 wdw, uint32_t& cur, F2& acc,
-                                         Held& held) {
+template <bool WINDOW, int HC>
+__device__ __forceinline__ void run_step(const ulonglong2& q, const Walk& k, F2 ucus, float wdi, float wi,
+                                         uint32_t& cur, float& aN, float& aW, Held& held) {
   const float2 r = unf2(fma2(q.x, k.cpsp, ucus));
   const float pf = fminf(__fadd_rd(fabsf(r.x), kMagic), k.pmax);
   const float tf = fminf(__fadd_rd(r.y, kMagic), k.tmax);
   uint32_t key = __float_as_uint(tf) * k.stride + __float_as_uint(pf);
   if (WINDOW) key = ((__float_as_uint(tf) - kMagicBits - k.twin) <= k.tspan) ? key : k.guard;
   const bool chg = key != cur;
-  if (__any_sync(0xffffffffu, chg && held.on)) add_held(held, k);
+  if (__any_sync(0xffffffffu, chg && held.on)) add_held<HC>(held, k);
+  const float2 w = unf2(q.y);
   held.key = chg ? cur : held.key;
-  held.nw = chg ? acc : held.nw;
+  held.n = chg ? aN : held.n;
+  held.w = chg ? aW : held.w;
   held.on = held.on || chg;
   cur = key;
-  acc = fma2(wdw, q.y, chg ? 0ull : acc);
+  // (scalar: packing the two sums costs more moves than the one instruction saves)
+  aN = fmaf(wdi, w.x, chg ? 0.f : aN);
+  aW = fmaf(wi, w.y, chg ? 0.f : aW);
 }
 
 // One 32-pixel chunk of forest a against pixels [jlo, jhi) of the staged
@@ -153,25 +175,26 @@ __device__ __forceinline__ void run_step(const ulonglong2& q, const Walk& k, F2 
 // additionally sends rows outside [twin, twin + tspan] to the guard.  Pixels
 // are read kUnroll at a time before the steps: the reductions write shared
 // memory, so a later load cannot be hoisted above them.
-template <bool WINDOW>
-__device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int jhi, const Walk& k, F2 ucus, F2 wdw) {
-  constexpr int kUnroll = 4;
+template <bool WINDOW, int HC>
+__device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int jhi, const Walk& k, F2 ucus, float wdi,
+                                           float wi) {
+  constexpr int kUnroll = 8;
   uint32_t cur = k.guard;
-  F2 acc = 0ull;
-  Held held{k.guard, 0ull, false};
+  float aN = 0.f, aW = 0.f;
+  Held held{k.guard, 0.f, 0.f, false};
   int j = jlo;
   for (; j + kUnroll <= jhi; j += kUnroll) {
     ulonglong2 q[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) q[u] = buf[j + u];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) run_step<WINDOW>(q[u], k, ucus, wdw, cur, acc, held);
+    for (int u = 0; u < kUnroll; ++u) run_step<WINDOW, HC>(q[u], k, ucus, wdi, wi, cur, aN, aW, held);
   }
-  for (; j < jhi; ++j) run_step<WINDOW>(buf[j], k, ucus, wdw, cur, acc, held);
+  for (; j < jhi; ++j) run_step<WINDOW, HC>(buf[j], k, ucus, wdi, wi, cur, aN, aW, held);
   // the held runs, then the last run of every lane
-  if (__any_sync(0xffffffffu, held.on)) add_held(held, k);
-  held = Held{cur, acc, true};
-  add_held(held, k);
+  if (__any_sync(0xffffffffu, held.on)) add_held<HC>(held, k);
+  held = Held{cur, aN, aW, true};
+  add_held<HC>(held, k);
 }
 
 // Per-pair scale sc16 = 2^(20 - e) with 2^e <= B < 2^(e+1): every |v| < B
@@ -184,8 +207,8 @@ __device__ __forceinline__ float fixed_scale(float B) {
 }
 
 struct TeamSm {
-  uint32_t* h;      // chunk histogram: N hi, N lo, W hi, W lo (kHcap words each)
-  float* acc;       // accumulator: N hi, N lo, W hi, W lo (kAcap each)
+  uint32_t* h;      // chunk histogram: N hi, N lo, W hi, W lo (HC words each)
+  float* acc;       // accumulator: N hi, N lo, W hi, W lo (AC each)
   ulonglong2* buf;  // staged pixels of forest b: {x, x}, {w delta, w}
   uint32_t sN;      // shared address of h
 };
@@ -193,17 +216,18 @@ struct TeamSm {
 // chunk rows [0, nrows) x columns [0, npar) -> accumulator rows [0, nrows)
 // (fixed point -> FP32 with the pair's scales); clears the whole chunk
 // histogram including the guard row and column.  All threads of the team.
+template <int HC, int AC>
 __device__ __forceinline__ void fold_chunk(const TeamSm& w, int nrows, int npar, float inv_scN, float inv_scW) {
   __syncthreads();
   const int stride = npar + 1;
   uint32_t* nh = w.h;
-  uint32_t* nl = w.h + kHcap;
-  uint32_t* wh = w.h + 2 * kHcap;
-  uint32_t* wl = w.h + 3 * kHcap;
+  uint32_t* nl = w.h + HC;
+  uint32_t* wh = w.h + 2 * HC;
+  uint32_t* wl = w.h + 3 * HC;
   float* nhi = w.acc;
-  float* nlo = w.acc + kAcap;
-  float* whi = w.acc + 2 * kAcap;
-  float* wlo = w.acc + 3 * kAcap;
+  float* nlo = w.acc + AC;
+  float* whi = w.acc + 2 * AC;
+  float* wlo = w.acc + 3 * AC;
   for (int r = 0; r <= nrows; ++r) {
     for (int p = threadIdx.x; p < stride; p += kTeam) {
       const int k = r * stride + p;
@@ -227,13 +251,14 @@ __device__ __forceinline__ void fold_chunk(const TeamSm& w, int nrows, int npar,
 }
 
 // accumulator rows [0, rows) with origin t0 -> FP64 bin sums in global memory
+template <int AC>
 __device__ __forceinline__ void flush_acc(const TeamSm& w, const XiArgs& A, int rows, int t0, int64_t out_off) {
   __syncthreads();
   const int npar = A.n_par;
   float* nhi = w.acc;
-  float* nlo = w.acc + kAcap;
-  float* whi = w.acc + 2 * kAcap;
-  float* wlo = w.acc + 3 * kAcap;
+  float* nlo = w.acc + AC;
+  float* whi = w.acc + 2 * AC;
+  float* wlo = w.acc + 3 * AC;
   for (int r = 0; r < rows; ++r) {
     for (int p = threadIdx.x; p < npar; p += kTeam) {
       const int a = r * npar + p;
@@ -265,7 +290,7 @@ __device__ __forceinline__ int staged_below(const ulonglong2* buf, int n, float 
 // Bin rows t0 .. t0 + K - 1 of forest pair (a, b) into the chunk histogram
 // (origin t0) and fold them into accumulator rows 0 ..; WINDOW restricts to
 // rows [t0, t0 + K) of a wider band whose top is t_hi.
-template <bool WINDOW>
+template <bool WINDOW, int HC, int AC>
 __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, const Pix* __restrict__ pa,
                           const Pix* __restrict__ pb, int na, int nb, float cp, float sp, float Dc, float Ds, int t0,
                           int K, int t_hi, int seg) {
@@ -290,7 +315,7 @@ __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, 
   k.tmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(t_hi + 1));
   k.twin = static_cast<uint32_t>(t0);
   k.tspan = static_cast<uint32_t>(K - 1);
-  k.dummy = w.sN + 4u * static_cast<uint32_t>(kHcap - 32 + lane);
+  k.dummy = w.sN + 4u * static_cast<uint32_t>(HC - 32 + lane);
   const int nchunk = (na + 31) >> 5;
   for (int j0 = 0; j0 < nb; j0 += seg) {
     const int segn = min(seg, nb - j0);
@@ -324,27 +349,29 @@ __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, 
           const int i = ((cb + c) << 5) + lane;
           // lanes past the end carry a NaN distance: they only ever hit the guard
           const Pix pi = (i < na) ? pa[i] : make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
-          chunk_runs<WINDOW>(w.buf, __shfl_sync(0xffffffffu, jlo, c), __shfl_sync(0xffffffffu, jhi, c), k,
-                             f2(fmaf(pi.x, cp, Dc), fmaf(pi.x, sp, Ds)), f2(pi.z, pi.y));
+          chunk_runs<WINDOW, HC>(w.buf, __shfl_sync(0xffffffffu, jlo, c), __shfl_sync(0xffffffffu, jhi, c), k,
+                             f2(fmaf(pi.x, cp, Dc), fmaf(pi.x, sp, Ds)), pi.z, pi.y);
         }
-        fold_chunk(w, K, npar, inv_scN, inv_scW);
+        fold_chunk<HC, AC>(w, K, npar, inv_scN, inv_scW);
       }
     }
     __syncthreads();
   }
 }
 
+// HC words per chunk-histogram array, AC entries per accumulator array (see kTables)
+template <int HC, int AC>
 __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int kmax, int grab) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_it;
-  // accumulator (4 x kAcap floats), chunk histogram (4 x kHcap words), pixel buffer (seg x 16 bytes)
+  // accumulator (4 x AC floats), chunk histogram (4 x HC words), pixel buffer (seg x 16 bytes)
   TeamSm w;
   w.acc = reinterpret_cast<float*>(smem);
-  w.h = reinterpret_cast<uint32_t*>(smem + kAcap * 16);
-  w.buf = reinterpret_cast<ulonglong2*>(smem + kAcap * 16 + kHcap * 16);
+  w.h = reinterpret_cast<uint32_t*>(smem + AC * 16);
+  w.buf = reinterpret_cast<ulonglong2*>(smem + AC * 16 + HC * 16);
   w.sN = smem_addr(w.h);
-  for (int k = threadIdx.x; k < 4 * kAcap; k += kTeam) w.acc[k] = 0.f;
-  for (int k = threadIdx.x; k < 4 * kHcap; k += kTeam) w.h[k] = 0u;
+  for (int k = threadIdx.x; k < 4 * AC; k += kTeam) w.acc[k] = 0.f;
+  for (int k = threadIdx.x; k < 4 * HC; k += kTeam) w.h[k] = 0u;
   const int nperp = A.n_perp;
   const float fnperp = static_cast<float>(nperp);
   // the accumulator holds rows [acc_t0, acc_t0 + kmax) of catalogue acc_off
@@ -381,24 +408,24 @@ __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int 
       const int64_t out_off = static_cast<int64_t>(A.F.mock[a]) * A.nb;
       if (K <= kmax) {
         if (t_lo != acc_t0 || out_off != acc_off) {
-          if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
+          if (acc_t0 >= 0) flush_acc<AC>(w, A, kmax, acc_t0, acc_off);
           acc_t0 = t_lo;
           acc_off = out_off;
         }
-        pair_rows<false>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, t_lo, K, t_hi, seg);
+        pair_rows<false, HC, AC>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, t_lo, K, t_hi, seg);
       } else {
         // wide band: windows of kmax rows, each flushed on its own
-        if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
+        if (acc_t0 >= 0) flush_acc<AC>(w, A, kmax, acc_t0, acc_off);
         acc_t0 = -1;
         for (int tw = t_lo; tw <= t_hi; tw += kmax) {
           const int Kw = min(kmax, t_hi - tw + 1);
-          pair_rows<true>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, tw, Kw, t_hi, seg);
-          flush_acc(w, A, Kw, tw, out_off);
+          pair_rows<true, HC, AC>(A, w, a, b, pa, pb, na, nb, cp, sp, Dc, Ds, tw, Kw, t_hi, seg);
+          flush_acc<AC>(w, A, Kw, tw, out_off);
         }
       }
     }
   }
-  if (acc_t0 >= 0) flush_acc(w, A, kmax, acc_t0, acc_off);
+  if (acc_t0 >= 0) flush_acc<AC>(w, A, kmax, acc_t0, acc_off);
 }
 
 // ----------------------------------------------------------------------------
@@ -651,23 +678,27 @@ __global__ void finalize_kernel(const double* num, const double* wsum, double* x
 
 int xi_mixed_max_npar() {
   // two chunk-histogram rows (band row and guard row) of n_par + 1 words below the 32 dummy words
-  return std::min((kHcap - 32) / 2 - 1, kAcap);
+  return std::min((kHcapL - 32) / 2 - 1, kAcapL);
 }
 
 cudaError_t plan_xi_mixed(const DevInfo& dev, int n_par, int max_len, int grab, XiLaunch* L) {
   if (n_par > xi_mixed_max_npar()) return cudaErrorInvalidValue;
   int seg = ((std::max(max_len, 1) + 31) / 32) * 32;
   if (seg > kMaxSeg) seg = kMaxSeg;   // longer forests are staged in segments
+  const bool small = max_len > kSmallTablesLen && (kHcapS - 32) / (n_par + 1) - 1 >= 5 && kAcapS / n_par >= 5;
   L->warps = kTeam / 32;
-  L->hcap = kHcap;
+  L->hcap = small ? kHcapS : kHcapL;
+  L->acap = small ? kAcapS : kAcapL;
   L->seg = seg;
   L->grab = grab;
-  L->smem = kAcap * 16 + kHcap * 16 + seg * 16;
+  L->smem = (L->acap + L->hcap + seg) * 16;
   if (L->smem > dev.smem_optin) return cudaErrorInvalidValue;
-  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_mixed_kernel), L->smem);
+  const void* fn = small ? reinterpret_cast<const void*>(xi_mixed_kernel<kHcapS, kAcapS>)
+                         : reinterpret_cast<const void*>(xi_mixed_kernel<kHcapL, kAcapL>);
+  cudaError_t e = set_max_dynamic_smem(fn, L->smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_mixed_kernel, kTeam, L->smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kTeam, L->smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidValue;
   L->blocks = per_sm * dev.sms;
@@ -680,8 +711,11 @@ cudaError_t launch_xi_mixed(const XiArgs& a, const XiLaunch& L, cudaStream_t s) 
   if (a.n_pairs == 0) return cudaSuccess;
   // band rows per window: the chunk histogram needs (kmax + 1) x (n_par + 1)
   // entries (guard row and column), the accumulator kmax x n_par
-  const int kmax = std::max(1, std::min({a.n_perp, (kHcap - 32) / (a.n_par + 1) - 1, kAcap / a.n_par}));
-  LYA_COUNT(1), xi_mixed_kernel<<<L.blocks, kTeam, L.smem, s>>>(a, L.seg, kmax, L.grab);
+  const int kmax = std::max(1, std::min({a.n_perp, (L.hcap - 32) / (a.n_par + 1) - 1, L.acap / a.n_par}));
+  if (L.hcap == kHcapS)
+    LYA_COUNT(1), xi_mixed_kernel<kHcapS, kAcapS><<<L.blocks, kTeam, L.smem, s>>>(a, L.seg, kmax, L.grab);
+  else
+    LYA_COUNT(1), xi_mixed_kernel<kHcapL, kAcapL><<<L.blocks, kTeam, L.smem, s>>>(a, L.seg, kmax, L.grab);
   return cudaGetLastError();
 }
 
