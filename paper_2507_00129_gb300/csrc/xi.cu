@@ -277,16 +277,6 @@ __device__ __forceinline__ void flush_acc(const TeamSm& w, const XiArgs& A, int 
   __syncthreads();
 }
 
-// Number of entries of the sorted array a[0..n) strictly below v (v NaN -> n).
-__device__ __forceinline__ int floats_below(const float* a, int n, float v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 // Number of staged pixels with distance strictly below v (v NaN -> n).
 __device__ __forceinline__ int staged_below(const ulonglong2* buf, int n, float v) {
   int lo = 0, hi = n;
@@ -442,111 +432,98 @@ __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int 
 // FP64 path
 // ----------------------------------------------------------------------------
 // FP64 arithmetic is the scarce unit of this part (1.7 fused multiply-adds per
-// clock and SM, against 126 in FP32), so the kernel spends it per run of
-// pixels in one bin and not per pixel pair, with the results of FP64:
+// clock and SM, against 126 in FP32), so the kernel uses it only where a bin
+// needs it, with the results of FP64:
 //  * bins: FP32 coordinates with a proven error bound; a pixel pair whose
 //    coordinate lies within the bound of a bin edge (about 1 step in 80 holds
 //    one) is binned by the definition in FP64, r = |d_i - d_j| * c, x = r * (1/D);
-//  * sums: with the forest's FP64 prefix sums P of w and w delta, the pixels
-//    [j0, j1) of one run add w_i (P[j1] - P[j0]).  A lane turns w_i P[j] into
-//    a 52-bit integer at every run edge (one fused multiply-add with 1.5 2^52)
-//    and adds the exact difference of two edges to the team's 64-bit integer
-//    histogram, which is added to the FP64 bin sums in global memory per pair.
-// Rounding: 2^-52 of the largest w_i P per edge, no error in any sum below the
-// bins of a forest pair.  Measured (SDSS-like, 3,000 forests, W and N against
-// 64-bit sums): see the error figures at launch_xi_fp64.
+//  * products and sums: per forest w and w delta become 55-bit integers
+//    V = round(v 2^s) = 2^28 H + L (H, L signed, at most 2^26 and 2^27), and
+//    w_i w_j is 2^56 H_i H_j + 2^28 (H_i L_j + L_i H_j), three 32 x 32 + 64
+//    bit multiply-adds without rounding (L_i L_j lies below the last bit kept);
+//  * the walk goes along the diagonals of the pixel-pair matrix: lane l takes
+//    the pairs (i, i + o + l), whose separation changes slowly with i, so a run
+//    of pixel pairs in one bin is tens of pairs long on any grid.  A lane that
+//    leaves a bin adds its run to the team's 64-bit integer histogram, which
+//    is added to the FP64 bin sums in global memory per tile of 256 x 256.
+// Rounding: 2^-54 of the forest's largest value per pixel, 2^-51 (2^-45 where a
+// bin may hold 65,536 pixel pairs) of the largest product per run, to nearest,
+// none in the sums below a tile.
+// What bounds it: issue (52%) and latencies of about 55 warp instructions per
+// step, of which the key and its edge test take 20, the six multiply-adds 6,
+// and the ends of runs (some lane in every second step) a quarter; a third of
+// the lanes' pairs lie off the grid at the ends of the diagonals.
+// Measured (SDSS-like, 3,000 forests): 370 ms with FP64 arithmetic and shared
+// FP64 atomics per pixel pair, 62 ms with FP64 run-edge integers along the
+// rows (FP64 pipe 74% busy), 47 ms as it is; the largest relative error of W
+// and N against 64-bit sums is that of the first form (6e-15).
 struct Fp64Args {
   XiArgs A;
-  const double2* dw;    // per packed pixel (d, w delta)
-  const double2* pre;   // exclusive prefix sums of (w, w delta): forest f's n + 1 entries from off[f] + f
-  const double4_32a* bound;   // per forest: max |w|, max |w delta|, max |prefix of w|, max |prefix of w delta|
+  const double* d;            // per packed pixel: distance
+  const int4* v;              // per packed pixel: H, L of w delta, H, L of w
+  const int2* scale;          // per forest: s of w delta, s of w
   double inv_dpar, inv_dperp;
 };
 
-constexpr double kM52 = 6755399441055744.0;   // 1.5 * 2^52
-constexpr int kGrab64 = 8;                    // most pairs per work grab
-
-// Power of two 2^(50 - e), 2^e <= B < 2^(e+1): |v| <= B maps below 2^51.
-__device__ __forceinline__ double edge_scale(double B) {
-  if (!(B > 1e-280) || !(B < 1e280)) return 1.0;
-  const int e = static_cast<int>((__double_as_longlong(B) >> 52) & 0x7FF) - 1023;
-  return __longlong_as_double(static_cast<long long>(50 - e + 1023) << 52);
-}
-
-// 1 / sc of a power of two (no FP64 division)
-__device__ __forceinline__ double inv_pow2(double sc) {
-  return __longlong_as_double((2046ll << 52) - __double_as_longlong(sc));
-}
+constexpr int kGrab64 = 8;      // most pairs per work grab
+constexpr int kTile64 = 256;    // pixels of a tile edge: a run of 256 products stays below 2^62
+constexpr int kPad64 = 40;      // sentinels on both sides of a staged tile of b (a block of 8 rows and 32 diagonals reaches 38 past it)
 
 struct Walk64 {
   float cp, sp;              // c/D_par, s/D_perp
   float hp, ht;              // 1/2 - guard of the two coordinates
   float pmax, tmin, tmax;
-  uint32_t stride, base, guard, twin, tspan, dummy;
+  uint32_t stride, base, guard, twin, tspan;
+  int shift;                 // bits a run's sum is rounded by before it is added to its bin
   double cp64, sp64;
-  const float* x;            // staged packed distances of b
-  const double2* pre;        // staged prefix sums of b
-  const double2* dw;         // b's (d, w delta) in global memory, at the segment
 };
 
-struct Lane64 {
-  float uc, us;
-  double d, w, wd;           // d_i, and w_i, (w delta)_i times the fixed-point scales
-  long long eN, eW;          // edge integers at the start of the run to add next
-  uint32_t cur, key;
-  int j;                     // end of the held run
-  bool on;
+struct Sum64 {
+  long long nh, nl, wh, wl;  // sums of H H and of H L + L H, of N and of W
 };
 
-// Adds every lane's held run [previous edge, j) to its bin.
-__device__ __forceinline__ void add_run64(Lane64& l, const Walk64& k) {
-  const double2 p = k.pre[l.on ? l.j : 0];
-  const long long n = __double_as_longlong(fma(l.wd, p.y, kM52));
-  const long long w = __double_as_longlong(fma(l.w, p.x, kM52));
-  const uint32_t addr = l.on ? k.base + (l.key << 4) : k.dummy;
-  const long long dn = l.on ? n - l.eN : 0, dw = l.on ? w - l.eW : 0;
-  asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(addr), "l"(dn), "l"(dw));
-  l.eN = l.on ? n : l.eN;
-  l.eW = l.on ? w : l.eW;
-  l.on = false;
+struct Run64 {
+  Sum64 s;                   // the current run
+  Sum64 held;                // an ended run, until the lane ends another
+  uint32_t cur, key;         // their bins
+  bool on;                   // a run is held
+};
+
+// v / 2^shift to nearest, ties to even (rounding ties up would add a bias
+// of 1e-14 to N, whose runs nearly cancel)
+__device__ __forceinline__ long long round_shift(long long v, int shift) {
+  return (v + ((1ll << (shift - 1)) - 1) + ((v >> shift) & 1)) >> shift;
 }
 
-template <bool WINDOW>
-__device__ __forceinline__ void step64(float xj, int j, const Walk64& k, Lane64& l) {
-  const float rp = fabsf(fmaf(-xj, k.cp, l.uc));
-  const float rt = fmaf(xj, k.sp, l.us);
-  const float pm = __fadd_rd(rp, kMagic), tm = __fadd_rd(rt, kMagic);
-  const bool near = fabsf((rp - (pm - kMagic)) - 0.5f) > k.hp || fabsf((rt - (tm - kMagic)) - 0.5f) > k.ht;
-  const uint32_t tb = __float_as_uint(fminf(WINDOW ? tm : fmaxf(tm, k.tmin), k.tmax));
-  uint32_t key = tb * k.stride + __float_as_uint(fminf(pm, k.pmax));
-  if (WINDOW) key = (tb - kMagicBits - k.twin <= k.tspan) ? key : k.guard;
-  if (__any_sync(0xffffffffu, near)) {
-    const double dj = k.dw[j].x;
-    const double x = fabs(l.d - dj) * k.cp64, y = (l.d + dj) * k.sp64;
-    uint32_t exact = k.guard;
-    // pmax and tmax hold n_par and the row past the band
-    if (x < static_cast<double>(k.pmax - kMagic) && y < static_cast<double>(k.tmax - kMagic)) {
-      const uint32_t t = static_cast<uint32_t>(static_cast<int>(y));
-      if (!WINDOW || t - k.twin <= k.tspan)
-        exact = (kMagicBits + t) * k.stride + kMagicBits + static_cast<uint32_t>(static_cast<int>(x));
-    }
-    key = near ? exact : key;
+// Adds every lane's held run to its bin.
+__device__ __forceinline__ void add_run64(Run64& r, const Walk64& k) {
+  if (r.on) {
+    const long long n = round_shift(r.held.nh + ((r.held.nl + (1ll << 27)) >> 28), k.shift);
+    const long long w = round_shift(r.held.wh + ((r.held.wl + (1ll << 27)) >> 28), k.shift);
+    asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(k.base + (r.key << 4)),
+                 "l"(n), "l"(w));
   }
-  const bool chg = key != l.cur;
-  if (__any_sync(0xffffffffu, chg && l.on)) add_run64(l, k);
-  l.key = chg ? l.cur : l.key;
-  l.j = chg ? j : l.j;
-  l.on = l.on || chg;
-  l.cur = key;
+  r.on = false;
+  __syncwarp();
+}
+
+// 2^e
+__device__ __forceinline__ double pow2(int e) {
+  return (e < -1022 || e > 1023) ? scalbn(1.0, e) : __longlong_as_double(static_cast<long long>(e + 1023) << 52);
 }
 
 // Bin rows [t0, t0 + K) of forest pair (a, b) into the FP64 sums; WINDOW
 // where the band goes on beyond them (its top row is t_hi).
 template <bool WINDOW>
-__device__ void pair64(const Fp64Args& P, unsigned long long* hist, double2* pbuf, float* xbuf, int a, int b, int na,
-                       int nb, double cp64, double sp64, int t0, int K, int t_hi, int seg, int hcap) {
+__device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int na, int nb, double cp64, double sp64,
+                       int t0, int K, int t_hi, int tile, int hcap) {
   const XiArgs& A = P.A;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long* hist = reinterpret_cast<unsigned long long*>(smem);
+  int4* av = reinterpret_cast<int4*>(smem + static_cast<size_t>(hcap) * 16);
+  int4* bv = av + tile + kPad64;
+  float2* au = reinterpret_cast<float2*>(bv + tile + kPad64);
+  float* bx = reinterpret_cast<float*>(au + tile) + kPad64;
   const int npar = A.n_par;
   const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(A.n_perp);
   const int64_t oa = A.F.off[a], ob = A.F.off[b];
@@ -570,92 +547,121 @@ __device__ void pair64(const Fp64Args& P, unsigned long long* hist, double2* pbu
   k.ht = 0.5f - gt - 1e-7f;
   k.stride = static_cast<uint32_t>(npar + 1);
   const uint32_t C = kMagicBits * (k.stride + 1u) + static_cast<uint32_t>(t0) * k.stride;
-  const uint32_t h0 = smem_addr(hist);
-  k.base = h0 - 16u * C;
+  k.base = smem_addr(hist) - 16u * C;
   k.guard = C + static_cast<uint32_t>(npar);
   k.pmax = kMagic + fnpar;
   k.tmin = kMagic + static_cast<float>(t0);
   k.tmax = kMagic + static_cast<float>(t_hi + 1);
   k.twin = static_cast<uint32_t>(t0);
   k.tspan = static_cast<uint32_t>(K - 1);
-  k.dummy = h0 + 16u * static_cast<uint32_t>(hcap - 32 + lane);
-  k.x = xbuf;
-  k.pre = pbuf;
-  const double4_32a ba = P.bound[a], bb = P.bound[b];
-  const double scW = edge_scale(ba.x * bb.z), scN = edge_scale(ba.y * bb.w);
-  const double inv_scW = inv_pow2(scW), inv_scN = inv_pow2(scN);
+  // products are below 2^52; a bin of a tile holds at most two runs of
+  // 2 D_par / (c gap_b) + 1 pixels per row, and its sum stays below 2^62
+  const float terms = fminf(512.f * (2.f / (k.cp * A.F.hmin[b]) + 1.f), 65536.f);
+  k.shift = max(1, 32 - __clz(static_cast<int>(terms)) - 10);
+  const int2 ea = P.scale[a], eb = P.scale[b];
   const int64_t out_off = static_cast<int64_t>(A.F.mock[a]) * A.nb;
-  const int nchunk = (na + 31) >> 5;
-  for (int j0 = 0; j0 < nb; j0 += seg) {
-    const int segn = min(seg, nb - j0);
-    for (int q = threadIdx.x; q <= segn; q += kTeam) {
-      pbuf[q] = P.pre[ob + b + j0 + q];
-      if (q < segn) xbuf[q] = pb[j0 + q].x;
-    }
-    k.dw = P.dw + ob + j0;
-    __syncthreads();
-    // batches of 32 chunks (1,024 rows): a bin's integer sum stays below 2^62
-    for (int cb = 0; cb < nchunk; cb += 32) {
-      const int i0 = (cb + lane) << 5;
-      int jlo = 0, jhi = 0;
-      if (i0 < na) {
-        const float xf = pa[i0].x, xl = pa[min(i0 + 31, na - 1)].x;
-        float dlo = (fmaf(xf, k.cp, Dc) - fnpar) / k.cp;
-        float dhi = (fmaf(xl, k.cp, Dc) + fnpar) / k.cp;
-        if (k.sp > 0.f) dhi = fminf(dhi, (fnperp - fmaf(xf, k.sp, Ds)) / k.sp);
-        dlo -= fabsf(dlo) * 1e-5f + 1e-2f;
-        dhi += fabsf(dhi) * 1e-5f + 1e-2f;
-        jlo = floats_below(xbuf, segn, dlo);
-        jhi = floats_below(xbuf, segn, dhi);
+  for (int ia = 0; ia < na; ia += tile) {
+    const int ta = min(tile, na - ia);
+    for (int jb = 0; jb < nb; jb += tile) {
+      const int tb = min(tile, nb - jb);
+      // rows up to a multiple of 8 and the padding of b lie at infinite distance, with zero weight
+      for (int q = threadIdx.x; q < ((ta + 7) & ~7); q += kTeam) {
+        const float x = (q < ta) ? pa[ia + q].x : INFINITY;
+        au[q] = (q < ta) ? make_float2(fmaf(x, k.cp, Dc), fmaf(x, k.sp, Ds)) : make_float2(INFINITY, INFINITY);
+        av[q] = (q < ta) ? P.v[oa + ia + q] : make_int4(0, 0, 0, 0);
       }
-      // the chunks with work, in turn to the two warps
-      unsigned todo = __ballot_sync(0xffffffffu, jlo < jhi);
-      for (int turn = 0; todo; ++turn) {
-        const int c = __ffs(todo) - 1;
-        todo &= todo - 1u;
-        if ((turn & 1) != wid) continue;
-        const int jb = __shfl_sync(0xffffffffu, jlo, c), je = __shfl_sync(0xffffffffu, jhi, c);
-        const int i = ((cb + c) << 5) + lane;
-        const int ic = min(i, na - 1);   // lanes past the end repeat the last pixel with zero weight
-        const Pix pi = pa[ic];
-        const double2 di = P.dw[oa + ic];
-        Lane64 l;
-        l.uc = fmaf(pi.x, k.cp, Dc);
-        l.us = fmaf(pi.x, k.sp, Ds);
-        l.d = di.x;
-        l.w = (i < na) ? static_cast<double>(pi.y) * scW : 0.0;
-        l.wd = (i < na) ? di.y * scN : 0.0;
-        l.cur = l.key = k.guard;
-        l.j = jb;
-        l.on = false;
-        const double2 p0 = pbuf[jb];
-        l.eN = __double_as_longlong(fma(l.wd, p0.y, kM52));
-        l.eW = __double_as_longlong(fma(l.w, p0.x, kM52));
-        int j = jb;
-        for (; j + 4 <= je; j += 4) {
-          float x[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) x[q] = xbuf[j + q];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) step64<WINDOW>(x[q], j + q, k, l);
+      for (int q = static_cast<int>(threadIdx.x) - kPad64; q < tb + kPad64; q += kTeam) {
+        const bool in = q >= 0 && q < tb;
+        bx[q] = in ? pb[jb + q].x : INFINITY;
+        bv[q] = in ? P.v[ob + jb + q] : make_int4(0, 0, 0, 0);
+      }
+      __syncthreads();
+      // groups of 32 diagonals j - i = o + lane, in turn to the two warps
+      const int ngroup = (ta + tb + 30) >> 5;
+      for (int g = wid; g < ngroup; g += kTeam / 32) {
+        const int o = 32 * g - (ta - 1);
+        // lane m: whether block m of 8 rows can hold an in-grid pixel pair (both coordinates are monotone in
+        // the sorted distances; 1e-2 bins cover the FP32 rounding)
+        bool work = false;
+        {
+          const int i0 = 8 * lane, i1 = min(i0 + 7, ta - 1);
+          const int jl = max(i0 + o, 0), jh = min(i1 + o + 31, tb - 1);
+          if (i0 < ta && jl <= jh) {
+            const float2 u0 = au[i0], u1 = au[i1];
+            const float xl = bx[jl], xh = bx[jh];
+            work = fmaf(-xh, k.cp, u0.x) < fnpar + 1e-2f && fmaf(-xl, k.cp, u1.x) > -fnpar - 1e-2f &&
+                   fmaf(xl, k.sp, u0.y) < fnperp + 1e-2f;
+          }
         }
-        for (; j < je; ++j) step64<WINDOW>(xbuf[j], j, k, l);
-        if (__any_sync(0xffffffffu, l.on)) add_run64(l, k);
-        l.key = l.cur;
-        l.j = je;
-        l.on = true;
-        add_run64(l, k);
+        unsigned todo = __ballot_sync(0xffffffffu, work);
+        Run64 r{{0, 0, 0, 0}, {0, 0, 0, 0}, k.guard, k.guard, false};
+        for (; todo; todo &= todo - 1u) {
+          const int i0 = 8 * (__ffs(todo) - 1);
+          const float* px = bx + i0 + o + lane;
+          const int4* pv = bv + i0 + o + lane;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float2 ui = au[i0 + q];
+            const float xj = px[q];
+            const float rp = fabsf(fmaf(-xj, k.cp, ui.x));
+            const float rt = fmaf(xj, k.sp, ui.y);
+            const float pm = __fadd_rd(rp, kMagic), tm = __fadd_rd(rt, kMagic);
+            const bool near = fabsf((rp - (pm - kMagic)) - 0.5f) > k.hp || fabsf((rt - (tm - kMagic)) - 0.5f) > k.ht;
+            const uint32_t tbits = __float_as_uint(fminf(WINDOW ? tm : fmaxf(tm, k.tmin), k.tmax));
+            uint32_t key = tbits * k.stride + __float_as_uint(fminf(pm, k.pmax));
+            if (WINDOW) key = (tbits - kMagicBits - k.twin <= k.tspan) ? key : k.guard;
+            if (__any_sync(0xffffffffu, near)) {
+              // (near is false for padding: its coordinates are infinite or NaN)
+              const int jc = min(max(i0 + q + o + lane, 0), tb - 1);
+              const double di = P.d[oa + ia + min(i0 + q, ta - 1)], dj = P.d[ob + jb + jc];
+              const double x = fabs(di - dj) * k.cp64, y = (di + dj) * k.sp64;
+              uint32_t exact = k.guard;
+              // pmax and tmax hold n_par and the row past the band
+              if (x < static_cast<double>(k.pmax - kMagic) && y < static_cast<double>(k.tmax - kMagic)) {
+                const uint32_t t = static_cast<uint32_t>(static_cast<int>(y));
+                if (t - k.twin <= k.tspan)
+                  exact = (kMagicBits + t) * k.stride + kMagicBits + static_cast<uint32_t>(static_cast<int>(x));
+              }
+              key = near ? exact : key;
+            }
+            const bool chg = key != r.cur;
+            if (__any_sync(0xffffffffu, chg)) {
+              if (__any_sync(0xffffffffu, chg && r.on)) add_run64(r, k);
+              if (chg) {
+                r.held = r.s;
+                r.key = r.cur;
+                r.on = true;
+                r.s = Sum64{0, 0, 0, 0};
+                r.cur = key;
+              }
+              __syncwarp();
+            }
+            const int4 vi = av[i0 + q], vj = pv[q];
+            r.s.nh += static_cast<long long>(vi.x) * vj.x;
+            r.s.nl += static_cast<long long>(vi.x) * vj.y;
+            r.s.nl += static_cast<long long>(vi.y) * vj.x;
+            r.s.wh += static_cast<long long>(vi.z) * vj.z;
+            r.s.wl += static_cast<long long>(vi.z) * vj.w;
+            r.s.wl += static_cast<long long>(vi.w) * vj.z;
+          }
+        }
+        add_run64(r, k);
+        r.held = r.s;
+        r.key = r.cur;
+        r.on = true;
+        add_run64(r, k);
       }
       // integer sums -> FP64 bin sums
       __syncthreads();
+      const double sn = pow2(56 + k.shift - ea.x - eb.x), sw = pow2(56 + k.shift - ea.y - eb.y);
       for (int q = threadIdx.x; q < (K + 1) * (npar + 1); q += kTeam) {
         const long long n = static_cast<long long>(hist[2 * q]), w = static_cast<long long>(hist[2 * q + 1]);
         if ((n | w) != 0) {
           const int tt = q / (npar + 1), p = q - tt * (npar + 1);
           if (tt < K && p < npar) {
             const int64_t bin = out_off + static_cast<int64_t>(p) * A.n_perp + t0 + tt;
-            red_add_f64_global(A.num + bin, static_cast<double>(n) * inv_scN);
-            red_add_f64_global(A.wsum + bin, static_cast<double>(w) * inv_scW);
+            red_add_f64_global(A.num + bin, static_cast<double>(n) * sn);
+            red_add_f64_global(A.wsum + bin, static_cast<double>(w) * sw);
           }
           hist[2 * q] = 0ull;
           hist[2 * q + 1] = 0ull;
@@ -666,16 +672,13 @@ __device__ void pair64(const Fp64Args& P, unsigned long long* hist, double2* pbu
   }
 }
 
-__global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int seg, int kmax, int hcap, int grab) {
+__global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int tile, int kmax, int hcap, int grab) {
+  // histogram (N, W) interleaved: hcap x 16 bytes | H, L of tile a and of tile b | (uc, us) of a | distances of b
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_it;
   __shared__ double2 s_cs[kGrab64];
   const XiArgs& A = P.A;
-  // histogram (N, W) interleaved: hcap x 16 bytes | prefix sums (seg + 1) x 16 | packed distances seg x 4
-  unsigned long long* hist = reinterpret_cast<unsigned long long*>(smem);
-  double2* pbuf = reinterpret_cast<double2*>(smem + static_cast<size_t>(hcap) * 16);
-  float* xbuf = reinterpret_cast<float*>(pbuf + seg + 1);
-  for (int q = threadIdx.x; q < 2 * hcap; q += kTeam) hist[q] = 0ull;
+  for (int q = threadIdx.x; q < 2 * hcap; q += kTeam) reinterpret_cast<unsigned long long*>(smem)[q] = 0ull;
   const double fnperp = A.n_perp;
   for (;;) {
     __syncthreads();
@@ -706,27 +709,33 @@ __global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int seg, int
       const int na = A.F.len[a], nb = A.F.len[b];
       if (na == 0 || nb == 0) continue;
       const double cp = s_cs[q].x, sp = s_cs[q].y;
-      const double2* da = P.dw + A.F.off[a];
-      const double2* db = P.dw + A.F.off[b];
-      const double rt_min = (da[0].x + db[0].x) * sp;
-      const double rt_max = (da[na - 1].x + db[nb - 1].x) * sp;
+      const double* da = P.d + A.F.off[a];
+      const double* db = P.d + A.F.off[b];
+      const double rt_min = (da[0] + db[0]) * sp;
+      const double rt_max = (da[na - 1] + db[nb - 1]) * sp;
       if (!(rt_min < fnperp)) continue;
       const int t_lo = static_cast<int>(rt_min);
       const int t_hi = (rt_max < fnperp) ? static_cast<int>(rt_max) : A.n_perp - 1;
       if (t_hi - t_lo < kmax) {
-        pair64<false>(P, hist, pbuf, xbuf, a, b, na, nb, cp, sp, t_lo, t_hi - t_lo + 1, t_hi, seg, hcap);
+        pair64<false>(P, smem, a, b, na, nb, cp, sp, t_lo, t_hi - t_lo + 1, t_hi, tile, hcap);
       } else {
         for (int tw = t_lo; tw <= t_hi; tw += kmax)
-          pair64<true>(P, hist, pbuf, xbuf, a, b, na, nb, cp, sp, tw, min(kmax, t_hi - tw + 1), t_hi, seg, hcap);
+          pair64<true>(P, smem, a, b, na, nb, cp, sp, tw, min(kmax, t_hi - tw + 1), t_hi, tile, hcap);
       }
     }
   }
 }
 
-// One warp per forest: FP64 distances and w delta, exclusive prefix sums of w
-// and w delta, and the bounds of their fixed-point scales.
-__global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, double2* dw, double2* pre,
-                              double4_32a* bound) {
+// H, L of round(v 2^s), |v| 2^s < 2^54: value = 2^28 H + L, L in [-2^27, 2^27)
+__device__ __forceinline__ int2 split55(double v, double scale) {
+  const long long q = __double2ll_rn(v * scale);
+  const int lo = static_cast<int>(((q + (1ll << 27)) & ((1ll << 28) - 1)) - (1ll << 27));
+  return make_int2(static_cast<int>((q - lo) >> 28), lo);
+}
+
+// One warp per forest: distances, and w delta and w as integers on the
+// forest's own power-of-two scales.
+__global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, double* d, int4* v, int2* scale) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -735,43 +744,24 @@ __global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, d
     const int n = F.len[gf];
     const int64_t o = cat.offsets[f];
     const int64_t g = F.off[gf];
-    double2* pf = pre + g + gf;
-    double cw = 0.0, cn = 0.0, mw = 0.0, mn = 0.0, mpw = 0.0, mpn = 0.0;
-    for (int base = 0; base < n; base += 32) {
-      const int k = base + lane;
-      double w = 0.0, wd = 0.0;
-      if (k < n) {
-        w = cat.weight[o + k];
-        wd = w * static_cast<double>(cat.delta[o + k]);
-        dw[g + k] = make_double2(cat.dist[o + k], wd);
-      }
+    double mw = 0.0, mn = 0.0;
+    for (int k = lane; k < n; k += 32) {
+      const double w = cat.weight[o + k];
       mw = fmax(mw, fabs(w));
-      mn = fmax(mn, fabs(wd));
-      double sw = w, sn = wd;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const double ow = __shfl_up_sync(0xffffffffu, sw, d), on = __shfl_up_sync(0xffffffffu, sn, d);
-        if (lane >= d) {
-          sw += ow;
-          sn += on;
-        }
-      }
-      sw += cw;
-      sn += cn;
-      if (k < n) pf[k + 1] = make_double2(sw, sn);
-      mpw = fmax(mpw, fabs(sw));
-      mpn = fmax(mpn, fabs(sn));
-      cw = __shfl_sync(0xffffffffu, sw, 31);
-      cn = __shfl_sync(0xffffffffu, sn, 31);
+      mn = fmax(mn, fabs(w * static_cast<double>(cat.delta[o + k])));
     }
     mw = warp_max_f64(mw);
     mn = warp_max_f64(mn);
-    mpw = warp_max_f64(mpw);
-    mpn = warp_max_f64(mpn);
-    if (lane == 0) {
-      if (n > 0) pf[0] = make_double2(0.0, 0.0);
-      bound[gf] = make_double4_32a(mw, mn, mpw, mpn);
+    // |value| < 2^(ilogb + 1): scaled below 2^54
+    const int en = (mn > 0.0) ? 53 - ilogb(mn) : 0, ew = (mw > 0.0) ? 53 - ilogb(mw) : 0;
+    const double sn = pow2(en), sw = pow2(ew);
+    for (int k = lane; k < n; k += 32) {
+      const double w = cat.weight[o + k];
+      d[g + k] = cat.dist[o + k];
+      const int2 a = split55(w * static_cast<double>(cat.delta[o + k]), sn), b = split55(w, sw);
+      v[g + k] = make_int4(a.x, a.y, b.x, b.y);
     }
+    if (lane == 0) scale[gf] = make_int2(en, ew);
   }
 }
 
@@ -943,37 +933,36 @@ cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats,
                            int max_len, double r_par_max, double r_perp_max, XiLaunch* used,
                            cudaStream_t s) {
   if (a.n_par > kMaxPar64) return cudaErrorInvalidValue;
-  // FP64 pixels, prefix sums and bounds, built on demand in one temporary buffer
+  // FP64 distances and integer pixels, built on demand in one temporary buffer
   int64_t npix = 0;
   for (int m = 0; m < n_cats; ++m) npix += cats[m].n_pix;
-  const int64_t nf = std::max<int64_t>(a.F.n, 1), np = std::max<int64_t>(npix, 1);
+  const int64_t nf = (std::max<int64_t>(a.F.n, 1) + 1) & ~int64_t{1}, np = std::max<int64_t>(npix, 1);
   char* tmp = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), static_cast<size_t>(32 * nf + 16 * (np + nf) + 16 * np), s);
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), static_cast<size_t>(8 * nf + 24 * np), s);
   if (e != cudaSuccess) return e;
-  double4_32a* bound = reinterpret_cast<double4_32a*>(tmp);
-  double2* pre = reinterpret_cast<double2*>(tmp + 32 * nf);
-  double2* dw = pre + np + nf;
+  int2* scale = reinterpret_cast<int2*>(tmp);
+  int4* v = reinterpret_cast<int4*>(tmp + 8 * nf);
+  double* d = reinterpret_cast<double*>(v + np);
   int64_t fb = 0;
   for (int m = 0; m < n_cats; ++m) {
     if (cats[m].n_forests > 0) {
       int64_t blocks = std::min<int64_t>((cats[m].n_forests * 32 + 255) / 256, 65535);
-      LYA_COUNT(1), pack64_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(cats[m], a.F, fb, dw, pre, bound);
+      LYA_COUNT(1), pack64_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(cats[m], a.F, fb, d, v, scale);
     }
     fb += cats[m].n_forests;
   }
   Fp64Args P;
   P.A = a;
-  P.dw = dw;
-  P.pre = pre;
-  P.bound = bound;
+  P.d = d;
+  P.v = v;
+  P.scale = scale;
   P.inv_dpar = static_cast<double>(a.n_par) / r_par_max;
   P.inv_dperp = static_cast<double>(a.n_perp) / r_perp_max;
-  int seg = ((std::max(max_len, 1) + 31) / 32) * 32;
-  if (seg > kMaxSeg) seg = kMaxSeg;
-  // at least one band row and the guard row; 32 dummy entries
-  const int hcap = std::max(408, 2 * (a.n_par + 1)) + 32;
-  const int kmax = std::min(a.n_perp, (hcap - 32) / (a.n_par + 1) - 1);
-  const int smem = hcap * 16 + (seg + 1) * 16 + seg * 4;
+  const int tile = std::min((std::max(max_len, 1) + 7) & ~7, kTile64);
+  // at least one band row and the guard row
+  const int hcap = std::max(408, 2 * (a.n_par + 1));
+  const int kmax = std::min(a.n_perp, hcap / (a.n_par + 1) - 1);
+  const int smem = hcap * 16 + (2 * tile + 2 * kPad64) * 16 + tile * 8 + (tile + 2 * kPad64) * 4;
   e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_fp64_kernel), smem);
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_fp64_kernel, kTeam, smem);
@@ -983,13 +972,13 @@ cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats,
   const int teams = per_sm * dev.sms;
   const int grab = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kGrab64, a.n_pairs / (16 * std::max(teams, 1)))));
   if (e == cudaSuccess && a.n_pairs > 0) {
-    LYA_COUNT(1), xi_fp64_kernel<<<teams, kTeam, smem, s>>>(P, seg, kmax, hcap, grab);
+    LYA_COUNT(1), xi_fp64_kernel<<<teams, kTeam, smem, s>>>(P, tile, kmax, hcap, grab);
     e = cudaGetLastError();
   }
   if (used) {
     used->warps = kTeam / 32;
     used->blocks = teams;
-    used->seg = seg;
+    used->seg = tile;
     used->smem = smem;
     used->hcap = hcap;
     used->grab = grab;
