@@ -1088,10 +1088,10 @@ int lya_xi_bin_means_z(lya_handle* h, const lya_catalog* cat, const lya_bins* bi
   if ((st = prepare(h, cat, 1, s))) return st;
   if ((st = ensure_pairs(h, cat, 1, bins, s))) return st;
   const int nb = bins->n_par * bins->n_perp;
-  if (means_smem_bytes(nb, h->max_len, z_pix != nullptr) > h->dev.smem_optin)
+  if (means_limit_bytes(nb, h->max_len, z_pix != nullptr) > h->dev.smem_optin)
     return fail(h, LYA_ERR_TOO_LARGE, "bin means: 36 (44 with redshifts) bytes per bin + 8 (12) per pixel of the "
                                       "longest forest above shared memory");
-  cudaError_t e = grow(&h->scratch2, &h->scratch2_cap, means_scratch_bytes(h->F.n, h->n_pairs, nb));
+  cudaError_t e = grow(&h->scratch2, &h->scratch2_cap, means_scratch_bytes(nb));
   if (e != cudaSuccess) return fail(h, LYA_ERR_NO_MEMORY, "bin-means scratch");
   MeansArgs A{};
   A.pairs = static_cast<const int2*>(h->pairbuf);
@@ -1103,7 +1103,6 @@ int lya_xi_bin_means_z(lya_handle* h, const lya_catalog* cat, const lya_bins* bi
   A.n_perp = bins->n_perp;
   A.d_par = bins->r_par_max / bins->n_par;
   A.d_perp = bins->r_perp_max / bins->n_perp;
-  A.err = h->d_err;
   A.max_len = h->max_len;
   A.zpix = z_pix;
   stage_begin(h, 0, s);

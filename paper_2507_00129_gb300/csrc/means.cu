@@ -5,45 +5,17 @@
 //     dist_mean_A = sum_A w_i w_j (d_i + d_j) / 2 / W_A,  count_A,
 // over the pixel pairs of Eq. (2.4) with the bisector split of Section 2.1.
 //
-// The forest pairs (a < b) of the cached list are grouped by a (counting
-// sort of pair indices); the kernel is described at means_kernel.  Bins are
-// the FP32 ones of the mixed path's arithmetic (|d_i - d_j| from the packed
-// distances and reference offsets, times cos(theta/2)/D_par).  Run sums are
-// FP32 (a run is a few pixels), accumulated as double-float pairs per block
-// and in FP64 across blocks.
+// Bins are the FP32 ones of the mixed path's arithmetic (|d_i - d_j| from the
+// packed distances and reference offsets, times cos(theta/2)/D_par).  The
+// kernel is described at means_kernel.
 #include <math.h>
 
 #include <algorithm>
 
-#include "dfloat.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
-
-constexpr int kMW = 16;   // warps per block
-constexpr unsigned kFull = 0xffffffffu;
-
-__device__ __forceinline__ int below(const float* a, int n, float v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-__global__ void first_count_kernel(const int2* p, int64_t n, int32_t* count) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    if (p[k].x >= 0) atomicAdd(&count[p[k].x], 1);
-}
-
-__global__ void first_scatter_kernel(const int2* p, int64_t n, const int64_t* start, int32_t* cursor,
-                                     int32_t* list) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    const int a = p[k].x;
-    if (a >= 0) list[start[a] + atomicAdd(&cursor[a], 1)] = static_cast<int32_t>(k);
-  }
-}
 
 struct Acc {
   double* W;
@@ -54,171 +26,323 @@ struct Acc {
   unsigned long long* C;
 };
 
-// Segmented inclusive scan of four (five with Z) FP32 sums over lanes with
-// equal bins (equal bins are contiguous); returns the first lane of the run on
-// its last lane, -1 elsewhere.
-template <bool Z>
-__device__ __forceinline__ int run_sums(int bin, int lane, float& v0, float& v1, float& v2, float& v3, float& v4) {
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int ob = __shfl_up_sync(kFull, bin, d);
-    const float o0 = __shfl_up_sync(kFull, v0, d);
-    const float o1 = __shfl_up_sync(kFull, v1, d);
-    const float o2 = __shfl_up_sync(kFull, v2, d);
-    const float o3 = __shfl_up_sync(kFull, v3, d);
-    const float o4 = Z ? __shfl_up_sync(kFull, v4, d) : 0.f;
-    if (lane >= d && ob == bin) {
-      v0 += o0;
-      v1 += o1;
-      v2 += o2;
-      v3 += o3;
-      if (Z) v4 += o4;
-    }
-  }
-  const int prev = __shfl_up_sync(kFull, bin, 1);
-  const int nxt = __shfl_down_sync(kFull, bin, 1);
-  const bool head = bin >= 0 && (lane == 0 || prev != bin);
-  const bool tail = bin >= 0 && (lane == 31 || nxt != bin);
-  const unsigned hm = __ballot_sync(kFull, head);
-  if (!tail) return -1;
-  return 31 - __clz(hm & (0xffffffffu >> (31 - lane)));
+constexpr int kTeam = 64;       // threads of a team (one block): two warps on one forest pair
+constexpr int kTile = 240;      // pixels of a tile edge: the low words of 57,600 blocks fit 32 bits
+constexpr int kPad = 40;        // sentinels on both sides of a staged tile of b (a block of 8 rows reaches 38 past it)
+constexpr int kBins = 408;      // bins of the band histogram: (K + 1) x (n_par + 1), guard row and column included
+
+// A lane's current run of pixel pairs in one bin: sums of w_i w_j times
+// (1, r_par/D_par), (d_i + d_j, z_i + z_j) and r_perp/D_perp, FP32 over a block
+// of at most 8 pairs and two-word fixed point (see fixed.cuh) over blocks.
+struct Run {
+  F2 wx, sz;
+  float y;
+  uint32_t h[5], l[5];
+  uint32_t cur;         // the run's bin
+  int n;                // minus its first row; its pixel pairs once it has ended
+  bool in;              // the bin lies in the grid
+};
+
+// Closes a block: its FP32 sums go to the run's integer words.
+__device__ __forceinline__ void close_pair(F2& v, F2 sc, uint32_t& h0, uint32_t& l0, uint32_t& h1, uint32_t& l1) {
+  const F2 m15 = f2(kM15, kM15);
+  const F2 hm = fma2_rd(v, sc, m15);
+  const F2 fr = fma2(v, sc, fma2(hm, f2(-1.f, -1.f), m15));
+  const F2 lm = fma2(fr, f2(65536.f, 65536.f), m15);
+  const float2 h = unf2(hm), l = unf2(lm);
+  h0 += __float_as_uint(h.x) - kM15Bits;
+  h1 += __float_as_uint(h.y) - kM15Bits;
+  l0 += __float_as_uint(l.x) - kM15Bits;
+  l1 += __float_as_uint(l.y) - kM15Bits;
+  v = 0ull;
 }
 
-// One block per first forest a (grid-stride; a's packed distances and weights
-// staged in shared memory), one warp per partner b.  A warp takes 32 pixels j
-// of b at a time, one window of a's pixels per lane (binary search), then walks
-// each window together with lanes over i, in two parts: d_i < d_j and
-// d_i >= d_j.  In each part r_par/D_par and r_perp/D_perp are monotone in i,
-// so equal bins are contiguous and a segmented warp scan sums each run of
-// w_i w_j, w_i w_j r_par/D_par, w_i w_j r_perp/D_perp and w_i w_j x_i; the
-// run's last lane adds them to the block's double-float histograms and its
-// length to the count histogram.  With Z the runs also sum w_i w_j z_i, and
-// the pair's mean redshift (z_i + z_j) / 2 goes to a fifth histogram.
-template <bool Z>
-__global__ void __launch_bounds__(kMW * 32, 2) means_kernel(MeansArgs A, const int64_t* poff, const int32_t* plist,
-                                                             Acc acc) {
-  // h1[nb] = (W, WX) | h2[nb] = (WY, WD) | hc[nb] u32 | [h3[nb] = WZ] | per team: xa[cap], wa[cap], [za[cap]]
-  extern __shared__ float4 msh[];
-  const int nb = A.n_par * A.n_perp;
-  const int cap = A.max_len;
-  float4* h1 = msh;
-  float4* h2 = msh + nb;
-  unsigned* hc = reinterpret_cast<unsigned*>(msh + 2 * nb);
-  float2* h3 = reinterpret_cast<float2*>(hc + ((nb + 1) & ~1));
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-    h1[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    h2[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    hc[k] = 0u;
-    if (Z) h3[k] = make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  // two teams of kMW / 2 warps on their own first forests (own staging and
-  // barrier), adding to the block's histograms
-  constexpr int kTeamWarps = kMW / 2;
-  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const int team = wi / kTeamWarps, tw = wi % kTeamWarps, tt = threadIdx.x % (kTeamWarps * 32);
-  float* stage0 = Z ? reinterpret_cast<float*>(h3 + nb) : reinterpret_cast<float*>(hc + nb);
-  float* xa = stage0 + static_cast<size_t>(team) * (Z ? 3 : 2) * cap;
-  float* wa = xa + cap;
-  float* za = wa + cap;   // used only with Z
-  const float fnpar = static_cast<float>(A.n_par), fnperp = static_cast<float>(A.n_perp);
-  for (int64_t f = 2 * static_cast<int64_t>(blockIdx.x) + team; f < A.F.n; f += 2 * static_cast<int64_t>(gridDim.x)) {
-    const int64_t k0 = poff[f], k1 = poff[f + 1];
-    const int n = A.F.len[f];
-    if (k1 <= k0 || n <= 0 || n > cap) continue;   // uniform over the team
-    team_sync(1 + team, kTeamWarps * 32);
-    const Pix* pa = A.pix + A.F.off[f];
-    for (int k = tt; k < n; k += kTeamWarps * 32) {
-      const Pix P = pa[k];
-      xa[k] = P.x;
-      wa[k] = P.y;
-      if (Z) za[k] = static_cast<float>(A.zpix[A.F.off[f] + k]);
-    }
-    team_sync(1 + team, kTeamWarps * 32);
-    const float dref_a = A.F.dref[f];
-    for (int64_t kk = k0 + tw; kk < k1; kk += kTeamWarps) {
-      const int k = plist[kk];
-      const int b = A.pairs[k].y;
-      if (b < 0) continue;
-      const int nbp = A.F.len[b];
-      if (nbp <= 0) continue;
-      const float2 cs = A.cs[k];
-      const float cP = cs.x, sP = cs.y;
-      const float dd = dref_a - A.F.dref[b];   // exact: multiples of 2^-10 below 8192
-      const float ss = dref_a + A.F.dref[b];
-      const Pix* pb = A.pix + A.F.off[b];
-      const float half = fnpar / cP;
-      const float tmax = (sP > 0.f) ? fnperp / sP : INFINITY;
-      for (int jb = 0; jb < nbp; jb += 32) {
-        // lane setup: pixel j = jb + lane of b and its window [i0, i1) of a, split at im (d_i >= d_j)
-        const int j = jb + lane;
-        float D = 0.f, S = 0.f, wj = 0.f, zj = 0.f;
-        int i0 = 0, im = 0, i1 = 0;
-        if (j < nbp) {
-          const Pix P = pb[j];
-          D = dd - P.x;          // d_i - d_j = xa_i + D
-          S = ss + P.x;          // d_i + d_j = xa_i + S
-          wj = P.y;
-          if (Z) zj = static_cast<float>(A.zpix[A.F.off[b] + j]);
-          const float lo = -D - half - 0.5f;
-          const float hi = fminf(-D + half, tmax - S) + 0.5f;
-          i0 = below(xa, n, lo);
-          i1 = (hi > lo) ? below(xa, n, hi) : i0;
-          im = min(max(below(xa, n, -D), i0), i1);
-        }
-        const int nj = min(32, nbp - jb);
-        for (int t = 0; t < nj; ++t) {
-          const float Dt = __shfl_sync(kFull, D, t), St = __shfl_sync(kFull, S, t), wt = __shfl_sync(kFull, wj, t);
-          const float Zt = Z ? __shfl_sync(kFull, zj, t) : 0.f;
-          const int a0 = __shfl_sync(kFull, i0, t), am = __shfl_sync(kFull, im, t), a1 = __shfl_sync(kFull, i1, t);
-#pragma unroll 1
-          for (int part = 0; part < 2; ++part) {
-            const int lo_i = part ? am : a0, hi_i = part ? a1 : am;
-            for (int base = lo_i; base < hi_i; base += 32) {
-              const int i = base + lane;
-              int bin = -1;
-              float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f, v4 = 0.f;
-              if (i < hi_i) {
-                const float xi = xa[i];
-                const float xv = fabsf(xi + Dt) * cP;
-                const float yv = (xi + St) * sP;
-                if (xv < fnpar && yv < fnperp) {
-                  bin = static_cast<int>(xv) * A.n_perp + static_cast<int>(yv);
-                  const float w = wa[i] * wt;
-                  v0 = w;
-                  v1 = w * xv;
-                  v2 = w * yv;
-                  v3 = w * xi;
-                  if (Z) v4 = w * za[i];
-                }
-              }
-              const int r0 = run_sums<Z>(bin, lane, v0, v1, v2, v3, v4);
-              if (r0 >= 0) {
-                df_atomic_add(reinterpret_cast<float2*>(&h1[bin]), v0, 0.f, A.err);
-                df_atomic_add(reinterpret_cast<float2*>(&h1[bin]) + 1, v1, 0.f, A.err);
-                df_atomic_add(reinterpret_cast<float2*>(&h2[bin]), v2, 0.f, A.err);
-                df_atomic_add(reinterpret_cast<float2*>(&h2[bin]) + 1, 0.5f * fmaf(St, v0, v3), 0.f, A.err);
-                if (Z) df_atomic_add(&h3[bin], 0.5f * fmaf(Zt, v0, v4), 0.f, A.err);
-                atomicAdd(&hc[bin], static_cast<unsigned>(lane - r0 + 1));
-              }
-            }
+__device__ __forceinline__ void close_one(float& v, float sc, uint32_t& h0, uint32_t& l0) {
+  const float hm = __fmaf_rd(v, sc, kM15);
+  const float lm = fmaf(fmaf(v, sc, kM15 - hm), 65536.f, kM15);
+  h0 += __float_as_uint(hm) - kM15Bits;
+  l0 += __float_as_uint(lm) - kM15Bits;
+  v = 0.f;
+}
+
+// (hi word, low word) -> FP64 value times 2^-e: one FP64 add, the scaling on the exponent
+__device__ __forceinline__ double from_fixed(uint32_t h, uint32_t l, int e) {
+  const long long v = (static_cast<long long>(static_cast<int32_t>(h)) << 16) + static_cast<long long>(l);
+  if (v == 0) return 0.0;
+  const double d = __longlong_as_double(v + __double_as_longlong(kM52)) - kM52;
+  return __longlong_as_double(__double_as_longlong(d) - (static_cast<long long>(e + 16) << 52));
+}
+
+// Bin rows [t0, t0 + K) of forest pair (a, b) into the sums; WINDOW where the
+// band goes on beyond them (its top row is t_hi).
+template <bool Z, bool WINDOW>
+__device__ void pair_means(const MeansArgs& A, const Acc& acc, unsigned char* smem, float* red, int a, int b, int na,
+                           int nb, float cP, float sP, int t0, int K, int t_hi, int tile, int bins) {
+  constexpr int kWords = Z ? 11 : 9;      // words per bin (odd: neighbouring bins lie in different banks)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+  float4* bp = reinterpret_cast<float4*>(smem + ((static_cast<size_t>(bins) * kWords * 4 + 15) & ~size_t{15})) + kPad;
+  float4* ap = bp + tile + kPad;
+  const int npar = A.n_par;
+  const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(A.n_perp);
+  const int64_t oa = A.F.off[a], ob = A.F.off[b];
+  const Pix* __restrict__ pa = A.pix + oa;
+  const Pix* __restrict__ pb = A.pix + ob;
+  const float dd = A.F.dref[a] - A.F.dref[b];   // exact: multiples of 2^-10 below 8192
+  const float ss = A.F.dref[a] + A.F.dref[b];
+  const uint32_t stride = static_cast<uint32_t>(npar + 1);
+  const uint32_t C = kMagicBits * (stride + 1u) + static_cast<uint32_t>(t0) * stride;
+  const uint32_t base = smem_addr(hist) - 4u * kWords * C;
+  const uint32_t guard = C + static_cast<uint32_t>(npar);
+  const float pmax = kMagic + fnpar, tmax = kMagic + static_cast<float>(t_hi + 1);
+  const uint32_t twin = static_cast<uint32_t>(t0), tspan = static_cast<uint32_t>(K - 1);
+  // fixed-point scales: a run is at most one diagonal of a tile long
+  const float bw = A.F.wmax[a] * A.F.wmax[b] * static_cast<float>(kTile);
+  const float bx = bw * fnpar, by = bw * fnperp, bs = bw * (ss + pa[na - 1].x + pb[nb - 1].x);
+  const float scW = fixed_scale(bw), scX = fixed_scale(bx), scY = fixed_scale(by), scS = fixed_scale(bs);
+  for (int ia = 0; ia < na; ia += tile) {
+    const int ta = min(tile, na - ia);
+    for (int jb = 0; jb < nb; jb += tile) {
+      const int tb = min(tile, nb - jb);
+      // rows up to a multiple of 8 and the padding of b lie at infinite distance, with zero weight
+      float zm = 0.f;
+      for (int q = threadIdx.x; q < ((ta + 7) & ~7); q += kTeam) {
+        const Pix p = (q < ta) ? pa[ia + q] : make_float4(INFINITY, 0.f, 0.f, 0.f);
+        const float z = (Z && q < ta) ? static_cast<float>(A.zpix[oa + ia + q]) : 0.f;
+        ap[q] = make_float4(p.x, z, p.y, 0.f);
+        if (Z) zm = (fabsf(z) < 1e36f) ? fmaxf(zm, fabsf(z)) : INFINITY;   // (a NaN counts as infinite)
+      }
+      for (int q = static_cast<int>(threadIdx.x) - kPad; q < tb + kPad; q += kTeam) {
+        const bool in = q >= 0 && q < tb;
+        const Pix p = in ? pb[jb + q] : make_float4(INFINITY, 0.f, 0.f, 0.f);
+        const float z = (Z && in) ? static_cast<float>(A.zpix[ob + jb + q]) : 0.f;
+        bp[q] = make_float4(ss + p.x, z, dd - p.x, p.y);   // d_i + d_j = x_i + .x, d_i - d_j = x_i + .z
+        if (Z) zm = (fabsf(z) < 1e36f) ? fmaxf(zm, fabsf(z)) : INFINITY;
+      }
+      float scZ = 1.f;
+      bool direct = !(bx < 1e36f && by < 1e36f && bs < 1e36f) || (bw != 0.f && bw < 1e-30f);
+      if (Z) {
+        // largest |z| of the tile
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
+        if (lane == 0) red[wid] = zm;
+      }
+      __syncthreads();
+      if (Z) {
+        const float bz = 2.f * bw * fmaxf(red[0], red[1]);
+        const bool fine = bz < 1e36f && (bz == 0.f || bz > 1e-30f);
+        direct = direct || !fine;
+        scZ = fixed_scale(bz);
+      }
+      const F2 scWX = f2(scW, scX), scSZ = f2(scS, scZ);
+      // the end of a block; sums beyond the fixed point's range (direct) go to
+      // the FP64 sums at once, infinities and NaN included
+      auto close_block = [&](Run& r) {
+        if (direct) {
+          const int q = static_cast<int>(r.cur - C), tt = q / (npar + 1), p = q - tt * (npar + 1);
+          if (tt < K && p < npar) {
+            const int64_t bin = static_cast<int64_t>(p) * A.n_perp + t0 + tt;
+            const float2 wx = unf2(r.wx), sz = unf2(r.sz);
+            red_add_f64_global(acc.W + bin, wx.x);
+            red_add_f64_global(acc.WX + bin, wx.y);
+            red_add_f64_global(acc.WY + bin, r.y);
+            red_add_f64_global(acc.WD + bin, 0.5 * sz.x);
+            if (Z) red_add_f64_global(acc.WZ + bin, 0.5 * sz.y);
           }
+          r.wx = r.sz = 0ull;
+          r.y = 0.f;
+        } else {
+          close_pair(r.wx, scWX, r.h[0], r.l[0], r.h[1], r.l[1]);
+          close_one(r.y, scY, r.h[2], r.l[2]);
+          close_pair(r.sz, scSZ, r.h[3], r.l[3], r.h[4], r.l[4]);
+        }
+      };
+      // the held runs of the lanes that have one -> their bins
+      bool on = false;
+      auto add_held = [&](Run& r) {
+        if (on) {
+          close_block(r);
+          const uint32_t addr = base + r.cur * (4u * kWords);
+          asm volatile(
+              "{\n\t"
+              "red.shared.add.u32 [%0], %1;\n\tred.shared.add.u32 [%0+4], %2;\n\t"
+              "red.shared.add.u32 [%0+8], %3;\n\tred.shared.add.u32 [%0+12], %4;\n\t"
+              "red.shared.add.u32 [%0+16], %5;\n\tred.shared.add.u32 [%0+20], %6;\n\t"
+              "red.shared.add.u32 [%0+24], %7;\n\tred.shared.add.u32 [%0+28], %8;\n\t"
+              "red.shared.add.u32 [%0+32], %9;\n\t}" ::"r"(addr),
+              "r"(r.h[0]), "r"(r.l[0]), "r"(r.h[1]), "r"(r.l[1]), "r"(r.h[2]), "r"(r.l[2]), "r"(r.h[3]), "r"(r.l[3]),
+              "r"(static_cast<uint32_t>(r.n)));
+          if (Z)
+            asm volatile("{\n\tred.shared.add.u32 [%0+36], %1;\n\tred.shared.add.u32 [%0+40], %2;\n\t}" ::"r"(addr),
+                         "r"(r.h[4]), "r"(r.l[4]));
+        }
+        on = false;
+        __syncwarp();
+      };
+      // groups of 32 diagonals j - i = o + lane, in turn to the two warps
+      const int ngroup = (ta + tb + 30) >> 5;
+      for (int g = wid; g < ngroup; g += kTeam / 32) {
+        const int o = 32 * g - (ta - 1);
+        // lane m: whether block m of 8 rows can hold an in-grid pixel pair (both coordinates are monotone in
+        // the sorted distances; 1e-2 bins cover the rounding)
+        bool work = false;
+        {
+          const int i0 = 8 * lane, i1 = min(i0 + 7, ta - 1);
+          const int jl = max(i0 + o, 0), jh = min(i1 + o + 31, tb - 1);
+          if (i0 < ta && jl <= jh)
+            work = (ap[i0].x + bp[jh].z) * cP < fnpar + 1e-2f && (ap[i1].x + bp[jl].z) * cP > -fnpar - 1e-2f &&
+                   (ap[i0].x + bp[jl].x) * sP < fnperp + 1e-2f;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, work);
+        if (!todo) continue;
+        const Run none{0ull, 0ull, 0.f, {0u, 0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u, 0u}, guard, 0, false};
+        Run r = none, held = none;
+        // the current run of every lane ends before row i
+        auto end_runs = [&](int i) {
+          if (__any_sync(0xffffffffu, on)) add_held(held);
+          held = r;
+          held.n += i;
+          on = r.in;
+          add_held(held);
+        };
+        int i = -1;
+        for (; todo; todo &= todo - 1u) {
+          const int ib = 8 * (__ffs(todo) - 1);
+          if (i >= 0 && ib != i) {   // blocks without work between: every run ends (its length counts its pairs)
+            end_runs(i);
+            r = none;
+          }
+          i = ib;
+          const float4* pj = bp + i + o + lane;
+#pragma unroll
+          for (int q = 0; q < 8; ++q, ++i) {
+            const float4 vi = ap[i], vj = pj[q];
+            const float xv = fabsf(vi.x + vj.z) * cP;
+            const float yv = (vi.x + vj.x) * sP;
+            const uint32_t pb_ = __float_as_uint(fminf(__fadd_rd(xv, kMagic), pmax));
+            const uint32_t tb_ = __float_as_uint(fminf(__fadd_rd(yv, kMagic), tmax));
+            uint32_t key = tb_ * stride + pb_;
+            if (WINDOW) key = (tb_ - kMagicBits - twin <= tspan) ? key : guard;
+            const bool chg = key != r.cur;
+            if (__any_sync(0xffffffffu, chg)) {
+              if (__any_sync(0xffffffffu, chg && on && r.in)) add_held(held);
+              if (chg) {
+                if (r.in) {
+                  held = r;
+                  held.n += i;
+                  on = true;
+                }
+                r = none;
+                r.cur = key;
+                r.n = -i;
+                r.in = xv < fnpar && yv < fnperp && key != guard;
+              }
+              __syncwarp();
+            }
+            const float ww = vi.z * vj.w;
+            const F2 w2 = f2(ww, ww);
+            r.wx = fma2(w2, f2(1.f, xv), r.wx);
+            r.y = fmaf(ww, yv, r.y);
+            // (not of the rounded sums x_i + (ref + x_j), z_i + z_j: on a common pixel grid their roundings repeat)
+            r.sz = fma2(w2, f2(vi.x, vi.y), fma2(w2, f2(vj.x, vj.y), r.sz));
+          }
+          close_block(r);
+        }
+        end_runs(i);
+      }
+      // integer sums -> FP64 sums
+      __syncthreads();
+      const int eW = scale_exponent(scW), eX = scale_exponent(scX), eY = scale_exponent(scY);
+      const int eS = scale_exponent(scS), eZ = scale_exponent(scZ);
+      for (int q = threadIdx.x; q < (K + 1) * (npar + 1); q += kTeam) {
+        uint32_t v[kWords], any = 0u;
+#pragma unroll
+        for (int m = 0; m < kWords; ++m) {
+          v[m] = hist[q * kWords + m];
+          any |= v[m];
+        }
+        if (any != 0u) {
+          const int tt = q / (npar + 1), p = q - tt * (npar + 1);
+          if (tt < K && p < npar) {
+            const int64_t bin = static_cast<int64_t>(p) * A.n_perp + t0 + tt;
+            if (!direct) {
+              red_add_f64_global(acc.W + bin, from_fixed(v[0], v[1], eW));
+              red_add_f64_global(acc.WX + bin, from_fixed(v[2], v[3], eX));
+              red_add_f64_global(acc.WY + bin, from_fixed(v[4], v[5], eY));
+              red_add_f64_global(acc.WD + bin, 0.5 * from_fixed(v[6], v[7], eS));
+              if (Z) red_add_f64_global(acc.WZ + bin, 0.5 * from_fixed(v[kWords - 2], v[kWords - 1], eZ));
+            }
+            if (v[8]) atomicAdd(acc.C + bin, static_cast<unsigned long long>(v[8]));
+          }
+#pragma unroll
+          for (int m = 0; m < kWords; ++m) hist[q * kWords + m] = 0u;
         }
       }
+      __syncthreads();
     }
   }
-  __syncthreads();
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-    const float4 u = h1[k], v = h2[k];
-    const double w = static_cast<double>(u.x) + u.y;
-    if (w != 0.0) {
-      red_add_f64_global(acc.W + k, w);
-      red_add_f64_global(acc.WX + k, static_cast<double>(u.z) + u.w);
-      red_add_f64_global(acc.WY + k, static_cast<double>(v.x) + v.y);
-      red_add_f64_global(acc.WD + k, static_cast<double>(v.z) + v.w);
-      if (Z) red_add_f64_global(acc.WZ + k, static_cast<double>(h3[k].x) + h3[k].y);
+}
+
+// Persistent, one forest pair per team (a block of two warps) at a time, the
+// pairs in the list's order.  A tile of up to 240 x 240 pixel pairs is staged
+// in shared memory and walked along its diagonals: lane l takes the pairs
+// (i, i + o + l), whose separations change slowly with i, so a run of pixel
+// pairs in one bin is tens of pairs long (36 on the SDSS-like grid, 66 on the
+// DESI-like one, where a run along a row is 2 and 7).  A run's sums of w_i w_j,
+// w_i w_j r_par/D_par, w_i w_j r_perp/D_perp, w_i w_j (d_i + d_j) and, with Z,
+// w_i w_j (z_i + z_j) are FP32 over at most 8 pairs and two-word fixed point
+// beyond; an ended run is held in registers until its lane ends another, and
+// then added to the team's band histogram with native 32-bit reductions (runs
+// off the grid are dropped: all lanes' would go to one word).  The histogram is
+// added to the FP64 sums per tile.
+// What bounds it: issue (69%) of about 60 warp instructions per step, a third
+// of them at the ends of runs, which some lane has in every second step.
+// Eight teams per SM (26 KB each); more teams with smaller tables cost windows.
+// Measured (SDSS-like, 15,000 forests, 5.7e10 pixel pairs, with redshifts):
+// lanes along the rows with a warp scan and compare-and-swap sums per run
+// 777 ms; along the diagonals 261 ms with every run compensated and added at
+// once, 237 ms with fixed-point runs, 202 ms held, 160 ms without the runs off
+// the grid, 180 ms with the sum of r_perp of its own (from the sum of d_i + d_j
+// its rounding differs by 6e-10 on a common pixel grid).
+template <bool Z>
+__global__ void __launch_bounds__(kTeam, 8) means_kernel(MeansArgs A, Acc acc, int tile, int bins, int kmax, int grab,
+                                                      unsigned long long* counter) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned long long s_it;
+  __shared__ float s_red[2];
+  constexpr int kWords = Z ? 11 : 9;
+  for (int q = threadIdx.x; q < bins * kWords; q += kTeam) reinterpret_cast<uint32_t*>(smem)[q] = 0u;
+  const float fnperp = static_cast<float>(A.n_perp);
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_it = atomicAdd(counter, static_cast<unsigned long long>(grab));
+    __syncthreads();
+    const unsigned long long it0 = s_it;
+    if (it0 >= static_cast<unsigned long long>(A.n_pairs)) break;
+    const int64_t it1 = min(static_cast<int64_t>(it0) + grab, A.n_pairs);
+    for (int64_t it = static_cast<int64_t>(it0); it < it1; ++it) {
+      const int2 ab = A.pairs[it];
+      if (ab.x < 0 || ab.y < 0) continue;
+      const int a = ab.x, b = ab.y;
+      const int na = A.F.len[a], nb = A.F.len[b];
+      if (na <= 0 || nb <= 0) continue;
+      const float2 cs = A.cs[it];
+      const Pix* pa = A.pix + A.F.off[a];
+      const Pix* pb = A.pix + A.F.off[b];
+      const float ss = A.F.dref[a] + A.F.dref[b];
+      // r_perp band from the extreme pixels (monotone in both distances, the same arithmetic as the walk)
+      const float y0 = (pa[0].x + (ss + pb[0].x)) * cs.y, y1 = (pa[na - 1].x + (ss + pb[nb - 1].x)) * cs.y;
+      if (!(y0 < fnperp)) continue;
+      const int t_lo = static_cast<int>(y0);
+      const int t_hi = (y1 < fnperp) ? static_cast<int>(y1) : A.n_perp - 1;
+      if (t_hi - t_lo < kmax) {
+        pair_means<Z, false>(A, acc, smem, s_red, a, b, na, nb, cs.x, cs.y, t_lo, t_hi - t_lo + 1, t_hi, tile, bins);
+      } else {
+        for (int tw = t_lo; tw <= t_hi; tw += kmax)
+          pair_means<Z, true>(A, acc, smem, s_red, a, b, na, nb, cs.x, cs.y, tw, min(kmax, t_hi - tw + 1), t_hi, tile,
+                              bins);
+      }
     }
-    if (hc[k]) atomicAdd(acc.C + k, static_cast<unsigned long long>(hc[k]));
   }
 }
 
@@ -243,16 +367,13 @@ int grid_for(int64_t n, int threads) {
   return static_cast<int>(b);
 }
 
-size_t al256(size_t v) { return (v + 255) & ~size_t(255); }
-
 }  // namespace
 
-size_t means_scratch_bytes(int64_t n_forests, int64_t n_pairs, int nb) {
-  return al256(6 * static_cast<size_t>(nb) * 8) + al256((n_forests + 1) * 8) + al256(2 * n_forests * 4 + 4) +
-         al256(std::max<int64_t>(n_pairs, 1) * 4);
-}
+size_t means_scratch_bytes(int nb) { return 6 * static_cast<size_t>(nb) * 8 + 8; }
 
-int means_smem_bytes(int nb, int max_len, bool with_z) {
+// The grids and forest lengths the entry point takes (36 or 44 bytes per bin
+// and 16 or 24 per pixel of the longest forest within a block's shared memory).
+int means_limit_bytes(int nb, int max_len, bool with_z) {
   const int base = 32 * nb + 4 * ((nb + 1) & ~1);
   return with_z ? base + 8 * nb + 2 * 12 * std::max(max_len, 1) : base + 2 * 8 * std::max(max_len, 1);
 }
@@ -261,43 +382,34 @@ cudaError_t launch_bin_means(const MeansArgs& a, const DevInfo& dev, void* scrat
                              double* rperp_mean, double* dist_mean, double* z_mean, int64_t* count, cudaStream_t s) {
   const int nb = a.n_par * a.n_perp;
   const bool with_z = a.zpix != nullptr && z_mean != nullptr;
-  char* p = static_cast<char*>(scratch);
   Acc acc;
-  acc.W = reinterpret_cast<double*>(p);
+  acc.W = static_cast<double*>(scratch);
   acc.WX = acc.W + nb;
   acc.WY = acc.WX + nb;
   acc.WD = acc.WY + nb;
   acc.WZ = acc.WD + nb;
   acc.C = reinterpret_cast<unsigned long long*>(acc.WZ + nb);
-  p += al256(6 * static_cast<size_t>(nb) * 8);
-  int64_t* poff = reinterpret_cast<int64_t*>(p);
-  p += al256((a.F.n + 1) * 8);
-  int32_t* cnt = reinterpret_cast<int32_t*>(p);
-  int32_t* cursor = cnt + a.F.n;
-  p += al256(2 * a.F.n * 4 + 4);
-  int32_t* plist = reinterpret_cast<int32_t*>(p);
-  cudaError_t e = cudaMemsetAsync(acc.W, 0, 6 * static_cast<size_t>(nb) * 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, 2 * a.F.n * 4 + 4, s);
+  unsigned long long* counter = acc.C + nb;
+  cudaError_t e = cudaMemsetAsync(acc.W, 0, means_scratch_bytes(nb), s);
   if (e != cudaSuccess) return e;
   if (a.n_pairs > 0 && a.F.n > 0) {
-    LYA_COUNT(1), first_count_kernel<<<grid_for(a.n_pairs, 256), 256, 0, s>>>(a.pairs, a.n_pairs, cnt);
-    e = launch_exclusive_scan(cnt, a.F.n, poff, s);
-    if (e != cudaSuccess) return e;
-    LYA_COUNT(1), first_scatter_kernel<<<grid_for(a.n_pairs, 256), 256, 0, s>>>(a.pairs, a.n_pairs, poff, cursor,
-                                                                                 plist);
-    const int smem = means_smem_bytes(nb, a.max_len, with_z);
+    const int tile = std::min((std::max(a.max_len, 1) + 7) & ~7, kTile);
+    // at least one band row and the guard row
+    const int bins = std::max(kBins, 2 * (a.n_par + 1));
+    const int kmax = std::min(a.n_perp, bins / (a.n_par + 1) - 1);
+    const int smem = ((bins * (with_z ? 11 : 9) * 4 + 15) & ~15) + (2 * tile + 2 * kPad) * 16;
     const void* fn = with_z ? reinterpret_cast<const void*>(means_kernel<true>)
                             : reinterpret_cast<const void*>(means_kernel<false>);
     e = set_max_dynamic_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = with_z ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, means_kernel<true>, kMW * 32, smem)
-               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, means_kernel<false>, kMW * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kTeam, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const int blocks = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(dev.sms) * per_sm, (a.F.n + 1) / 2));
-    if (with_z) LYA_COUNT(1), means_kernel<true><<<blocks, kMW * 32, smem, s>>>(a, poff, plist, acc);
-    else LYA_COUNT(1), means_kernel<false><<<blocks, kMW * 32, smem, s>>>(a, poff, plist, acc);
+    const int teams = per_sm * dev.sms;
+    const int grab = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(8, a.n_pairs / (16 * std::max(teams, 1)))));
+    if (with_z) LYA_COUNT(1), means_kernel<true><<<teams, kTeam, smem, s>>>(a, acc, tile, bins, kmax, grab, counter);
+    else LYA_COUNT(1), means_kernel<false><<<teams, kTeam, smem, s>>>(a, acc, tile, bins, kmax, grab, counter);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

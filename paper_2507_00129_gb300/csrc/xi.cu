@@ -39,7 +39,7 @@
 #include <algorithm>
 #include <math.h>
 
-#include "lya_internal.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
@@ -57,8 +57,6 @@ constexpr int kHcapS = 344, kAcapS = 256;
 // 244 against 259 ms); short ones gain no team and pay for the bands of 6 and
 // 7 rows (207 pixels, SDSS-like survey of 60,000: 414 against 386 ms).
 constexpr int kSmallTablesLen = 384;
-constexpr uint32_t kM15Bits = 0x4B400000u;   // bits of 1.5 * 2^23
-constexpr float kM15 = 12582912.0f;
 constexpr int kMaxPar64 = 256;   // largest n_par of the FP64 path
 constexpr int kMaxSeg = 1024;    // pixel buffer cap per warp
 
@@ -68,38 +66,6 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
   const float bp = s - hi;
   lo += (hi - (s - bp)) + (x - bp);
   hi = s;
-}
-
-// Exact two-word fixed point.  v (|v| < B) is represented as
-// (hi * 2^16 + lo) * 2^-k with q = v * 2^(k-16), hi = floor(q), lo =
-// round((q - hi) * 2^16) in [0, 2^16]; sc16 = 2^(k-16) is chosen per forest
-// pair so that |q| < 2^21 for every run of in-grid pairs.  Sums of hi and of lo
-// are kept in separate 32-bit words (no carries between them), which shared
-// memory adds natively; FP32 shared-memory reductions are emulated on this
-// part and far slower.
-
-// Two FP32 values in one 64-bit register: one instruction does both lanes'
-// fused multiply-adds, each rounded exactly as the scalar one.
-using F2 = uint64_t;
-__device__ __forceinline__ F2 f2(float lo, float hi) {
-  F2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unf2(F2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-  F2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ F2 fma2_rd(F2 a, F2 b, F2 c) {
-  F2 r;
-  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 
 // A lane's ended run, held in registers until the warp adds the held runs to
@@ -195,15 +161,6 @@ __device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int j
   if (__any_sync(0xffffffffu, held.on)) add_held<HC>(held, k);
   held = Held{cur, aN, aW, true};
   add_held<HC>(held, k);
-}
-
-// Per-pair scale sc16 = 2^(20 - e) with 2^e <= B < 2^(e+1): every |v| < B
-// maps to |q| < 2^21.
-__device__ __forceinline__ float fixed_scale(float B) {
-  if (!(B > 0.f) || !(B < 1e37f)) return 1.f;
-  const int e = static_cast<int>((__float_as_uint(B) >> 23) & 0xFFu) - 127;
-  const int ex = 20 - e + 127;
-  return __uint_as_float(static_cast<uint32_t>(min(max(ex, 1), 254)) << 23);
 }
 
 struct TeamSm {

@@ -65,3 +65,52 @@ def test_fp64_sums_are_those_of_the_definition(api, handle, lengths, step, bins,
     assert np.all(np.abs(w - ref["wsum"]) <= 1e-12 * ref["wsum"])
     wd = float(np.abs(cat.weight.astype(np.float64) * cat.delta).max())
     assert np.all(np.abs(n - ref["num"]) <= ref["count"] * 2.0 ** -44 * wd * wd + 1e-300)
+
+
+@pytest.mark.parametrize("lengths,step,bins,seed,kind", [
+    ((1, 2, 7, 8, 9), 1.0, (25, 25, 100.0, 100.0), 11, "z"),       # below one block of rows
+    ((31, 33, 65, 239, 240, 241), 0.6, (20, 40, 80.0, 60.0), 12, "z"),   # edges of groups and of a tile
+    ((500, 90), 0.25, (250, 4, 125.0, 16.0), 13, ""),              # many r_par bins, three tiles
+    ((40, 70, 110), 0.25, (1, 300, 60.0, 30.0), 14, "z"),          # one r_par bin, bands of many rows
+    ((96, 130, 64), 1.0, (25, 10, 100.0, 50.0), 15, "gap"),        # a gap: diagonals that leave the grid and return
+    ((64, 80), 1.0, (25, 10, 100.0, 50.0), 16, "huge"),            # weights whose products exceed the fixed point
+    ((64, 80), 1.0, (25, 10, 100.0, 50.0), 17, "nan"),             # a redshift that is not a number
+])
+def test_bin_means_forms(api, handle, lengths, step, bins, seed, kind):
+    """Counts are whole numbers, equal up to the oracle's edge allowance.  The means are FP32 sums of 8 terms and
+    integers beyond: 8 x 2^-24 relative to a sum of positive terms is the worst case (5e-7), next to the edge
+    allowance of one bin width (one range for the distances and redshifts) times twice the ambiguous weight."""
+    cat = _catalog(lengths, step, seed, patch=6e-3)
+    if kind == "gap":
+        cat.dist[int(cat.offsets[1]) // 2:int(cat.offsets[1])] += 60.0
+    if kind == "huge":
+        cat.weight *= np.float32(1e16)
+    z = np.exp(cat.loglam) / 1215.67 - 1.0
+    b = synth.Bins(*bins)
+    ref = oracle.xi.bin_means(cat, b, eps_edge=6e-5, z=z)
+    dc = api.DeviceCatalog.from_host(cat)
+    zt = torch.from_numpy(z).cuda()
+    if kind == "nan":
+        zt[3] = float("nan")
+    got = api.lya_xi_bin_means(handle, dc, b, z_pix=None if kind == "" else zt)
+    api.lya_sync_status(handle)
+    got = {k: v.cpu().numpy() for k, v in got.items()}
+    W = ref["wsum"]
+    on = W > 4.0 * ref["edge_w"]
+    assert on.sum() > 0
+    assert np.all(np.abs(got["count"] - ref["count"]) <= ref["edge_c"])
+    assert np.all(np.abs(got["wsum"] - W) <= 1e-6 * W + ref["edge_w"])
+    frac = 2.0 * ref["edge_w"][on] / (W[on] - ref["edge_w"][on])
+    spread = float(cat.dist.max() - cat.dist.min())
+    for key, width in (("rpar_mean", b.r_par_max / b.n_par), ("rperp_mean", b.r_perp_max / b.n_perp),
+                       ("dist_mean", spread), ("z_mean", float(z.max() - z.min()))):
+        if key not in got:
+            continue
+        err = np.abs(got[key][on] - ref[key][on])
+        if kind == "nan" and key == "z_mean":
+            bad = np.isnan(got[key][on])
+            assert bad.any()     # ... reaches the bins that hold it
+            err = err[~bad]
+            assert np.all(err <= 1e-6 * np.abs(ref[key][on][~bad]) + (frac * width)[~bad])
+            continue
+        assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width)
