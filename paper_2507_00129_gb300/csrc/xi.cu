@@ -32,7 +32,8 @@
 // reduction).  A team of two shares 12.7 KB of tables and the staged forest,
 // so 9-13 teams (18-26 warps) fit on an SM where 8 single warps did.
 // Measured (survey pass): 60,000 SDSS-like forests 624 -> 386 ms, 9,000
-// DESI-like forests 414 -> 244 ms.
+// DESI-like forests 414 -> 244 ms; 365 and 238 ms without the reductions of
+// guard runs at the ends of a chunk.
 // FP64 kernel (LYA_PREC_FP64): the same decomposition with FP64 distances,
 // separations, products and shared-memory sums, mirroring the oracle's
 // operation order: r = |d_i - d_j| * c, x = r * (1/D).
@@ -107,6 +108,17 @@ __device__ __forceinline__ void add_held(Held& h, const Walk& k) {
   h.on = false;
 }
 
+// Bin of a lane's pixel and the pixel {x, x} of b, as the key
+// (2^23 bits + row) * (n_par + 1) + (2^23 bits + column).
+template <bool WINDOW>
+__device__ __forceinline__ uint32_t step_key(F2 xx, const Walk& k, F2 ucus) {
+  const float2 r = unf2(fma2(xx, k.cpsp, ucus));
+  const float pf = fminf(__fadd_rd(fabsf(r.x), kMagic), k.pmax);
+  const float tf = fminf(__fadd_rd(r.y, kMagic), k.tmax);
+  const uint32_t key = __float_as_uint(tf) * k.stride + __float_as_uint(pf);
+  return (!WINDOW || (__float_as_uint(tf) - kMagicBits - k.twin) <= k.tspan) ? key : k.guard;
+}
+
 // One pixel pair of a run walk (see chunk_runs).  A run that ends here is
 // held in the lane's registers; the warp adds its held runs to the histogram
 // only when some lane that already holds one ends another.  On the DESI-like
@@ -115,11 +127,7 @@ __device__ __forceinline__ void add_held(Held& h, const Walk& k) {
 template <bool WINDOW, int HC>
 __device__ __forceinline__ void run_step(const ulonglong2& q, const Walk& k, F2 ucus, float wdi, float wi,
                                          uint32_t& cur, float& aN, float& aW, Held& held) {
-  const float2 r = unf2(fma2(q.x, k.cpsp, ucus));
-  const float pf = fminf(__fadd_rd(fabsf(r.x), kMagic), k.pmax);
-  const float tf = fminf(__fadd_rd(r.y, kMagic), k.tmax);
-  uint32_t key = __float_as_uint(tf) * k.stride + __float_as_uint(pf);
-  if (WINDOW) key = ((__float_as_uint(tf) - kMagicBits - k.twin) <= k.tspan) ? key : k.guard;
+  const uint32_t key = step_key<WINDOW>(q.x, k, ucus);
   const bool chg = key != cur;
   if (__any_sync(0xffffffffu, chg && held.on)) add_held<HC>(held, k);
   const float2 w = unf2(q.y);
@@ -145,7 +153,9 @@ template <bool WINDOW, int HC>
 __device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int jhi, const Walk& k, F2 ucus, float wdi,
                                            float wi) {
   constexpr int kUnroll = 8;
-  uint32_t cur = k.guard;
+  // the first run starts in the first pixel's bin: ending one of the guard
+  // bin there would send all lanes' reductions to one word
+  uint32_t cur = step_key<WINDOW>(buf[jlo].x, k, ucus);
   float aN = 0.f, aW = 0.f;
   Held held{k.guard, 0.f, 0.f, false};
   int j = jlo;
@@ -159,7 +169,8 @@ __device__ __forceinline__ void chunk_runs(const ulonglong2* buf, int jlo, int j
   for (; j < jhi; ++j) run_step<WINDOW, HC>(buf[j], k, ucus, wdi, wi, cur, aN, aW, held);
   // the held runs, then the last run of every lane
   if (__any_sync(0xffffffffu, held.on)) add_held<HC>(held, k);
-  held = Held{cur, aN, aW, true};
+  // (not of the lanes that have left the grid: their key's column is the guard's)
+  held = Held{cur, aN, aW, (cur - (k.guard - (k.stride - 1u))) % k.stride != k.stride - 1u};
   add_held<HC>(held, k);
 }
 
@@ -443,7 +454,7 @@ struct Run64 {
   Sum64 s;                   // the current run
   Sum64 held;                // an ended run, until the lane ends another
   uint32_t cur, key;         // their bins
-  bool on;                   // a run is held
+  bool in, on;               // the current bin lies in the grid; a run is held
 };
 
 // v / 2^shift to nearest, ties to even (rounding ties up would add a bias
@@ -551,7 +562,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
           }
         }
         unsigned todo = __ballot_sync(0xffffffffu, work);
-        Run64 r{{0, 0, 0, 0}, {0, 0, 0, 0}, k.guard, k.guard, false};
+        Run64 r{{0, 0, 0, 0}, {0, 0, 0, 0}, k.guard, k.guard, false, false};
         for (; todo; todo &= todo - 1u) {
           const int i0 = 8 * (__ffs(todo) - 1);
           const float* px = bx + i0 + o + lane;
@@ -583,13 +594,18 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
             }
             const bool chg = key != r.cur;
             if (__any_sync(0xffffffffu, chg)) {
-              if (__any_sync(0xffffffffu, chg && r.on)) add_run64(r, k);
+              // (runs off the grid are dropped: all lanes' would go to a few words)
+              if (__any_sync(0xffffffffu, chg && r.on && r.in)) add_run64(r, k);
               if (chg) {
-                r.held = r.s;
-                r.key = r.cur;
-                r.on = true;
+                if (r.in) {
+                  r.held = r.s;
+                  r.key = r.cur;
+                  r.on = true;
+                }
                 r.s = Sum64{0, 0, 0, 0};
                 r.cur = key;
+                const uint32_t q = key - C;   // row * (n_par + 1) + column
+                r.in = q < static_cast<uint32_t>(K) * k.stride && q % k.stride != static_cast<uint32_t>(npar);
               }
               __syncwarp();
             }
@@ -605,7 +621,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
         add_run64(r, k);
         r.held = r.s;
         r.key = r.cur;
-        r.on = true;
+        r.on = r.in;
         add_run64(r, k);
       }
       // integer sums -> FP64 bin sums
