@@ -1317,7 +1317,7 @@ int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max
   unsigned flags = 0;
   if ((st = read_flags(h, s, &flags))) return st;
   if ((st = flags_to_status(h, flags))) return st;
-  if (xi1d_smem_bytes(n_bins, ml) > h->dev.smem_optin)
+  if (xi1d_limit_bytes(n_bins, ml) > h->dev.smem_optin)
     return fail(h, LYA_ERR_TOO_LARGE, "1D correlation: 16 bytes per bin + 24 per pixel of the longest forest above shared memory");
   CK(cudaMemsetAsync(num, 0, static_cast<size_t>(n_bins) * 8, s), "zero num");
   CK(cudaMemsetAsync(wsum, 0, static_cast<size_t>(n_bins) * 8, s), "zero wsum");
@@ -1332,7 +1332,7 @@ int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max
   A.wsum = wsum;
   A.max_len = ml;
   stage_begin(h, 0, s);
-  CK(launch_xi1d(A, static_cast<const Pix*>(h->pixbuf), h->dev, s), "1D correlation kernel");
+  CK(launch_xi1d(A, static_cast<const Pix*>(h->pixbuf), h->d_counter, h->dev, s), "1D correlation kernel");
   stage_end(h, 0, s);
   if (xi) CK(launch_finalize(num, wsum, xi, n_bins, s), "finalize");
   return LYA_OK;

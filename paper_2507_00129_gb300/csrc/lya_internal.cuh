@@ -312,8 +312,8 @@ struct X1Args {
   double* wsum;
   int max_len;
 };
-int xi1d_smem_bytes(int n_bins, int max_len);
-cudaError_t launch_xi1d(const X1Args& a, const Pix* pix, const DevInfo& dev, cudaStream_t s);
+int xi1d_limit_bytes(int n_bins, int max_len);
+cudaError_t launch_xi1d(const X1Args& a, const Pix* pix, unsigned long long* counter, const DevInfo& dev, cudaStream_t s);
 
 // means.cu: per-bin weighted means of r_par, r_perp and the pair distance, and
 // pixel-pair counts, over the cached forest-pair list

@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <math.h>
 
+#include "exact.cuh"
 #include "fixed.cuh"
 
 namespace lya {
@@ -405,10 +406,7 @@ __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int 
 //  * bins: FP32 coordinates with a proven error bound; a pixel pair whose
 //    coordinate lies within the bound of a bin edge (about 1 step in 80 holds
 //    one) is binned by the definition in FP64, r = |d_i - d_j| * c, x = r * (1/D);
-//  * products and sums: per forest w and w delta become 55-bit integers
-//    V = round(v 2^s) = 2^28 H + L (H, L signed, at most 2^26 and 2^27), and
-//    w_i w_j is 2^56 H_i H_j + 2^28 (H_i L_j + L_i H_j), three 32 x 32 + 64
-//    bit multiply-adds without rounding (L_i L_j lies below the last bit kept);
+//  * products and sums are exact integers (see exact.cuh);
 //  * the walk goes along the diagonals of the pixel-pair matrix: lane l takes
 //    the pairs (i, i + o + l), whose separation changes slowly with i, so a run
 //    of pixel pairs in one bin is tens of pairs long on any grid.  A lane that
@@ -446,10 +444,6 @@ struct Walk64 {
   double cp64, sp64;
 };
 
-struct Sum64 {
-  long long nh, nl, wh, wl;  // sums of H H and of H L + L H, of N and of W
-};
-
 struct Run64 {
   Sum64 s;                   // the current run
   Sum64 held;                // an ended run, until the lane ends another
@@ -457,27 +451,15 @@ struct Run64 {
   bool in, on;               // the current bin lies in the grid; a run is held
 };
 
-// v / 2^shift to nearest, ties to even (rounding ties up would add a bias
-// of 1e-14 to N, whose runs nearly cancel)
-__device__ __forceinline__ long long round_shift(long long v, int shift) {
-  return (v + ((1ll << (shift - 1)) - 1) + ((v >> shift) & 1)) >> shift;
-}
-
 // Adds every lane's held run to its bin.
 __device__ __forceinline__ void add_run64(Run64& r, const Walk64& k) {
   if (r.on) {
-    const long long n = round_shift(r.held.nh + ((r.held.nl + (1ll << 27)) >> 28), k.shift);
-    const long long w = round_shift(r.held.wh + ((r.held.wl + (1ll << 27)) >> 28), k.shift);
+    const long long n = run_value(r.held.nh, r.held.nl, k.shift), w = run_value(r.held.wh, r.held.wl, k.shift);
     asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(k.base + (r.key << 4)),
                  "l"(n), "l"(w));
   }
   r.on = false;
   __syncwarp();
-}
-
-// 2^e
-__device__ __forceinline__ double pow2(int e) {
-  return (e < -1022 || e > 1023) ? scalbn(1.0, e) : __longlong_as_double(static_cast<long long>(e + 1023) << 52);
 }
 
 // Bin rows [t0, t0 + K) of forest pair (a, b) into the FP64 sums; WINDOW
@@ -610,12 +592,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
               __syncwarp();
             }
             const int4 vi = av[i0 + q], vj = pv[q];
-            r.s.nh += static_cast<long long>(vi.x) * vj.x;
-            r.s.nl += static_cast<long long>(vi.x) * vj.y;
-            r.s.nl += static_cast<long long>(vi.y) * vj.x;
-            r.s.wh += static_cast<long long>(vi.z) * vj.z;
-            r.s.wl += static_cast<long long>(vi.z) * vj.w;
-            r.s.wl += static_cast<long long>(vi.w) * vj.z;
+            add_products(r.s, vi, vj);
           }
         }
         add_run64(r, k);
@@ -697,13 +674,6 @@ __global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int tile, in
       }
     }
   }
-}
-
-// H, L of round(v 2^s), |v| 2^s < 2^54: value = 2^28 H + L, L in [-2^27, 2^27)
-__device__ __forceinline__ int2 split55(double v, double scale) {
-  const long long q = __double2ll_rn(v * scale);
-  const int lo = static_cast<int>(((q + (1ll << 27)) & ((1ll << 28) - 1)) - (1ll << 27));
-  return make_int2(static_cast<int>((q - lo) >> 28), lo);
 }
 
 // One warp per forest: distances, and w delta and w as integers on the

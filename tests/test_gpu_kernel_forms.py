@@ -114,3 +114,27 @@ def test_bin_means_forms(api, handle, lengths, step, bins, seed, kind):
             assert np.all(err <= 1e-6 * np.abs(ref[key][on][~bad]) + (frac * width)[~bad])
             continue
         assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width)
+
+
+@pytest.mark.parametrize("lengths,step,n_bins,r_max,seed", [
+    ((1, 2, 8, 9, 33, 34), 1.0, 20, 40.0, 21),           # below and above a block of rows and a group of lags
+    ((255, 257, 264, 300), 0.5, 50, 200.0, 22),          # edges of a batch of 256 rows
+    ((1200, 5), 0.25, 4096, 300.0, 23),                  # most bins, sums straight to the FP64 outputs
+    ((90, 70), 1.0, 513, 60.0, 24),                      # one more than the bins summed per warp
+    ((90, 70, 40), 0.5, 1, 30.0, 25),                    # one bin
+    ((96, 130, 64), 0.25, 25, 100.0, -26),               # separations on 1/16 bin
+    ((64, 64, 200), 4.0, 25, 100.0, -27),                # every separation exactly on a bin edge
+])
+def test_xi1d_forms(api, handle, lengths, step, n_bins, r_max, seed):
+    """Bins are the definition's, sums exact up to the tolerance of test_fp64_sums_are_those_of_the_definition."""
+    cat = _catalog(lengths, step, seed)
+    ref = oracle.xi1d.xi1d_sums(cat, n_bins, r_max)
+    num, wsum, xi = api.lya_xi1d(handle, api.DeviceCatalog.from_host(cat), n_bins, r_max)
+    api.lya_sync_status(handle)
+    n, w = num.cpu().numpy(), wsum.cpu().numpy()
+    assert (ref["wsum"] > 0).any()
+    assert np.all((w > 0) == (ref["wsum"] > 0))
+    assert np.all(np.abs(w - ref["wsum"]) <= 1e-12 * ref["wsum"])
+    wd = float(np.abs(cat.weight.astype(np.float64) * cat.delta).max())
+    # pixel pairs of a bin <= W, the weights being at least 1
+    assert np.all(np.abs(n - ref["num"]) <= ref["wsum"] * 2.0 ** -44 * wd * wd + 1e-300)
