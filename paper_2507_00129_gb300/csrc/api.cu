@@ -724,7 +724,7 @@ int run_dmat_cats(lya_handle* h, const lya_catalog* cats, int n, const lya_bins*
   stage_begin(h, 1, s);
   CK(run_dmat(A, h->dev, &h->scratch2, &h->scratch2_cap, s), "dmat");
   stage_end(h, 1, s);
-  CK(launch_dm_finalize(G, wdm, dmat, wsum_dm, nb, n, s), "dmat finalize");
+  CK(launch_dm_finalize(G, wdm, dmat, wsum_dm, bins->n_par, bins->n_perp, n, s), "dmat finalize");
   return LYA_OK;
 }
 
@@ -1297,7 +1297,7 @@ int lya_xdmat(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, con
   stage_begin(h, 1, s);
   CK(launch_xdm(A, h->dev, s), "cross distortion-matrix kernel");
   stage_end(h, 1, s);
-  CK(launch_dm_finalize(G, wdm, dmat, wsum_dm, nb, 1, s), "finalize");
+  CK(launch_dm_finalize(G, wdm, dmat, wsum_dm, bins->n_par, bins->n_perp, 1, s), "finalize");
   return LYA_OK;
 }
 

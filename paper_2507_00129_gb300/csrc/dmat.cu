@@ -136,7 +136,7 @@ constexpr int kCB2 = 32;
 
 // Shared-memory layout of one block (offsets in bytes)
 struct Lay {
-  int U, T4, Va, Vb, mark, inv, S, ucs, pixa, pixb, tv, cf, gbin, misc, end;
+  int U, T4, Va, Vb, mark, inv, S, ucs, pixa, pixb, tv, cf, misc, end;
 };
 
 __host__ __device__ inline int scap_for(int L, int npar, int K, int cb) {
@@ -149,12 +149,13 @@ __host__ __device__ inline int scap_for(int L, int npar, int K, int cb) {
 }
 
 // Row stride of the batch vectors V[cb][.]: at least the support capacity
-// rounded up to 16 (the tensor-core tiles read 16-row blocks) and 8 modulo 32,
-// so that the fragment loads of the tensor-core tiles (rows t and t + 4 of a
-// k step, 8 consecutive support entries) hit 32 different banks.
+// rounded up to 16 (the tensor-core tiles read 16-row blocks), a multiple of 4
+// (the FP32 tiles read float4) and 4 modulo 32: the histograms of neighbouring
+// vectors, one per lane, fall on 8 x 4 banks (with 8 modulo 32 on 4 x 8: D on
+// 12,000 SDSS-like forests 106.1 -> 101.9 ms).
 __host__ __device__ inline int ldv_for(int scap) {
   int v = (scap + 15) & ~15;
-  while ((v & 31) != 8) v += 8;
+  while ((v & 31) != 4) v += 4;
   return v;
 }
 
@@ -175,7 +176,6 @@ __host__ __device__ inline Lay layout(int L, int scap, int max_len, bool global_
   y.pixb = o; o += al(max_len * 16);
   y.tv = o; o += al(max_len * 8);
   y.cf = o; o += al(max_len * 16);
-  y.gbin = o; o += al(L * 4);
   y.misc = o; o += 64;
   y.end = o;
   return y;
@@ -306,9 +306,8 @@ __device__ void dm_tiles_tc(const float* Va, const float* Vb, int ldv, int ns, i
 // order) cover each unordered pair of its bins once; the symmetric entry goes
 // to (min, max) of the two local bins.
 template <bool GLOBAL>
-__device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t* S, const int32_t* gbin,
-                                              int ns, int L, int nbins, int rblk, int cblk,
-                                              const float (&acc)[4][4]) {
+__device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t* S, int g0, int ns, int L, int nbins,
+                                              int rblk, int cblk, const float (&acc)[4][4]) {
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int r = 4 * rblk + u;
@@ -323,8 +322,7 @@ __device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t
         const int lo = min(lr, lc), hi = max(lr, lc);
         U[tri_rowbase(lo, L) + hi] -= acc[u][v];
       } else {
-        const int Ar = gbin[lr], Ac = gbin[lc];
-        red_add_f64_global(G + static_cast<int64_t>(min(Ar, Ac)) * nbins + max(Ar, Ac),
+        red_add_f64_global(G + static_cast<int64_t>(g0 + min(lr, lc)) * nbins + g0 + max(lr, lc),
                            -static_cast<double>(acc[u][v]));
       }
     }
@@ -367,7 +365,7 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
   float2* ucs = reinterpret_cast<float2*>(sm + y.ucs);
   Pix* pxa = reinterpret_cast<Pix*>(sm + y.pixa);
   Pix* pxb = reinterpret_cast<Pix*>(sm + y.pixb);
-  const int32_t* gbin = reinterpret_cast<const int32_t*>(sm + y.gbin);
+  const int g0 = t0 * A.n_par;   // accumulator row of local bin 0 (see dm_finalize_kernel)
   int* misc = reinterpret_cast<int*>(sm + y.misc);   // [0] = |S|
 
   const Pix* ga = A.pix + A.F.off[a];
@@ -535,7 +533,7 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
             float acc[4][4];
             int rblk, cblk;
             dm_tile(Va, Vb, ldv, q, 0, cbn, acc, &rblk, &cblk);
-            dm_tile_store<GLOBAL>(G, U, S, gbin, ns, L, nbins, rblk, cblk, acc);
+            dm_tile_store<GLOBAL>(G, U, S, g0, ns, L, nbins, rblk, cblk, acc);
           }
         }
       }
@@ -569,38 +567,24 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
       float v = f1 * tc.x + fy * tc.z + fx * tc.y + fxy * tc.w;
       const float v2 = f1 * tc2.x + fy * tc2.z + fx * tc2.y + fxy * tc2.w;
       if (c == r) v += tr.x;
+      // consecutive lanes add to consecutive entries of the accumulator's row
+      double* row = G + static_cast<int64_t>(g0 + r) * nbins + g0;
       if (!GLOBAL) {
-        // (r, c), (r, c2) owned by this lane: flush and clear
-        const int Ar = gbin[r];
-        const float t1 = U[rb + c] + v;
-        if (t1 != 0.f) {
-          const int Ac = gbin[c];
-          red_add_f64_global(G + static_cast<int64_t>(min(Ar, Ac)) * nbins + max(Ar, Ac), static_cast<double>(t1));
-          U[rb + c] = 0.f;
-        }
+        // (r, c), (r, c2) owned by this lane: flush and clear (also where the sum cancels to 0)
+        const float u1 = U[rb + c];
+        if (u1 + v != 0.f) red_add_f64_global(row + c, static_cast<double>(u1 + v));
+        if (u1 != 0.f) U[rb + c] = 0.f;
         if (c2 < L) {
-          const float t2 = U[rb + c2] + v2;
-          if (t2 != 0.f) {
-            const int Ac = gbin[c2];
-            red_add_f64_global(G + static_cast<int64_t>(min(Ar, Ac)) * nbins + max(Ar, Ac), static_cast<double>(t2));
-            U[rb + c2] = 0.f;
-          }
+          const float u2 = U[rb + c2];
+          if (u2 + v2 != 0.f) red_add_f64_global(row + c2, static_cast<double>(u2 + v2));
+          if (u2 != 0.f) U[rb + c2] = 0.f;
         }
       } else {
-        const int Ar = gbin[r];
-        if (v != 0.f) {
-          const int Ac = gbin[c];
-          red_add_f64_global(G + static_cast<int64_t>(min(Ar, Ac)) * nbins + max(Ar, Ac),
-                             static_cast<double>(v));
-        }
-        if (v2 != 0.f) {
-          const int Ac = gbin[c2];
-          red_add_f64_global(G + static_cast<int64_t>(min(Ar, Ac)) * nbins + max(Ar, Ac),
-                             static_cast<double>(v2));
-        }
+        if (v != 0.f) red_add_f64_global(row + c, static_cast<double>(v));
+        if (v2 != 0.f) red_add_f64_global(row + c2, static_cast<double>(v2));
       }
     }
-    if (lane == 0) red_add_f64_global(wdm + gbin[r], static_cast<double>(tr.x));
+    if (lane == 0) red_add_f64_global(wdm + g0 + r, static_cast<double>(tr.x));
   }
   __syncthreads();
   for (int k = tid; k < L; k += blockDim.x) T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -622,7 +606,6 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
   float* U = reinterpret_cast<float*>(sm + y.U);
   float4* T4 = reinterpret_cast<float4*>(sm + y.T4);
   unsigned char* mark = sm + y.mark;
-  int32_t* gbin = reinterpret_cast<int32_t*>(sm + y.gbin);
   // clear all accumulators once
   if (!GLOBAL) {
     const int nt = Lalloc * (Lalloc + 1) / 2;
@@ -654,11 +637,6 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
     double* G = A.G + static_cast<int64_t>(mock) * nbins * nbins;
     double* wdm = A.wdm + static_cast<int64_t>(mock) * nbins;
     const int L = K * A.n_par;
-    for (int k = tid; k < L; k += blockDim.x) {
-      const int tt = k / A.n_par, p = k - tt * A.n_par;
-      gbin[k] = p * A.n_perp + t0 + tt;
-    }
-    __syncthreads();
     for (int q = 0; q < cnt; ++q) {
       const int pi = GLOBAL ? wide[item] : order[first + q];
       dm_pair<GLOBAL, CB>(A, G, wdm, pi, t0, K, L, scap, sm, y);
@@ -666,18 +644,35 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
   }
 }
 
-__global__ void dm_finalize_kernel(const double* G, const double* wdm, double* D, double* wout, int nb,
-                                   int n_mocks) {
-  const int64_t nb2 = static_cast<int64_t>(nb) * nb;
-  const int64_t n = nb2 * n_mocks;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t m = k / nb2, e = k - m * nb2;
-    const int r = static_cast<int>(e / nb), c = static_cast<int>(e - static_cast<int64_t>(r) * nb);
-    const int lo = min(r, c), hi = max(r, c);
-    const double w = wdm[m * nb + r];
-    D[k] = (w != 0.0) ? G[m * nb2 + static_cast<int64_t>(lo) * nb + hi] / w : 0.0;
-    if (wout && c == 0) wout[m * nb + r] = w;
+// D and W from the accumulators, one block per (catalogue, row of D).  The
+// accumulators number bin (p, t) as t n_par + p, so that a pair's local bins,
+// and with them the 32 lanes of an atomic, are consecutive (L2 takes atomics a
+// 32-byte sector at a time); the outputs number it p n_perp + t.
+template <bool STAGED>
+__global__ void __launch_bounds__(256) dm_finalize_kernel(const double* G, const double* wdm, double* D, double* wout,
+                                                          int n_par, int n_perp, int64_t rows) {
+  extern __shared__ double frow[];   // the row in the accumulators' numbering
+  const int nb = n_par * n_perp;
+  for (int64_t q = blockIdx.x; q < rows; q += gridDim.x) {
+    const int64_t m = q / nb;
+    const int r = static_cast<int>(q - m * nb);
+    const int rp = (r % n_perp) * n_par + r / n_perp;
+    const double w = wdm[m * nb + rp];
+    const double* Gm = G + m * nb * nb;
+    auto at = [&](int c) {
+      return (c >= rp) ? Gm[static_cast<int64_t>(rp) * nb + c] : Gm[static_cast<int64_t>(c) * nb + rp];
+    };
+    if (STAGED && w != 0.0) {
+      for (int c = threadIdx.x; c < nb; c += blockDim.x) frow[c] = at(c);
+      __syncthreads();
+    }
+    double* out = D + q * nb;
+    for (int c = threadIdx.x; c < nb; c += blockDim.x) {
+      const int cp = (c % n_perp) * n_par + c / n_perp;
+      out[c] = (w != 0.0) ? (STAGED ? frow[cp] : at(cp)) / w : 0.0;
+    }
+    if (wout && threadIdx.x == 0) wout[q] = w;
+    __syncthreads();
   }
 }
 
@@ -941,11 +936,15 @@ cudaError_t run_dmat(const DmArgs& a, const DevInfo& dev, void** scratch, size_t
   return cudaSuccess;
 }
 
-cudaError_t launch_dm_finalize(const double* G, const double* wdm, double* D, double* wdm_out, int nb,
+cudaError_t launch_dm_finalize(const double* G, const double* wdm, double* D, double* wdm_out, int n_par, int n_perp,
                                int n_mocks, cudaStream_t s) {
-  const int64_t n = static_cast<int64_t>(nb) * nb * n_mocks;
-  if (n == 0) return cudaSuccess;
-  LYA_COUNT(1), dm_finalize_kernel<<<grid_for(n, 256), 256, 0, s>>>(G, wdm, D, wdm_out, nb, n_mocks);
+  const int64_t rows = static_cast<int64_t>(n_par) * n_perp * n_mocks;
+  if (rows == 0) return cudaSuccess;
+  const int smem = n_par * n_perp * 8;   // staged up to 48 KB a row (6,144 bins)
+  if (smem <= 48 * 1024)
+    LYA_COUNT(1), dm_finalize_kernel<true><<<grid_for(rows, 1), 256, smem, s>>>(G, wdm, D, wdm_out, n_par, n_perp, rows);
+  else
+    LYA_COUNT(1), dm_finalize_kernel<false><<<grid_for(rows, 1), 256, 0, s>>>(G, wdm, D, wdm_out, n_par, n_perp, rows);
   return cudaGetLastError();
 }
 

@@ -196,7 +196,7 @@ struct DmArgs {
   int eta_mean_slope;
   double p_subsample;
   uint64_t seed;
-  double* G;        // [n_mocks][nb*nb] upper-triangle accumulators (A <= B)
+  double* G;        // [n_mocks][nb*nb] upper-triangle accumulators (A <= B, bin (p, t) at t n_par + p)
   double* wdm;      // [n_mocks][nb]
   int max_len;
   int n_mocks;      // catalogues in the batch (forest f belongs to F.mock[f])
@@ -205,8 +205,9 @@ struct DmArgs {
 };
 cudaError_t run_dmat(const DmArgs& a, const DevInfo& dev, void** scratch, size_t* scratch_cap,
                      cudaStream_t s);
-cudaError_t launch_dm_finalize(const double* G, const double* wdm, double* D, double* wdm_out,
-                               int nb, int n_mocks, cudaStream_t s);
+// G and wdm number bin (p, t) as t n_par + p, the outputs as p n_perp + t
+cudaError_t launch_dm_finalize(const double* G, const double* wdm, double* D, double* wdm_out, int n_par, int n_perp,
+                               int n_mocks, cudaStream_t s);
 // work counts of the closed form over the kept pairs (single catalogue)
 struct DmWork {
   unsigned long long pairs;   // kept forest pairs with an in-grid band
@@ -287,7 +288,7 @@ struct XcfArgs {
   int eta_mean_slope;    // distortion matrix
   double p_subsample;
   uint64_t seed;
-  double* G;             // [nb*nb] upper triangle (A <= B) of D~
+  double* G;             // [nb*nb] upper triangle (A <= B, bin (p, t) at t n_par + p) of D~
   double* wdm;           // [nb]
   int max_len;
 };

@@ -22,11 +22,8 @@
 //
 // Distortion matrix.  With eta = I - 1 u^T - x v^T the pair (a, q) adds
 // w_q (diag(alpha) - alpha alpha^T / W_a - beta beta^T / S_a) on the bins its
-// window touches, alpha[B] = sum_{k in B} w_k, beta[B] = sum_{k in B} w_k x_k.
-// One warp per kept pair: the same segmented scan yields (bin, alpha, beta)
-// per run, kept as the pair's run list in shared memory; the warp adds the
-// upper triangle (bins ascend along the list) to D~ with FP64 global
-// reductions; D = D~ / W_A row by row.
+// window touches, alpha[B] = sum_{k in B} w_k, beta[B] = sum_{k in B} w_k x_k:
+// xdm_kernel; D = D~ / W_A row by row.
 //
 // 1D correlation.  Described at xi1d_kernel.
 #include <math.h>
@@ -267,81 +264,146 @@ __global__ void __launch_bounds__(kXCW * 32, 2) xcf_kernel(XcfArgs A, int cap) {
   }
 }
 
-// one warp per kept (forest, quasar) pair; per warp: run list of `cap` entries
+// Kept (forest, quasar) pairs, one per warp at a time.  A warp draws its pairs
+// 32 at a time and queues the kept ones; with 32 in the queue (or at the end)
+// each lane computes one pair's geometry, window and normalisers in FP64 (with
+// all lanes on one pair that cost as much as the pair's updates), and the warp
+// takes the pairs in turn: the runs of its window in shared memory, scaled to
+// al = alpha sqrt(w_q / W_a) and be = beta sqrt(w_q / S_a), then the upper
+// triangle -(al al^T + be be^T), two FP64 operations per entry, rows r and
+// L - 1 - r together so that the lanes stay full.
+// What bounds it: the FP64 pipe (two operations of 19 clocks per 32 entries)
+// and L2's atomics (entries of consecutive runs are consecutive in G).
+// Measured (60,000 x 90,000, 2% of the pairs): 31.0 ms with the geometry in all
+// lanes, five FP64 operations per entry and G numbered p n_perp + t; with the
+// rest of its call 12 ms as it is.
 __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
   extern __shared__ double dsh[];
+  __shared__ int2 s_queue[kXW][64];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   double* lal = dsh + static_cast<size_t>(wi) * 2 * cap;
   double* lbe = lal + cap;
   int* lA = reinterpret_cast<int*>(dsh + static_cast<size_t>(nwb) * 2 * cap) + static_cast<size_t>(wi) * cap;
+  int2* queue = s_queue[wi];
   const int nb = A.n_par * A.n_perp;
   const int all = A.p_subsample >= 1.0;
-  const uint64_t thr = static_cast<uint64_t>(A.p_subsample * 18446744073709551616.0);
+  const uint64_t thr = all ? 0 : static_cast<uint64_t>(A.p_subsample * 18446744073709551616.0);
   const int64_t nw = static_cast<int64_t>(gridDim.x) * nwb;
-  for (int64_t k = blockIdx.x * (int64_t)nwb + wi; k < A.n_pairs; k += nw) {
-    const int2 pr = A.pairs[k];
-    const int a = pr.x, q = pr.y;
-    if (a < 0 || q < 0) continue;
-    if (!all && !(splitmix64(A.seed ^ ((static_cast<uint64_t>(a) << 32) | static_cast<uint64_t>(q))) < thr)) continue;
-    const int n = A.F.len[a];
-    if (n <= 0 || A.Q.len[q] <= 0) continue;
-    const Pix* fp = A.pix + A.F.off[a];
-    const XGeo g = pair_geo(A, a, q, fp, n);
-    int L = 0, lastA = -1;
-    for (int base = g.i0; base < g.i1; base += 32) {
-      const int i = base + lane;
-      int bin = -1;
-      float ha = 0.f, la = 0.f, hb = 0.f, lb = 0.f;
-      if (i < g.i1) {
-        const Pix P = fp[i];
-        bin = pixel_bin(g, P.x, A.n_par, A.n_perp);
-        if (bin >= 0) {
-          ha = P.y;
-          hb = P.y * P.w;
-          lb = fmaf(P.y, P.w, -hb);
-        }
+  int queued = 0;   // pairs in the queue (uniform)
+  for (int64_t k0 = (blockIdx.x * static_cast<int64_t>(nwb) + wi) * 32;; k0 += nw * 32) {
+    const bool last = k0 >= A.n_pairs;
+    bool keep = false;
+    int2 pr = make_int2(-1, -1);
+    if (k0 + lane < A.n_pairs) {
+      pr = A.pairs[k0 + lane];
+      keep = pr.x >= 0 && pr.y >= 0 &&
+             (all || splitmix64(A.seed ^ ((static_cast<uint64_t>(pr.x) << 32) | static_cast<uint64_t>(pr.y))) < thr);
+      keep = keep && A.F.len[pr.x] > 0 && A.Q.len[pr.y] > 0;
+    }
+    const unsigned km = __ballot_sync(kFull, keep);
+    if (keep) queue[queued + __popc(km & ((1u << lane) - 1u))] = pr;
+    queued += __popc(km);
+    __syncwarp();
+    if (queued < 32 && !last) continue;
+    const int nq = min(queued, 32);
+    // one pair's geometry per lane
+    XGeo mine{0.f, 0.f, 0.f, 0.f, 0, 0};
+    double cw = 0.0, cs = 0.0;   // sqrt(w_q / W_a), sqrt(w_q / S_a) (0 where eta lacks the term)
+    if (lane < nq) {
+      pr = queue[lane];
+      mine = pair_geo(A, pr.x, pr.y, A.pix + A.F.off[pr.x], A.F.len[pr.x]);
+      const double wq = static_cast<double>(A.wq[pr.y]);
+      const double Wa = A.F.wsum[pr.x], Sa = A.F.ssum[pr.x];
+      if (A.eta_mean_slope && Wa > 0.0) {
+        cw = sqrt(wq / Wa);
+        cs = (Sa > 0.0) ? sqrt(wq / Sa) : 0.0;
       }
-      const bool tail = run_scan(bin, lane, ha, la, hb, lb);
-      const unsigned tm = __ballot_sync(kFull, tail);
-      if (tm) {
-        const int fbin = __shfl_sync(kFull, bin, __ffs(tm) - 1);
-        const int merged = (fbin == lastA) ? 1 : 0;   // run continued from the previous chunk
-        if (tail) {
-          const int r = __popc(tm & ((1u << lane) - 1u));
-          const double va = static_cast<double>(ha) + static_cast<double>(la);
-          const double vb = static_cast<double>(hb) + static_cast<double>(lb);
-          if (r == 0 && merged) {
-            lal[L - 1] += va;
-            lbe[L - 1] += vb;
-          } else {
-            const int slot = L + r - merged;
-            lA[slot] = bin;
-            lal[slot] = va;
-            lbe[slot] = vb;
+    }
+    for (int m = 0; m < nq; ++m) {
+      const int a = __shfl_sync(kFull, pr.x, m), q = __shfl_sync(kFull, pr.y, m);
+      XGeo g;
+      g.i0 = __shfl_sync(kFull, mine.i0, m);
+      g.i1 = __shfl_sync(kFull, mine.i1, m);
+      g.cP = __shfl_sync(kFull, mine.cP, m);
+      g.sP = __shfl_sync(kFull, mine.sP, m);
+      g.X0 = __shfl_sync(kFull, mine.X0, m);
+      g.Y0 = __shfl_sync(kFull, mine.Y0, m);
+      const double sw = __shfl_sync(kFull, cw, m), ss = __shfl_sync(kFull, cs, m);
+      const Pix* fp = A.pix + A.F.off[a];
+      int L = 0, lastA = -1;
+      for (int base = g.i0; base < g.i1; base += 32) {
+        const int i = base + lane;
+        int bin = -1;
+        float ha = 0.f, la = 0.f, hb = 0.f, lb = 0.f;
+        if (i < g.i1) {
+          const Pix P = fp[i];
+          bin = pixel_bin(g, P.x, A.n_par, A.n_perp);
+          if (bin >= 0) {
+            bin = (bin % A.n_perp) * A.n_par + bin / A.n_perp;   // as G numbers it; also ascending along the window
+            ha = P.y;
+            hb = P.y * P.w;
+            lb = fmaf(P.y, P.w, -hb);
           }
         }
-        lastA = __shfl_sync(kFull, bin, 31 - __clz(tm));
-        L += __popc(tm) - merged;
+        const bool tail = run_scan(bin, lane, ha, la, hb, lb);
+        const unsigned tm = __ballot_sync(kFull, tail);
+        if (tm) {
+          const int fbin = __shfl_sync(kFull, bin, __ffs(tm) - 1);
+          const int merged = (fbin == lastA) ? 1 : 0;   // run continued from the previous chunk
+          if (tail) {
+            const int r = __popc(tm & ((1u << lane) - 1u));
+            const double va = static_cast<double>(ha) + static_cast<double>(la);
+            const double vb = static_cast<double>(hb) + static_cast<double>(lb);
+            if (r == 0 && merged) {
+              lal[L - 1] += va;
+              lbe[L - 1] += vb;
+            } else {
+              const int slot = L + r - merged;
+              lA[slot] = bin;
+              lal[slot] = va;
+              lbe[slot] = vb;
+            }
+          }
+          lastA = __shfl_sync(kFull, bin, 31 - __clz(tm));
+          L += __popc(tm) - merged;
+        }
+        __syncwarp();
+      }
+      if (L == 0) continue;
+      const double wq = static_cast<double>(A.wq[q]);
+      for (int r = lane; r < L; r += 32) {
+        const double v = wq * lal[r];
+        const int64_t b = lA[r];
+        red_add_f64_global(A.wdm + b, v);
+        if (v != 0.0) red_add_f64_global(A.G + b * nb + b, v);
+        lal[r] *= sw;
+        lbe[r] *= ss;
+      }
+      __syncwarp();
+      if (sw != 0.0) {
+        for (int r = 0; 2 * r < L; ++r) {
+          // row r from its diagonal on, then row L - 1 - r (L + 1 entries together; once where they are the same row)
+          const int r2 = L - 1 - r;
+          const int n1 = L - r, n = (r2 > r) ? L + 1 : n1;
+          for (int e = lane; e < n; e += 32) {
+            const int row = (e < n1) ? r : r2;
+            const int c = (e < n1) ? r + e : r2 + (e - n1);
+            const double v = fma(lbe[row], lbe[c], lal[row] * lal[c]);
+            if (v != 0.0) red_add_f64_global(A.G + static_cast<int64_t>(lA[row]) * nb + lA[c], -v);
+          }
+        }
       }
       __syncwarp();
     }
-    if (L == 0) continue;
-    const double wq = static_cast<double>(A.wq[q]);
-    const double Wa = A.F.wsum[a], Sa = A.F.ssum[a];
-    const bool use_w = A.eta_mean_slope && Wa > 0.0;
-    const bool use_s = use_w && Sa > 0.0;
-    const double iW = use_w ? wq / Wa : 0.0, iS = use_s ? wq / Sa : 0.0;
-    for (int r = lane; r < L; r += 32) red_add_f64_global(A.wdm + lA[r], wq * lal[r]);
-    for (int r = 0; r < L; ++r) {
-      const double ar = lal[r], br = lbe[r];
-      double* row = A.G + static_cast<int64_t>(lA[r]) * nb;
-      for (int c = r + lane; c < L; c += 32) {
-        double v = -(ar * lal[c]) * iW - (br * lbe[c]) * iS;
-        if (c == r) v += wq * ar;
-        if (v != 0.0) red_add_f64_global(row + lA[c], v);
-      }
-    }
+    // the rest of the queue moves to its front
+    const int rest = queued - nq;
+    int2 moved = make_int2(-1, -1);
+    if (lane < rest) moved = queue[32 + lane];
     __syncwarp();
+    if (lane < rest) queue[lane] = moved;
+    queued = rest;
+    __syncwarp();
+    if (last && queued == 0) break;
   }
 }
 
