@@ -11,17 +11,26 @@
 // atomics, deterministic.  Each pixel pair is binned with the same FP32
 // operations, in the same operand roles, as the forward kernel (first forest
 // of the stored pair on the "i" side), so forward and backward agree on every
-// bin.  The table has a zero guard row and column; out-of-grid pairs are
-// clamped into them, so the inner loop has no branch.  Per-neighbour FP32
+// bin.  The table has a zero guard row and column; pairs that may lie off the
+// grid are clamped into them, and the range of a neighbour that lies in the
+// grid for all 32 pixels is walked without the clamps.  Per-neighbour FP32
 // partial sums are added into two-term (hi, lo) accumulators (Knuth's TwoSum).
+// What bounds it: the shared-memory pipe (77%: per visit one broadcast 16-byte
+// load and one gathered 8-byte table load).  Neighbours are staged 256 pixels
+// at a time, which leaves room for 32 warps per SM, and the separations and the
+// two sums are packed FP32 pairs.  Measured (gradient of a DESI-like catalogue
+// of 4,000 forests): 70.8 ms with whole neighbours staged (16 warps), 58 ms
+// with 256 pixels, 47 ms as it is; shorter segments (192: +1 ms, 128: +7 ms)
+// and larger blocks (12 or 16 warps: +0.5 to +3 ms) are slower.
 #include <algorithm>
 
-#include "lya_internal.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
 
 constexpr int kAdjWarps = 8;
+constexpr int kAdjSeg = 256;   // staged pixels of a neighbour per warp
 
 __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
   const float s = hi + x;
@@ -31,21 +40,52 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
   lo += e;
 }
 
-__device__ __forceinline__ int count_below_x(const float4* a, int n, float v) {
+// Number of staged pixels whose key (the 32-bit word at `word` of each 16-byte
+// record, ascending) lies strictly below v (v NaN -> n).
+__device__ __forceinline__ int staged_below(const ulonglong2* a, int word, int n, float v) {
   int lo = 0, hi = n;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (a[mid].x < v) lo = mid + 1; else hi = mid;
+    if (reinterpret_cast<const float*>(a + mid)[word] < v) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
-__device__ __forceinline__ int count_below_y(const float4* a, int n, float v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid].y < v) lo = mid + 1; else hi = mid;
+
+// Constants of a visit: the table's address, the pair's factors and the clamps
+// into the guard row and column.
+struct Visit {
+  F2 cpsp;             // (-c/D_par, s/D_perp)
+  float pmax, tmax;
+  uint32_t stride, tbase;
+};
+
+// One pixel pair: acc += (gamma (w delta), rho w).  The separations are
+// a * cpsp + b; CLAMP sends pairs off the grid to the zero guard.
+template <bool CLAMP>
+__device__ __forceinline__ void visit(F2 a, F2 b, F2 wdw, const Visit& k, F2& acc) {
+  const float2 r = unf2(fma2(a, k.cpsp, b));
+  float pf = __fadd_rd(fabsf(r.x), kMagic), tf = __fadd_rd(r.y, kMagic);
+  if (CLAMP) {
+    pf = fminf(pf, k.pmax);
+    tf = fminf(tf, k.tmax);
   }
-  return lo;
+  const uint32_t idx = __float_as_uint(pf) * k.stride + __float_as_uint(tf);
+  F2 gr;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(gr) : "r"(k.tbase + (idx << 3)));
+  acc = fma2(gr, wdw, acc);
+}
+
+// Pixels [j0, j1) of the staged neighbour.  FIRST: the lane is a first-forest
+// pixel (lane = its (uc, us), record = {x, x}); else a second-forest pixel
+// (lane = {x, x}, record = (uc, us)).
+template <bool FIRST, bool CLAMP>
+__device__ __forceinline__ void visits(const ulonglong2* buf, int j0, int j1, F2 lane, const Visit& k, F2& acc) {
+#pragma unroll 8
+  for (int j = j0; j < j1; ++j) {
+    const ulonglong2 q = buf[j];
+    if (FIRST) visit<CLAMP>(q.x, lane, q.y, k, acc);
+    else visit<CLAMP>(lane, q.x, q.y, k, acc);
+  }
 }
 
 __global__ void degree_kernel(const int2* pairs, int64_t n, int32_t* deg) {
@@ -134,7 +174,7 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_kernel(AdjArgs A, cons
   float2* table = reinterpret_cast<float2*>(sm);
   const int tab_bytes = ((tab_n * 8) + 15) & ~15;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float4* buf = reinterpret_cast<float4*>(sm + tab_bytes + wid * seg * 16);
+  ulonglong2* buf = reinterpret_cast<ulonglong2*>(sm + tab_bytes + wid * seg * 16);
   for (int k = threadIdx.x; k < tab_n; k += blockDim.x) {
     const int p = k / tstride, t = k - p * tstride;
     float2 e = make_float2(0.f, 0.f);
@@ -150,11 +190,12 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_kernel(AdjArgs A, cons
   }
   __syncthreads();
   // key (M + p) * tstride + (M + t), M = bits of 2^23, minus this offset is p * tstride + t
-  const uint32_t tbase = smem_addr(table) -
-                         8u * (kMagicBits * static_cast<uint32_t>(tstride) + kMagicBits);
+  Visit vk;
+  vk.stride = static_cast<uint32_t>(tstride);
+  vk.tbase = smem_addr(table) - 8u * (kMagicBits * vk.stride + kMagicBits);
   const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(nperp);
-  const float pmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(npar));
-  const float tmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(nperp));
+  vk.pmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(npar));
+  vk.tmax = __uint_as_float(kMagicBits + static_cast<uint32_t>(nperp));
   const int64_t n_items = *n_items_dev;
   for (;;) {
     unsigned long long it = 0;
@@ -166,7 +207,9 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_kernel(AdjArgs A, cons
     const int nf = A.F.len[f];
     const int i = item.y * 32 + lane;
     const bool valid = i < nf;
-    const Pix me = valid ? A.pix[A.F.off[f] + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    // (lanes past the end repeat the last pixel; nothing of them is stored)
+    const Pix me = (nf > 0) ? A.pix[A.F.off[f] + min(i, nf - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float me_first = __shfl_sync(0xffffffffu, me.x, 0), me_last = __shfl_sync(0xffffffffu, me.x, 31);
     const float ref_f = A.F.dref[f];
     float g1h = 0.f, g1l = 0.f, g2h = 0.f, g2l = 0.f;
     const int64_t e0 = adj_start[f], e1 = adj_start[f + 1];
@@ -184,73 +227,62 @@ __global__ void __launch_bounds__(kAdjWarps * 32) adjoint_kernel(AdjArgs A, cons
       // pair constants with the stored (first, second) roles
       const float ref1 = first ? ref_f : ref_o, ref2 = first ? ref_o : ref_f;
       const float Dc = (ref1 - ref2) * cp, Ds = (ref1 + ref2) * sp;
-      float a1 = 0.f, a2 = 0.f;
+      vk.cpsp = f2(-cp, sp);
+      const float eps = 1e-3f + 1e-5f * (fabsf(Dc) + (me_last + po[no - 1].x) * cp);
+      // no pixel pair of this chunk and this neighbour within r_par of each other
+      {
+        const float lo = first ? fmaf(me_first - po[no - 1].x, cp, Dc) : fmaf(po[0].x - me_last, cp, Dc);
+        const float hi = first ? fmaf(me_last - po[0].x, cp, Dc) : fmaf(po[no - 1].x - me_first, cp, Dc);
+        if (lo > fnpar + eps || hi < -fnpar - eps) continue;
+      }
+      const F2 mine = first ? f2(fmaf(me.x, cp, Dc), fmaf(me.x, sp, Ds)) : f2(me.x, me.x);
+      F2 acc = 0ull;
       for (int j0 = 0; j0 < no; j0 += seg) {
         const int segn = min(seg, no - j0);
         __syncwarp();
-        if (first) {
-          for (int k = lane; k < segn; k += 32) buf[k] = po[j0 + k];
-        } else {
-          for (int k = lane; k < segn; k += 32) {
-            const Pix q = po[j0 + k];
-            buf[k] = make_float4(fmaf(q.x, cp, Dc), fmaf(q.x, sp, Ds), q.y, q.z);
-          }
+        for (int k = lane; k < segn; k += 32) {
+          const Pix q = po[j0 + k];
+          buf[k] = make_ulonglong2(first ? f2(q.x, q.x) : f2(fmaf(q.x, cp, Dc), fmaf(q.x, sp, Ds)), f2(q.z, q.y));
         }
         __syncwarp();
+        // the range [j0, j3) that some lane can reach and the part [j1, j2) that lies in the grid for all of
+        // them: six searches, one per lane (the staged keys ascend)
+        float v = 0.f;
+        int word = 0;
         if (first) {
-          // lanes are first-forest pixels; loop over second-forest pixels (d~ in .x)
-          const float uc = fmaf(me.x, cp, Dc), us = fmaf(me.x, sp, Ds);
-          const int last = max(0, min(31, nf - 1 - item.y * 32));
-          const float ucf = __shfl_sync(0xffffffffu, uc, 0);
-          const float usf = __shfl_sync(0xffffffffu, us, 0);
-          const float ucl = __shfl_sync(0xffffffffu, uc, last);
-          float dlo = (ucf - fnpar) / cp, dhi = (ucl + fnpar) / cp;
-          if (sp > 0.f) dhi = fminf(dhi, (fnperp - usf) / sp);
-          dlo -= fabsf(dlo) * 1e-5f + 1e-2f;
-          dhi += fabsf(dhi) * 1e-5f + 1e-2f;
-          const int jlo = count_below_x(buf, segn, dlo), jhi = count_below_x(buf, segn, dhi);
-#pragma unroll 4
-          for (int j = jlo; j < jhi; ++j) {
-            const float4 q = buf[j];
-            const float rp = fabsf(fmaf(-q.x, cp, uc));
-            const float rt = fmaf(q.x, sp, us);
-            const float pf = fminf(__fadd_rd(rp, kMagic), pmax), tf = fminf(__fadd_rd(rt, kMagic), tmax);
-            const uint32_t idx = __float_as_uint(pf) * static_cast<uint32_t>(tstride) + __float_as_uint(tf);
-            float2 gr;
-            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(gr.x), "=f"(gr.y) : "r"(tbase + (idx << 3)));
-            a1 = fmaf(gr.x, q.z, a1);
-            a2 = fmaf(gr.y, q.y, a2);
-          }
+          // |uc - x cp| < npar and x sp + us < nperp, x the staged distance
+          const float uf = fmaf(me_first, cp, Dc), ul = fmaf(me_last, cp, Dc);
+          const float tf = (fnperp - fmaf(me_first, sp, Ds)) / sp, tl = (fnperp - fmaf(me_last, sp, Ds)) / sp;
+          const float far = (sp > 0.f) ? 1.f : 0.f;
+          v = lane == 0 ? (uf - fnpar) / cp : lane == 1 ? (ul + fnpar) / cp : lane == 2 ? (far != 0.f ? tf : INFINITY)
+            : lane == 3 ? (ul - fnpar) / cp : lane == 4 ? (uf + fnpar) / cp : (far != 0.f ? tl : INFINITY);
+          const float m = fabsf(v) * 1e-5f + 1e-2f;
+          v += (lane == 0 || lane >= 4) ? -m : m;
         } else {
-          // lanes are second-forest pixels; loop over first-forest pixels
-          // (buf: .x = uc_i, .y = us_i, .z = w_i, .w = (w d)_i)
-          const float dme = me.x;
-          const float dmin_l = __shfl_sync(0xffffffffu, dme, 0);
-          const int last = max(0, min(31, nf - 1 - item.y * 32));
-          const float dmax_l = __shfl_sync(0xffffffffu, dme, last);
-          // |uc_i - d cp| < npar  ->  uc_i in (dmin cp - npar, dmax cp + npar)
-          float ulo = fmaf(dmin_l, cp, -fnpar), uhi = fmaf(dmax_l, cp, fnpar);
-          ulo -= fabsf(ulo) * 1e-5f + 1e-3f;
-          uhi += fabsf(uhi) * 1e-5f + 1e-3f;
-          // rt = d sp + us_i < nperp  ->  us_i < nperp - dmin sp
-          float vhi = fmaf(-dmin_l, sp, fnperp);
-          vhi += fabsf(vhi) * 1e-5f + 1e-3f;
-          const int ilo = count_below_x(buf, segn, ulo);
-          const int ihi = min(count_below_x(buf, segn, uhi), count_below_y(buf, segn, vhi));
-#pragma unroll 4
-          for (int j = ilo; j < ihi; ++j) {
-            const float4 q = buf[j];
-            const float rp = fabsf(fmaf(-dme, cp, q.x));
-            const float rt = fmaf(dme, sp, q.y);
-            const float pf = fminf(__fadd_rd(rp, kMagic), pmax), tf = fminf(__fadd_rd(rt, kMagic), tmax);
-            const uint32_t idx = __float_as_uint(pf) * static_cast<uint32_t>(tstride) + __float_as_uint(tf);
-            float2 gr;
-            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(gr.x), "=f"(gr.y) : "r"(tbase + (idx << 3)));
-            a1 = fmaf(gr.x, q.w, a1);
-            a2 = fmaf(gr.y, q.z, a2);
-          }
+          // |uc - d cp| < npar and d sp + us < nperp, (uc, us) the staged pair
+          word = (lane == 2 || lane == 5) ? 1 : 0;
+          v = lane == 0 ? fmaf(me_first, cp, -fnpar) : lane == 1 ? fmaf(me_last, cp, fnpar)
+            : lane == 2 ? fmaf(-me_first, sp, fnperp) : lane == 3 ? fmaf(me_last, cp, -fnpar)
+            : lane == 4 ? fmaf(me_first, cp, fnpar) : fmaf(-me_last, sp, fnperp);
+          const float m = fabsf(v) * 1e-5f + 1e-3f;
+          v += (lane == 0 || lane >= 4) ? -m : m;
+        }
+        const int pos = (lane < 6) ? staged_below(buf, word, segn, v) : 0;
+        const int lo = __shfl_sync(0xffffffffu, pos, 0);
+        const int hi = min(__shfl_sync(0xffffffffu, pos, 1), __shfl_sync(0xffffffffu, pos, 2));
+        const int in0 = min(max(__shfl_sync(0xffffffffu, pos, 3), lo), max(hi, lo));
+        const int in1 = min(max(min(__shfl_sync(0xffffffffu, pos, 4), __shfl_sync(0xffffffffu, pos, 5)), in0), max(hi, lo));
+        if (first) {
+          visits<true, true>(buf, lo, in0, mine, vk, acc);
+          visits<true, false>(buf, in0, in1, mine, vk, acc);
+          visits<true, true>(buf, in1, hi, mine, vk, acc);
+        } else {
+          visits<false, true>(buf, lo, in0, mine, vk, acc);
+          visits<false, false>(buf, in0, in1, mine, vk, acc);
+          visits<false, true>(buf, in1, hi, mine, vk, acc);
         }
       }
+      const float a1 = unf2(acc).x, a2 = unf2(acc).y;
       two_sum_add(g1h, g1l, a1);
       two_sum_add(g2h, g2l, a2);
     }
@@ -316,7 +348,7 @@ cudaError_t run_adjoint(const AdjArgs& a, const DevInfo& dev, void** scratch, si
   LYA_TRY(cudaGetLastError());
   const int tab_n = (a.n_par + 1) * (a.n_perp + 1);
   int seg = ((std::max(a.max_len, 1) + 31) / 32) * 32;
-  if (seg > 1024) seg = 1024;
+  if (seg > kAdjSeg) seg = kAdjSeg;
   const int smem = ((tab_n * 8 + 15) & ~15) + kAdjWarps * seg * 16;
   if (smem > dev.smem_optin) return cudaErrorInvalidValue;
   LYA_TRY(set_max_dynamic_smem(reinterpret_cast<const void*>(adjoint_kernel), smem));
