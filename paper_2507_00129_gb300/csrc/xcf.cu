@@ -540,9 +540,17 @@ __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int
       hist[2 * q + 1] = 0ull;
     }
   }
-  for (int q = lane; q < acc_bins; q += 32) {
-    if (acc[q].x != 0.0) red_add_f64_global(A.num + q, acc[q].x);
-    if (acc[q].y != 0.0) red_add_f64_global(A.wsum + q, acc[q].y);
+  // the block's warps together, so that the FP64 sums in global memory take few terms
+  __syncthreads();
+  for (int q = threadIdx.x; q < acc_bins; q += blockDim.x) {
+    double n = 0.0, w = 0.0;
+    for (int m = 0; m < static_cast<int>(blockDim.x >> 5); ++m) {
+      const double2 t = reinterpret_cast<const double2*>(dyn + static_cast<size_t>(m) * per_warp + 16 * (A.n_bins + 1))[q];
+      n += t.x;
+      w += t.y;
+    }
+    if (n != 0.0) red_add_f64_global(A.num + q, n);
+    if (w != 0.0) red_add_f64_global(A.wsum + q, w);
   }
 }
 
