@@ -1232,6 +1232,8 @@ XcfArgs xcf_args(lya_handle* h, const lya_catalog* cat, const lya_quasars* q, co
   A.n_perp = b->n_perp;
   A.r_par_max = b->r_par_max;
   A.r_perp_max = b->r_perp_max;
+  A.inv_dpar = b->n_par / (2.0 * b->r_par_max);
+  A.inv_dperp = b->n_perp / b->r_perp_max;
   A.max_len = max_len;
   A.err = h->d_err;
   return A;
@@ -1248,13 +1250,13 @@ int lya_xcf(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, const
   if (st) return st;
   if (!num || !wsum) return fail(h, LYA_ERR_INVALID_ARG, "num and wsum are required");
   const int nb = bins->n_par * bins->n_perp;
-  if (xcf_smem_bytes(nb, 1) > h->dev.smem_optin)
+  if (xcf_limit_bytes(nb, 1) > h->dev.smem_optin)
     return fail(h, LYA_ERR_TOO_LARGE, "cross-correlation grid above the shared-memory histogram (16 bytes per bin)");
   if ((st = refuse_in_capture(h, "lya_xcf"))) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int ml = 0;
   if ((st = build_xpairs(h, cat, qso, forest_qso, bins, &ml, s))) return st;
-  if (xcf_smem_bytes(nb, ml) > h->dev.smem_optin)
+  if (xcf_limit_bytes(nb, ml) > h->dev.smem_optin)
     return fail(h, LYA_ERR_TOO_LARGE, "cross-correlation: 16 bytes per bin + 20 per pixel of the longest forest above shared memory");
   CK(cudaMemsetAsync(num, 0, static_cast<size_t>(nb) * 8, s), "zero num");
   CK(cudaMemsetAsync(wsum, 0, static_cast<size_t>(nb) * 8, s), "zero wsum");
@@ -1262,7 +1264,7 @@ int lya_xcf(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, const
   A.num = num;
   A.wsum = wsum;
   stage_begin(h, 0, s);
-  CK(launch_xcf(A, h->dev, s), "cross-correlation kernel");
+  CK(launch_xcf(A, h->d_counter, h->dev, s), "cross-correlation kernel");
   stage_end(h, 0, s);
   if (xi) CK(launch_finalize(num, wsum, xi, nb, s), "finalize");
   return LYA_OK;

@@ -282,6 +282,7 @@ struct XcfArgs {
   const float* wq;       // quasar weights
   int n_par, n_perp;     // r_par over [-r_par_max, r_par_max) in n_par bins
   double r_par_max, r_perp_max;
+  double inv_dpar, inv_dperp;   // 1 / bin widths
   double* num;           // [nb] cross-correlation sums
   double* wsum;
   unsigned* err;         // device flags
@@ -297,10 +298,10 @@ cudaError_t launch_qso_prep(const lya_quasars& q, Forests Q, unsigned* err, unsi
                             cudaStream_t s);
 // adds a fingerprint of own[0..n) (own-quasar indices; nothing for NULL) to *fp
 cudaError_t launch_own_hash(const int64_t* own, int64_t n, unsigned long long* fp, cudaStream_t s);
-cudaError_t launch_xcf(const XcfArgs& a, const DevInfo& dev, cudaStream_t s);
+cudaError_t launch_xcf(const XcfArgs& a, unsigned long long* counter, const DevInfo& dev, cudaStream_t s);
 cudaError_t launch_xdm(const XcfArgs& a, const DevInfo& dev, cudaStream_t s);
 // shared memory the kernels need: 0 when the grid or forest length is beyond their limits
-int xcf_smem_bytes(int nb, int max_len);
+int xcf_limit_bytes(int nb, int max_len);
 int xdm_warps(const DevInfo& dev, int max_len);
 struct X1Args {
   Forests F;

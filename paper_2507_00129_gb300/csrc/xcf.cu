@@ -8,17 +8,8 @@
 //     N_A = sum_{(i,q) in A} (w delta)_i w_q,   W_A = sum_{(i,q) in A} w_i w_q,
 // r_par = (d_i - d_q) cos(theta/2) signed and binned over [-r_par_max, r_par_max),
 // r_perp = (d_i + d_q) sin(theta/2).  The (forest, quasar) list is grouped by
-// forest; a block holds two teams of warps, each staging one forest's packed
-// pixels in shared memory.  A warp takes 32 of the forest's quasars, one
-// pair's geometry per lane (FP64, then the window of pixels that can land in
-// the grid by binary search in shared memory), and walks each window with all
-// lanes: a lane bins one pixel in FP32 as x = fma(x_i, c/D_par, X0),
-// y = fma(x_i, s/D_perp, Y0) (X0, Y0 formed in FP64).  Both grow with the pixel
-// distance, so the bin never decreases along the window and equal bins sit in
-// adjacent lanes: a segmented warp scan sums each run (error-free FP32
-// products w_q w_i and w_q (w delta)_i, TwoSum-compensated additions) and the
-// run's last lane adds it to the block's double-float histogram (bounded
-// compare-and-swap), flushed to the FP64 sums once per block.
+// forest: xcf_kernel.  A lane bins one pixel in FP32 as x = fma(x_i, c/D_par, X0),
+// y = fma(x_i, s/D_perp, Y0) (X0, Y0 formed in FP64).
 //
 // Distortion matrix.  With eta = I - 1 u^T - x v^T the pair (a, q) adds
 // w_q (diag(alpha) - alpha alpha^T / W_a - beta beta^T / S_a) on the bins its
@@ -37,7 +28,7 @@ namespace lya {
 namespace {
 
 constexpr int kXW = 8;    // warps per block (distortion matrix)
-constexpr int kXCW = 16;  // warps per block of the cross-correlation (two blocks per SM share the shared memory)
+constexpr int kXCW = 32;  // warps per block of the cross-correlation (one block per SM)
 constexpr int kPad1 = 48;   // sentinels past a forest (a block of 8 rows and 32 lags reaches 39 past it)
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -150,68 +141,137 @@ __device__ __forceinline__ int count_below_s(const float* a, int n, float v) {
   return lo;
 }
 
+// w S f as an unevaluated float pair (h, l): S = 2^27 H + L, |H| < 2^22, with f = 2^27 times the unit of S.
+__device__ __forceinline__ void run_times(long long S, float w, float f, float& h, float& l) {
+  const float H = static_cast<float>(static_cast<int>(S >> 27));
+  const float L = static_cast<float>(static_cast<int>(S) & 0x7FFFFFF) * 7.450580596923828125e-9f;   // 2^-27
+  const float p = H * w;
+  h = p * f;
+  l = (fmaf(H, w, -p) + L * w) * f;
+}
+
+// sqrt(q) to 2e-14 (one Newton step from FP32; exact FP64 roots and divisions
+// cost twenty FP64 operations each)
+__device__ __forceinline__ double root(double q) {
+  const float qf = static_cast<float>(q);
+  if (!(qf > 1e-30f)) return sqrt(q);
+  const double y = rsqrtf(qf);
+  return q * fma(0.5 * y, fma(-(q * y), y, 1.0), y);
+}
+
 // Window geometry of one (forest, quasar) pair against the forest's staged
-// packed distances xs[0..n): as pair_geo, searched in shared memory.
+// packed distances xs[0..n): as pair_geo, searched in shared memory, the
+// window's ends in FP32.
 __device__ __forceinline__ XGeo pair_geo_s(const XcfArgs& A, int a, int q, const float* xs, int n) {
   const double ax = A.F.ux[a], ay = A.F.uy[a], az = A.F.uz[a];
   const double qx = A.Q.ux[q], qy = A.Q.uy[q], qz = A.Q.uz[q];
   const double dx = ax - qx, dy = ay - qy, dz = az - qz;
   const double sx = ax + qx, sy = ay + qy, sz = az + qz;
-  const double s = 0.5 * sqrt(dx * dx + dy * dy + dz * dz);
-  const double c = 0.5 * sqrt(sx * sx + sy * sy + sz * sz);
-  const double inv_dpar = A.n_par / (2.0 * A.r_par_max), inv_dperp = A.n_perp / A.r_perp_max;
+  const double s = 0.5 * root(dx * dx + dy * dy + dz * dz);
+  const double c = 0.5 * root(sx * sx + sy * sy + sz * sz);
   const double dref = static_cast<double>(A.F.dref[a]), dq = A.Q.dmin[q];
+  const double cp = c * A.inv_dpar, sp = s * A.inv_dperp;
   XGeo g;
-  g.cP = static_cast<float>(c * inv_dpar);
-  g.sP = static_cast<float>(s * inv_dperp);
-  g.X0 = static_cast<float>((dref - dq) * c * inv_dpar + 0.5 * A.n_par);
-  g.Y0 = static_cast<float>((dref + dq) * s * inv_dperp);
-  const double xq = dq - dref;
-  const double half = A.r_par_max / c;
-  const double lo = xq - half - 0.5;
-  double hi = xq + half + 0.5;
-  if (s > 0.0) hi = fmin(hi, A.r_perp_max / s - dref - dq + 0.5);
-  g.i0 = count_below_s(xs, n, static_cast<float>(lo));
-  g.i1 = (hi > lo) ? count_below_s(xs, n, static_cast<float>(hi)) : g.i0;
+  g.cP = static_cast<float>(cp);
+  g.sP = static_cast<float>(sp);
+  g.X0 = static_cast<float>((dref - dq) * cp + 0.5 * A.n_par);
+  g.Y0 = static_cast<float>((dref + dq) * sp);
+  // 0 <= x cP + X0 < n_par and x sP + Y0 < n_perp, 0.5 Mpc/h wider (and 1e-5 of the terms)
+  const float fnpar = static_cast<float>(A.n_par), fnperp = static_cast<float>(A.n_perp);
+  const float lo = -g.X0 / g.cP;
+  float hi = (fnpar - g.X0) / g.cP;
+  if (g.sP > 0.f) hi = fminf(hi, (fnperp - g.Y0) / g.sP);
+  g.i0 = count_below_s(xs, n, lo - (0.5f + 1e-5f * fabsf(lo)));
+  g.i1 = count_below_s(xs, n, hi + (0.5f + 1e-5f * fabsf(hi)));
   if (g.i1 < g.i0) g.i1 = g.i0;
   return g;
 }
 
-// One block per forest (grid-stride): the forest's packed pixels are staged in
-// shared memory; warps take 32 of the forest's quasars at a time, one pair's
-// geometry per lane (FP64), then walk each pair's window together.  Per lane
-// the products w_q w_j and w_q (w delta)_j are exact FP32 pairs (TwoProduct),
-// a segmented TwoSum scan forms each run's sum, and the run's last lane adds
-// it to the block's double-float histogram: no FP64 arithmetic per pixel.
-__global__ void __launch_bounds__(kXCW * 32, 2) xcf_kernel(XcfArgs A, int cap) {
-  // [nb] (num hi, num lo, w hi, w lo) | per team: staged pixels [cap], xs [cap]
+// One block per SM: teams of warps, each staging one forest at a time (atomic
+// counter) with integer prefix sums of its packed w delta and w on the forest's
+// own power-of-two scales (43 bits: 2^-44 of the largest value per pixel, exact
+// sums).  Warps take 32 of the forest's quasars at a time, one pair's geometry
+// per lane, then walk each pair's window together: bins ascend along the
+// window, so a run of equal bins [j0, j] sits in adjacent lanes, and its last
+// lane adds w_q (P[j + 1] - P[j0]) as a float pair to the block's double-float
+// histogram (bounded compare-and-swap), flushed to FP64 once per block.  The
+// teams are as many and as small as shared memory allows (single warps up to
+// about 230 pixels at 5,000 bins): a team waits for its slowest warp at every
+// forest.
+// What bounds it: issue, about 100 warp instructions per 32 pixels.
+// Measured (60,000 x 90,000, 100 x 50 bins): 27.5 ms with a compensated
+// segmented scan over the lanes per 32 pixels and FP64 square roots, divisions
+// and window ends per pair; 18 ms with the prefix sums in teams of eight warps,
+// 16 ms as it is.
+__global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, int team_warps, unsigned long long* counter) {
+  // [nb] (num hi, num lo, w hi, w lo) | per team: inclusive prefix sums (w delta, w) [cap] | per team: distances [cap]
   extern __shared__ float4 xs4[];
   const int nb = A.n_par * A.n_perp;
   float4* hist = xs4;
   for (int k = threadIdx.x; k < nb; k += blockDim.x) hist[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
-  // two teams of kXCW / 2 warps, each on its own forests with its own staging
-  // buffer and barrier, so that one team's wait for its slowest warp leaves
-  // the other team issuing; both add to the block's histogram
-  constexpr int kTeamWarps = kXCW / 2;
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const int team = wi / kTeamWarps, tw = wi % kTeamWarps, tt = threadIdx.x % (kTeamWarps * 32);
-  Pix* sp = reinterpret_cast<Pix*>(xs4 + nb) + static_cast<size_t>(team) * cap;
-  float* xs = reinterpret_cast<float*>(reinterpret_cast<Pix*>(xs4 + nb) + 2 * static_cast<size_t>(cap)) +
+  const int teams = kXCW / team_warps;
+  const int team = wi / team_warps, tw = wi % team_warps, tt = threadIdx.x % (team_warps * 32);
+  longlong2* pre = reinterpret_cast<longlong2*>(xs4 + nb) + static_cast<size_t>(team) * cap;
+  float* xs = reinterpret_cast<float*>(reinterpret_cast<longlong2*>(xs4 + nb) + static_cast<size_t>(teams) * cap) +
               static_cast<size_t>(team) * cap;
-  for (int64_t f = 2 * static_cast<int64_t>(blockIdx.x) + team; f < A.F.n; f += 2 * static_cast<int64_t>(gridDim.x)) {
+  auto sync = [&]() {
+    if (team_warps == 1) __syncwarp();
+    else team_sync(1 + team, team_warps * 32);   // (at most 8 teams of more than one warp)
+  };
+  for (;;) {
+    sync();   // the team's previous forest's readers are done
+    long long f = 0;
+    if (tt == 0) f = static_cast<long long>(atomicAdd(counter, 1ull));
+    if (team_warps == 1) {
+      f = __shfl_sync(kFull, f, 0);
+    } else {   // by way of the staging buffer
+      if (tt == 0) pre[0].x = f;
+      sync();
+      f = pre[0].x;
+      sync();
+    }
+    if (f >= A.F.n) break;
     const int64_t q0 = A.qoff[f], q1 = A.qoff[f + 1];
     const int n = A.F.len[f];
     if (q1 <= q0 || n <= 0 || n > cap) continue;   // uniform over the team
-    team_sync(1 + team, kTeamWarps * 32);          // the team's previous forest's readers are done
     const Pix* fp = A.pix + A.F.off[f];
-    for (int k = tt; k < n; k += kTeamWarps * 32) {
-      const Pix P = fp[k];
-      sp[k] = P;
-      xs[k] = P.x;
+    const float mn = A.F.wdmax[f], mw = A.F.wmax[f];
+    // |value| 2^e < 2^43; values beyond FP32's range (their sums are infinite or NaN) are summed pixel by pixel
+    const bool plain = !(mn < 1e38f && mw < 1e38f);
+    const int en = (mn > 0.f && !plain) ? 42 - ilogbf(mn) : 0, ew = (mw > 0.f && !plain) ? 42 - ilogbf(mw) : 0;
+    for (int k = tt; k < n; k += team_warps * 32) xs[k] = fp[k].x;
+    if (tw == 0 && !plain) {
+      const double sn = pow2(en), sw = pow2(ew);
+      long long cn = 0, cw = 0;
+      for (int base = 0; base < n; base += 32) {
+        const int k = base + lane;
+        long long vn = 0, vw = 0;
+        if (k < n) {
+          const Pix P = fp[k];
+          vn = __double2ll_rn(static_cast<double>(P.z) * sn);
+          vw = __double2ll_rn(static_cast<double>(P.y) * sw);
+        }
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const long long on = __shfl_up_sync(kFull, vn, d), ow = __shfl_up_sync(kFull, vw, d);
+          if (lane >= d) {
+            vn += on;
+            vw += ow;
+          }
+        }
+        vn += cn;
+        vw += cw;
+        if (k < n) pre[k] = make_longlong2(vn, vw);
+        cn = __shfl_sync(kFull, vn, 31);
+        cw = __shfl_sync(kFull, vw, 31);
+      }
     }
-    team_sync(1 + team, kTeamWarps * 32);
-    for (int64_t qb = q0 + static_cast<int64_t>(tw) * 32; qb < q1; qb += kTeamWarps * 32) {
+    sync();
+    // a run's integer sum S = 2^27 H + L as floats: H 2^27 2^-e and L 2^-e, the factor 2^(27 - e) applied last
+    const float fn = ldexpf(1.f, 27 - en), fw = ldexpf(1.f, 27 - ew);
+    for (int64_t qb = q0 + static_cast<int64_t>(tw) * 32; qb < q1; qb += team_warps * 32) {
       XGeo g{0.f, 0.f, 0.f, 0.f, 0, 0};
       float wq = 0.f;
       const int64_t k = qb + lane;
@@ -234,22 +294,32 @@ __global__ void __launch_bounds__(kXCW * 32, 2) xcf_kernel(XcfArgs A, int cap) {
         const float wqt = __shfl_sync(kFull, wq, t);
         for (int base = i0; base < i1; base += 32) {
           const int j = base + lane;
-          int bin = -1;
-          float hn = 0.f, ln = 0.f, hw = 0.f, lw = 0.f;
-          if (j < i1) {
-            const Pix P = sp[j];
-            bin = pixel_bin(h, P.x, A.n_par, A.n_perp);
-            if (bin >= 0) {
-              hn = wqt * P.z;
-              ln = fmaf(wqt, P.z, -hn);
-              hw = wqt * P.y;
-              lw = fmaf(wqt, P.y, -hw);
+          const int bin = (j < i1) ? pixel_bin(h, xs[j], A.n_par, A.n_perp) : -1;
+          const int prev = __shfl_up_sync(kFull, bin, 1), nxt = __shfl_down_sync(kFull, bin, 1);
+          const unsigned heads = __ballot_sync(kFull, lane == 0 || prev != bin);
+          if (bin >= 0 && (lane == 31 || nxt != bin)) {
+            const int j0 = base + 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+            float hn, ln, hw, lw;
+            if (!plain) {
+              longlong2 S = pre[j];
+              if (j0 > 0) {
+                const longlong2 p = pre[j0 - 1];
+                S.x -= p.x;
+                S.y -= p.y;
+              }
+              run_times(S.x, wqt, fn, hn, ln);
+              run_times(S.y, wqt, fw, hw, lw);
+            } else {
+              hn = ln = hw = lw = 0.f;
+              for (int i = j0; i <= j; ++i) {
+                hn += wqt * fp[i].z;
+                hw += wqt * fp[i].y;
+              }
             }
-          }
-          if (run_scan(bin, lane, hn, ln, hw, lw)) {
             df_atomic_add(reinterpret_cast<float2*>(&hist[bin]), hn, ln, A.err);
             df_atomic_add(reinterpret_cast<float2*>(&hist[bin]) + 1, hw, lw, A.err);
           }
+          __syncwarp();
         }
       }
     }
@@ -563,7 +633,9 @@ int grid_for(int64_t n, int threads) {
 
 }  // namespace
 
-int xcf_smem_bytes(int nb, int max_len) {
+// The grids and forest lengths the entry point takes (16 bytes per bin and 40
+// per pixel of the longest forest within a block's shared memory).
+int xcf_limit_bytes(int nb, int max_len) {
   const int cap = std::max(max_len, 1);
   return 16 * nb + 2 * 20 * cap;
 }
@@ -594,18 +666,19 @@ cudaError_t launch_own_hash(const int64_t* own, int64_t n, unsigned long long* f
   return cudaGetLastError();
 }
 
-cudaError_t launch_xcf(const XcfArgs& a, const DevInfo& dev, cudaStream_t s) {
+cudaError_t launch_xcf(const XcfArgs& a, unsigned long long* counter, const DevInfo& dev, cudaStream_t s) {
   if (a.n_pairs == 0) return cudaSuccess;
-  const int cap = std::max(a.max_len, 1);
-  const int smem = xcf_smem_bytes(a.n_par * a.n_perp, cap);
+  const int cap = std::max(a.max_len, 1), nb = a.n_par * a.n_perp;
+  // the most teams whose staging fits beside the histogram (power of two; named barriers serve up to 8)
+  int team_warps = 1;
+  while (team_warps < kXCW && (team_warps == 2 || 16 * nb + (kXCW / team_warps) * 20 * cap > dev.smem_optin))
+    team_warps *= 2;
+  const int smem = 16 * nb + (kXCW / team_warps) * 20 * cap;
   cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xcf_kernel), smem);
+  if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xcf_kernel, kXCW * 32, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int blocks = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(dev.sms) * per_sm, (a.F.n + 1) / 2));
-  LYA_COUNT(1), xcf_kernel<<<blocks, kXCW * 32, smem, s>>>(a, cap);
+  const int blocks = static_cast<int>(std::min<int64_t>(dev.sms, a.F.n));
+  LYA_COUNT(1), xcf_kernel<<<blocks, kXCW * 32, smem, s>>>(a, cap, team_warps, counter);
   return cudaGetLastError();
 }
 

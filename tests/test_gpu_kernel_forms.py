@@ -170,3 +170,30 @@ def test_dmat_on_a_grid_of_unequal_sides(api, handle):
     edge = np.divide(ref["edge_d"] + np.abs(R) * E[:, None], den, out=np.zeros_like(R), where=den > 0)
     assert np.all(np.abs(D.cpu().numpy() - R) <= 1e-5 * np.abs(R).max(axis=1)[:, None] + edge + 1e-12)
     assert np.all(np.abs(w.cpu().numpy() - W) <= 1e-6 * W + E + 1e-9)
+
+
+@pytest.mark.parametrize("lengths,n_qso,bins,seed", [
+    ((1, 2, 31, 32, 33), 40, (10, 8, 60.0, 40.0), 31),          # edges of a warp's window step
+    ((300, 700, 90), 90, (100, 50, 200.0, 200.0), 32),          # teams of several warps
+    ((2600, 1500), 33, (64, 40, 200.0, 200.0), 33),             # one team per block
+    ((60, 50), 20, (1, 1, 100.0, 100.0), 34),                   # one bin: the longest runs
+])
+def test_xcf_forms(api, handle, lengths, n_qso, bins, seed):
+    """Pixels are rounded at 2^-44 of the forest's largest value and the sums are double-float, so off the bin edges
+    only the FP32 rounding of the packed w delta (2^-24 of each term) remains: 1e-6 of W and of the sum of |terms|,
+    next to the oracle's edge allowance."""
+    cat = _catalog(lengths, 0.3, seed, patch=8e-3)
+    rng = np.random.default_rng(seed)
+    q = synth.Quasars(ra=rng.uniform(0, 8e-3, n_qso), dec=rng.uniform(0, 8e-3, n_qso),
+                      dist=rng.uniform(2900.0, 3400.0, n_qso), weight=rng.uniform(0.5, 2.0, n_qso).astype(np.float32),
+                      z=np.full(n_qso, 2.5))
+    b = synth.Bins(*bins)
+    own = np.arange(cat.n_forests, dtype=np.int64)
+    ref = oracle.xcf.xcf_sums(cat, q, b, forest_qso=own, eps_edge=6e-5)
+    num, wsum, _ = api.lya_xcf(handle, api.DeviceCatalog.from_host(cat), api.DeviceQuasars.from_host(q), b, own)
+    api.lya_sync_status(handle)
+    n, w = num.cpu().numpy(), wsum.cpu().numpy()
+    assert ref["wsum"].sum() > 0
+    assert np.all(np.abs(w - ref["wsum"]) <= 1e-6 * ref["wsum"] + ref["edge_w"])
+    top = float(np.abs(cat.delta).max())
+    assert np.all(np.abs(n - ref["num"]) <= 1e-6 * top * ref["wsum"] + ref["edge_n"] + 1e-300)
