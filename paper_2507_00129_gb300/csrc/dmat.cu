@@ -570,14 +570,21 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
       // consecutive lanes add to consecutive entries of the accumulator's row
       double* row = G + static_cast<int64_t>(g0 + r) * nbins + g0;
       if (!GLOBAL) {
-        // (r, c), (r, c2) owned by this lane: flush and clear (also where the sum cancels to 0)
-        const float u1 = U[rb + c];
-        if (u1 + v != 0.f) red_add_f64_global(row + c, static_cast<double>(u1 + v));
-        if (u1 != 0.f) U[rb + c] = 0.f;
+        // (r, c), (r, c2) owned by this lane: flush and clear.  Where the sum is
+        // exactly 0 (u = -v, about one entry in 1e7) the rank-1 part u stays and
+        // goes out with the block's next pair that has the entry.  Clearing it too
+        // makes two calls agree to 1e-18, but moves D by 1e-7 to 1e-5 of its norm.
+        const float x = U[rb + c] + v;
+        if (x != 0.f) {
+          red_add_f64_global(row + c, static_cast<double>(x));
+          U[rb + c] = 0.f;
+        }
         if (c2 < L) {
-          const float u2 = U[rb + c2];
-          if (u2 + v2 != 0.f) red_add_f64_global(row + c2, static_cast<double>(u2 + v2));
-          if (u2 != 0.f) U[rb + c2] = 0.f;
+          const float x2 = U[rb + c2] + v2;
+          if (x2 != 0.f) {
+            red_add_f64_global(row + c2, static_cast<double>(x2));
+            U[rb + c2] = 0.f;
+          }
         }
       } else {
         if (v != 0.f) red_add_f64_global(row + c, static_cast<double>(v));
