@@ -21,15 +21,25 @@
 // to the FP64 accumulator G (entries A <= B) with FP64 atomics at the end of
 // the pair, so that the sum over pairs is FP64.  The rank-1 terms are applied a
 // batch of up to CB vectors (consecutive columns, then rows) at a time:
-//  (a1) every thread bins pixel pairs and marks the local bins the batch
-//       touches; (b) one warp compacts the marks into the batch's sorted union
+//  (a1) every thread bins pixel pairs of the batch's vectors and the other
+//       forest's pixels within their reach (dm_windows) and marks the local
+//       bins; (b) the marks are compacted into the batch's ascending union
 //       support S (|S| is a little above one vector's support, because
-//       neighbouring columns visit nearly the same bins);
+//       neighbouring columns visit nearly the same bins: 62 on average on
+//       SDSS-like forests, 35 on DESI-like ones);
 //  (a2) the batch's histograms are summed densely on S with shared atomics;
 //       column histograms also feed the T vectors;
-//  (d)  each thread owns a 4 x 4 tile of the S x S upper triangle and adds
+//  (d)  each thread owns a 2 x 4 tile of the S x S upper triangle and adds
 //       sum_v (a_v a_v^T + b_v b_v^T) over the batch in registers (FP32 FMA,
-//       float4 loads), then updates its 16 triangle entries -- no atomics.
+//       float4 loads), then updates its 8 triangle entries -- no atomics.
+// What bounds it: 8.4 batches a pair, each with four block-wide phases of 1,000
+// to 4,600 cycles; (d) takes 40% (4 x 4 tiles left three quarters of the
+// threads idle at |S| = 62, and 2 x 8 ones half), (a2) 17%, half of it the
+// shared atomics, the flush to G 12%.  D on 12,000 SDSS-like forests, 5% of the
+// pairs: windows, one division per lane, floors without conversions and four
+// phases instead of six a batch 101.9 -> 72 ms, tiles of 2 x 4 (2 x 8: 58.9) and
+// V cleared only where used -> 57.7 ms (384, 640, 768, 1024 threads: 61, 60,
+// 62, 63).
 // Pairs whose band is too wide for shared memory take the same code with the
 // triangle replaced by FP64 atomics into G.  Binning uses exactly the FP32
 // arithmetic of the xi kernel, so W^DM equals the xi weights of the kept
@@ -37,7 +47,7 @@
 #include <algorithm>
 #include <math.h>
 
-#include "lya_internal.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
@@ -136,8 +146,10 @@ constexpr int kCB2 = 32;
 
 // Shared-memory layout of one block (offsets in bytes)
 struct Lay {
-  int U, T4, Va, Vb, mark, inv, S, ucs, pixa, pixb, tv, cf, misc, end;
+  int U, T4, V, mark, inv, S, ucs, db, tv, cf, win, misc, end;
 };
+
+constexpr int kWin = 16;   // vectors per search window
 
 __host__ __device__ inline int scap_for(int L, int npar, int K, int cb) {
   // union-support capacity: at least one vector's support bound 2 (n_par + K) + 2,
@@ -148,16 +160,12 @@ __host__ __device__ inline int scap_for(int L, int npar, int K, int cb) {
   return (c + 3) & ~3;
 }
 
-// Row stride of the batch vectors V[cb][.]: at least the support capacity
-// rounded up to 16 (the tensor-core tiles read 16-row blocks), a multiple of 4
-// (the FP32 tiles read float4) and 4 modulo 32: the histograms of neighbouring
-// vectors, one per lane, fall on 8 x 4 banks (with 8 modulo 32 on 4 x 8: D on
-// 12,000 SDSS-like forests 106.1 -> 101.9 ms).
-__host__ __device__ inline int ldv_for(int scap) {
-  int v = (scap + 15) & ~15;
-  while ((v & 31) != 4) v += 4;
-  return v;
-}
+// Row stride, in (a, b) entries, of the batch vectors V[cb][.]: at least the
+// support capacity rounded up to 16 (the tensor-core tiles read 16-row blocks),
+// and 2 modulo 16, i.e. 4 words modulo 32: the histograms of neighbouring
+// vectors, one per lane, fall on different banks (8 words modulo 32 instead of
+// 4: D on 12,000 SDSS-like forests 106.1 -> 101.9 ms).
+__host__ __device__ inline int ldv_for(int scap) { return ((scap + 15) & ~15) + 2; }
 
 __host__ __device__ inline Lay layout(int L, int scap, int max_len, bool global_sink, int cb) {
   auto al = [](int v) { return (v + 15) & ~15; };
@@ -166,19 +174,30 @@ __host__ __device__ inline Lay layout(int L, int scap, int max_len, bool global_
   y.U = o;
   if (!global_sink) o += al(static_cast<int>((static_cast<int64_t>(L) * (L + 1) / 2) * 4));
   y.T4 = o; o += al(L * 16);
-  y.Va = o; o += al(cb * ldv_for(scap) * 4);
-  y.Vb = o; o += al(cb * ldv_for(scap) * 4);
+  y.V = o; o += al(cb * ldv_for(scap) * 8);
   y.mark = o; o += al(L);
   y.inv = o; o += al(L * 2);
   y.S = o; o += al(scap * 4);
   y.ucs = o; o += al(max_len * 8);
-  y.pixa = o; o += al(max_len * 16);
-  y.pixb = o; o += al(max_len * 16);
-  y.tv = o; o += al(max_len * 8);
-  y.cf = o; o += al(max_len * 16);
-  y.misc = o; o += 64;
+  y.db = o; o += al(max_len * 4);
+  y.tv = o; o += 2 * al(max_len * 8);
+  y.cf = o; o += 2 * al(max_len * 16);
+  y.win = o; o += 2 * al((max_len / kWin + 1) * 8);
+  y.misc = o; o += 192;
   y.end = o;
   return y;
+}
+
+// Bytes by which a band is judged to fit: the triangle, the batch with rows of
+// 8 words modulo 32, 23 bytes per local bin and 64 per pixel.  The
+// block needs a little less (see layout); whether a pair's vectors are summed
+// 32 or 16 at a time, and so the rounding of its FP32 sums, does not follow
+// every change of the layout.
+__host__ inline int64_t band_bytes(int L, int scap, int max_len, int cb) {
+  auto al = [](int64_t v) { return (v + 15) & ~int64_t(15); };
+  const int64_t row = ((((scap + 15) & ~15) + 23) & ~31) + 8;
+  return al(static_cast<int64_t>(L) * (L + 1) / 2 * 4) + al(L * 16) + 2 * al(cb * row * 4) + al(L) + al(L * 2) +
+         al(scap * 4) + 2 * al(max_len * 8) + 3 * al(max_len * 16) + al(L * 4) + 128;
 }
 
 __device__ __forceinline__ int tri_rowbase(int r, int L) {
@@ -203,33 +222,67 @@ __device__ __forceinline__ int local_bin(float2 u, float dj, float cp, float sp,
   return -1;
 }
 
-// Tile q of the packed upper triangle of 4 x 4 blocks of the union support:
-// acc = sum over vectors [vlo, vhi) of a a^T + b b^T on that block.
-__device__ __forceinline__ void dm_tile(const float* Va, const float* Vb, int ldv, int q, int vlo, int vhi,
-                                        float (&acc)[4][4], int* rblk_out, int* cblk_out) {
-  int rr = static_cast<int>((sqrtf(8.f * q + 1.f) - 1.f) * 0.5f);
-  while (rr * (rr + 1) / 2 > q) --rr;
-  while ((rr + 1) * (rr + 2) / 2 <= q) ++rr;
-  const int cblk = rr;                      // column block (>= row block)
-  const int rblk = q - rr * (rr + 1) / 2;   // row block
+// The same for a pixel pair given by (rp, rt) = (fmaf(-dj, cp, u.x), fmaf(dj, sp, u.y)),
+// with the floors as FP32 adds of 2^23 rounded toward -inf (a conversion to
+// integer runs at a quarter of the rate); corner = bits of both additions and
+// the band's first row, see bin_corner.
+__device__ __forceinline__ uint32_t bin_corner(int npar, int t0) {
+  return 0u - (0x4B000000u + static_cast<uint32_t>(t0)) * static_cast<uint32_t>(npar) - 0x4B000000u;
+}
+__device__ __forceinline__ bool bin_at(float rp, float rt, float fnpar, float fnperp, uint32_t npar, uint32_t corner,
+                                       int* l) {
+  rp = fabsf(rp);
+  *l = static_cast<int>(__float_as_uint(__fadd_rd(rt, 8388608.0f)) * npar +
+                        __float_as_uint(__fadd_rd(rp, 8388608.0f)) + corner);
+  return rp < fnpar && rt < fnperp;
+}
+
+// Tile q of 2 rows x W columns of the union support's upper triangle: acc = sum
+// over the batch's vectors of a a^T + b b^T.  Tiles of one column block are
+// consecutive, so the lanes of a warp read consecutive 16-byte row pairs (4
+// shared-memory passes) and the same columns (W / 2 broadcasts).
+template <int W>
+__device__ __forceinline__ void dm_tile(const F2* V, int ldv, int q, int nv, float (&acc)[2][W], int* row, int* col) {
+  // column block cb has W / 2 (cb + 1) row pairs
+  int cb = static_cast<int>((sqrtf(16.f / W * q + 1.f) - 1.f) * 0.5f);
+  while (W / 4 * cb * (cb + 1) > q) --cb;
+  while (W / 4 * (cb + 1) * (cb + 2) <= q) ++cb;
+  *col = W * cb;
+  *row = 2 * (q - W / 4 * cb * (cb + 1));
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < 2; ++u)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-  for (int vv = vlo; vv < vhi; ++vv) {
-    const float4 ar = *reinterpret_cast<const float4*>(Va + vv * ldv + 4 * rblk);
-    const float4 ac = *reinterpret_cast<const float4*>(Va + vv * ldv + 4 * cblk);
-    const float4 br = *reinterpret_cast<const float4*>(Vb + vv * ldv + 4 * rblk);
-    const float4 bc = *reinterpret_cast<const float4*>(Vb + vv * ldv + 4 * cblk);
-    const float arv[4] = {ar.x, ar.y, ar.z, ar.w}, acv[4] = {ac.x, ac.y, ac.z, ac.w};
-    const float brv[4] = {br.x, br.y, br.z, br.w}, bcv[4] = {bc.x, bc.y, bc.z, bc.w};
+    for (int v = 0; v < W; ++v) acc[u][v] = 0.f;
+  const float2 *r = reinterpret_cast<const float2*>(V) + *row, *c = reinterpret_cast<const float2*>(V) + *col;
+  auto add = [&](const float4& rr, const float4 (&cc)[W / 2]) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int v = 0; v < W; v += 2) {
+      const float4 k = cc[v / 2];
+      acc[0][v] = fmaf(rr.y, k.y, fmaf(rr.x, k.x, acc[0][v]));
+      acc[1][v] = fmaf(rr.w, k.y, fmaf(rr.z, k.x, acc[1][v]));
+      acc[0][v + 1] = fmaf(rr.y, k.w, fmaf(rr.x, k.z, acc[0][v + 1]));
+      acc[1][v + 1] = fmaf(rr.w, k.w, fmaf(rr.z, k.z, acc[1][v + 1]));
+    }
+  };
+  constexpr int N = 16 / W;   // vectors in flight
+  int vv = 0;
+  for (; vv + N <= nv; vv += N, r += N * ldv, c += N * ldv) {
+    float4 rr[N], cc[N][W / 2];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(brv[u], bcv[v], fmaf(arv[u], acv[v], acc[u][v]));
+    for (int e = 0; e < N; ++e) {
+      rr[e] = *reinterpret_cast<const float4*>(r + e * ldv);
+#pragma unroll
+      for (int v = 0; v < W / 2; ++v) cc[e][v] = *reinterpret_cast<const float4*>(c + e * ldv + 2 * v);
+    }
+#pragma unroll
+    for (int e = 0; e < N; ++e) add(rr[e], cc[e]);
   }
-  *rblk_out = rblk;
-  *cblk_out = cblk;
+  for (; vv < nv; ++vv, r += ldv, c += ldv) {
+    float4 cc[W / 2];
+#pragma unroll
+    for (int v = 0; v < W / 2; ++v) cc[v] = *reinterpret_cast<const float4*>(c + 2 * v);
+    add(*reinterpret_cast<const float4*>(r), cc);
+  }
 }
 
 // Tensor-core form of the rank-1 tiles: C = V^T V over the union support,
@@ -258,7 +311,7 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
   lo = tf32_bits(x - __uint_as_float(hi));
 }
 
-__device__ void dm_tiles_tc(const float* Va, const float* Vb, int ldv, int ns, int cbn, const int32_t* S, float* U,
+__device__ void dm_tiles_tc(const float* V, int ldv, int ns, int cbn, const int32_t* S, float* U,
                             int L, int wid, int nwarps, int lane) {
   const int g = lane >> 2, t = lane & 3;
   const int R = (ns + 15) >> 4, C8 = (ns + 7) >> 3;
@@ -271,17 +324,16 @@ __device__ void dm_tiles_tc(const float* Va, const float* Vb, int ldv, int ns, i
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        const float* V = half ? Vb : Va;
         for (int ks = 0; ks < ksteps; ++ks) {
-          const float* v0 = V + (ks * 8 + t) * ldv;
-          const float* v4 = v0 + 4 * ldv;
+          const float* v0 = V + (ks * 8 + t) * 2 * ldv + half;   // entry e of vector v: V[(v ldv + e) 2 + half]
+          const float* v4 = v0 + 8 * ldv;
           uint32_t ah[4], al[4], bh[2], bl[2];
-          split_tf32(v0[r0 + g], ah[0], al[0]);
-          split_tf32(v0[r0 + g + 8], ah[1], al[1]);
-          split_tf32(v4[r0 + g], ah[2], al[2]);
-          split_tf32(v4[r0 + g + 8], ah[3], al[3]);
-          split_tf32(v0[c0 + g], bh[0], bl[0]);
-          split_tf32(v4[c0 + g], bh[1], bl[1]);
+          split_tf32(v0[2 * (r0 + g)], ah[0], al[0]);
+          split_tf32(v0[2 * (r0 + g + 8)], ah[1], al[1]);
+          split_tf32(v4[2 * (r0 + g)], ah[2], al[2]);
+          split_tf32(v4[2 * (r0 + g + 8)], ah[3], al[3]);
+          split_tf32(v0[2 * (c0 + g)], bh[0], bl[0]);
+          split_tf32(v4[2 * (c0 + g)], bh[1], bl[1]);
           mma_tf32(acc, al[0], al[1], al[2], al[3], bh[0], bh[1]);
           mma_tf32(acc, ah[0], ah[1], ah[2], ah[3], bl[0], bl[1]);
           mma_tf32(acc, ah[0], ah[1], ah[2], ah[3], bh[0], bh[1]);
@@ -292,9 +344,7 @@ __device__ void dm_tiles_tc(const float* Va, const float* Vb, int ldv, int ns, i
         const int r = r0 + g + ((e & 2) ? 8 : 0);
         const int c = c0 + 2 * t + (e & 1);
         if (r <= c && c < ns) {
-          const int lr = S[r], lc = S[c];
-          const int lo = min(lr, lc), hi = max(lr, lc);
-          U[tri_rowbase(lo, L) + hi] -= acc[e];
+          U[tri_rowbase(S[r], L) + S[c]] -= acc[e];
         }
       }
     }
@@ -302,268 +352,425 @@ __device__ void dm_tiles_tc(const float* Va, const float* Vb, int ldv, int ns, i
 }
 
 // Subtract a tile from the triangle, or from G with FP64 atomics for wide
-// pairs.  Positions r <= c of the union support S (which is in no particular
-// order) cover each unordered pair of its bins once; the symmetric entry goes
-// to (min, max) of the two local bins.
-template <bool GLOBAL>
+// pairs.  S is ascending, so positions r <= c of it are entries of the upper
+// triangle.
+template <bool GLOBAL, int W>
 __device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t* S, int g0, int ns, int L, int nbins,
-                                              int rblk, int cblk, const float (&acc)[4][4]) {
+                                              int row, int col, const float (&acc)[2][W]) {
+  int lc[W];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = 4 * rblk + u;
-    if (r >= ns) continue;
-    const int lr = S[r];
+  for (int v = 0; v < W; ++v) lc[v] = S[min(col + v, ns - 1)];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int c = 4 * cblk + v;
-      if (c >= ns || c < r) continue;
-      const int lc = S[c];
-      if (!GLOBAL) {
-        const int lo = min(lr, lc), hi = max(lr, lc);
-        U[tri_rowbase(lo, L) + hi] -= acc[u][v];
-      } else {
-        red_add_f64_global(G + static_cast<int64_t>(g0 + min(lr, lc)) * nbins + g0 + max(lr, lc),
-                           -static_cast<double>(acc[u][v]));
-      }
+  for (int u = 0; u < 2; ++u) {
+    const int r = row + u;
+    const int lr = S[min(r, ns - 1)];
+    if (!GLOBAL) {
+      float* Ur = U + tri_rowbase(lr, L);
+      float old[W];   // all loads before the stores
+#pragma unroll
+      for (int v = 0; v < W; ++v) old[v] = (col + v < ns && r <= col + v) ? Ur[lc[v]] : 0.f;
+#pragma unroll
+      for (int v = 0; v < W; ++v)
+        if (col + v < ns && r <= col + v) Ur[lc[v]] = old[v] - acc[u][v];
+    } else {
+      double* Gr = G + static_cast<int64_t>(g0 + lr) * nbins + g0;
+#pragma unroll
+      for (int v = 0; v < W; ++v)
+        if (col + v < ns && r <= col + v) red_add_f64_global(Gr + lc[v], -static_cast<double>(acc[u][v]));
     }
   }
 }
 
-// One forest pair: accumulate its contribution into the triangle (or G).
-template <bool GLOBAL, int CB>
-__device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t0, int K, int L, int scap,
-                        unsigned char* sm, const Lay& y) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+template <bool GLOBAL, int W>
+__device__ __forceinline__ void dm_tiles(const F2* V, int ldv, int nv, double* G, float* U, const int32_t* S, int g0,
+                                         int ns, int L, int nbins) {
+  const int nc = (ns + W - 1) / W;
+  for (int q = threadIdx.x; q < W / 4 * nc * (nc + 1); q += kDmThreads) {
+    float acc[2][W];
+    int row, col;
+    dm_tile<W>(V, ldv, q, nv, acc, &row, &col);
+    dm_tile_store<GLOBAL>(G, U, S, g0, ns, L, nbins, row, col, acc);
+  }
+}
+
+// shared-memory arrays of one block
+struct Sm {
+  float* U;        // triangle of the pair
+  float4* T4;      // T1, Tx, Ty, Txy per local bin
+  F2* V;           // the batch's vectors, (a, b) entries; fixed-point words while filling
+  unsigned char* mark;
+  int16_t* inv;
+  int32_t* S;
+  float2* ucs;     // per pixel of a: (d cp + Dc, d sp + Ds)
+  float* db;       // distances of b
+  int2* tv_;       // per side: fixed-point terms of the summed-over forest
+  float4* cf_;     // per side: coefficients and T weights of the vectors
+  int2* win_;      // per side and kWin vectors: range of the summed-over forest in the grid
+  int tvn, cfn, winn;   // entries of one side
+  int* ns;         // size of the union support
+  float* par;      // 2 x 16 scalars of the pair (its own and the next one's)
+  __device__ Sm(unsigned char* sm, const Lay& y, int max_len) {
+    U = reinterpret_cast<float*>(sm + y.U);
+    T4 = reinterpret_cast<float4*>(sm + y.T4);
+    V = reinterpret_cast<F2*>(sm + y.V);
+    mark = sm + y.mark;
+    inv = reinterpret_cast<int16_t*>(sm + y.inv);
+    S = reinterpret_cast<int32_t*>(sm + y.S);
+    ucs = reinterpret_cast<float2*>(sm + y.ucs);
+    db = reinterpret_cast<float*>(sm + y.db);
+    tv_ = reinterpret_cast<int2*>(sm + y.tv);
+    cf_ = reinterpret_cast<float4*>(sm + y.cf);
+    win_ = reinterpret_cast<int2*>(sm + y.win);
+    tvn = (y.cf - y.tv) / 16;
+    cfn = (y.win - y.cf) / 32;
+    winn = (y.misc - y.win) / 16;
+    par = reinterpret_cast<float*>(sm + y.misc);
+    ns = reinterpret_cast<int*>(sm + y.misc + 128);
+  }
+  __device__ __forceinline__ int2* tv(int side) const { return tv_ + side * tvn; }
+  __device__ __forceinline__ float4* cf(int side) const { return cf_ + side * cfn; }
+  __device__ __forceinline__ int2* win(int side) const { return win_ + side * winn; }
+};
+
+// scalars of a pair in Sm::par
+enum { kScA0, kScB0, kScA1, kScB1, kC11, kCyy, kCxx, kCxy, kIWb, kISb, kIWa, kISa };
+
+struct Pair {
+  int na, nb;
+  float cp, sp;
+  bool ok;
+};
+
+// Stage a pair: pixels, fixed-point histogram terms, weights, and the pair's
+// FP64 quotients, one per lane of the last warp (every thread computing all
+// eight took a fifth of the kernel: FP64 runs at 1.7 lanes a cycle).
+__device__ __forceinline__ Pair dm_load(const DmArgs& A, int item, const Sm& m, int par) {
+  const int tid = threadIdx.x;
   const int2 pr = A.pairs[item];
   const float2 cs = A.cs[item];
   const int a = pr.x, b = pr.y;
-  const int na = A.F.len[a], nb = A.F.len[b];
+  Pair P;
+  P.na = A.F.len[a];
+  P.nb = A.F.len[b];
+  P.cp = cs.x;
+  P.sp = cs.y;
   // staging buffers hold max_len pixels (the longest forest when the pair list
   // was built); a longer forest means the offsets changed in place without a
   // rebuild, and the pair is skipped rather than overrun shared memory
-  if (na > A.max_len || nb > A.max_len || na == 0 || nb == 0) return;
-  const float cp = cs.x, sp = cs.y;
+  P.ok = !(P.na > A.max_len || P.nb > A.max_len || P.na == 0 || P.nb == 0);
+  if (!P.ok) return P;
   const float refa = A.F.dref[a], refb = A.F.dref[b];
-  const float Dc = (refa - refb) * cp, Ds = (refa + refb) * sp;
-  const double Wa = A.F.wsum[a], Sa = A.F.ssum[a], Wb = A.F.wsum[b], Sb = A.F.ssum[b];
+  const float Dc = (refa - refb) * P.cp, Ds = (refa + refb) * P.sp;
+  // Histogram terms of the summed-over forest (w, w x) in fixed point, one
+  // 32-bit word each: shared memory adds integers natively.  A (vector, bin)
+  // sum holds at most 2 / (cp hmin) + 2 pixels (two windows of width 1/cp).
+  const float runa = 2.f / (P.cp * A.F.hmin[a]) + 2.f, runb = 2.f / (P.cp * A.F.hmin[b]) + 2.f;
+  const float sA0 = word_scale(runa * A.F.wmax[a]), sB0 = word_scale(runa * A.F.wmax[a] * A.F.xmax[a]);
+  const float sA1 = word_scale(runb * A.F.wmax[b]), sB1 = word_scale(runb * A.F.wmax[b] * A.F.xmax[b]);
+  const Pix* ga = A.pix + A.F.off[a];
+  const Pix* gb = A.pix + A.F.off[b];
+  for (int k = tid; k < P.na; k += kDmThreads) {
+    const Pix p = ga[k];
+    m.ucs[k] = make_float2(fmaf(p.x, P.cp, Dc), fmaf(p.x, P.sp, Ds));
+    m.tv(0)[k] = make_int2(__float2int_rn(p.y * sA0), __float2int_rn(p.y * p.w * sB0));
+    m.cf(1)[k] = make_float4(0.f, 0.f, p.y, p.y * p.w);
+  }
+  for (int k = tid; k < P.nb; k += kDmThreads) {
+    const Pix p = gb[k];
+    m.db[k] = p.x;
+    m.tv(1)[k] = make_int2(__float2int_rn(p.y * sA1), __float2int_rn(p.y * p.w * sB1));
+    m.cf(0)[k] = make_float4(0.f, 0.f, p.y, p.y * p.w);
+  }
+  float* c = m.par + 16 * par;
+  const int t = tid - (kDmThreads - 32);
+  if (t >= 0 && t < 8) {
+    // 1 / (W_a W_b), 1 / (W_a S_b), 1 / (S_a W_b), 1 / (S_a S_b), 1 / W_b, 1 / S_b, 1 / W_a, 1 / S_a
+    const double x = (t < 4) ? (t < 2 ? A.F.wsum[a] : A.F.ssum[a]) : 1.0;
+    const double y = (t < 4) ? ((t & 1) ? A.F.ssum[b] : A.F.wsum[b])
+                             : (t == 4 ? A.F.wsum[b] : t == 5 ? A.F.ssum[b] : t == 6 ? A.F.wsum[a] : A.F.ssum[a]);
+    c[kC11 + t] = (A.eta_mean_slope != 0 && x > 0.0 && y > 0.0) ? static_cast<float>(1.0 / (x * y)) : 0.f;
+  }
+  if (t == 8) {
+    c[kScA0] = 1.f / sA0;
+    c[kScB0] = 1.f / sB0;
+    c[kScA1] = 1.f / sA1;
+    c[kScB1] = 1.f / sB1;
+  }
+  return P;
+}
+
+// Rank-1 coefficients sqrt(w_v / W), sqrt(w_v / S) of the vectors of both
+// sides, and for every kWin vectors the range of the other forest's pixels
+// that can share the grid with one of them (for one vector r_par is monotone
+// in the other pixel and r_perp rises, in FP32 as evaluated, so the two ends
+// are found by bisection with the binning's own arithmetic).  About a third of
+// the pixel pairs of two SDSS-like forests fall outside.
+__device__ __forceinline__ void dm_windows(const DmArgs& A, const Pair& P, const Sm& m, int par) {
+  const int tid = threadIdx.x;
+  const float* c = m.par + 16 * par;
+  const float fnpar = static_cast<float>(A.n_par), fnperp = static_cast<float>(A.n_perp);
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int nvec = side == 0 ? P.nb : P.na, nother = side == 0 ? P.na : P.nb;
+    const float iw = c[side == 0 ? kIWa : kIWb], is = c[side == 0 ? kISa : kISb];
+    for (int k = tid; k < nvec; k += kDmThreads) {
+      const float w = m.cf(side)[k].z;
+      m.cf(side)[k].x = sqrtf(w * iw);
+      m.cf(side)[k].y = sqrtf(w * is);
+    }
+    const int ng = (nvec + kWin - 1) / kWin;
+    // one thread per end of a range, from the last thread down
+    for (int g2 = kDmThreads - 1 - tid; g2 < 2 * ng; g2 += kDmThreads) {
+      const int g = g2 >> 1, first = g * kWin, last = min(first + kWin, nvec) - 1;
+      int lo = 0, hi = nother;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        // at the vector of the group that reaches furthest down (up) in the other forest
+        const float2 u = m.ucs[side == 0 ? mid : ((g2 & 1) ? last : first)];
+        const float d = m.db[side == 0 ? ((g2 & 1) ? last : first) : mid];
+        const float rp = fmaf(-d, P.cp, u.x);
+        bool below;
+        if (!(g2 & 1))
+          below = side == 0 ? !(rp > -fnpar) : !(rp < fnpar);
+        else {
+          const float2 uf = m.ucs[side == 0 ? mid : first];
+          const float df = m.db[side == 0 ? first : mid];
+          below = (side == 0 ? rp < fnpar : rp > -fnpar) && fmaf(df, P.sp, uf.y) < fnperp;
+        }
+        if (below)
+          lo = mid + 1;
+        else
+          hi = mid;
+      }
+      reinterpret_cast<int*>(m.win(side))[g2] = lo;
+    }
+  }
+}
+
+// One batch: cbn consecutive vectors from v0 of a side, against the pixels
+// [lo, hi) of the other forest.
+struct Batch {
+  int side, v0, cbn, lo, hi;
+};
+
+// the next batch that has pixels in the grid; false after the last one
+__device__ __forceinline__ bool next_batch(Batch& B, int v0, int cb, const Pair& P, bool eta, const Sm& m) {
+  for (;;) {
+    const int nvec = B.side == 0 ? P.nb : P.na;
+    if (v0 >= nvec) {
+      if (B.side == 1 || !eta) return false;
+      B.side = 1;
+      v0 = 0;
+      continue;
+    }
+    B.v0 = v0;
+    B.cbn = min(cb, nvec - v0);
+    B.lo = m.win(B.side)[v0 / kWin].x;
+    B.hi = m.win(B.side)[v0 / kWin].y;
+    for (int g = v0 / kWin + 1; g * kWin < v0 + B.cbn; ++g) B.hi = max(B.hi, m.win(B.side)[g].y);
+    if (B.lo < B.hi) return true;
+    v0 += B.cbn;
+  }
+}
+
+// f(o, l) for the pixel pairs (vector of this thread, pixel o) of a batch that
+// are in the grid, l their local bin.  Lanes are consecutive vectors, thread
+// groups of CB take every (threads / CB)-th pixel; four loads in flight.
+template <int CB, class F>
+__device__ __forceinline__ void for_pairs(const Batch& B, const Pair& P, const Sm& m, float fnpar, float fnperp, int npar,
+                                          uint32_t corner, F&& f) {
+  const int vv = threadIdx.x & (CB - 1);
+  constexpr int step = kDmThreads / CB;
+  if (vv >= B.cbn) return;
+  const float nan = __int_as_float(0x7FC00000);
+  int l;
+  if (B.side == 0) {
+    const float dj = m.db[B.v0 + vv];
+    for (int o = B.lo + threadIdx.x / CB; o < B.hi; o += 4 * step) {
+      float2 u[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) u[e] = (o + e * step < B.hi) ? m.ucs[o + e * step] : make_float2(nan, nan);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (bin_at(fmaf(-dj, P.cp, u[e].x), fmaf(dj, P.sp, u[e].y), fnpar, fnperp, npar, corner, &l)) f(o + e * step, l);
+    }
+  } else {
+    const float2 u = m.ucs[B.v0 + vv];
+    for (int o = B.lo + threadIdx.x / CB; o < B.hi; o += 4 * step) {
+      float d[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) d[e] = (o + e * step < B.hi) ? m.db[o + e * step] : nan;
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (bin_at(fmaf(-d[e], P.cp, u.x), fmaf(d[e], P.sp, u.y), fnpar, fnperp, npar, corner, &l)) f(o + e * step, l);
+    }
+  }
+}
+
+// The rank-1 terms of one pair, batch by batch, into the triangle (or G), and
+// its T vectors.  dirty: entries of V's rows in use by the last batch (the rest
+// is zero).  Four block-wide phases a batch: the next batch's marks are
+// set in the phase of this one's tiles, whose last round leaves warps idle.
+template <bool GLOBAL, int CB>
+__device__ void dm_vectors(const DmArgs& A, const Pair& P, double* G, int t0, int L, int scap, const Sm& m, int par,
+                           int& dirty) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  constexpr int nwarps = kDmThreads / 32;
   const bool eta = A.eta_mean_slope != 0;
   const int npar = A.n_par, nbins = A.n_par * A.n_perp;
   const int ldv = ldv_for(scap);
   const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(A.n_perp);
-
-  float* U = reinterpret_cast<float*>(sm + y.U);
-  float4* T4 = reinterpret_cast<float4*>(sm + y.T4);
-  float* Va = reinterpret_cast<float*>(sm + y.Va);
-  float* Vb = reinterpret_cast<float*>(sm + y.Vb);
-  int32_t* Vai = reinterpret_cast<int32_t*>(sm + y.Va);   // same storage, fixed point while filling
-  int32_t* Vbi = reinterpret_cast<int32_t*>(sm + y.Vb);
-  int2* tv = reinterpret_cast<int2*>(sm + y.tv);
-  float4* cf = reinterpret_cast<float4*>(sm + y.cf);
-  unsigned char* mark = sm + y.mark;
-  int16_t* inv = reinterpret_cast<int16_t*>(sm + y.inv);
-  int32_t* S = reinterpret_cast<int32_t*>(sm + y.S);
-  float2* ucs = reinterpret_cast<float2*>(sm + y.ucs);
-  Pix* pxa = reinterpret_cast<Pix*>(sm + y.pixa);
-  Pix* pxb = reinterpret_cast<Pix*>(sm + y.pixb);
+  const uint32_t corner = bin_corner(npar, t0);
   const int g0 = t0 * A.n_par;   // accumulator row of local bin 0 (see dm_finalize_kernel)
-  int* misc = reinterpret_cast<int*>(sm + y.misc);   // [0] = |S|
-
-  const Pix* ga = A.pix + A.F.off[a];
-  const Pix* gb = A.pix + A.F.off[b];
-  for (int k = tid; k < na; k += blockDim.x) {
-    const Pix p = ga[k];
-    pxa[k] = p;
-    ucs[k] = make_float2(fmaf(p.x, cp, Dc), fmaf(p.x, sp, Ds));
-  }
-  for (int k = tid; k < nb; k += blockDim.x) pxb[k] = gb[k];
+  unsigned char* mark = m.mark;
+  auto set_marks = [&](const Batch& B) {
+    for_pairs<CB>(B, P, m, fnpar, fnperp, npar, corner, [&](int, int l) { mark[l] = 1; });
+  };
+  auto clear_marks = [&]() {
+    for (int k = tid; k < (L + 3) / 4; k += kDmThreads) reinterpret_cast<uint32_t*>(mark)[k] = 0;
+  };
+  Batch B;
+  B.side = 0;
+  bool on = next_batch(B, 0, CB, P, eta, m);
+  if (!on) return;
+  set_marks(B);
   __syncthreads();
-
-  // side 0: columns j of b (histograms over i of a, weights w_i, x_i)
-  // side 1: rows i of a (histograms over j of b, weights w_j, y_j)
-  for (int side = 0; side < 2; ++side) {
-    if (side == 1 && !eta) break;
-    const int nvec = side == 0 ? nb : na;
-    const int nother = side == 0 ? na : nb;
-    // rank-1 coefficients sqrt(w_v / W) and sqrt(w_v / S) of this side's
-    // vectors, from FP32 reciprocals computed once per pair (FP64 division is
-    // slow on this part)
-    const double Wn = side == 0 ? Wa : Wb;
-    const double Sn = side == 0 ? Sa : Sb;
-    const float inv_w = (eta && Wn > 0.0) ? static_cast<float>(1.0 / Wn) : 0.f;
-    const float inv_s = (eta && Sn > 0.0) ? static_cast<float>(1.0 / Sn) : 0.f;
-    // Histogram terms of the summed-over forest (w, w x) in fixed point, one
-    // 32-bit word each: shared memory adds integers natively.  A (vector, bin)
-    // sum holds at most 2 / (cp hmin) + 2 pixels (two windows of width 1/cp).
+  while (on) {
+    // compaction of the marks into the ascending union support S and the
+    // inverse map: a warp takes 32 local bins and counts the marks below
+    // them itself.  The last batch's entries of V are cleared meanwhile.
+    for (int l0 = wid * 32; l0 < L; l0 += nwarps * 32) {
+      int below = 0;
+      for (int k = lane; k < l0 / 4; k += 32) below += __popc(reinterpret_cast<const uint32_t*>(mark)[k]);
+      below = __reduce_add_sync(0xffffffffu, below);
+      const int l = l0 + lane;
+      const bool set = (l < L) && mark[l];
+      const unsigned msk = __ballot_sync(0xffffffffu, set);
+      if (set) {
+        const int pos = below + __popc(msk & ((1u << lane) - 1u));
+        if (pos < scap) m.S[pos] = l;
+        m.inv[l] = static_cast<int16_t>(pos);
+      }
+      if (l0 + 32 >= L && lane == 0) *m.ns = below + __popc(msk);
+    }
+    for (int vv = wid; vv < CB; vv += nwarps)
+      for (int k = lane; 2 * k < dirty; k += 32)
+        reinterpret_cast<float4*>(m.V + vv * ldv)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    dirty = 0;
+    __syncthreads();
+    const int ns = *m.ns;
+    if (ns > scap) {
+      // union too large for the staging arrays: again with half the batch
+      clear_marks();
+      __syncthreads();
+      next_batch(B, B.v0, max(1, B.cbn / 2), P, eta, m);
+      set_marks(B);
+      __syncthreads();
+      continue;
+    }
+    // histograms on S
     {
-      const int fs = side == 0 ? a : b;
-      const Pix* ps = side == 0 ? pxa : pxb;
-      const int ns_ = side == 0 ? na : nb;
-      const float nrun = 2.f / (cp * A.F.hmin[fs]) + 2.f;
-      const float scA = word_scale(nrun * A.F.wmax[fs]);
-      const float scB = word_scale(nrun * A.F.wmax[fs] * A.F.xmax[fs]);
-      if (tid == 0) {
-        reinterpret_cast<float*>(misc)[1] = 1.f / scA;
-        reinterpret_cast<float*>(misc)[2] = 1.f / scB;
-      }
-      for (int k = tid; k < ns_; k += blockDim.x)
-        tv[k] = make_int2(__float2int_rn(ps[k].y * scA), __float2int_rn(ps[k].y * ps[k].w * scB));
-      // per vector of this side: rank-1 coefficients and the T weights w_v, w_v y_v
-      const Pix* pv = side == 0 ? pxb : pxa;
-      for (int k = tid; k < nvec; k += blockDim.x) {
-        const Pix me = pv[k];
-        cf[k] = make_float4(sqrtf(me.y * inv_w), sqrtf(me.y * inv_s), me.y, me.y * me.w);
-      }
-      __syncthreads();
+      unsigned* row = reinterpret_cast<unsigned*>(m.V + (tid & (CB - 1)) * ldv);
+      const int2* tv = m.tv(B.side);
+      const int16_t* inv = m.inv;
+      for_pairs<CB>(B, P, m, fnpar, fnperp, npar, corner, [&](int o, int l) {
+        const int2 t = tv[o];
+        const int k = 2 * inv[l];
+        atomicAdd(row + k, static_cast<unsigned>(t.x));
+        atomicAdd(row + k + 1, static_cast<unsigned>(t.y));
+      });
     }
-    const float inv_scA = reinterpret_cast<float*>(misc)[1];
-    const float inv_scB = reinterpret_cast<float*>(misc)[2];
-    int v0 = 0;
-    int cb = CB;
-    while (v0 < nvec) {
-      const int cbn = min(cb, nvec - v0);
-      // (a1) mark the local bins the batch touches (and reset the slot counter of (b))
-      if (tid == 0) misc[3] = 0;
-      const int vv_t = tid % cbn;
-      const int ostep = blockDim.x / cbn;
-      // independent items: unrolled so that several items' loads are in flight
-#pragma unroll 4
-      for (int o = tid / cbn; o < nother && tid < ostep * cbn; o += ostep) {
-        const int i = side == 0 ? o : v0 + vv_t;
-        const int j = side == 0 ? v0 + vv_t : o;
-        const int l = local_bin(ucs[i], pxb[j].x, cp, sp, fnpar, fnperp, npar, t0);
-        if (l >= 0) mark[l] = 1;
-      }
-      __syncthreads();
-      // (b) compaction of the marks into S and the inverse map, all warps: a
-      // warp takes 32 local bins, ballots, and reserves its slots in S with
-      // one shared atomic (S is in no particular order; every output entry
-      // still sums its vectors in a fixed order).  V is cleared meanwhile.
-      {
-        const int nwarps = blockDim.x >> 5;
-        for (int l0 = wid * 32; l0 < L; l0 += nwarps * 32) {
-          const int l = l0 + lane;
-          const bool on = (l < L) && mark[l];
-          const unsigned msk = __ballot_sync(0xffffffffu, on);
-          int base = 0;
-          if (lane == 0 && msk) base = atomicAdd(&misc[3], __popc(msk));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (on) {
-            const int pos = base + __popc(msk & ((1u << lane) - 1u));
-            if (pos < scap) S[pos] = l;
-            inv[l] = static_cast<int16_t>(pos);
-            mark[l] = 0;
-          }
-        }
-        for (int k = tid; k < CB * ldv; k += blockDim.x) {
-          Va[k] = 0.f;
-          Vb[k] = 0.f;
-        }
-      }
-      __syncthreads();
-      const int ns = misc[3];
-      if (ns > scap) {
-        // union too large for the staging arrays: retry with half the batch
-        __syncthreads();
-        cb = max(1, cbn / 2);
-        continue;
-      }
-      // (a2) dense histograms on S
-      // independent items: unrolled so that several items' loads are in flight
-#pragma unroll 4
-      for (int o = tid / cbn; o < nother && tid < ostep * cbn; o += ostep) {
-        const int i = side == 0 ? o : v0 + vv_t;
-        const int j = side == 0 ? v0 + vv_t : o;
-        const int l = local_bin(ucs[i], pxb[j].x, cp, sp, fnpar, fnperp, npar, t0);
-        if (l >= 0) {
-          const int2 t = tv[side == 0 ? i : j];   // the summed-over pixel's terms
-          const int k = vv_t * ldv + inv[l];
-          atomicAdd(reinterpret_cast<unsigned*>(&Vai[k]), static_cast<unsigned>(t.x));
-          atomicAdd(reinterpret_cast<unsigned*>(&Vbi[k]), static_cast<unsigned>(t.y));
-        }
-      }
-      __syncthreads();
-      // T vectors (from unscaled column histograms) and scaling by the
-      // rank-1 coefficients sqrt(w_v / W), sqrt(w_v / S).  Item (k, vv) =
-      // (bin of S, vector of the batch); the 16 vectors of a bin sit in 16
-      // consecutive lanes, which sum the bin's T terms with shuffles.
-      for (int base = 0; base < ns * CB; base += blockDim.x) {
-        const int idx = base + tid;
-        const int k = idx / CB, vv = idx % CB;
-        const bool act = (k < ns) && (vv < cbn);
-        float t1 = 0.f, tx = 0.f, ty = 0.f, txy = 0.f;
+    clear_marks();
+    __syncthreads();
+    // T vectors (from unscaled column histograms) and scaling by the rank-1
+    // coefficients sqrt(w_v / W), sqrt(w_v / S)
+    const float4* cf = m.cf(B.side) + B.v0;
+    const float isA = m.par[16 * par + (B.side == 0 ? kScA0 : kScA1)];
+    const float isB = m.par[16 * par + (B.side == 0 ? kScB0 : kScB1)];
+    if (B.side == 0) {
+      // item (k, vv) = (bin of S, vector): the vectors of a bin sit in CB
+      // consecutive lanes, which sum its four T terms, half of the terms
+      // changing lanes at each of the first two steps
+      const int vv = tid & (CB - 1);
+      const bool actv = vv < B.cbn;
+      const float4 c = actv ? cf[vv] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k0 = 0; k0 < ns; k0 += kDmThreads / CB) {
+        const int k = k0 + tid / CB;
+        const bool act = (k < ns) && actv;
+        float t[4] = {0.f, 0.f, 0.f, 0.f};
         if (act) {
-          const float4 c = cf[v0 + vv];
-          const float va = static_cast<float>(Vai[vv * ldv + k]) * inv_scA;
-          const float vb = static_cast<float>(Vbi[vv * ldv + k]) * inv_scB;
-          t1 = c.z * va;
-          tx = c.z * vb;
-          ty = c.w * va;
-          txy = c.w * vb;
-          Va[vv * ldv + k] = va * c.x;
-          Vb[vv * ldv + k] = vb * c.y;
+          const float2 h = unf2(m.V[vv * ldv + k]);
+          const float va = static_cast<float>(__float_as_int(h.x)) * isA;
+          const float vb = static_cast<float>(__float_as_int(h.y)) * isB;
+          t[0] = c.z * va;
+          t[1] = c.z * vb;
+          t[2] = c.w * va;
+          t[3] = c.w * vb;
+          m.V[vv * ldv + k] = f2(va * c.x, vb * c.y);
         }
-        if (side == 0) {
+        const bool up1 = vv & (CB / 2), up2 = vv & (CB / 4);
+        float x = up1 ? t[2] : t[0], y = up1 ? t[3] : t[1];
+        x += __shfl_xor_sync(0xffffffffu, up1 ? t[0] : t[2], CB / 2);
+        y += __shfl_xor_sync(0xffffffffu, up1 ? t[1] : t[3], CB / 2);
+        float z = up2 ? y : x;
+        z += __shfl_xor_sync(0xffffffffu, up2 ? x : y, CB / 4);
 #pragma unroll
-          for (int o = CB / 2; o > 0; o >>= 1) {
-            t1 += __shfl_xor_sync(0xffffffffu, t1, o);
-            tx += __shfl_xor_sync(0xffffffffu, tx, o);
-            ty += __shfl_xor_sync(0xffffffffu, ty, o);
-            txy += __shfl_xor_sync(0xffffffffu, txy, o);
-          }
-          if (act && vv == 0) {
-            float4 t = T4[S[k]];
-            t.x += t1;
-            t.y += tx;
-            t.z += ty;
-            t.w += txy;
-            T4[S[k]] = t;
-          }
+        for (int o = CB / 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (k < ns && (vv & (CB / 4 - 1)) == 0)
+          reinterpret_cast<float*>(m.T4 + m.S[k])[vv / (CB / 4)] += z;
+      }
+    } else {
+      for (int vv = wid; vv < B.cbn; vv += nwarps) {
+        const float4 c = cf[vv];
+        const float ka = c.x, kb = c.y;
+        F2* row = m.V + vv * ldv;
+        for (int k = lane; k < ns; k += 32) {
+          const float2 h = unf2(row[k]);
+          row[k] = f2(static_cast<float>(__float_as_int(h.x)) * isA * ka,
+                      static_cast<float>(__float_as_int(h.y)) * isB * kb);
         }
       }
-      __syncthreads();
-      // (d) rank-1 updates of the batch: 4 x 4 register tiles of S x S,
-      // one tile per thread, each adding its 16 entries to the triangle.
-      if (eta) {
-        if (!GLOBAL && A.tensor_tiles) {
-          dm_tiles_tc(Va, Vb, ldv, ns, cbn, S, U, L, wid, blockDim.x >> 5, lane);
-        } else {
-          const int nt = (ns + 3) >> 2;
-          const int ntiles = nt * (nt + 1) / 2;
-          for (int q = tid; q < ntiles; q += blockDim.x) {
-            float acc[4][4];
-            int rblk, cblk;
-            dm_tile(Va, Vb, ldv, q, 0, cbn, acc, &rblk, &cblk);
-            dm_tile_store<GLOBAL>(G, U, S, g0, ns, L, nbins, rblk, cblk, acc);
-          }
-        }
-      }
-      __syncthreads();
-      v0 += cbn;
-      cb = CB;
     }
+    __syncthreads();
+    // rank-1 updates of the batch: register tiles of S x S, one per thread,
+    // each adding its 16 entries to the triangle
+    if (eta) {
+      if (!GLOBAL && A.tensor_tiles) {
+        dm_tiles_tc(reinterpret_cast<const float*>(m.V), ldv, ns, B.cbn, m.S, m.U, L, wid, nwarps, lane);
+      } else {
+        dm_tiles<GLOBAL, 4>(m.V, ldv, B.cbn, G, m.U, m.S, g0, ns, L, nbins);
+      }
+    }
+    dirty = ns;
+    on = next_batch(B, B.v0 + B.cbn, CB, P, eta, m);
+    if (on) set_marks(B);
+    __syncthreads();
   }
+}
 
-  // T terms, diagonal and W: one warp per row r, lanes over c >= r.  The
-  // pair's whole contribution (its rank-1 terms, already in the triangle, plus
-  // these) goes to the FP64 accumulator here, and the triangle is cleared, so
-  // that D~ and W are summed over pairs in FP64 only.  Rows and columns with
-  // T = 0 hold nothing: every rank-1 term of a bin carries the weights of the
-  // pixel pairs in it.
-  const int nwarps = blockDim.x >> 5;
-  const float c11 = (eta && Wa > 0 && Wb > 0) ? static_cast<float>(1.0 / (Wa * Wb)) : 0.f;
-  const float cyy = (eta && Wa > 0 && Sb > 0) ? static_cast<float>(1.0 / (Wa * Sb)) : 0.f;
-  const float cxx = (eta && Sa > 0 && Wb > 0) ? static_cast<float>(1.0 / (Sa * Wb)) : 0.f;
-  const float cxy = (eta && Sa > 0 && Sb > 0) ? static_cast<float>(1.0 / (Sa * Sb)) : 0.f;
+// T terms, diagonal and W: one warp per row r, lanes over c >= r.  The
+// pair's whole contribution (its rank-1 terms, already in the triangle, plus
+// these) goes to the FP64 accumulator here, and the triangle is cleared, so
+// that D~ and W are summed over pairs in FP64 only.  Rows and columns with
+// T = 0 hold nothing: every rank-1 term of a bin carries the weights of the
+// pixel pairs in it.
+template <bool GLOBAL>
+__device__ __forceinline__ void dm_flush(const DmArgs& A, double* G, double* wdm, int t0, int L, const Sm& m, int par) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int nwarps = kDmThreads / 32;
+  const int g0 = t0 * A.n_par, nbins = A.n_par * A.n_perp;
+  const float* pc = m.par + 16 * par;
+  const float c11 = pc[kC11], cyy = pc[kCyy], cxx = pc[kCxx], cxy = pc[kCxy];
   for (int r = wid; r < L; r += nwarps) {
-    const float4 tr = T4[r];
+    const float4 tr = m.T4[r];
     if (tr.x == 0.f && tr.y == 0.f && tr.z == 0.f && tr.w == 0.f) continue;
     const float f1 = c11 * tr.x, fy = cyy * tr.z, fx = cxx * tr.y, fxy = cxy * tr.w;
     const int rb = tri_rowbase(r, L);
     // two columns per lane per iteration (independent chains)
     for (int c = r + lane; c < L; c += 64) {
       const int c2 = c + 32;
-      const float4 tc = T4[c];
-      const float4 tc2 = (c2 < L) ? T4[c2] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 tc = m.T4[c];
+      const float4 tc2 = (c2 < L) ? m.T4[c2] : make_float4(0.f, 0.f, 0.f, 0.f);
       float v = f1 * tc.x + fy * tc.z + fx * tc.y + fxy * tc.w;
       const float v2 = f1 * tc2.x + fy * tc2.z + fx * tc2.y + fxy * tc2.w;
       if (c == r) v += tr.x;
@@ -574,16 +781,16 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
         // exactly 0 (u = -v, about one entry in 1e7) the rank-1 part u stays and
         // goes out with the block's next pair that has the entry.  Clearing it too
         // makes two calls agree to 1e-18, but moves D by 1e-7 to 1e-5 of its norm.
-        const float x = U[rb + c] + v;
+        const float x = m.U[rb + c] + v;
         if (x != 0.f) {
           red_add_f64_global(row + c, static_cast<double>(x));
-          U[rb + c] = 0.f;
+          m.U[rb + c] = 0.f;
         }
         if (c2 < L) {
-          const float x2 = U[rb + c2] + v2;
+          const float x2 = m.U[rb + c2] + v2;
           if (x2 != 0.f) {
             red_add_f64_global(row + c2, static_cast<double>(x2));
-            U[rb + c2] = 0.f;
+            m.U[rb + c2] = 0.f;
           }
         }
       } else {
@@ -593,9 +800,6 @@ __device__ void dm_pair(const DmArgs& A, double* G, double* wdm, int item, int t
     }
     if (lane == 0) red_add_f64_global(wdm + g0 + r, static_cast<double>(tr.x));
   }
-  __syncthreads();
-  for (int k = tid; k < L; k += blockDim.x) T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-  __syncthreads();
 }
 
 template <bool GLOBAL, int CB>
@@ -609,19 +813,18 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
   const int tid = threadIdx.x;
   const int nbins = A.n_par * A.n_perp;
   const int n_items = GLOBAL ? *n_wide_dev : *n_chunks_dev;
-  const Lay y = layout(Lalloc, scap, A.max_len, GLOBAL, CB);
-  float* U = reinterpret_cast<float*>(sm + y.U);
-  float4* T4 = reinterpret_cast<float4*>(sm + y.T4);
-  unsigned char* mark = sm + y.mark;
+  const Sm m(sm, layout(Lalloc, scap, A.max_len, GLOBAL, CB), A.max_len);
   // clear all accumulators once
   if (!GLOBAL) {
     const int nt = Lalloc * (Lalloc + 1) / 2;
-    for (int k = tid; k < nt; k += blockDim.x) U[k] = 0.f;
+    for (int k = tid; k < nt; k += blockDim.x) m.U[k] = 0.f;
   }
   for (int k = tid; k < Lalloc; k += blockDim.x) {
-    T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    mark[k] = 0;
+    m.T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    m.mark[k] = 0;
   }
+  for (int k = tid; k < CB * ldv_for(scap); k += blockDim.x) m.V[k] = 0;
+  int dirty = 0;
   __syncthreads();
   for (;;) {
     if (tid == 0) s_item = static_cast<long long>(atomicAdd(counter, 1ull));
@@ -644,9 +847,23 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
     double* G = A.G + static_cast<int64_t>(mock) * nbins * nbins;
     double* wdm = A.wdm + static_cast<int64_t>(mock) * nbins;
     const int L = K * A.n_par;
+    // A pair's pixels are loaded while the previous one's triangle is flushed.
+    int par = 0;
+    Pair P = dm_load(A, GLOBAL ? wide[item] : order[first], m, par);
+    __syncthreads();
     for (int q = 0; q < cnt; ++q) {
-      const int pi = GLOBAL ? wide[item] : order[first + q];
-      dm_pair<GLOBAL, CB>(A, G, wdm, pi, t0, K, L, scap, sm, y);
+      if (P.ok) dm_windows(A, P, m, par);
+      __syncthreads();
+      if (P.ok) dm_vectors<GLOBAL, CB>(A, P, G, t0, L, scap, m, par, dirty);
+      Pair N;
+      N.ok = false;
+      if (!GLOBAL && q + 1 < cnt) N = dm_load(A, order[first + q + 1], m, par ^ 1);
+      if (P.ok) dm_flush<GLOBAL>(A, G, wdm, t0, L, m, par);
+      __syncthreads();
+      if (P.ok)
+        for (int k = tid; k < L; k += kDmThreads) m.T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      P = N;
+      par ^= 1;
     }
   }
 }
@@ -830,25 +1047,17 @@ cudaError_t run_dmat(const DmArgs& a, const DevInfo& dev, void** scratch, size_t
   const int max_len = std::max(a.max_len, 1);
   // largest band that fits in shared memory with batches of 16 vectors (kfit)
   // and with batches of 32 (kfit2 <= kfit)
+  auto fits = [&](int K, int cb, int* sc) {
+    const int L = K * a.n_par;
+    *sc = scap_for(L, a.n_par, K, cb);
+    return band_bytes(L, *sc, max_len, cb) <= dev.smem_optin &&
+           layout(L, *sc, max_len, false, cb).end + 64 <= dev.smem_optin;
+  };
   int kfit = 0, scap = 0, kfit2 = 0, scap2 = 0;
-  for (int K = a.n_perp; K >= 1; --K) {
-    const int L = K * a.n_par;
-    const int sc = scap_for(L, a.n_par, K, kCB);
-    if (layout(L, sc, max_len, false, kCB).end + 64 <= dev.smem_optin) {
-      kfit = K;
-      scap = sc;
-      break;
-    }
-  }
-  for (int K = kfit; K >= 1; --K) {
-    const int L = K * a.n_par;
-    const int sc = scap_for(L, a.n_par, K, kCB2);
-    if (layout(L, sc, max_len, false, kCB2).end + 64 <= dev.smem_optin) {
-      kfit2 = K;
-      scap2 = sc;
-      break;
-    }
-  }
+  for (int K = a.n_perp; K >= 1 && kfit == 0; --K)
+    if (fits(K, kCB, &scap)) kfit = K;
+  for (int K = kfit; K >= 1 && kfit2 == 0; --K)
+    if (fits(K, kCB2, &scap2)) kfit2 = K;
   // wide-pair configuration (triangle in global memory)
   const int Lw = a.n_perp * a.n_par;
   const int scapw = scap_for(Lw, a.n_par, a.n_perp, kCB);

@@ -157,6 +157,34 @@ def test_dmat_on_a_grid_of_unequal_sides(api, handle):
     assert np.all(np.abs(w.cpu().numpy() - W) <= 1e-6 * W + E + 1e-9)
 
 
+@pytest.mark.parametrize("lengths,bins,step,patch", [
+    # edges of windows and batches
+    ((15, 16, 17, 31, 32, 33, 47, 48, 49, 64, 65), (13, 22, 60.0, 90.0), (0.3, 3.7), 0.016),
+    # far apart pixels: 32 vectors reach more bins than the staging holds, and the batch is halved
+    ((40, 36, 44, 38, 33), (20, 40, 100.0, 4.0), (2.0, 20.0), 0.0028),
+    # every pixel of a forest in the window
+    ((40, 33, 130, 20, 64), (7, 3, 300.0, 6.0), (0.3, 3.7), 0.004),
+])
+def test_dmat_windows_and_batches(api, handle, lengths, bins, step, patch):
+    """Pixels at random spacings, so that neighbouring vectors visit different bins.  Allowance as above."""
+    rng = np.random.default_rng(sum(lengths))
+    fs = [(*rng.uniform(0, patch, 2), 500.0 + rng.uniform(0, 20) + np.cumsum(rng.uniform(*step, n)),
+           8.2 + np.cumsum(rng.uniform(1e-4, 6e-4, n)), rng.standard_normal(n), rng.uniform(0.5, 2.0, n))
+          for n in lengths]
+    cat = line_catalog(fs)
+    b = synth.Bins(*bins)
+    pr = oracle.pairs.forest_pairs(cat, b)
+    fwd = oracle.xi.xi_sums(cat, b, pr, eps_edge=6e-5)
+    ref = oracle.dmat.dmat(cat, b, pr, processes=0, eps_edge=6e-5)
+    D, w = api.lya_dmat(handle, api.DeviceCatalog.from_host(cat), b, 1.0, 3)
+    api.lya_sync_status(handle)
+    W, E, R = fwd["wsum"], fwd["edge_w"], ref["dmat"]
+    den = (W - E)[:, None]
+    edge = np.divide(ref["edge_d"] + np.abs(R) * E[:, None], den, out=np.zeros_like(R), where=den > 0)
+    assert np.all(np.abs(D.cpu().numpy() - R) <= 1e-5 * np.abs(R).max(axis=1)[:, None] + edge + 1e-12)
+    assert np.all(np.abs(w.cpu().numpy() - W) <= 1e-6 * W + E + 1e-9)
+
+
 @pytest.mark.parametrize("lengths,n_qso,bins,seed", [
     ((1, 2, 31, 32, 33), 40, (10, 8, 60.0, 40.0), 31),          # edges of a warp's window step
     ((300, 700, 90), 90, (100, 50, 200.0, 200.0), 32),          # teams of several warps
