@@ -8,7 +8,9 @@
 // r1 and r2.  Every pixel is a main vertex, the other two pixels take
 // (r1, r2) in both orders, and a record needs |r1|, |r2| < r_max.
 //
-// One block per main-vertex pixel (work taken from an atomic counter):
+// Two kernels with the same arithmetic: xi3_group_kernel (several vertices a block,
+// sums of a class in shared memory; see there) where it pays, and xi3_kernel: one
+// block per main-vertex pixel (work taken from an atomic counter):
 //  1. gather: for every forest in the vertex forest's neighbour list, the chord
 //     of pixels within r_max of the vertex (a contiguous range of the sorted
 //     distances, one forest per lane), then the chords' pixels, one per thread:
@@ -26,7 +28,7 @@
 // shared-memory capacity is sized to them; a vertex with more neighbours than
 // one block can hold raises a device flag (reported as LYA_ERR_TOO_LARGE)
 // instead of being truncated silently.
-// What bounds it: the FP64 atomics in L2, which takes one 32-byte sector per
+// What bounds xi3_kernel: the FP64 atomics in L2, which takes one 32-byte sector per
 // 2.3 clocks and SM wherever the bins are random; N and W of a bin therefore
 // lie side by side and two lanes add a record, so a record costs one sector and
 // not two.  Measured (5,000 SDSS-like forests, r_max 40, 200,000 bins): 411 ms
@@ -35,7 +37,8 @@
 #include <algorithm>
 #include <math.h>
 
-#include "lya_internal.cuh"
+#include "exact.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
@@ -121,6 +124,64 @@ __device__ __forceinline__ Chord chord(const X3Args& A, int f, int o, double di,
   return c;
 }
 
+// Bins of a neighbour pixel: |r| and the angle to the vertex's line of sight,
+// from FP32, and near a bin edge from the definition in FP64.
+struct X3Bin {
+  double rmax2, inv_dr, inv_dt;
+  float inv_dr_f, inv_dt_f, guard_r, guard_t;
+  int nr, nt;
+  // pixel p of forest o against the vertex at x with line of sight u: false beyond r_max
+  __device__ __forceinline__ bool candidate(const X3Args& A, int o, int64_t p, const double* x, const double* u,
+                                            float4* r4, int* ir, int* it) const {
+    const double dj = A.dist[p];
+    const double dx = dj * A.F.ux[o] - x[0], dy = dj * A.F.uy[o] - x[1], dz = dj * A.F.uz[o] - x[2];
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    if (!(r2 < rmax2 && r2 > 0.0)) return false;
+    // 1 / |r| to 2e-14: one Newton step from FP32 (an FP64 square root and division cost 20 times that)
+    const float r2f = static_cast<float>(r2);
+    const float y0f = rsqrtf(r2f);
+    const double y0 = y0f;
+    const double y = fma(0.5 * y0, fma(-(r2 * y0), y0, 1.0), y0);
+    const double dot = dx * u[0] + dy * u[1] + dz * u[2];
+    const float ctf = static_cast<float>(dot * y);
+    const float fr = r2f * y0f * inv_dr_f, ft = acosf(fminf(1.f, fmaxf(-1.f, ctf))) * inv_dt_f;
+    const float gr = fr - floorf(fr), gt = ft - floorf(ft);
+    int jr = static_cast<int>(fr), jt = static_cast<int>(ft);
+    const bool sure = r2f > 1e-30f && fabsf(gr - 0.5f) < 0.5f - guard_r && fabsf(gt - 0.5f) < 0.5f - guard_t &&
+                      fabsf(ctf) <= 0.9999f;
+    if (!sure) {   // the definition, near a bin edge
+      const double r = sqrt(r2);
+      const double ct = dot / r;
+      jr = static_cast<int>(r * inv_dr);
+      jt = static_cast<int>(acos(fmin(1.0, fmax(-1.0, ct))) * inv_dt);
+      r4->w = static_cast<float>(1.0 / r);
+    } else {
+      r4->w = static_cast<float>(y);
+    }
+    r4->x = static_cast<float>(dx);
+    r4->y = static_cast<float>(dy);
+    r4->z = static_cast<float>(dz);
+    *ir = min(jr, nr - 1);
+    *it = min(jt, nt - 1);
+    return true;
+  }
+};
+__device__ __forceinline__ X3Bin x3_bin(const X3Args& A) {
+  X3Bin b;
+  b.rmax2 = A.r_max * A.r_max;
+  b.inv_dr = A.n_r / A.r_max;
+  b.inv_dt = A.n_theta / M_PI;
+  b.inv_dr_f = static_cast<float>(b.inv_dr);
+  b.inv_dt_f = static_cast<float>(b.inv_dt);
+  // FP32 errors of |r| and theta in bins, doubled: |r| n_r / r_max <= n_r is good to 4 roundings; theta =
+  // acos(c) to 5e-6 rad where |c| <= 0.9999 (the FP32 rounding of c over sin theta, and of acosf)
+  b.guard_r = 1e-6f * static_cast<float>(A.n_r) + 1e-6f;
+  b.guard_t = 1e-5f * b.inv_dt_f + 1e-6f;
+  b.nr = A.n_r;
+  b.nt = A.n_theta;
+  return b;
+}
+
 __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int32_t* nbr, const int64_t* nstart,
                                                          int cap, double* sums, unsigned long long* counter, unsigned* err) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -131,12 +192,8 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
   __shared__ long long s_item;
   __shared__ int s_o[kX3Batch], s_lo[kX3Batch], s_pre[kX3Batch + 1];   // chords of a batch of neighbours
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = blockDim.x >> 5;
-  const double rmax = A.r_max, rmax2 = rmax * rmax;
-  const double inv_dr = A.n_r / rmax, inv_dt = A.n_theta / M_PI;
-  const float inv_dr_f = static_cast<float>(inv_dr), inv_dt_f = static_cast<float>(inv_dt);
-  // FP32 errors of |r| and theta in bins, doubled: |r| n_r / r_max <= n_r is good to 4 roundings; theta =
-  // acos(c) to 5e-6 rad where |c| <= 0.9999 (the FP32 rounding of c over sin theta, and of acosf)
-  const float guard_r = 1e-6f * static_cast<float>(A.n_r) + 1e-6f, guard_t = 1e-5f * inv_dt_f + 1e-6f;
+  const double rmax2 = A.r_max * A.r_max;
+  const X3Bin bin3 = x3_bin(A);
   const float half_na = 0.5f * static_cast<float>(A.n_alpha);
   const int nr = A.n_r, nt = A.n_theta, na = A.n_alpha;
   for (;;) {
@@ -155,7 +212,7 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
     if (i_in >= A.F.len[f]) continue;    // pixel of a forest that failed the input checks
     const double nax = A.F.ux[f], nay = A.F.uy[f], naz = A.F.uz[f];
     const double di = A.dist[g];
-    const double xi = di * nax, yi = di * nay, zi = di * naz;
+    const double xv[3] = {di * nax, di * nay, di * naz}, uv[3] = {nax, nay, naz};
     const Pix pv = A.pix[g];
     const float w_i = pv.y, wd_i = pv.z;
     // 1. gather the vertex's neighbours within r_max: the chords of up to 64
@@ -201,37 +258,11 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
           }
           o = s_o[lo];
           const int64_t p = A.F.off[o] + s_lo[lo] + (k - s_pre[lo]);
-          const double dj = A.dist[p];
-          const double dx = dj * A.F.ux[o] - xi, dy = dj * A.F.uy[o] - yi, dz = dj * A.F.uz[o] - zi;
-          const double r2 = dx * dx + dy * dy + dz * dz;
-          in = r2 < rmax2 && r2 > 0.0;
+          int ir, it;
+          in = bin3.candidate(A, o, p, xv, uv, &r4, &ir, &it);
           if (in) {
             q = A.pix[p];
-            // 1 / |r| to 2e-14: one Newton step from FP32 (an FP64 square root and division cost 20 times that)
-            const float r2f = static_cast<float>(r2);
-            const float y0f = rsqrtf(r2f);
-            const double y0 = y0f;
-            const double y = fma(0.5 * y0, fma(-(r2 * y0), y0, 1.0), y0);
-            const double dot = dx * nax + dy * nay + dz * naz;
-            const float ctf = static_cast<float>(dot * y);
-            const float fr = r2f * y0f * inv_dr_f, ft = acosf(fminf(1.f, fmaxf(-1.f, ctf))) * inv_dt_f;
-            const float gr = fr - floorf(fr), gt = ft - floorf(ft);
-            int ir = static_cast<int>(fr), it = static_cast<int>(ft);
-            const bool sure = r2f > 1e-30f && fabsf(gr - 0.5f) < 0.5f - guard_r && fabsf(gt - 0.5f) < 0.5f - guard_t &&
-                              fabsf(ctf) <= 0.9999f;
-            if (!sure) {   // the definition, near a bin edge
-              const double r = sqrt(r2);
-              const double ct = dot / r;
-              ir = static_cast<int>(r * inv_dr);
-              it = static_cast<int>(acos(fmin(1.0, fmax(-1.0, ct))) * inv_dt);
-              r4.w = static_cast<float>(1.0 / r);
-            } else {
-              r4.w = static_cast<float>(y);
-            }
-            r4.x = static_cast<float>(dx);
-            r4.y = static_cast<float>(dy);
-            r4.z = static_cast<float>(dz);
-            key = (min(ir, nr - 1) << 16) | min(it, nt - 1);
+            key = (ir << 16) | it;
           }
         }
         const unsigned msk = __ballot_sync(0xffffffffu, in);
@@ -296,14 +327,437 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
   }
 }
 
-// largest number of pixels on any main vertex's chords (an upper bound of its
-// neighbours within r_max, 1e-2 Mpc/h wider), one warp per vertex pixel
-__global__ void xi3_count_kernel(X3Args A, const int32_t* nbr, const int64_t* nstart, int* max_count) {
+// ----------------------------------------------------------------------------
+// Several main vertices per block: their records of one (r1, r2) class, whose
+// n_alpha n_theta^2 bins fit in shared memory, are summed there before they go
+// to the FP64 bin sums, so L2 sees one reduction per touched bin, group of
+// vertices and sum instead of one per record.
+//  * The block takes kXGVerts consecutive pixels, finds the chords of all of them
+//    at once (a warp per vertex), and gathers as many of them as its list holds;
+//    the list is then counting-sorted by (vertex, |r| bin).
+//  * A class (r1 <= r2) is walked by all warps: 16 neighbours q of bin r2 in the
+//    half-warps' registers against two neighbours p of bin r1 a step; steps are
+//    dealt evenly over the warps.
+//  * Sums are exact integers in two words of 16 to 20 bits of a record's value (as
+//    many as leave room for all records of the class), 32 to 40 bits below the
+//    group's largest product, which shared memory adds natively.  A class with
+//    few records (below kXGDirect a bin) or more than a word can hold, and a
+//    group whose products leave the scales, adds its records to L2 as
+//    xi3_kernel does; with two blocks per SM the one's reductions in L2 run
+//    beside the other's in shared memory.
+// What bounds it: the shared-memory pipe (four reductions a record, 25 of 32
+// lanes on random bins) and L2's atomics.  Measured (5,000 SDSS-like forests,
+// r_max 40, 200,000 bins): xi3_kernel 204 ms,
+// this 158 ms; three words 227 ms, one block of 1,024 threads per SM 171 ms, no
+// direct classes 185 ms, kXGDirect 3, 12, 20: 160, 161, 186 ms; 64-bit words 449
+// ms (emulated).  Smaller grids gain more: 13 x 6^2 bins of 100 classes, 1,300
+// forests of a denser sky: 163 -> 54 ms.
+// ----------------------------------------------------------------------------
+constexpr int kXGThreads = 512;
+constexpr int kXGSmem = 113 * 1024;   // shared memory of a block: two per SM
+constexpr int kXGVerts = 8;     // vertices a work item
+constexpr int kXGBatch = 96;     // most neighbour forests of a vertex
+constexpr int kXGMaxR = 16;      // most |r| bins
+constexpr int kXGMove = 4;       // list entries a thread moves in the sort (list <= 2,048)
+constexpr int kXGClasses = kXGMaxR * (kXGMaxR + 1) / 2;
+constexpr double kXGGain = 0.5;  // see x3_group_cap
+constexpr int kXGDirect = 6;     // records a bin below which a class goes to L2
+constexpr int kXGWords = 5;      // words of a bin: N and W in 2 each, and an odd stride
+
+struct XGLay {
+  int cr, cw, ck, hist, ch, end;
+};
+__host__ __device__ inline XGLay xg_layout(int cap, int nbc) {
+  XGLay y;
+  int o = 0;
+  y.cr = o; o += cap * 16;
+  y.cw = o; o += cap * 8;
+  y.ck = o; o += cap * 8;
+  y.hist = o; o += (nbc * kXGWords * 4 + 15) & ~15;
+  y.ch = o; o += kXGVerts * (3 * kXGBatch + 1) * 4;
+  y.end = o;
+  return y;
+}
+
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float(static_cast<uint32_t>(e + 127) << 23); }
+
+// steps of a class for one vertex: tiles of 16 q, two p a step; within one |r|
+// bin (same) tile t meets the p below its end only
+__device__ __forceinline__ int xg_steps(int np, int nq, bool same) {
+  if (np == 0 || nq == 0) return 0;
+  if (!same) return ((nq + 15) >> 4) * ((np + 1) >> 1);
+  const int T = (nq + 15) >> 4;
+  return nq < 2 ? 0 : 4 * T * (T - 1) + ((nq + 1) >> 1);
+}
+
+__global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, const int32_t* nbr, const int64_t* nstart,
+                                                                  int cap, double* sums, unsigned long long* counter,
+                                                                  unsigned* err) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ long long s_item;
+  __shared__ double s_x[kXGVerts][3], s_u[kXGVerts][3];
+  __shared__ float2 s_w[kXGVerts];                       // (w delta, w) of the vertex
+  __shared__ int s_f[kXGVerts], s_nb[kXGVerts], s_tot[kXGVerts];
+  __shared__ int s_n, s_wd, s_ww;                        // list length, largest |w delta| and w of the list (bits)
+  __shared__ int s_st[kXGVerts * kXGMaxR + 1], s_pos[kXGVerts * kXGMaxR];
+  __shared__ int s_steps[kXGClasses], s_recs[kXGClasses];
+  __shared__ int s_e[2];                                 // every |product| is below 2^e; 999: beyond the scales
+  const int nr = A.n_r, nt = A.n_theta, na = A.n_alpha, nbc = na * nt * nt, ncls = nr * (nr + 1) / 2;
+  const XGLay y = xg_layout(cap, nbc);
+  float4* cr = reinterpret_cast<float4*>(sm + y.cr);     // r (FP32) and 1 / |r|
+  float2* cw = reinterpret_cast<float2*>(sm + y.cw);     // (w delta, w)
+  int2* ck = reinterpret_cast<int2*>(sm + y.ck);         // ((vertex << 24) | (|r| bin << 16) | theta bin, forest)
+  unsigned* hist = reinterpret_cast<unsigned*>(sm + y.hist);
+  int* s_o = reinterpret_cast<int*>(sm + y.ch);          // chords: forest, first pixel, exclusive counts
+  int* s_lo = s_o + kXGVerts * kXGBatch;
+  int* s_pre = s_lo + kXGVerts * kXGBatch;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  constexpr int nwarps = kXGThreads / 32;
+  const double rmax2 = A.r_max * A.r_max;
+  const X3Bin bin = x3_bin(A);
+  const float half_na = 0.5f * static_cast<float>(na);
+  for (int k = tid; k < nbc * kXGWords; k += kXGThreads) hist[k] = 0u;
+  for (;;) {
+    __syncthreads();
+    if (wid == 0) {
+      long long it = 0;
+      if (lane == 0) it = static_cast<long long>(atomicAdd(counter, static_cast<unsigned long long>(kXGVerts)));
+      it = __shfl_sync(0xffffffffu, it, 0);
+      if (lane == 0) s_item = it;
+      if (lane < kXGVerts) {
+        const long long g = it + lane;
+        int f = -1;
+        if (g < A.n_pix) {
+          f = forest_of(A.F, g);
+          if (g - A.F.off[f] >= A.F.len[f]) f = -1;    // pixel of a forest that failed the input checks
+        }
+        s_f[lane] = f;
+        if (f >= 0) {
+          const double d = A.dist[g], ux = A.F.ux[f], uy = A.F.uy[f], uz = A.F.uz[f];
+          s_u[lane][0] = ux; s_u[lane][1] = uy; s_u[lane][2] = uz;
+          s_x[lane][0] = d * ux; s_x[lane][1] = d * uy; s_x[lane][2] = d * uz;
+          const Pix p = A.pix[g];
+          s_w[lane] = make_float2(p.z, p.y);
+        }
+      }
+    }
+    __syncthreads();
+    if (s_item >= A.n_pix) break;
+    for (int v = wid; v < kXGVerts; v += nwarps) {
+      const int f = s_f[v];
+      const int nb = (f < 0) ? 0 : static_cast<int>(min(nstart[f + 1] - nstart[f], static_cast<int64_t>(kXGBatch)));
+      const double di = (f < 0) ? 0.0 : A.dist[s_item + v];
+      int carry = 0;
+      if (lane == 0) s_pre[v * (kXGBatch + 1)] = 0;
+      for (int m0 = 0; m0 < nb; m0 += 32) {
+        const int m = m0 + lane;
+        int cnt = 0;
+        if (m < nb) {
+          const int o = nbr[nstart[f] + m];
+          const Chord c = chord(A, f, o, di, rmax2);
+          s_o[v * kXGBatch + m] = o;
+          s_lo[v * kXGBatch + m] = c.lo;
+          cnt = c.hi - c.lo;
+        }
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int up = __shfl_up_sync(0xffffffffu, cnt, d);
+          if (lane >= d) cnt += up;
+        }
+        cnt += carry;
+        if (m < nb) s_pre[v * (kXGBatch + 1) + m + 1] = cnt;
+        carry = __shfl_sync(0xffffffffu, cnt, 31);
+      }
+      if (lane == 0) {
+        s_nb[v] = nb;
+        s_tot[v] = carry;
+      }
+    }
+    __syncthreads();
+    int v1 = 0;
+    for (int v0 = 0; v0 < kXGVerts; v0 = v1) {
+      // the next vertices whose chords fit the list (a single vertex's always do)
+      int sum = 0;
+      for (v1 = v0; v1 < kXGVerts && sum + s_tot[v1] <= cap; ++v1) sum += s_tot[v1];
+      if (v1 == v0) {   // cannot happen: cap is at least the longest
+        if (tid == 0) atomicOr(err, FLAG_X3_CAP);
+        v1 = v0 + 1;
+        continue;
+      }
+      const int nkey = (v1 - v0) * nr;
+      for (int k = tid; k < nkey; k += kXGThreads) s_pos[k] = 0;
+      if (tid == 0) {
+        s_n = 0;
+        s_wd = 0;
+        s_ww = 0;
+      }
+      __syncthreads();
+      // gather, 32 candidates a warp
+      int before = 0, mwd = 0, mww = 0;
+      for (int v = v0; v < v1; ++v) {
+        const int tot = s_tot[v], units = (tot + 31) >> 5;
+        const int* pre = s_pre + v * (kXGBatch + 1);
+        for (int u = (wid - before) & (nwarps - 1); u < units; u += nwarps) {
+          const int k = 32 * u + lane;
+          bool in = false;
+          float4 r4 = make_float4(0.f, 0.f, 0.f, 0.f);
+          Pix q = r4;
+          int key = 0, o = 0;
+          if (k < tot) {
+            int lo = 0, hi = s_nb[v] - 1;   // neighbour whose pixels hold candidate k: the last with pre <= k
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (pre[mid] <= k) lo = mid; else hi = mid - 1;
+            }
+            o = s_o[v * kXGBatch + lo];
+            const int64_t p = A.F.off[o] + s_lo[v * kXGBatch + lo] + (k - pre[lo]);
+            int ir, it;
+            in = bin.candidate(A, o, p, s_x[v], s_u[v], &r4, &ir, &it);
+            if (in) {
+              q = A.pix[p];
+              key = ((v - v0) << 24) | (ir << 16) | it;
+              mwd = max(mwd, __float_as_int(fabsf(q.z)));
+              mww = max(mww, __float_as_int(fabsf(q.y)));
+              atomicAdd(&s_pos[(v - v0) * nr + ir], 1);
+            }
+          }
+          const unsigned msk = __ballot_sync(0xffffffffu, in);
+          int slot = 0;
+          if (lane == 0 && msk) slot = atomicAdd(&s_n, __popc(msk));
+          slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(msk & ((1u << lane) - 1u));
+          if (in) {   // slot < cap: the chords' pixels fit
+            cr[slot] = r4;
+            cw[slot] = make_float2(q.z, q.y);
+            ck[slot] = make_int2(key, o);
+          }
+        }
+        before += units;
+      }
+      mwd = __reduce_max_sync(0xffffffffu, mwd);
+      mww = __reduce_max_sync(0xffffffffu, mww);
+      if (lane == 0) {
+        atomicMax(&s_wd, mwd);
+        atomicMax(&s_ww, mww);
+      }
+      __syncthreads();
+      // bucket starts (warp 0), scales (warp 1)
+      if (wid == 0) {
+        int carry = 0;
+        for (int k0 = 0; k0 < nkey; k0 += 32) {
+          const int k = k0 + lane;
+          const int c = (k < nkey) ? s_pos[k] : 0;
+          int x = c;
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += up;
+          }
+          if (k < nkey) {
+            s_st[k] = carry + x - c;
+            s_pos[k] = carry + x - c;
+          }
+          carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) s_st[nkey] = carry;
+      } else if (wid == 1 && lane < 2) {
+        float vm = 0.f;
+        for (int v = v0; v < v1; ++v)
+          if (s_f[v] >= 0) vm = fmaxf(vm, fabsf(lane ? s_w[v].y : s_w[v].x));
+        const float m = __int_as_float(lane ? s_ww : s_wd);
+        const float B = m * m * vm * 2.001f;   // |product| of any record, mirror weight included
+        const int e = static_cast<int>((__float_as_uint(B) >> 23) & 0xFFu) - 126;
+        s_e[lane] = (B == 0.f) ? 0 : (B > 1e-25f && B < 1e30f) ? e : 999;
+      }
+      __syncthreads();
+      // sort the list by (vertex, |r| bin): places first, then the fields; the
+      // classes' steps and records meanwhile
+      const int n = s_n;
+      {
+        int pos[kXGMove];
+        float4 mr[kXGMove];
+#pragma unroll
+        for (int e = 0; e < kXGMove; ++e) {
+          const int k = tid + e * kXGThreads;
+          pos[e] = -1;
+          if (k < n) {
+            const int key = ck[k].x;
+            pos[e] = atomicAdd(&s_pos[(key >> 24) * nr + ((key >> 16) & 0xff)], 1);
+            mr[e] = cr[k];
+          }
+        }
+        for (int c = tid; c < ncls; c += kXGThreads) {
+          int ra = 0, left = c;
+          while (left >= nr - ra) {
+            left -= nr - ra;
+            ++ra;
+          }
+          const int rb = ra + left;
+          int steps = 0, recs = 0;
+          for (int v = 0; v < v1 - v0; ++v) {
+            const int np = s_st[v * nr + ra + 1] - s_st[v * nr + ra], nq = s_st[v * nr + rb + 1] - s_st[v * nr + rb];
+            steps += xg_steps(np, nq, ra == rb);
+            recs += (ra == rb) ? nq * (nq - 1) / 2 : np * nq;
+          }
+          s_steps[c] = steps;
+          s_recs[c] = recs;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < kXGMove; ++e)
+          if (pos[e] >= 0) cr[pos[e]] = mr[e];
+        float2 mw[kXGMove];
+        int2 mk[kXGMove];
+#pragma unroll
+        for (int e = 0; e < kXGMove; ++e) {
+          const int k = tid + e * kXGThreads;
+          if (k < n) {
+            mw[e] = cw[k];
+            mk[e] = ck[k];
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < kXGMove; ++e)
+          if (pos[e] >= 0) {
+            cw[pos[e]] = mw[e];
+            ck[pos[e]] = mk[e];
+          }
+      }
+      __syncthreads();
+      const int en = s_e[0], ew = s_e[1];
+      const F2 M2 = f2(kM15, kM15), neg2 = f2(-1.f, -1.f);
+      int cls = 0;
+      for (int ra = 0; ra < nr; ++ra) {
+        for (int rb = ra; rb < nr; ++rb, ++cls) {
+          const int S = s_steps[cls];
+          if (S == 0) continue;
+          const bool same = ra == rb;
+          // bits of a word: its sum over the class's records stays below 2^32
+          const int recs = s_recs[cls], bits = min(20, __clz(recs));
+          const bool direct = max(en, ew) > 900 || bits < 16 || recs < kXGDirect * nbc;
+          const F2 sc2 = f2(pow2f(bits - 1 - en), pow2f(bits - 1 - ew)), up2 = f2(pow2f(bits), pow2f(bits));
+          double* const base = sums + 2 * (static_cast<int64_t>(ra * nr + rb) * nbc);
+          int b = static_cast<int>(static_cast<int64_t>(S) * wid / nwarps);
+          int left = static_cast<int>(static_cast<int64_t>(S) * (wid + 1) / nwarps) - b;
+          int v = -1, np = 0, nq = 0, p0 = 0, q0 = 0, t = 0;
+          // step b of the class: vertex v, tile t, step k of the tile
+          int k = b;
+          bool find = true;
+          while (left > 0) {
+            if (find) {
+              for (;;) {
+                ++v;
+                p0 = s_st[v * nr + ra];
+                np = s_st[v * nr + ra + 1] - p0;
+                q0 = s_st[v * nr + rb];
+                nq = s_st[v * nr + rb + 1] - q0;
+                const int sv = xg_steps(np, nq, same);
+                if (k < sv) break;
+                k -= sv;
+              }
+              t = 0;
+              find = false;
+            }
+            const int lim = same ? min(np, 16 * (t + 1)) : np;
+            const int ks = (lim + 1) >> 1;
+            if (k >= ks) {
+              k -= ks;
+              ++t;
+              continue;
+            }
+            const int ql = 16 * t + (lane & 15);
+            const bool qv = ql < nq;
+            const int q = q0 + min(ql, nq - 1);
+            const float4 rq = cr[q];
+            const float2 wq = cw[q], wv = s_w[v0 + v];
+            const int2 kq = ck[q];
+            const float wdq = wq.x * wv.x, wwq = wq.y * wv.y;
+            const int tq = kq.x & 0xffff;
+            const int m = min(ks - k, left);
+            left -= m;
+            for (int e = 0; e < m; ++e, ++k) {
+              const int pl = 2 * k + (lane >> 4);
+              const int p = p0 + min(pl, np - 1);
+              const float4 rp = cr[p];
+              const float2 wp = cw[p];
+              const int2 kp = ck[p];
+              const bool on = qv && pl < lim && (!same || pl < ql) && kp.y != kq.y;
+              const float ca = (rp.x * rq.x + rp.y * rq.y + rp.z * rq.z) * (rp.w * rq.w);
+              const int ia = min(max(static_cast<int>(floorf((ca + 1.0f) * half_na)), 0), na - 1);
+              const int tp = kp.x & 0xffff;
+              int t1 = tp, t2 = tq;
+              float mult = 1.f;
+              if (same) {
+                t1 = min(tp, tq);
+                t2 = max(tp, tq);
+                mult = (tp == tq) ? 2.f : 1.f;
+              }
+              const int l = (ia * nt + t1) * nt + t2;
+              const float vn = wp.x * wdq * mult, vw = wp.y * wwq * mult;
+              if (direct) {
+                const int bb = on ? l : -1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  const int src = (lane >> 1) + 16 * h;
+                  const int b2 = __shfl_sync(0xffffffffu, bb, src);
+                  const float n2 = __shfl_sync(0xffffffffu, vn, src), w2 = __shfl_sync(0xffffffffu, vw, src);
+                  if (b2 >= 0) red_add_f64_global(base + 2 * static_cast<int64_t>(b2) + (lane & 1), static_cast<double>((lane & 1) ? w2 : n2));
+                }
+              } else if (on) {
+                // floor(q) and the rest, rounded, in units of 2^-bits
+                const F2 v2 = f2(vn, vw);
+                const F2 hm = fma2_rd(v2, sc2, M2);
+                const F2 lm = fma2(fma2(v2, sc2, fma2(hm, neg2, M2)), up2, M2);
+                const float2 h = unf2(hm), lo = unf2(lm);
+                unsigned* w = hist + l * kXGWords;
+                atomicAdd(w + 0, __float_as_uint(h.x) - kM15Bits);
+                atomicAdd(w + 1, __float_as_uint(lo.x) - kM15Bits);
+                atomicAdd(w + 2, __float_as_uint(h.y) - kM15Bits);
+                atomicAdd(w + 3, __float_as_uint(lo.y) - kM15Bits);
+              }
+            }
+            if (k == ks) {
+              k = 0;
+              ++t;
+            }
+            if (16 * t >= nq) find = true;
+          }
+          if (!direct) {
+            __syncthreads();
+            const double inv = pow2(1 - 2 * bits + ((tid & 1) ? ew : en));
+            for (int k2 = tid; k2 < 2 * nbc; k2 += kXGThreads) {
+              unsigned* w = hist + (k2 >> 1) * kXGWords + 2 * (k2 & 1);
+              const unsigned h = w[0], lo = w[1];
+              if ((h | lo) != 0u) {
+                const long long x = (static_cast<long long>(static_cast<int>(h)) << bits) + lo;
+                if (x != 0) red_add_f64_global(base + k2, static_cast<double>(x) * inv);
+                w[0] = 0u;
+                w[1] = 0u;
+              }
+            }
+            __syncthreads();
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+struct X3Count {
+  unsigned long long total;   // pixels on the chords of all vertices
+  int most, degree;           // of any vertex; most neighbour forests of one
+};
+
+// pixels on every main vertex's chords (an upper bound of its neighbours within
+// r_max, 1e-2 Mpc/h wider): the longest and the sum, one warp per vertex pixel
+__global__ void xi3_count_kernel(X3Args A, const int32_t* nbr, const int64_t* nstart, X3Count* out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const double rmax2 = A.r_max * A.r_max;
   int best = 0;
+  unsigned long long total = 0, degree = 0;
   for (int64_t g = warp; g < A.n_pix; g += nw) {
     const int f = forest_of(A.F, g);
     if (g - A.F.off[f] >= A.F.len[f]) continue;
@@ -312,9 +766,16 @@ __global__ void xi3_count_kernel(X3Args A, const int32_t* nbr, const int64_t* ns
       const Chord c = chord(A, f, nbr[e], A.dist[g], rmax2);
       cnt += c.hi - c.lo;
     }
-    best = max(best, __reduce_add_sync(0xffffffffu, cnt));
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    best = max(best, cnt);
+    total += cnt;
+    degree = max(degree, static_cast<unsigned long long>(nstart[f + 1] - nstart[f]));
   }
-  if (lane == 0 && best > 0) atomicMax(max_count, best);
+  if (lane == 0 && best > 0) {
+    atomicMax(&out->most, best);
+    atomicMax(&out->degree, static_cast<int>(min(degree, 0x7fffffffull)));
+    atomicAdd(&out->total, total);
+  }
 }
 
 // num, wsum and xi of every bin: the sums of its canonical bin (side-1 key <=
@@ -351,6 +812,26 @@ int grid_for(int64_t n, int threads) {
     if (e_ != cudaSuccess) return e_; \
   } while (0)
 
+// List length of the grouped kernel, or 0 where xi3_kernel is the better or the
+// only one: the (r1, r2) class has to leave room in shared memory for a list of
+// every vertex's neighbours, and a group's records (at most mean^2 / 2 a vertex)
+// have to reach half the number of canonical bins (half of all), which are walked
+// once a group.  Both kernels, against that ratio: 0.16: 8.0 against 6.8 ms for
+// xi3_kernel; 0.29: 4.9 against 5.2; 0.37: 10.3 against 10.1; 1.4: 3.5 against
+// 4.8; 2.2: 158 against 204; 3.3: 23.7 against 63 ms.
+int x3_group_cap(const X3Args& a, const DevInfo& dev, const X3Count& c) {
+  const int64_t nbc = static_cast<int64_t>(a.n_alpha) * a.n_theta * a.n_theta;
+  if (a.n_r > kXGMaxR || a.n_theta > 0xffff || c.degree > kXGBatch || c.most < 1 || nbc > 7000) return 0;
+  // two blocks per SM (1 KB of each reserved), less 6 KB for the static arrays
+  const int room = std::min(dev.smem_optin, kXGSmem) - 6144 - xg_layout(0, static_cast<int>(nbc)).end;
+  const int cap = std::min(room / 32 & ~3, kXGMove * kXGThreads);
+  if (cap < c.most) return 0;
+  const double mean = static_cast<double>(c.total) / static_cast<double>(std::max<int64_t>(a.n_pix, 1));
+  const double verts = std::min<double>(kXGVerts, cap / std::max(mean, 1.0));
+  const double records = verts * mean * mean / 2, bins = 0.5 * a.n_r * a.n_r * static_cast<double>(nbc);
+  return records >= kXGGain * bins ? cap : 0;
+}
+
 }  // namespace
 
 cudaError_t run_xi3(const X3Args& a, const DevInfo& dev, void** scratch, size_t* scratch_cap, unsigned* err,
@@ -385,13 +866,24 @@ cudaError_t run_xi3(const X3Args& a, const DevInfo& dev, void** scratch, size_t*
   // pass, synchronising); a list beyond one block's shared memory is reported,
   // not truncated
   const int per_cand = 32;
-  int* dmax = reinterpret_cast<int*>(sc + o_misc + 64);
-  LYA_TRY(cudaMemsetAsync(dmax, 0, 4, s));
+  X3Count* dcount = reinterpret_cast<X3Count*>(sc + o_misc + 64);
+  LYA_TRY(cudaMemsetAsync(dcount, 0, sizeof(X3Count), s));
   if (a.n_pix > 0 && nf > 0)
-    LYA_COUNT(1), xi3_count_kernel<<<dev.sms * 8, 256, 0, s>>>(a, nbr, start, dmax);
-  int hmax = 0;
-  LYA_TRY(cudaMemcpyAsync(&hmax, dmax, 4, cudaMemcpyDeviceToHost, s));
+    LYA_COUNT(1), xi3_count_kernel<<<dev.sms * 8, 256, 0, s>>>(a, nbr, start, dcount);
+  X3Count count{};
+  LYA_TRY(cudaMemcpyAsync(&count, dcount, sizeof(count), cudaMemcpyDeviceToHost, s));
   LYA_TRY(cudaStreamSynchronize(s));
+  const int hmax = count.most;
+  const int gcap = x3_group_cap(a, dev, count);
+  if (gcap > 0) {
+    const int smem = xg_layout(gcap, a.n_alpha * a.n_theta * a.n_theta).end;
+    LYA_TRY(set_max_dynamic_smem(reinterpret_cast<const void*>(xi3_group_kernel), smem));
+    LYA_COUNT(1), xi3_group_kernel<<<2 * dev.sms, kXGThreads, smem, s>>>(a, nbr, start, gcap, sums, counter, err);
+    LYA_TRY(cudaGetLastError());
+    LYA_COUNT(1), xi3_finalize_kernel<<<grid_for(nbins, 256), 256, 0, s>>>(sums, a.num, a.wsum, a.xi, a.n_r, a.n_theta,
+                                                                          a.n_alpha);
+    return cudaGetLastError();
+  }
   const int cap_max = (dev.smem_optin - 1024) / per_cand;
   const int cap = std::max(std::min(hmax, cap_max), 256);
   const int smem = cap * per_cand;

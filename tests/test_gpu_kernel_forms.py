@@ -210,3 +210,26 @@ def test_xcf_forms(api, handle, lengths, n_qso, bins, seed):
     assert np.all(np.abs(w - ref["wsum"]) <= 1e-6 * ref["wsum"] + ref["edge_w"])
     top = float(np.abs(cat.delta).max())
     assert np.all(np.abs(n - ref["num"]) <= 1e-6 * top * ref["wsum"] + ref["edge_n"] + 1e-300)
+
+
+@pytest.mark.parametrize("n_r,n_alpha,n_theta,nf,factor", [
+    (4, 5, 3, 14, 1.0),      # classes summed in shared memory
+    (16, 1, 1, 14, 1.0),     # the most |r| bins
+    (1, 3, 2, 24, 1.0),      # one class, more records than a word holds
+    (4, 5, 3, 14, 1e9),      # products beyond the fixed-point scale
+    (4, 5, 3, 14, 0.0),      # all weights zero
+])
+def test_xi3_grouped_vertices(api, handle, n_r, n_alpha, n_theta, nf, factor):
+    """Grids with fewer bins than a group of vertices has records.  Tolerances as in test_gpu_xi3."""
+    spec = synth.Spec(n_forests=nf, seed=8, region="box", box_deg=0.3, grid="log10", delta_sigma=0.2)
+    cat = synth.generate(spec)
+    cat.weight[:] *= np.float32(factor)
+    g = oracle.xi3.Grid3(n_r=n_r, n_theta=n_theta, n_alpha=n_alpha, r_max=15.0)
+    num, wsum, xi = api.lya_xi3(handle, api.DeviceCatalog.from_host(cat), g)
+    api.lya_sync_status(handle)
+    ref = oracle.xi3.xi3_sums(cat, g, eps_r=1e-9, eps_c=2e-6)
+    W, N, unit = wsum.cpu().numpy(), num.cpu().numpy(), max(float(factor), 1.0) ** 3
+    assert np.all(np.abs(W - ref["wsum"]) <= 1e-6 * ref["wsum"] + ref["edge_w"] + 1e-9 * unit)
+    assert np.all(np.abs(N - ref["num"]) <= 1e-5 * np.sqrt(ref["num_sq"]) + ref["edge_n"] + 1e-12 * unit)
+    Wr = W.reshape(n_r, n_r, n_alpha, n_theta, n_theta)
+    np.testing.assert_array_equal(Wr, Wr.transpose(1, 0, 2, 4, 3))
