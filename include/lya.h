@@ -207,7 +207,8 @@ int lya_xi_batched(lya_handle* h, const lya_catalog* mocks, int32_t n_mocks, con
 /* Tuning: pick launch parameters of the pair kernel by timing candidates on
  * the cached pair list of `cat` (synchronising); the choice is kept in the
  * handle for later lya_xi calls with the same bin grid.  *choice (optional,
- * host) receives an index into the candidate table. */
+ * host) receives an index into the candidate table: 1, 2, 4, 8 or 16 forest
+ * pairs per work grab. */
 int lya_autotune(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, int32_t* choice,
                  void* stream);
 

@@ -1,5 +1,5 @@
-// Double-float accumulation helpers shared by the cross-correlation and the
-// per-bin-means kernels: error-free FP32 addition and a shared-memory
+// Double-float accumulation helpers of the cross-correlation kernel: error-free
+// FP32 addition and a shared-memory
 // histogram entry held as an unevaluated sum hi + lo of two floats.
 #pragma once
 

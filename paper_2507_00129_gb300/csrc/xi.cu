@@ -27,16 +27,16 @@
 //  * the j loop of each 32-pixel chunk of a is restricted to the pixels that
 //    can be in range (distances are sorted; binary searches, one chunk per lane).
 // What bounds it: issue slots and fixed latencies (28 warp instructions per
-// step of 32 pixel pairs, issue 65-70%), and on the SDSS-like grid, whose runs
-// are two pixels long, the shared-memory pipe (81%: 3.6 wavefronts per
+// step of 32 pixel pairs, issue 74-76%), and on the SDSS-like grid, whose runs
+// are two pixels long, the shared-memory pipe (77%: 2.9 wavefronts per
 // reduction).  A team of two shares 12.7 KB of tables and the staged forest,
 // so 9-13 teams (18-26 warps) fit on an SM where 8 single warps did.
 // Measured (survey pass): 60,000 SDSS-like forests 624 -> 386 ms, 9,000
 // DESI-like forests 414 -> 244 ms; 365 and 238 ms without the reductions of
 // guard runs at the ends of a chunk.
-// FP64 kernel (LYA_PREC_FP64): the same decomposition with FP64 distances,
-// separations, products and shared-memory sums, mirroring the oracle's
-// operation order: r = |d_i - d_j| * c, x = r * (1/D).
+// FP64 kernel (LYA_PREC_FP64): the results of FP64 distances, separations and
+// products in the oracle's operation order, r = |d_i - d_j| * c, x = r * (1/D);
+// see "FP64 path" below.
 #include <algorithm>
 #include <math.h>
 
