@@ -748,12 +748,19 @@ __device__ void dm_vectors(const DmArgs& A, const Pair& P, double* G, int t0, in
   }
 }
 
+// T1 of a local bin that no pixel pair of this pair has reached: -0, which any
+// sum of weights replaces (-0 + 0 is +0)
+constexpr uint32_t kUntouched = 0x80000000u;
+__device__ __forceinline__ float4 untouched() { return make_float4(__uint_as_float(kUntouched), 0.f, 0.f, 0.f); }
+
 // T terms, diagonal and W: one warp per row r, lanes over c >= r.  The
 // pair's whole contribution (its rank-1 terms, already in the triangle, plus
 // these) goes to the FP64 accumulator here, and the triangle is cleared, so
-// that D~ and W are summed over pairs in FP64 only.  Rows and columns with
-// T = 0 hold nothing: every rank-1 term of a bin carries the weights of the
-// pixel pairs in it.
+// that D~ and W are summed over pairs in FP64 only and nothing of a pair stays
+// for the block's next one, which may have other bins in the same words or
+// belong to another catalogue.  Rows that no pixel pair touched (kUntouched)
+// hold nothing; a row whose T is 0 can (weights that the fixed point of one
+// side rounds to 0 and that of the other does not).
 template <bool GLOBAL>
 __device__ __forceinline__ void dm_flush(const DmArgs& A, double* G, double* wdm, int t0, int L, const Sm& m, int par) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -763,7 +770,7 @@ __device__ __forceinline__ void dm_flush(const DmArgs& A, double* G, double* wdm
   const float c11 = pc[kC11], cyy = pc[kCyy], cxx = pc[kCxx], cxy = pc[kCxy];
   for (int r = wid; r < L; r += nwarps) {
     const float4 tr = m.T4[r];
-    if (tr.x == 0.f && tr.y == 0.f && tr.z == 0.f && tr.w == 0.f) continue;
+    if (__float_as_uint(tr.x) == kUntouched) continue;
     const float f1 = c11 * tr.x, fy = cyy * tr.z, fx = cxx * tr.y, fxy = cxy * tr.w;
     const int rb = tri_rowbase(r, L);
     // two columns per lane per iteration (independent chains)
@@ -777,21 +784,15 @@ __device__ __forceinline__ void dm_flush(const DmArgs& A, double* G, double* wdm
       // consecutive lanes add to consecutive entries of the accumulator's row
       double* row = G + static_cast<int64_t>(g0 + r) * nbins + g0;
       if (!GLOBAL) {
-        // (r, c), (r, c2) owned by this lane: flush and clear.  Where the sum is
-        // exactly 0 (u = -v, about one entry in 1e7) the rank-1 part u stays and
-        // goes out with the block's next pair that has the entry.  Clearing it too
-        // makes two calls agree to 1e-18, but moves D by 1e-7 to 1e-5 of its norm.
-        const float x = m.U[rb + c] + v;
-        if (x != 0.f) {
-          red_add_f64_global(row + c, static_cast<double>(x));
-          m.U[rb + c] = 0.f;
-        }
+        // (r, c), (r, c2) owned by this lane: flush, and clear also where the
+        // rank-1 part u and v cancel to exactly 0 (about one entry in 1e7)
+        const float u = m.U[rb + c], x = u + v;
+        if (x != 0.f) red_add_f64_global(row + c, static_cast<double>(x));
+        if (u != 0.f) m.U[rb + c] = 0.f;
         if (c2 < L) {
-          const float x2 = m.U[rb + c2] + v2;
-          if (x2 != 0.f) {
-            red_add_f64_global(row + c2, static_cast<double>(x2));
-            m.U[rb + c2] = 0.f;
-          }
+          const float u2 = m.U[rb + c2], x2 = u2 + v2;
+          if (x2 != 0.f) red_add_f64_global(row + c2, static_cast<double>(x2));
+          if (u2 != 0.f) m.U[rb + c2] = 0.f;
         }
       } else {
         if (v != 0.f) red_add_f64_global(row + c, static_cast<double>(v));
@@ -820,7 +821,7 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
     for (int k = tid; k < nt; k += blockDim.x) m.U[k] = 0.f;
   }
   for (int k = tid; k < Lalloc; k += blockDim.x) {
-    m.T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    m.T4[k] = untouched();
     m.mark[k] = 0;
   }
   for (int k = tid; k < CB * ldv_for(scap); k += blockDim.x) m.V[k] = 0;
@@ -861,7 +862,7 @@ __global__ void __launch_bounds__(kDmThreads, 1) dm_kernel(DmArgs A, const Chunk
       if (P.ok) dm_flush<GLOBAL>(A, G, wdm, t0, L, m, par);
       __syncthreads();
       if (P.ok)
-        for (int k = tid; k < L; k += kDmThreads) m.T4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = tid; k < L; k += kDmThreads) m.T4[k] = untouched();
       P = N;
       par ^= 1;
     }

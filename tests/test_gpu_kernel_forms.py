@@ -140,6 +140,37 @@ def test_xi1d_forms(api, handle, lengths, step, n_bins, r_max, seed):
     assert np.all(np.abs(n - ref["num"]) <= ref["wsum"] * 2.0 ** -44 * wd * wd + 1e-300)
 
 
+def test_dmat_is_reproducible(api, handle):
+    """Every forest pair's contribution is formed in a fixed order and summed in FP64, so two calls differ by the
+    order of the FP64 sums only: at most n 2^-53 of the sum of magnitudes, n < 2^16 pairs per entry (1e-11).  (A
+    triangle entry left behind where a pair's terms cancel to zero would be added to another pair's entry.)"""
+    cat = synth.subset(synth.make(1, n_forests=20000), np.arange(12000))
+    dc = api.DeviceCatalog.from_host(cat)
+    b = synth.Bins(50, 50, 200.0, 200.0)
+    first, w1 = api.lya_dmat(handle, dc, b, 0.05, 7)
+    scale = first.abs().amax(dim=1, keepdim=True)
+    for _ in range(3):
+        again, w2 = api.lya_dmat(handle, dc, b, 0.05, 7)
+        assert bool(((again - first).abs() <= 1e-11 * scale).all())
+        assert bool(((w2 - w1).abs() <= 1e-11 * w1).all())
+
+
+def test_dmat_of_a_mock_does_not_depend_on_the_batch(api, handle):
+    """D of four catalogues in one call against each one's own call, where the blocks meet the pairs in another
+    order: the allowance of test_dmat_is_reproducible."""
+    cats = []
+    for k in range(4):
+        spec = synth.spec_for(4, seed=k, n_forests=3000)
+        spec.area_deg2 = 60.0
+        cats.append(api.DeviceCatalog.from_host(synth.generate(spec)))
+    b = synth.Bins(50, 50, 200.0, 200.0)
+    D, w = api.lya_dmat_batched(handle, cats, b, 0.1, 1234)
+    for k, c in enumerate(cats):
+        own, w1 = api.lya_dmat(handle, c, b, 0.1, 1234)
+        assert bool(((w[k] - w1).abs() <= 1e-11 * w1).all())
+        assert bool(((D[k] - own).abs() <= 1e-11 * own.abs().amax(dim=1, keepdim=True)).all())
+
+
 def test_dmat_on_a_grid_of_unequal_sides(api, handle):
     """n_par != n_perp: the accumulators' bin numbering (t n_par + p) against the outputs' (p n_perp + t).  The
     allowance is the one of the square grids (1e-5 of the row maximum and the quotient rule of the edge terms)."""
