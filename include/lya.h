@@ -299,8 +299,10 @@ typedef struct {
  * line of sight.  Triangle index
  *   A = (((i_r1 n_r + i_r2) n_alpha + i_alpha) n_theta + i_theta1) n_theta + i_theta2.
  * num, wsum (required), xi (optional): [n_r^2 n_alpha n_theta^2] float64.
- * The |r| and theta bins are computed in FP64, cos alpha in FP32; products
- * in FP32 are added to FP64 bin sums.  Builds (and caches) the forest-pair
+ * The |r| and theta bins are those of FP64, cos alpha is FP32; products in
+ * FP32 are added to FP64 bin sums, several vertices' together by way of exact
+ * integers where the rounding to them (of the smallest W term and of a typical
+ * N term of the integers' own bins) is no more than the products' own.  Builds (and caches) the forest-pair
  * list for r_par_max = r_perp_max = r_max.  Synchronises (a counting pass
  * sizes the kernel's neighbour capacity to the largest list); not allowed
  * during graph capture.  A main vertex with more neighbours within r_max

@@ -338,17 +338,21 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
 //  * A class (r1 <= r2) is walked by all warps: 16 neighbours q of bin r2 in the
 //    half-warps' registers against two neighbours p of bin r1 a step; steps are
 //    dealt evenly over the warps.
-//  * Sums are exact integers in two words of 16 to 20 bits of a record's value (as
-//    many as leave room for all records of the class), 32 to 40 bits below the
-//    group's largest product, which shared memory adds natively.  A class with
-//    few records (below kXGDirect a bin) or more than a word can hold, and a
-//    group whose products leave the scales, adds its records to L2 as
-//    xi3_kernel does; with two blocks per SM the one's reductions in L2 run
-//    beside the other's in shared memory.
+//  * Sums are exact integers in two words, which shared memory adds natively: the
+//    high one in units of 2^eh as fine as the class's largest record (2^21 units)
+//    and the sum of all (2^30) allow, the low one with as many bits below as leave
+//    room for all records (xg_scale).  A record of a class is summed so only where
+//    the rounding is no more than that of its FP32 product (2^-24): of the
+//    smallest record for W, whose terms are positive, and of one of typical
+//    size for N, whose terms come arbitrarily close to 0.  Weights a few thousand times
+//    apart between neighbours are beyond that.  Such a class, one with few
+//    records (below kXGDirect a bin) and one whose products leave the FP32 range
+//    add their records to L2 as xi3_kernel does; with two blocks per SM the one's
+//    reductions in L2 run beside the other's in shared memory.
 // What bounds it: the shared-memory pipe (four reductions a record, 25 of 32
 // lanes on random bins) and L2's atomics.  Measured (5,000 SDSS-like forests,
 // r_max 40, 200,000 bins): xi3_kernel 204 ms,
-// this 158 ms; three words 227 ms, one block of 1,024 threads per SM 171 ms, no
+// this 157 ms; three words 227 ms, one block of 1,024 threads per SM 171 ms, no
 // direct classes 185 ms, kXGDirect 3, 12, 20: 160, 161, 186 ms; 64-bit words 449
 // ms (emulated).  Smaller grids gain more: 13 x 6^2 bins of 100 classes, 1,300
 // forests of a denser sky: 163 -> 54 ms.
@@ -390,6 +394,14 @@ __device__ __forceinline__ int xg_steps(int np, int nq, bool same) {
   return nq < 2 ? 0 : 4 * T * (T - 1) + ((nq + 1) >> 1);
 }
 
+// Scale of one word pair: records of magnitude up to B and total magnitude up to
+// T (both with the FP32 rounding of their own sums) as integers of 2^eh, k bits
+// below: the smallest eh with B <= 2^21 2^eh and T <= 2^30 2^eh.
+__device__ __forceinline__ int xg_scale(float B, float T) {
+  const float u = fmaxf(B * 4.76837158e-7f, T * 9.31322575e-10f);   // 2^-21, 2^-30
+  return (u > 0.f) ? static_cast<int>((__float_as_uint(u) >> 23) & 0xFFu) - 126 : 0;   // 2^eh > u
+}
+
 __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, const int32_t* nbr, const int64_t* nstart,
                                                                   int cap, double* sums, unsigned long long* counter,
                                                                   unsigned* err) {
@@ -398,10 +410,15 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
   __shared__ double s_x[kXGVerts][3], s_u[kXGVerts][3];
   __shared__ float2 s_w[kXGVerts];                       // (w delta, w) of the vertex
   __shared__ int s_f[kXGVerts], s_nb[kXGVerts], s_tot[kXGVerts];
-  __shared__ int s_n, s_wd, s_ww;                        // list length, largest |w delta| and w of the list (bits)
+  __shared__ int s_n;                                    // list length
+  __shared__ int s_ne, s_nc;                             // sum of the exponents and number of the list's |w delta| > 0
+  __shared__ float s_typ;                                // log2 of a typical |N| record
   __shared__ int s_st[kXGVerts * kXGMaxR + 1], s_pos[kXGVerts * kXGMaxR];
   __shared__ int s_steps[kXGClasses], s_recs[kXGClasses];
-  __shared__ int s_e[2];                                 // every |product| is below 2^e; 999: beyond the scales
+  // per (vertex, |r| bin): sum and largest |w delta|; sum, largest and smallest w > 0 (infinite without one)
+  __shared__ float s_sn[kXGVerts * kXGMaxR], s_mn[kXGVerts * kXGMaxR], s_sw[kXGVerts * kXGMaxR];
+  __shared__ float s_mw[kXGVerts * kXGMaxR], s_lw[kXGVerts * kXGMaxR];
+  __shared__ int s_eh[kXGClasses];                       // a class's scales, (N + 256) 2^16 + (W + 256); -1: direct
   const int nr = A.n_r, nt = A.n_theta, na = A.n_alpha, nbc = na * nt * nt, ncls = nr * (nr + 1) / 2;
   const XGLay y = xg_layout(cap, nbc);
   float4* cr = reinterpret_cast<float4*>(sm + y.cr);     // r (FP32) and 1 / |r|
@@ -488,12 +505,12 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
       for (int k = tid; k < nkey; k += kXGThreads) s_pos[k] = 0;
       if (tid == 0) {
         s_n = 0;
-        s_wd = 0;
-        s_ww = 0;
+        s_ne = 0;
+        s_nc = 0;
       }
       __syncthreads();
       // gather, 32 candidates a warp
-      int before = 0, mwd = 0, mww = 0;
+      int before = 0, ne = 0, nc = 0;
       for (int v = v0; v < v1; ++v) {
         const int tot = s_tot[v], units = (tot + 31) >> 5;
         const int* pre = s_pre + v * (kXGBatch + 1);
@@ -516,8 +533,10 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
             if (in) {
               q = A.pix[p];
               key = ((v - v0) << 24) | (ir << 16) | it;
-              mwd = max(mwd, __float_as_int(fabsf(q.z)));
-              mww = max(mww, __float_as_int(fabsf(q.y)));
+              if (q.z != 0.f) {
+                ne += static_cast<int>((__float_as_uint(q.z) >> 23) & 0xFFu) - 127;
+                ++nc;
+              }
               atomicAdd(&s_pos[(v - v0) * nr + ir], 1);
             }
           }
@@ -533,14 +552,14 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
         }
         before += units;
       }
-      mwd = __reduce_max_sync(0xffffffffu, mwd);
-      mww = __reduce_max_sync(0xffffffffu, mww);
-      if (lane == 0) {
-        atomicMax(&s_wd, mwd);
-        atomicMax(&s_ww, mww);
+      ne = __reduce_add_sync(0xffffffffu, ne);
+      nc = __reduce_add_sync(0xffffffffu, nc);
+      if (lane == 0 && nc > 0) {
+        atomicAdd(&s_ne, ne);
+        atomicAdd(&s_nc, nc);
       }
       __syncthreads();
-      // bucket starts (warp 0), scales (warp 1)
+      // bucket starts (warp 0), typical N record (warp 1)
       if (wid == 0) {
         int carry = 0;
         for (int k0 = 0; k0 < nkey; k0 += 32) {
@@ -559,14 +578,17 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
           carry += __shfl_sync(0xffffffffu, x, 31);
         }
         if (lane == 0) s_st[nkey] = carry;
-      } else if (wid == 1 && lane < 2) {
-        float vm = 0.f;
-        for (int v = v0; v < v1; ++v)
-          if (s_f[v] >= 0) vm = fmaxf(vm, fabsf(lane ? s_w[v].y : s_w[v].x));
-        const float m = __int_as_float(lane ? s_ww : s_wd);
-        const float B = m * m * vm * 2.001f;   // |product| of any record, mirror weight included
-        const int e = static_cast<int>((__float_as_uint(B) >> 23) & 0xFFu) - 126;
-        s_e[lane] = (B == 0.f) ? 0 : (B > 1e-25f && B < 1e30f) ? e : 999;
+      } else if (wid == 1 && lane == 0) {
+        int e = 0, c = 0;
+        for (int v = v0; v < v1; ++v) {
+          const float x = s_w[v].x;
+          if (s_f[v] >= 0 && x != 0.f) {
+            e += static_cast<int>((__float_as_uint(x) >> 23) & 0xFFu) - 127;
+            ++c;
+          }
+        }
+        s_typ = (c > 0 && s_nc > 0) ? 2.f * static_cast<float>(s_ne) / static_cast<float>(s_nc) +
+                                          static_cast<float>(e) / static_cast<float>(c) : 0.f;
       }
       __syncthreads();
       // sort the list by (vertex, |r| bin): places first, then the fields; the
@@ -624,7 +646,65 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
           }
       }
       __syncthreads();
-      const int en = s_e[0], ew = s_e[1];
+      // magnitudes of every bucket, a warp each
+      for (int key = wid; key < nkey; key += nwarps) {
+        float sn = 0.f, sw = 0.f;
+        unsigned mn = 0u, mw = 0u, lw = 0x7F800000u;
+        for (int k = s_st[key] + lane; k < s_st[key + 1]; k += 32) {
+          const float2 q = cw[k];
+          sn += fabsf(q.x);
+          sw += q.y;
+          mn = max(mn, __float_as_uint(fabsf(q.x)));
+          mw = max(mw, __float_as_uint(q.y));
+          if (q.y > 0.f) lw = min(lw, __float_as_uint(q.y));
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+          sn += __shfl_xor_sync(0xffffffffu, sn, d);
+          sw += __shfl_xor_sync(0xffffffffu, sw, d);
+        }
+        mn = __reduce_max_sync(0xffffffffu, mn);
+        mw = __reduce_max_sync(0xffffffffu, mw);
+        lw = __reduce_min_sync(0xffffffffu, lw);
+        if (lane == 0) {
+          s_sn[key] = sn;
+          s_sw[key] = sw;
+          s_mn[key] = __uint_as_float(mn);
+          s_mw[key] = __uint_as_float(mw);
+          s_lw[key] = __uint_as_float(lw);
+        }
+      }
+      __syncthreads();
+      for (int c = tid; c < ncls; c += kXGThreads) {
+        int ra = 0, left = c;
+        while (left >= nr - ra) {
+          left -= nr - ra;
+          ++ra;
+        }
+        const int rb = ra + left, recs = s_recs[c];
+        s_eh[c] = -1;
+        if (recs < kXGDirect * nbc || recs < 1) continue;
+        // largest and total magnitude (with mirror weights), smallest W record that is not 0
+        float bn = 0.f, bw = 0.f, tn = 0.f, tw = 0.f, lw = INFINITY;
+        for (int v = 0; v < v1 - v0; ++v) {
+          const float2 wv = s_f[v0 + v] >= 0 ? s_w[v0 + v] : make_float2(0.f, 0.f);
+          const int a = v * nr + ra, b = v * nr + rb;
+          // (multiplied in the records' order, so that no record is larger or, if not 0, smaller)
+          bn = fmaxf(bn, s_mn[a] * (s_mn[b] * fabsf(wv.x)));
+          bw = fmaxf(bw, s_mw[a] * (s_mw[b] * wv.y));
+          tn += s_sn[a] * (s_sn[b] * fabsf(wv.x));
+          tw += s_sw[a] * (s_sw[b] * wv.y);
+          if (wv.y > 0.f) lw = fminf(lw, s_lw[a] * (s_lw[b] * wv.y));
+        }
+        const bool fn = tn == 0.f || (bn > 1e-25f && tn < 1e30f), fw = tw == 0.f || (bw > 1e-25f && tw < 1e30f);
+        if (!fn || !fw) continue;   // (sums that are infinite or not numbers among them)
+        const int en = xg_scale(2.002f * bn, 1.01f * tn), ew = xg_scale(2.002f * bw, 1.01f * tw);
+        const int k = min(21, __clz(recs));
+        if (tw != 0.f && !(lw >= pow2f(ew - k + 23))) continue;
+        if (tn != 0.f && !(static_cast<float>(en - k + 24) <= s_typ)) continue;
+        s_eh[c] = ((en + 256) << 16) | (ew + 256);
+      }
+      __syncthreads();
       const F2 M2 = f2(kM15, kM15), neg2 = f2(-1.f, -1.f);
       int cls = 0;
       for (int ra = 0; ra < nr; ++ra) {
@@ -632,10 +712,11 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
           const int S = s_steps[cls];
           if (S == 0) continue;
           const bool same = ra == rb;
-          // bits of a word: its sum over the class's records stays below 2^32
-          const int recs = s_recs[cls], bits = min(20, __clz(recs));
-          const bool direct = max(en, ew) > 900 || bits < 16 || recs < kXGDirect * nbc;
-          const F2 sc2 = f2(pow2f(bits - 1 - en), pow2f(bits - 1 - ew)), up2 = f2(pow2f(bits), pow2f(bits));
+          // bits of the low word: its sum over the class's records stays below 2^32
+          const int eh = s_eh[cls], bits = min(21, __clz(s_recs[cls]));
+          const int en = (eh >> 16) - 256, ew = (eh & 0xffff) - 256;
+          const bool direct = eh < 0;
+          const F2 sc2 = direct ? 0ull : f2(pow2f(-en), pow2f(-ew)), up2 = f2(pow2f(bits), pow2f(bits));
           double* const base = sums + 2 * (static_cast<int64_t>(ra * nr + rb) * nbc);
           int b = static_cast<int>(static_cast<int64_t>(S) * wid / nwarps);
           int left = static_cast<int>(static_cast<int64_t>(S) * (wid + 1) / nwarps) - b;
@@ -704,7 +785,7 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
                   if (b2 >= 0) red_add_f64_global(base + 2 * static_cast<int64_t>(b2) + (lane & 1), static_cast<double>((lane & 1) ? w2 : n2));
                 }
               } else if (on) {
-                // floor(q) and the rest, rounded, in units of 2^-bits
+                // floor in units of 2^eh, and the rest, rounded, `bits` below
                 const F2 v2 = f2(vn, vw);
                 const F2 hm = fma2_rd(v2, sc2, M2);
                 const F2 lm = fma2(fma2(v2, sc2, fma2(hm, neg2, M2)), up2, M2);
@@ -724,7 +805,7 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
           }
           if (!direct) {
             __syncthreads();
-            const double inv = pow2(1 - 2 * bits + ((tid & 1) ? ew : en));
+            const double inv = pow2(((tid & 1) ? ew : en) - bits);
             for (int k2 = tid; k2 < 2 * nbc; k2 += kXGThreads) {
               unsigned* w = hist + (k2 >> 1) * kXGWords + 2 * (k2 & 1);
               const unsigned h = w[0], lo = w[1];

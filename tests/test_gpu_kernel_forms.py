@@ -264,3 +264,26 @@ def test_xi3_grouped_vertices(api, handle, n_r, n_alpha, n_theta, nf, factor):
     assert np.all(np.abs(N - ref["num"]) <= 1e-5 * np.sqrt(ref["num_sq"]) + ref["edge_n"] + 1e-12 * unit)
     Wr = W.reshape(n_r, n_r, n_alpha, n_theta, n_theta)
     np.testing.assert_array_equal(Wr, Wr.transpose(1, 0, 2, 4, 3))
+
+
+@pytest.mark.parametrize("factor", [30.0, 1e3, 1e6])
+def test_xi3_light_triplets_beside_a_heavy_forest(api, handle, factor):
+    """One forest, 13.2 Mpc/h from the others, weighs `factor` times as much, so that its records fill bins of their
+    own (the outermost |r| bin, theta near 90 degrees) and every other bin holds light ones only.  W to 1e-6 of each
+    bin's own value (FP32 products, and at most 2^-24 of a record in its rounding), N as in test_gpu_xi3."""
+    rng = np.random.default_rng(3)
+    forests = []
+    for k in range(8):
+        ra, dec = (0.0132, 0.0) if k == 0 else (0.0, 4e-4 * k)
+        forests.append((ra, dec, 1000.0 + rng.uniform(0, 1) + np.arange(60) * 1.0, 8.2 + 1e-4 * np.arange(60),
+                        rng.normal(0.05, 0.3, 60), rng.uniform(1, 4, 60) * (factor if k == 0 else 1.0)))
+    cat = line_catalog(forests)
+    g = oracle.xi3.Grid3(n_r=4, n_theta=3, n_alpha=5, r_max=15.0)
+    num, wsum, xi = api.lya_xi3(handle, api.DeviceCatalog.from_host(cat), g)
+    api.lya_sync_status(handle)
+    ref = oracle.xi3.xi3_sums(cat, g, eps_r=1e-9, eps_c=2e-6)
+    W, N = wsum.cpu().numpy(), num.cpu().numpy()
+    assert ref["count"].sum() > 1e5
+    assert np.all(W[ref["wsum"] > ref["edge_w"]] > 0)
+    assert np.all(np.abs(W - ref["wsum"]) <= 1e-6 * ref["wsum"] + ref["edge_w"])
+    assert np.all(np.abs(N - ref["num"]) <= 1e-5 * np.sqrt(ref["num_sq"]) + ref["edge_n"])
