@@ -321,8 +321,9 @@ int lya_xi3(lya_handle* h, const lya_catalog* cat, const lya_bins3* bins, double
  *                   follows from the caller's d(z)),   npairs[A] = pixel pairs in A,
  * 0 where W_A = 0; wsum (optional) receives W_A.  Each [n_par*n_perp]
  * (float64; npairs int64).  Same pair list and FP32 bin arithmetic as the
- * mixed path of lya_xi; run sums in FP32, accumulation in double-float then
- * FP64.  Builds the pair list if none is cached (synchronises); refused
+ * mixed path of lya_xi; sums of up to 8 pixel pairs in FP32, then exact integers
+ * (where these would round such a sum by more than 2^-21 of its smallest pair,
+ * weights being too far apart: FP64) and FP64.  Builds the pair list if none is cached (synchronises); refused
  * during graph capture.  Limit: 36 bytes per bin + 8 per pixel of the longest
  * forest of shared memory. */
 int lya_xi_bin_means(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, double* wsum, double* rpar_mean,

@@ -96,47 +96,71 @@ __device__ void pair_means(const MeansArgs& A, const Acc& acc, unsigned char* sm
   const uint32_t guard = C + static_cast<uint32_t>(npar);
   const float pmax = kMagic + fnpar, tmax = kMagic + static_cast<float>(t_hi + 1);
   const uint32_t twin = static_cast<uint32_t>(t0), tspan = static_cast<uint32_t>(K - 1);
-  // fixed-point scales: a run is at most one diagonal of a tile long
-  const float bw = A.F.wmax[a] * A.F.wmax[b] * static_cast<float>(kTile);
-  const float bx = bw * fnpar, by = bw * fnperp, bs = bw * (ss + pa[na - 1].x + pb[nb - 1].x);
-  const float scW = fixed_scale(bw), scX = fixed_scale(bx), scY = fixed_scale(by), scS = fixed_scale(bs);
   for (int ia = 0; ia < na; ia += tile) {
     const int ta = min(tile, na - ia);
     for (int jb = 0; jb < nb; jb += tile) {
       const int tb = min(tile, nb - jb);
-      // rows up to a multiple of 8 and the padding of b lie at infinite distance, with zero weight
-      float zm = 0.f;
+      // rows up to a multiple of 8 and the padding of b lie at infinite distance, with zero weight;
+      // of the tile: sums of w^2, smallest weights that are not 0, smallest and largest |z|
+      float zm = 0.f, zl = INFINITY, qa = 0.f, qb = 0.f, la = INFINITY, lb = INFINITY;
       for (int q = threadIdx.x; q < ((ta + 7) & ~7); q += kTeam) {
         const Pix p = (q < ta) ? pa[ia + q] : make_float4(INFINITY, 0.f, 0.f, 0.f);
         const float z = (Z && q < ta) ? static_cast<float>(A.zpix[oa + ia + q]) : 0.f;
         ap[q] = make_float4(p.x, z, p.y, 0.f);
+        qa = fmaf(p.y, p.y, qa);
+        if (p.y != 0.f) la = fminf(la, p.y);
         if (Z) zm = (fabsf(z) < 1e36f) ? fmaxf(zm, fabsf(z)) : INFINITY;   // (a NaN counts as infinite)
+        if (Z && z != 0.f) zl = fminf(zl, fabsf(z));
       }
       for (int q = static_cast<int>(threadIdx.x) - kPad; q < tb + kPad; q += kTeam) {
         const bool in = q >= 0 && q < tb;
         const Pix p = in ? pb[jb + q] : make_float4(INFINITY, 0.f, 0.f, 0.f);
         const float z = (Z && in) ? static_cast<float>(A.zpix[ob + jb + q]) : 0.f;
         bp[q] = make_float4(ss + p.x, z, dd - p.x, p.y);   // d_i + d_j = x_i + .x, d_i - d_j = x_i + .z
+        qb = fmaf(p.y, p.y, qb);
+        if (p.y != 0.f) lb = fminf(lb, p.y);
         if (Z) zm = (fabsf(z) < 1e36f) ? fmaxf(zm, fabsf(z)) : INFINITY;
+        if (Z && z != 0.f) zl = fminf(zl, fabsf(z));
       }
-      float scZ = 1.f;
-      bool direct = !(bx < 1e36f && by < 1e36f && bs < 1e36f) || (bw != 0.f && bw < 1e-30f);
-      if (Z) {
-        // largest |z| of the tile
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-        if (lane == 0) red[wid] = zm;
+      for (int o = 16; o > 0; o >>= 1) {
+        qa += __shfl_xor_sync(0xffffffffu, qa, o);
+        qb += __shfl_xor_sync(0xffffffffu, qb, o);
+      }
+      // (none of them is negative: their bits order like the values)
+      la = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(la)));
+      lb = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lb)));
+      if (Z) {
+        zm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(zm)));
+        zl = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(zl)));
+      }
+      if (lane == 0) {
+        float* r = red + 6 * wid;
+        r[0] = qa, r[1] = qb, r[2] = la, r[3] = lb, r[4] = zm, r[5] = zl;
       }
       __syncthreads();
+      // Fixed-point scales: a run meets every pixel of the tile's rows and columns at most once, so its sum of
+      // w_i w_j is at most the geometric mean of the sums of w^2 (Cauchy-Schwarz).  The integers hold 2^-37 of that
+      // bound; where it is more than 2^16 of the smallest product (survey weights: 2^13 to 2^15), so that they
+      // would round a block by more than 2^-21 of its smallest pair, or the sums leave the fixed point's range,
+      // the blocks go to the FP64 sums at once (direct).
+      const float bw = 1.001f * sqrtf(red[0] + red[6]) * sqrtf(red[1] + red[7]);
+      const float bx = bw * fnpar, by = bw * static_cast<float>(t0 + K), bs = bw * (ss + pa[na - 1].x + pb[nb - 1].x);
+      const float scW = fixed_scale(bw), scX = fixed_scale(bx), scY = fixed_scale(by), scS = fixed_scale(bs);
+      const float wa = fminf(red[2], red[8]), wb = fminf(red[3], red[9]);   // infinite where all weights are 0
+      bool direct = wa < INFINITY && wb < INFINITY &&
+                    !(bx < 1e36f && by < 1e36f && bs < 1e36f && bw > 1e-30f && bw <= 65536.f * (wa * wb));
+      float scZ = 1.f;
       if (Z) {
-        const float bz = 2.f * bw * fmaxf(red[0], red[1]);
-        const bool fine = bz < 1e36f && (bz == 0.f || bz > 1e-30f);
-        direct = direct || !fine;
+        const float zmax = fmaxf(red[4], red[10]), bz = 2.f * bw * zmax;
+        direct = direct || !(zmax == 0.f || (zmax <= 16.f * fminf(red[5], red[11]) && bz < 1e36f && (bz == 0.f || bz > 1e-30f)));
         scZ = fixed_scale(bz);
       }
-      const F2 scWX = f2(scW, scX), scSZ = f2(scS, scZ);
-      // the end of a block; sums beyond the fixed point's range (direct) go to
-      // the FP64 sums at once, infinities and NaN included
+      F2 scWX = f2(scW, scX), scSZ = f2(scS, scZ);
+      // (kept from being recomputed inside the walk: 185.6 -> 182.5 ms)
+      asm volatile("" : "+l"(scWX), "+l"(scSZ));
+      // the end of a block; with `direct` its sums go to the FP64 sums at once,
+      // infinities and NaN included
       auto close_block = [&](Run& r) {
         if (direct) {
           const int q = static_cast<int>(r.cur - C), tt = q / (npar + 1), p = q - tt * (npar + 1);
@@ -302,14 +326,14 @@ __device__ void pair_means(const MeansArgs& A, const Acc& acc, unsigned char* sm
 // lanes along the rows with a warp scan and compare-and-swap sums per run
 // 777 ms; along the diagonals 261 ms with every run compensated and added at
 // once, 237 ms with fixed-point runs, 202 ms held, 160 ms without the runs off
-// the grid, 180 ms with the sum of r_perp of its own (from the sum of d_i + d_j
+// the grid, 182 ms with the sum of r_perp of its own (from the sum of d_i + d_j
 // its rounding differs by 6e-10 on a common pixel grid).
 template <bool Z>
 __global__ void __launch_bounds__(kTeam, 8) means_kernel(MeansArgs A, Acc acc, int tile, int bins, int kmax, int grab,
                                                       unsigned long long* counter) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_it;
-  __shared__ float s_red[2];
+  __shared__ float s_red[12];
   constexpr int kWords = Z ? 11 : 9;
   for (int q = threadIdx.x; q < bins * kWords; q += kTeam) reinterpret_cast<uint32_t*>(smem)[q] = 0u;
   const float fnperp = static_cast<float>(A.n_perp);

@@ -116,6 +116,46 @@ def test_bin_means_forms(api, handle, lengths, step, bins, seed, kind):
         assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width)
 
 
+def _light_and_heavy(factor, seed=41):
+    """Forests of 40 light pixels and 40 of `factor` times their weight: every pixel pair less than 40 Mpc/h apart
+    along the line of sight is one of light pixels (of two forests of different kinds)."""
+    rng = np.random.default_rng(seed)
+    forests = []
+    for k in range(2):
+        d = np.concatenate([3000.0 + np.arange(40), 3000.0 + (250.0 if k else 100.0) + np.arange(40)])
+        forests.append((rng.uniform(0, 2e-3), rng.uniform(0, 2e-3), d + rng.uniform(0.0, 0.2, 80),
+                        np.log(3600.0) + 1e-4 * np.arange(80), rng.normal(0.05, 0.3, 80),
+                        rng.uniform(1, 4, 80) * np.repeat([1.0, factor], 40)))
+    return line_catalog(forests)
+
+
+@pytest.mark.parametrize("factor", [30.0, 1e3, 1e5, 1e12])
+@pytest.mark.parametrize("with_z", [True, False])
+def test_bin_means_of_light_pixels(api, handle, factor, with_z):
+    """Bins that hold light pixels only, beside heavy ones of the same forests: W and the means to 1e-6 of the bin's
+    own values (FP32 products and sums of 8 terms; the integers round a block by at most 2^-21 of its smallest pair,
+    5e-7), next to the edge allowance of test_bin_means_forms."""
+    cat = _light_and_heavy(factor)
+    z = np.exp(cat.loglam) / 1215.67 - 1.0
+    b = synth.Bins(60, 5, 300.0, 25.0)
+    ref = oracle.xi.bin_means(cat, b, eps_edge=6e-5, z=z)
+    got = api.lya_xi_bin_means(handle, api.DeviceCatalog.from_host(cat), b, z_pix=torch.from_numpy(z).cuda() if with_z else None)
+    api.lya_sync_status(handle)
+    got = {k: v.cpu().numpy() for k, v in got.items()}
+    W = ref["wsum"]
+    on = W > 4.0 * ref["edge_w"]
+    light = on & (np.arange(b.n_par * b.n_perp) // b.n_perp < 8)
+    assert light.sum() >= 8 and np.all(W[light] <= 16.0 * ref["count"][light])
+    assert np.all(np.abs(got["count"] - ref["count"]) <= ref["edge_c"])
+    assert np.all(np.abs(got["wsum"] - W) <= 1e-6 * W + ref["edge_w"])
+    frac = 2.0 * ref["edge_w"][on] / (W[on] - ref["edge_w"][on])
+    for key, width in (("rpar_mean", 5.0), ("rperp_mean", 5.0), ("dist_mean", float(cat.dist.max() - cat.dist.min())),
+                       ("z_mean", float(z.max() - z.min()))):
+        if key in got:
+            err = np.abs(got[key][on] - ref[key][on])
+            assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width), key
+
+
 @pytest.mark.parametrize("lengths,step,n_bins,r_max,seed", [
     ((1, 2, 8, 9, 33, 34), 1.0, 20, 40.0, 21),           # below and above a block of rows and a group of lags
     ((255, 257, 264, 300), 0.5, 50, 200.0, 22),          # edges of a batch of 256 rows
