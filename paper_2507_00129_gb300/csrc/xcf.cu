@@ -28,6 +28,7 @@ namespace lya {
 namespace {
 
 constexpr int kXW = 8;    // warps per block (distortion matrix)
+constexpr int kXdmCap = 32;   // least entries of a warp's run list: it passes 64 pairs
 constexpr int kXCW = 32;  // warps per block of the cross-correlation (one block per SM)
 constexpr int kPad1 = 48;   // sentinels past a forest (a block of 8 rows and 32 lags reaches 39 past it)
 constexpr unsigned kFull = 0xffffffffu;
@@ -335,8 +336,8 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
 }
 
 // Kept (forest, quasar) pairs, one per warp at a time.  A warp draws its pairs
-// 32 at a time and queues the kept ones; with 32 in the queue (or at the end)
-// each lane computes one pair's geometry, window and normalisers in FP64 (with
+// 32 at a time and collects the kept ones, at most one per lane and the next 31
+// by way of its run lists' memory; with 32 of them (or at the end) each lane computes one pair's geometry, window and normalisers in FP64 (with
 // all lanes on one pair that cost as much as the pair's updates), and the warp
 // takes the pairs in turn: the runs of its window in shared memory, scaled to
 // al = alpha sqrt(w_q / W_a) and be = beta sqrt(w_q / S_a), then the upper
@@ -349,17 +350,17 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
 // rest of its call 12 ms as it is.
 __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
   extern __shared__ double dsh[];
-  __shared__ int2 s_queue[kXW][64];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   double* lal = dsh + static_cast<size_t>(wi) * 2 * cap;
   double* lbe = lal + cap;
   int* lA = reinterpret_cast<int*>(dsh + static_cast<size_t>(nwb) * 2 * cap) + static_cast<size_t>(wi) * cap;
-  int2* queue = s_queue[wi];
+  int2* pass = reinterpret_cast<int2*>(lal);   // 64 pairs: cap >= kXdmCap
   const int nb = A.n_par * A.n_perp;
   const int all = A.p_subsample >= 1.0;
   const uint64_t thr = all ? 0 : static_cast<uint64_t>(A.p_subsample * 18446744073709551616.0);
   const int64_t nw = static_cast<int64_t>(gridDim.x) * nwb;
-  int queued = 0;   // pairs in the queue (uniform)
+  int held = 0;   // pairs kept so far (uniform), one in `own` of each of the first lanes
+  int2 own = make_int2(-1, -1);
   for (int64_t k0 = (blockIdx.x * static_cast<int64_t>(nwb) + wi) * 32;; k0 += nw * 32) {
     const bool last = k0 >= A.n_pairs;
     bool keep = false;
@@ -371,16 +372,25 @@ __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
       keep = keep && A.F.len[pr.x] > 0 && A.Q.len[pr.y] > 0;
     }
     const unsigned km = __ballot_sync(kFull, keep);
-    if (keep) queue[queued + __popc(km & ((1u << lane) - 1u))] = pr;
-    queued += __popc(km);
-    __syncwarp();
-    if (queued < 32 && !last) continue;
-    const int nq = min(queued, 32);
+    if (km) {
+      // the new ones behind those held
+      __syncwarp();
+      if (lane < held) pass[lane] = own;
+      if (keep) pass[held + __popc(km & ((1u << lane) - 1u))] = pr;
+      held += __popc(km);
+      __syncwarp();
+      if (lane < held) own = pass[lane];
+      if (lane + 32 < held) pr = pass[lane + 32];
+      __syncwarp();
+    }
+    if (held < 32 && !last) continue;
+    const int nq = min(held, 32);
+    const int2 rest = pr;   // of the first held - 32 lanes: kept for the next turn
     // one pair's geometry per lane
     XGeo mine{0.f, 0.f, 0.f, 0.f, 0, 0};
     double cw = 0.0, cs = 0.0;   // sqrt(w_q / W_a), sqrt(w_q / S_a) (0 where eta lacks the term)
     if (lane < nq) {
-      pr = queue[lane];
+      pr = own;
       mine = pair_geo(A, pr.x, pr.y, A.pix + A.F.off[pr.x], A.F.len[pr.x]);
       const double wq = static_cast<double>(A.wq[pr.y]);
       const double Wa = A.F.wsum[pr.x], Sa = A.F.ssum[pr.x];
@@ -465,15 +475,9 @@ __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
       }
       __syncwarp();
     }
-    // the rest of the queue moves to its front
-    const int rest = queued - nq;
-    int2 moved = make_int2(-1, -1);
-    if (lane < rest) moved = queue[32 + lane];
-    __syncwarp();
-    if (lane < rest) queue[lane] = moved;
-    queued = rest;
-    __syncwarp();
-    if (last && queued == 0) break;
+    held -= nq;
+    if (lane < held) own = rest;
+    if (last) break;   // (a turn leaves pairs only where it has drawn some)
   }
 }
 
@@ -641,7 +645,7 @@ int xcf_limit_bytes(int nb, int max_len) {
 }
 
 int xdm_warps(const DevInfo& dev, int max_len) {
-  const int64_t per_warp = 20LL * std::max(max_len, 1);
+  const int64_t per_warp = 20LL * std::max(max_len, kXdmCap);
   int w = static_cast<int>(std::min<int64_t>(kXW, dev.smem_optin / per_warp));
   return w;   // 0: forests too long for the run lists
 }
@@ -686,7 +690,7 @@ cudaError_t launch_xdm(const XcfArgs& a, const DevInfo& dev, cudaStream_t s) {
   if (a.n_pairs == 0 || a.p_subsample <= 0.0) return cudaSuccess;
   const int warps = xdm_warps(dev, a.max_len);
   if (warps < 1) return cudaErrorInvalidConfiguration;
-  const int cap = std::max(a.max_len, 1);
+  const int cap = std::max(a.max_len, kXdmCap);
   const int smem = warps * 20 * cap;
   cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xdm_kernel), smem);
   if (e != cudaSuccess) return e;

@@ -283,6 +283,36 @@ def test_xcf_forms(api, handle, lengths, n_qso, bins, seed):
     assert np.all(np.abs(n - ref["num"]) <= 1e-6 * top * ref["wsum"] + ref["edge_n"] + 1e-300)
 
 
+@pytest.mark.parametrize("lengths,n_qso,step,bins,p,seed", [
+    ((1, 2, 31, 32, 33, 64), 12, 0.3, (10, 8, 60.0, 40.0), 1.0, 51),     # two batches of 32 pairs and a remainder
+    ((32,), 32, 0.3, (10, 8, 60.0, 40.0), 1.0, 52),                      # exactly one batch
+    ((70, 40), 33, 0.3, (1, 1, 100.0, 100.0), 1.0, 53),                  # one bin: runs over more than 32 pixels
+    ((90, 200), 60, 0.3, (41, 7, 200.0, 100.0), 0.4, 54),                # batches filled from several draws
+    ((1440, 30), 20, 0.3, (64, 40, 200.0, 200.0), 1.0, 55),              # run lists of eight warps fill shared memory
+    ((5780,), 3, 0.15, (64, 40, 200.0, 200.0), 1.0, 56),                 # ... of two warps
+])
+def test_xdmat_forms(api, handle, lengths, n_qso, step, bins, p, seed):
+    """Allowance as in test_gpu_xcf: 1e-5 of the row's largest entry and the edge terms' quotient rule."""
+    cat = _catalog(lengths, step, seed, patch=8e-3)
+    rng = np.random.default_rng(seed)
+    q = synth.Quasars(ra=rng.uniform(0, 8e-3, n_qso), dec=rng.uniform(0, 8e-3, n_qso),
+                      dist=rng.uniform(2900.0, 3400.0, n_qso), weight=rng.uniform(0.5, 2.0, n_qso).astype(np.float32),
+                      z=np.full(n_qso, 2.5))
+    b = synth.Bins(*bins)
+    D, Wd = api.lya_xdmat(handle, api.DeviceCatalog.from_host(cat), api.DeviceQuasars.from_host(q), b, p, seed)
+    api.lya_sync_status(handle)
+    pl = oracle.xcf.forest_quasar_pairs(cat, q, b, np.full(cat.n_forests, -1))
+    m = oracle.xcf.keep_xpairs(pl[0], pl[1], seed, p)
+    ref = oracle.xcf.xdmat(cat, q, b, (pl[0][m], pl[1][m]), eps_edge=6e-5)
+    W = ref["wsum"]
+    assert np.count_nonzero(W) > 0
+    rel = np.divide(ref["edge_w"], W, out=np.zeros_like(W), where=W > 0)
+    col = np.divide(ref["edge_d"], W[:, None], out=np.zeros_like(ref["edge_d"]), where=W[:, None] > 0)
+    tol = (1e-5 + 3 * rel)[:, None] * np.abs(ref["dmat"]).max(axis=1)[:, None] + col
+    assert np.all(np.abs(D.cpu().numpy() - ref["dmat"]) <= tol + 1e-12)
+    assert np.all(np.abs(Wd.cpu().numpy() - W) <= 1e-6 * W + ref["edge_w"] + 1e-9)
+
+
 @pytest.mark.parametrize("n_r,n_alpha,n_theta,nf,factor", [
     (4, 5, 3, 14, 1.0),      # classes summed in shared memory
     (16, 1, 1, 14, 1.0),     # the most |r| bins
