@@ -82,7 +82,9 @@ typedef struct {
 } lya_bins;
 
 typedef enum {
-  LYA_PREC_FP64 = 0,  /* separations, binning, products and sums in FP64 */
+  LYA_PREC_FP64 = 0,  /* the bins of FP64 separations; products and sums to 2^-36 of the
+                         smallest product of a run of pixel pairs or better (64-bit
+                         integers, FP64 where the weights lie too far apart) */
   LYA_PREC_MIXED = 1  /* FP32 separations/binning/products, FP64 bin sums */
 } lya_precision;
 

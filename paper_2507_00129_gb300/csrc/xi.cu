@@ -38,6 +38,8 @@
 // products in the oracle's operation order, r = |d_i - d_j| * c, x = r * (1/D);
 // see "FP64 path" below.
 #include <algorithm>
+#include <type_traits>
+
 #include <math.h>
 
 #include "exact.cuh"
@@ -406,30 +408,42 @@ __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int 
 //  * bins: FP32 coordinates with a proven error bound; a pixel pair whose
 //    coordinate lies within the bound of a bin edge (about 1 step in 80 holds
 //    one) is binned by the definition in FP64, r = |d_i - d_j| * c, x = r * (1/D);
-//  * products and sums are exact integers (see exact.cuh);
+//  * products and sums are exact integers (see exact.cuh), except for forest
+//    pairs whose values lie too far apart for them (see wide_pair), which a
+//    second launch sums in FP64 on the same walk;
 //  * the walk goes along the diagonals of the pixel-pair matrix: lane l takes
 //    the pairs (i, i + o + l), whose separation changes slowly with i, so a run
 //    of pixel pairs in one bin is tens of pairs long on any grid.  A lane that
 //    leaves a bin adds its run to the team's 64-bit integer histogram, which
 //    is added to the FP64 bin sums in global memory per tile of 256 x 256.
-// Rounding: 2^-54 of the forest's largest value per pixel, 2^-51 (2^-45 where a
-// bin may hold 65,536 pixel pairs) of the largest product per run, to nearest,
-// none in the sums below a tile.
+// Rounding: 2^-54 of the forest's largest value per pixel, 2^-51 to 2^-45 of the
+// largest product per run (as the sums leave room), to nearest, none in the sums
+// below a tile; the run's is at most 2^-36 of the pair's smallest product w_i w_j.
 // What bounds it: issue (52%) and latencies of about 55 warp instructions per
 // step, of which the key and its edge test take 20, the six multiply-adds 6,
 // and the ends of runs (some lane in every second step) a quarter; a third of
 // the lanes' pairs lie off the grid at the ends of the diagonals.
 // Measured (SDSS-like, 3,000 forests): 370 ms with FP64 arithmetic and shared
 // FP64 atomics per pixel pair, 62 ms with FP64 run-edge integers along the
-// rows (FP64 pipe 74% busy), 47 ms as it is; the largest relative error of W
+// rows (FP64 pipe 74% busy), 45 ms as it is; the largest relative error of W
 // and N against 64-bit sums is that of the first form (6e-15).
 struct Fp64Args {
   XiArgs A;
   const double* d;            // per packed pixel: distance
   const int4* v;              // per packed pixel: H, L of w delta, H, L of w
+  const double* wd;           // per packed pixel: w delta
   const int2* scale;          // per forest: s of w delta, s of w
+  const float4* spread;       // per forest: see Spread64
+  unsigned* wide;             // set where a forest pair is left to the FP64 sums
   double inv_dpar, inv_dperp;
 };
+
+// Sizes of a forest's values, for w delta and w: log2 of the largest over the
+// smallest (rn, rw), and the largest sum of |values| over a tile's pixels in units
+// of the largest (qn, qw).  The smallest weight is the smallest that is not 0;
+// w delta comes arbitrarily close to 0, so its smallest is that of the largest of
+// 32 consecutive pixels (all of them 0 apart, and less than 16 at the forest's end).
+using Spread64 = float4;   // (rn, rw, qn, qw)
 
 constexpr int kGrab64 = 8;      // most pairs per work grab
 constexpr int kTile64 = 256;    // pixels of a tile edge: a run of 256 products stays below 2^62
@@ -444,29 +458,62 @@ struct Walk64 {
   double cp64, sp64;
 };
 
+// Sums of N and W in FP64 (forest pairs beyond the integers).
+struct SumF64 {
+  double n, w;
+};
+
+template <class S>
 struct Run64 {
-  Sum64 s;                   // the current run
-  Sum64 held;                // an ended run, until the lane ends another
+  S s;                       // the current run
+  S held;                    // an ended run, until the lane ends another
   uint32_t cur, key;         // their bins
   bool in, on;               // the current bin lies in the grid; a run is held
 };
 
+__device__ __forceinline__ void add_bin64(const Sum64& s, uint32_t addr, int shift) {
+  const long long n = run_value(s.nh, s.nl, shift), w = run_value(s.wh, s.wl, shift);
+  asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(addr), "l"(n), "l"(w));
+}
+__device__ __forceinline__ void add_bin64(const SumF64& s, uint32_t addr, int) {
+  asm volatile("{\n\tred.shared.add.f64 [%0], %1;\n\tred.shared.add.f64 [%0+8], %2;\n\t}" ::"r"(addr), "d"(s.n), "d"(s.w));
+}
+
+__device__ __forceinline__ void add_products(SumF64& s, const int4& a, const int4& b) {
+  s.n = fma(__hiloint2double(a.y, a.x), __hiloint2double(b.y, b.x), s.n);
+  s.w = fma(__hiloint2double(a.w, a.z), __hiloint2double(b.w, b.z), s.w);
+}
+
 // Adds every lane's held run to its bin.
-__device__ __forceinline__ void add_run64(Run64& r, const Walk64& k) {
-  if (r.on) {
-    const long long n = run_value(r.held.nh, r.held.nl, k.shift), w = run_value(r.held.wh, r.held.wl, k.shift);
-    asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(k.base + (r.key << 4)),
-                 "l"(n), "l"(w));
-  }
+template <class S>
+__device__ __forceinline__ void add_run64(Run64<S>& r, const Walk64& k) {
+  if (r.on) add_bin64(r.held, k.base + (r.key << 4), k.shift);
   r.on = false;
   __syncwarp();
 }
 
+// Bits a run's sum is rounded by: products are below 2^52, and a bin's sum has to
+// stay below 2^62.  A bin of a tile holds at most two runs of 2 D_par / (c gap_b) + 1
+// pixels per row, and no more than the product of the two tiles' sums.
+__device__ __forceinline__ int shift64(const XiArgs& A, const Spread64& a, const Spread64& b, int bi, float cp) {
+  const float terms = fminf(fminf(512.f * (2.f / (cp * A.F.hmin[bi]) + 1.f), 65536.f),
+                            1.001f * fmaxf(a.z * b.z, a.w * b.w) + 1.f);
+  return max(1, 32 - __clz(static_cast<int>(terms)) - 10);
+}
+
+// Whether the integers would round a run by more than 2^-36 of the pair's
+// smallest product: half of 2^shift against products of 2^(50 - r) and more.
+// (Survey weights: r about 9.5 on the SDSS-like and 11 on the DESI-like grid.)
+__device__ __forceinline__ bool wide_pair(const Spread64& a, const Spread64& b, int shift) {
+  return fmaxf(a.x + b.x, a.y + b.y) + static_cast<float>(shift) > 15.f;
+}
+
 // Bin rows [t0, t0 + K) of forest pair (a, b) into the FP64 sums; WINDOW
 // where the band goes on beyond them (its top row is t_hi).
-template <bool WINDOW>
+template <bool WINDOW, class S>
 __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int na, int nb, double cp64, double sp64,
-                       int t0, int K, int t_hi, int tile, int hcap) {
+                       int shift, int t0, int K, int t_hi, int tile, int hcap) {
+  constexpr bool kExact = std::is_same<S, Sum64>::value;   // integers
   const XiArgs& A = P.A;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(smem);
@@ -504,12 +551,15 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
   k.tmax = kMagic + static_cast<float>(t_hi + 1);
   k.twin = static_cast<uint32_t>(t0);
   k.tspan = static_cast<uint32_t>(K - 1);
-  // products are below 2^52; a bin of a tile holds at most two runs of
-  // 2 D_par / (c gap_b) + 1 pixels per row, and its sum stays below 2^62
-  const float terms = fminf(512.f * (2.f / (k.cp * A.F.hmin[b]) + 1.f), 65536.f);
-  k.shift = max(1, 32 - __clz(static_cast<int>(terms)) - 10);
+  k.shift = shift;
   const int2 ea = P.scale[a], eb = P.scale[b];
   const int64_t out_off = static_cast<int64_t>(A.F.mock[a]) * A.nb;
+  // a pixel's (w delta, w): integers, or the FP64 values
+  auto value = [&](int64_t g, float w) {
+    if (kExact) return P.v[g];
+    const double n = P.wd[g], d = w;
+    return make_int4(__double2loint(n), __double2hiint(n), __double2loint(d), __double2hiint(d));
+  };
   for (int ia = 0; ia < na; ia += tile) {
     const int ta = min(tile, na - ia);
     for (int jb = 0; jb < nb; jb += tile) {
@@ -518,12 +568,12 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
       for (int q = threadIdx.x; q < ((ta + 7) & ~7); q += kTeam) {
         const float x = (q < ta) ? pa[ia + q].x : INFINITY;
         au[q] = (q < ta) ? make_float2(fmaf(x, k.cp, Dc), fmaf(x, k.sp, Ds)) : make_float2(INFINITY, INFINITY);
-        av[q] = (q < ta) ? P.v[oa + ia + q] : make_int4(0, 0, 0, 0);
+        av[q] = (q < ta) ? value(oa + ia + q, pa[ia + q].y) : make_int4(0, 0, 0, 0);
       }
       for (int q = static_cast<int>(threadIdx.x) - kPad64; q < tb + kPad64; q += kTeam) {
         const bool in = q >= 0 && q < tb;
         bx[q] = in ? pb[jb + q].x : INFINITY;
-        bv[q] = in ? P.v[ob + jb + q] : make_int4(0, 0, 0, 0);
+        bv[q] = in ? value(ob + jb + q, pb[jb + q].y) : make_int4(0, 0, 0, 0);
       }
       __syncthreads();
       // groups of 32 diagonals j - i = o + lane, in turn to the two warps
@@ -544,7 +594,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
           }
         }
         unsigned todo = __ballot_sync(0xffffffffu, work);
-        Run64 r{{0, 0, 0, 0}, {0, 0, 0, 0}, k.guard, k.guard, false, false};
+        Run64<S> r{S{}, S{}, k.guard, k.guard, false, false};
         for (; todo; todo &= todo - 1u) {
           const int i0 = 8 * (__ffs(todo) - 1);
           const float* px = bx + i0 + o + lane;
@@ -584,7 +634,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
                   r.key = r.cur;
                   r.on = true;
                 }
-                r.s = Sum64{0, 0, 0, 0};
+                r.s = S{};
                 r.cur = key;
                 const uint32_t q = key - C;   // row * (n_par + 1) + column
                 r.in = q < static_cast<uint32_t>(K) * k.stride && q % k.stride != static_cast<uint32_t>(npar);
@@ -601,7 +651,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
         r.on = r.in;
         add_run64(r, k);
       }
-      // integer sums -> FP64 bin sums
+      // the tile's sums -> FP64 bin sums
       __syncthreads();
       const double sn = pow2(56 + k.shift - ea.x - eb.x), sw = pow2(56 + k.shift - ea.y - eb.y);
       for (int q = threadIdx.x; q < (K + 1) * (npar + 1); q += kTeam) {
@@ -610,8 +660,8 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
           const int tt = q / (npar + 1), p = q - tt * (npar + 1);
           if (tt < K && p < npar) {
             const int64_t bin = out_off + static_cast<int64_t>(p) * A.n_perp + t0 + tt;
-            red_add_f64_global(A.num + bin, static_cast<double>(n) * sn);
-            red_add_f64_global(A.wsum + bin, static_cast<double>(w) * sw);
+            red_add_f64_global(A.num + bin, kExact ? static_cast<double>(n) * sn : __longlong_as_double(n));
+            red_add_f64_global(A.wsum + bin, kExact ? static_cast<double>(w) * sw : __longlong_as_double(w));
           }
           hist[2 * q] = 0ull;
           hist[2 * q + 1] = 0ull;
@@ -622,9 +672,14 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
   }
 }
 
+// S: Sum64, the forest pairs that the integers serve (the others set P.wide), or
+// SumF64, the others.  Both over the whole list.
+template <class S>
 __global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int tile, int kmax, int hcap, int grab) {
-  // histogram (N, W) interleaved: hcap x 16 bytes | H, L of tile a and of tile b | (uc, us) of a | distances of b
+  // histogram (N, W) interleaved: hcap x 16 bytes | values of tile a and of tile b | (uc, us) of a | distances of b
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool kExact = std::is_same<S, Sum64>::value;
+  if (!kExact && *P.wide == 0u) return;
   __shared__ unsigned long long s_it;
   __shared__ double2 s_cs[kGrab64];
   const XiArgs& A = P.A;
@@ -659,6 +714,12 @@ __global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int tile, in
       const int na = A.F.len[a], nb = A.F.len[b];
       if (na == 0 || nb == 0) continue;
       const double cp = s_cs[q].x, sp = s_cs[q].y;
+      const Spread64 ra = P.spread[a], rb = P.spread[b];
+      const int shift = shift64(A, ra, rb, b, static_cast<float>(cp));
+      if (wide_pair(ra, rb, shift) == kExact) {
+        if (kExact && threadIdx.x == 0) *P.wide = 1u;
+        continue;
+      }
       const double* da = P.d + A.F.off[a];
       const double* db = P.d + A.F.off[b];
       const double rt_min = (da[0] + db[0]) * sp;
@@ -667,18 +728,19 @@ __global__ void __launch_bounds__(kTeam) xi_fp64_kernel(Fp64Args P, int tile, in
       const int t_lo = static_cast<int>(rt_min);
       const int t_hi = (rt_max < fnperp) ? static_cast<int>(rt_max) : A.n_perp - 1;
       if (t_hi - t_lo < kmax) {
-        pair64<false>(P, smem, a, b, na, nb, cp, sp, t_lo, t_hi - t_lo + 1, t_hi, tile, hcap);
+        pair64<false, S>(P, smem, a, b, na, nb, cp, sp, shift, t_lo, t_hi - t_lo + 1, t_hi, tile, hcap);
       } else {
         for (int tw = t_lo; tw <= t_hi; tw += kmax)
-          pair64<true>(P, smem, a, b, na, nb, cp, sp, tw, min(kmax, t_hi - tw + 1), t_hi, tile, hcap);
+          pair64<true, S>(P, smem, a, b, na, nb, cp, sp, shift, tw, min(kmax, t_hi - tw + 1), t_hi, tile, hcap);
       }
     }
   }
 }
 
-// One warp per forest: distances, and w delta and w as integers on the
-// forest's own power-of-two scales.
-__global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, double* d, int4* v, int2* scale) {
+// One warp per forest: distances, w delta, and w delta and w as integers on the
+// forest's own power-of-two scales, and their spread.
+__global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, double* d, double* wd, int4* v,
+                              int2* scale, Spread64* spread) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -687,24 +749,44 @@ __global__ void pack64_kernel(lya_catalog cat, Forests F, int64_t forest_base, d
     const int n = F.len[gf];
     const int64_t o = cat.offsets[f];
     const int64_t g = F.off[gf];
-    double mw = 0.0, mn = 0.0;
-    for (int k = lane; k < n; k += 32) {
-      const double w = cat.weight[o + k];
-      mw = fmax(mw, fabs(w));
-      mn = fmax(mn, fabs(w * static_cast<double>(cat.delta[o + k])));
+    // largest values; smallest weight; smallest of the 32-pixel segments' largest |w delta|; tiles' sums
+    double mw = 0.0, mn = 0.0, lw = INFINITY, ln = INFINITY, qw = 0.0, qn = 0.0, tw = 0.0, tn = 0.0;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      if (k0 % kTile64 == 0) tw = tn = 0.0;
+      const int k = k0 + lane;
+      const double w = (k < n) ? static_cast<double>(cat.weight[o + k]) : 0.0;
+      const double x = (k < n) ? fabs(w * static_cast<double>(cat.delta[o + k])) : 0.0;
+      mw = fmax(mw, w);
+      if (w > 0.0) lw = fmin(lw, w);
+      const double top = warp_max_f64(x);
+      mn = fmax(mn, top);
+      if (top > 0.0 && (n - k0 >= 16 || k0 == 0)) ln = fmin(ln, top);
+      tw += w;
+      tn += x;
+      if (k0 + 32 >= n || (k0 + 32) % kTile64 == 0) {
+        qw = fmax(qw, warp_sum_f64(tw));
+        qn = fmax(qn, warp_sum_f64(tn));
+      }
     }
     mw = warp_max_f64(mw);
-    mn = warp_max_f64(mn);
+    lw = -warp_max_f64(-lw);
     // |value| < 2^(ilogb + 1): scaled below 2^54
     const int en = (mn > 0.0) ? 53 - ilogb(mn) : 0, ew = (mw > 0.0) ? 53 - ilogb(mw) : 0;
     const double sn = pow2(en), sw = pow2(ew);
     for (int k = lane; k < n; k += 32) {
-      const double w = cat.weight[o + k];
+      const double w = cat.weight[o + k], x = w * static_cast<double>(cat.delta[o + k]);
       d[g + k] = cat.dist[o + k];
-      const int2 a = split55(w * static_cast<double>(cat.delta[o + k]), sn), b = split55(w, sw);
+      wd[g + k] = x;
+      const int2 a = split55(x, sn), b = split55(w, sw);
       v[g + k] = make_int4(a.x, a.y, b.x, b.y);
     }
-    if (lane == 0) scale[gf] = make_int2(en, ew);
+    if (lane == 0) {
+      scale[gf] = make_int2(en, ew);
+      // (a forest without a segment of its own, its values in the last pixels: as wide as the type)
+      const float rn = (mn > 0.0) ? (ln < INFINITY ? log2f(static_cast<float>(mn / ln)) : 128.f) : 0.f;
+      const float rw = (mw > 0.0) ? log2f(static_cast<float>(mw / lw)) : 0.f;
+      spread[gf] = make_float4(rn, rw, mn > 0.0 ? static_cast<float>(qn / mn) : 0.f, mw > 0.0 ? static_cast<float>(qw / mw) : 0.f);
+    }
   }
 }
 
@@ -881,16 +963,19 @@ cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats,
   for (int m = 0; m < n_cats; ++m) npix += cats[m].n_pix;
   const int64_t nf = (std::max<int64_t>(a.F.n, 1) + 1) & ~int64_t{1}, np = std::max<int64_t>(npix, 1);
   char* tmp = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), static_cast<size_t>(8 * nf + 24 * np), s);
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), static_cast<size_t>(16 + 24 * nf + 32 * np), s);
   if (e != cudaSuccess) return e;
-  int2* scale = reinterpret_cast<int2*>(tmp);
-  int4* v = reinterpret_cast<int4*>(tmp + 8 * nf);
+  unsigned* wide = reinterpret_cast<unsigned*>(tmp);
+  Spread64* spread = reinterpret_cast<Spread64*>(tmp + 16);
+  int2* scale = reinterpret_cast<int2*>(spread + nf);
+  int4* v = reinterpret_cast<int4*>(scale + nf);
   double* d = reinterpret_cast<double*>(v + np);
+  double* wd = d + np;
   int64_t fb = 0;
   for (int m = 0; m < n_cats; ++m) {
     if (cats[m].n_forests > 0) {
       int64_t blocks = std::min<int64_t>((cats[m].n_forests * 32 + 255) / 256, 65535);
-      LYA_COUNT(1), pack64_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(cats[m], a.F, fb, d, v, scale);
+      LYA_COUNT(1), pack64_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(cats[m], a.F, fb, d, wd, v, scale, spread);
     }
     fb += cats[m].n_forests;
   }
@@ -898,7 +983,10 @@ cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats,
   P.A = a;
   P.d = d;
   P.v = v;
+  P.wd = wd;
   P.scale = scale;
+  P.spread = spread;
+  P.wide = wide;
   P.inv_dpar = static_cast<double>(a.n_par) / r_par_max;
   P.inv_dperp = static_cast<double>(a.n_perp) / r_perp_max;
   const int tile = std::min((std::max(max_len, 1) + 7) & ~7, kTile64);
@@ -906,17 +994,25 @@ cudaError_t launch_xi_fp64(const XiArgs& a, const lya_catalog* cats, int n_cats,
   const int hcap = std::max(408, 2 * (a.n_par + 1));
   const int kmax = std::min(a.n_perp, hcap / (a.n_par + 1) - 1);
   const int smem = hcap * 16 + (2 * tile + 2 * kPad64) * 16 + tile * 8 + (tile + 2 * kPad64) * 4;
-  e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_fp64_kernel), smem);
+  e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_fp64_kernel<Sum64>), smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi_fp64_kernel<SumF64>), smem);
   int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_fp64_kernel, kTeam, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi_fp64_kernel<Sum64>, kTeam, smem);
   if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidValue;
   if (e == cudaSuccess) e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(wide, 0, sizeof(unsigned), s);
   // pairs per grab: one thread each computes the geometry; few at a time where the list is short
   const int teams = per_sm * dev.sms;
   const int grab = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kGrab64, a.n_pairs / (16 * std::max(teams, 1)))));
   if (e == cudaSuccess && a.n_pairs > 0) {
-    LYA_COUNT(1), xi_fp64_kernel<<<teams, kTeam, smem, s>>>(P, tile, kmax, hcap, grab);
+    LYA_COUNT(1), xi_fp64_kernel<Sum64><<<teams, kTeam, smem, s>>>(P, tile, kmax, hcap, grab);
     e = cudaGetLastError();
+    // the forest pairs left by it (the kernel ends at once where there are none)
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+    if (e == cudaSuccess) {
+      LYA_COUNT(1), xi_fp64_kernel<SumF64><<<teams, kTeam, smem, s>>>(P, tile, kmax, hcap, grab);
+      e = cudaGetLastError();
+    }
   }
   if (used) {
     used->warps = kTeam / 32;

@@ -129,6 +129,26 @@ def _light_and_heavy(factor, seed=41):
     return line_catalog(forests)
 
 
+@pytest.mark.parametrize("factor", [30.0, 1e4, 1e8, 1e16])
+def test_fp64_sums_of_light_pixels(api, handle, factor):
+    """Bins that hold light pixels only, beside heavy ones of the same forests.  A run is rounded by at most 2^-36 of
+    its smallest product, its products by 2^-38 each and their low halves' sum by 2^-37: W to 2^-35 of the bin's own
+    value, N to 2^-35 of its number of pairs times the square of the largest light |w delta|."""
+    cat = _light_and_heavy(factor)
+    b = synth.Bins(60, 5, 300.0, 25.0)
+    ref = oracle.xi.xi_sums(cat, b)
+    num, wsum, xi = api.lya_xi(handle, api.DeviceCatalog.from_host(cat), b, "fp64")
+    api.lya_sync_status(handle)
+    n, w = num.cpu().numpy(), wsum.cpu().numpy()
+    light = (ref["count"] > 0) & (np.arange(b.n_par * b.n_perp) // b.n_perp < 8)
+    assert light.sum() >= 8 and np.all(ref["wsum"][light] <= 16.0 * ref["count"][light])
+    assert np.all((w > 0) == (ref["count"] > 0))
+    assert np.all(np.abs(w - ref["wsum"]) <= 2.0 ** -35 * ref["wsum"])
+    pix = np.arange(80) < 40
+    wd = np.abs(cat.weight.astype(np.float64) * cat.delta).reshape(2, 80)[:, pix].max()
+    assert np.all(np.abs(n - ref["num"])[light] <= 2.0 ** -35 * wd * wd * ref["count"][light])
+
+
 @pytest.mark.parametrize("factor", [30.0, 1e3, 1e5, 1e12])
 @pytest.mark.parametrize("with_z", [True, False])
 def test_bin_means_of_light_pixels(api, handle, factor, with_z):
