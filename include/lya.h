@@ -395,7 +395,7 @@ int lya_xdmat(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, con
  * i < j of one forest that the three-dimensional estimator excludes
  * (Section 2.1), binned in p = floor(|d_i - d_j| / (r_max / n_bins)),
  * p < n_bins.  num, wsum required, xi optional, each [n_bins] float64.
- * FP64 throughout (bin decisions identical to the definition's).
+ * Bins are the definition's in FP64; products and sums as with LYA_PREC_FP64.
  * Synchronises; refused during graph capture.  Limits: 1 <= n_bins <= 4096;
  * 16 bytes per bin + 24 per pixel of the longest forest of shared memory. */
 int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max, double* num, double* wsum,

@@ -1336,6 +1336,9 @@ int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max
   A.num = num;
   A.wsum = wsum;
   A.max_len = ml;
+  cudaError_t e = grow(&h->scratch2, &h->scratch2_cap, static_cast<size_t>(std::max<int64_t>(h->F.n, 1)) * 4);
+  if (e != cudaSuccess) return fail(h, LYA_ERR_NO_MEMORY, "1D correlation scratch");
+  A.wide = static_cast<int32_t*>(h->scratch2);
   stage_begin(h, 0, s);
   CK(launch_xi1d(A, static_cast<const Pix*>(h->pixbuf), h->d_counter, h->dev, s), "1D correlation kernel");
   stage_end(h, 0, s);

@@ -47,4 +47,29 @@ __device__ __forceinline__ long long run_value(long long h, long long l, int shi
   return round_shift(h + ((l + (1ll << 27)) >> 28), shift);
 }
 
+// Sums of N and W in FP64, on the same records (the two FP64 values in place of
+// the four integers): for values that lie too far apart for the integers.
+struct SumF64 {
+  double n, w;
+};
+
+__device__ __forceinline__ int4 pack_f64(double n, double w) {
+  return make_int4(__double2loint(n), __double2hiint(n), __double2loint(w), __double2hiint(w));
+}
+
+__device__ __forceinline__ void add_products(SumF64& s, const int4& a, const int4& b) {
+  s.n = fma(__hiloint2double(a.y, a.x), __hiloint2double(b.y, b.x), s.n);
+  s.w = fma(__hiloint2double(a.w, a.z), __hiloint2double(b.w, b.z), s.w);
+}
+
+// Adds a run's sums to its bin (N, W at a shared-memory address), integers in
+// units of 2^(56 + shift).
+__device__ __forceinline__ void add_bin64(const Sum64& s, uint32_t addr, int shift) {
+  const long long n = run_value(s.nh, s.nl, shift), w = run_value(s.wh, s.wl, shift);
+  asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(addr), "l"(n), "l"(w));
+}
+__device__ __forceinline__ void add_bin64(const SumF64& s, uint32_t addr, int) {
+  asm volatile("{\n\tred.shared.add.f64 [%0], %1;\n\tred.shared.add.f64 [%0+8], %2;\n\t}" ::"r"(addr), "d"(s.n), "d"(s.w));
+}
+
 }  // namespace lya

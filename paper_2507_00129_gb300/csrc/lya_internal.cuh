@@ -313,8 +313,10 @@ struct X1Args {
   double* num;
   double* wsum;
   int max_len;
+  int32_t* wide;         // [F.n] scratch
 };
 int xi1d_limit_bytes(int n_bins, int max_len);
+// counter: two words of scratch
 cudaError_t launch_xi1d(const X1Args& a, const Pix* pix, unsigned long long* counter, const DevInfo& dev, cudaStream_t s);
 
 // means.cu: per-bin weighted means of r_par, r_perp and the pair distance, and

@@ -20,6 +20,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "dfloat.cuh"
 #include "exact.cuh"
@@ -485,16 +486,26 @@ __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
 // (i, i + lag + l) of a group of 32 lags, whose separations change slowly with
 // i, so a run of pairs in one bin is tens of pairs long; products and sums are
 // the exact integers of exact.cuh, added to the warp's 64-bit histogram per run
-// and to FP64 sums per forest.  p = floor((d_j - d_i) / D) is taken from the
+// and to FP64 sums per forest.  With S = SumF64 they are FP64: a second launch
+// for the forests, left by the first, whose values lie so far apart that a run
+// would be rounded by more than 2^-36 of its smallest product (survey weights
+// reach 12 of the 15 bits).  p = floor((d_j - d_i) / D) is taken from the
 // FP32 packed distances when that value lies farther than `guard` from an
 // integer (the FP32 error is below guard / 2), else from the FP64 division of
 // the definition, so every bin is the definition's.
 // What bounds it: issue (73%), about 55 warp instructions per step of 32 pairs.
 // Measured (60,000 SDSS-like forests, 8.5e8 pairs): one warp per pixel with
 // FP64 prefix sums and two shared FP64 atomics per run of two pixels 25.1 ms,
-// this form 2.5 ms.
+// this form 2.5 ms, and 0.05 ms for 21 forests of the second launch (0.13 ms with
+// a warp on a whole forest).
+template <class S>
 __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int acc_bins, int stage, int per_warp,
-                                                   unsigned long long* counter) {
+                                                   unsigned long long* counter, unsigned* n_wide) {
+  constexpr bool kExact = std::is_same<S, Sum64>::value;
+  // with FP64 sums an item is one group of 32 lags: a few forests have to fill the GPU
+  const unsigned groups = kExact ? 1u : static_cast<unsigned>(A.max_len + 30) / 32u;
+  const unsigned long long n_items = kExact ? static_cast<unsigned long long>(A.F.n) : static_cast<unsigned long long>(*n_wide) * groups;
+  if (n_items == 0ull) return;
   // per warp: histogram (N, W) of n_bins + 1 bins, u64 | FP64 sums of acc_bins bins | H, L [stage] | distances [stage]
   extern __shared__ __align__(16) unsigned char dyn[];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
@@ -513,45 +524,76 @@ __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int
     unsigned long long f = 0;
     if (lane == 0) f = atomicAdd(counter, 1ull);
     f = __shfl_sync(kFull, f, 0);
-    if (f >= static_cast<unsigned long long>(A.F.n)) break;
+    if (f >= n_items) break;
+    int first = 1;   // first lag
+    if (!kExact) {
+      first += 32 * static_cast<int>(f % groups);
+      f = static_cast<unsigned long long>(A.wide[f / groups]);
+    }
     const int n = A.F.len[f];
     if (n < 2 || n > A.max_len) continue;
     const int64_t o = A.F.off[f];
     __syncwarp();
-    // largest |w delta| and |w|, by the high words of the FP64 values
-    uint32_t mn = 0u, mw = 0u;
-    for (int k = lane; k < n; k += 32) {
-      const double w = static_cast<double>(A.weight[o + k]), wd = w * static_cast<double>(A.delta[o + k]);
-      mn = max(mn, static_cast<uint32_t>(__double2hiint(wd)) & 0x7FFFFFFFu);
-      mw = max(mw, static_cast<uint32_t>(__double2hiint(w)) & 0x7FFFFFFFu);
+    // by the high words of the FP64 values: largest |w delta| and |w|, smallest w that is not 0, and smallest of
+    // the 32-pixel segments' largest |w delta| that is not 0 (not of less than 16 pixels at the forest's end)
+    uint32_t mn = 0u, mw = 0u, ln = 0xFFFFFFFFu, lw = 0xFFFFFFFFu;
+    float tn = 0.f, tw = 0.f;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      const int k = k0 + lane;
+      const float wf = (k < n) ? A.weight[o + k] : 0.f;
+      const double w = static_cast<double>(wf), wd = (k < n) ? fabs(w * static_cast<double>(A.delta[o + k])) : 0.0;
+      const uint32_t hw = static_cast<uint32_t>(__double2hiint(w)) & 0x7FFFFFFFu;
+      const uint32_t top = __reduce_max_sync(kFull, static_cast<uint32_t>(__double2hiint(wd)));
+      mn = max(mn, top);
+      mw = max(mw, hw);
+      if (hw) lw = min(lw, hw);
+      if (top && (n - k0 >= 16 || k0 == 0)) ln = min(ln, top);
+      tn += static_cast<float>(wd);
+      tw += wf;
     }
-    mn = __reduce_max_sync(kFull, mn);
     mw = __reduce_max_sync(kFull, mw);
+    lw = __reduce_min_sync(kFull, lw);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      tn += __shfl_xor_sync(kFull, tn, d);
+      tw += __shfl_xor_sync(kFull, tw, d);
+    }
     // |value| < 2^(exponent + 1) scaled below 2^54
     const int en = (mn >> 20) ? 53 - (static_cast<int>(mn >> 20) - 1023) : 0;
     const int ew = (mw >> 20) ? 53 - (static_cast<int>(mw >> 20) - 1023) : 0;
     const double sn = pow2(en), sw = pow2(ew);
+    // a bin holds at most D / gap + 2 partners of a pixel, and no more than half the square of the values' sum
+    // (in units of 2^54); its sum stays below 2^62
+    const float qn = static_cast<float>(static_cast<double>(tn) * pow2(en - 54)), qw = static_cast<float>(static_cast<double>(tw) * pow2(ew - 54));
+    const float terms = fminf(fminf(static_cast<float>(n) * (static_cast<float>(dr) / A.F.hmin[f] + 2.f),
+                                    0.5f * static_cast<float>(n) * static_cast<float>(n)),
+                              0.501f * fmaxf(qn * qn, qw * qw) + 1.f);
+    const int shift = max(1, static_cast<int>((__float_as_uint(fmaxf(terms, 1.f)) >> 23) & 0xFFu) - 126 - 10);
+    // log2 of largest over smallest, from exponent and mantissa in one (0.1: their log2 is less than 0.09 off)
+    const float rn = mn ? (ln != 0xFFFFFFFFu ? static_cast<float>(mn - ln) * 9.5367431640625e-7f + 0.1f : 128.f) : 0.f;
+    const float rw = mw ? static_cast<float>(mw - lw) * 9.5367431640625e-7f + 0.1f : 0.f;
+    if (kExact && 2.f * fmaxf(rn, rw) + static_cast<float>(shift) > 15.f) {
+      if (lane == 0) A.wide[atomicAdd(n_wide, 1u)] = static_cast<int32_t>(f);
+      continue;
+    }
     for (int k = lane; k < n + kPad1; k += 32) {
       const bool in = k < n;
       xs[k] = in ? pix[o + k].x : INFINITY;
-      int2 a = make_int2(0, 0), b = a;
-      if (in) {
-        const double w = static_cast<double>(A.weight[o + k]);
-        a = split55(w * static_cast<double>(A.delta[o + k]), sn);
-        b = split55(w, sw);
+      const double w = in ? static_cast<double>(A.weight[o + k]) : 0.0;
+      const double wd = in ? w * static_cast<double>(A.delta[o + k]) : 0.0;
+      if (kExact) {
+        const int2 a = split55(wd, sn), b = split55(w, sw);
+        v[k] = make_int4(a.x, a.y, b.x, b.y);
+      } else {
+        v[k] = pack_f64(wd, w);
       }
-      v[k] = make_int4(a.x, a.y, b.x, b.y);
     }
     __syncwarp();
     // |FP32 value - exact quotient| < 2^-22 (2 xs_max + r_max) / D + 2^-22 n_bins  (half of the guard)
     const float guard = 2.384185791015625e-7f * ((2.0f * xs[n - 1] + static_cast<float>(A.r_max)) * inv_dr + fbins) + 1e-6f;
     const float half = 0.5f - guard;
-    // a bin holds at most D / gap + 2 partners of a pixel, and its sum stays below 2^62
-    const float terms = fminf(static_cast<float>(n) * (static_cast<float>(dr) / A.F.hmin[f] + 2.f),
-                              0.5f * static_cast<float>(n) * static_cast<float>(n));
-    const int shift = max(1, static_cast<int>((__float_as_uint(fmaxf(terms, 1.f)) >> 23) & 0xFFu) - 126 - 10);
     bool more = true;
-    for (int lag = 1; lag < n && more; lag += 32) {
+    for (int lag = first; lag < n && more; lag += 32) {
       // separations grow with the lag: a group none of whose rows can be in range ends the walk
       more = false;
       for (int r0 = 0; r0 < n - lag; r0 += 256) {
@@ -561,12 +603,8 @@ __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int
         const bool work = i0 + lag < n && (xs[i0 + lag] - xs[i1]) * inv_dr < fbins + 1e-2f;
         unsigned todo = __ballot_sync(kFull, work);
         more = more || todo != 0u;
-        Sum64 run{0, 0, 0, 0};
+        S run{};
         uint32_t cur = off_grid;
-        auto add_run = [&]() {
-          asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(base + (cur << 4)),
-                       "l"(run_value(run.nh, run.nl, shift)), "l"(run_value(run.wh, run.wl, shift)));
-        };
         for (; todo; todo &= todo - 1u) {
           const int ib = r0 + 8 * (__ffs(todo) - 1);
 #pragma unroll
@@ -584,8 +622,8 @@ __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int
             const bool chg = key != cur;
             if (__any_sync(kFull, chg)) {
               if (chg) {
-                if (cur != off_grid) add_run();
-                run = Sum64{0, 0, 0, 0};
+                if (cur != off_grid) add_bin64(run, base + (cur << 4), shift);
+                run = S{};
                 cur = key;
               }
               __syncwarp();
@@ -593,16 +631,18 @@ __global__ void __launch_bounds__(256) xi1d_kernel(X1Args A, const Pix* pix, int
             add_products(run, v[i], v[j]);
           }
         }
-        if (cur != off_grid) add_run();
+        if (cur != off_grid) add_bin64(run, base + (cur << 4), shift);
         __syncwarp();
       }
+      if (!kExact) break;
     }
-    // integer sums -> FP64 sums
+    // the forest's sums -> FP64 sums
     const double un = pow2(56 + shift - 2 * en), uw = pow2(56 + shift - 2 * ew);
     for (int q = lane; q < A.n_bins; q += 32) {
       const long long hn = static_cast<long long>(hist[2 * q]), hw = static_cast<long long>(hist[2 * q + 1]);
       if ((hn | hw) == 0) continue;
-      const double dn = static_cast<double>(hn) * un, dw = static_cast<double>(hw) * uw;
+      const double dn = kExact ? static_cast<double>(hn) * un : __longlong_as_double(hn);
+      const double dw = kExact ? static_cast<double>(hw) * uw : __longlong_as_double(hw);
       if (q < acc_bins) {
         acc[q].x += dn;
         acc[q].y += dw;
@@ -712,17 +752,24 @@ cudaError_t launch_xi1d(const X1Args& a, const Pix* pix, unsigned long long* cou
   const int per_warp = (16 * (a.n_bins + 1 + acc_bins) + 20 * stage + 15) & ~15;
   const int warps = std::max(1, std::min(8, dev.smem_optin / per_warp));
   const int smem = warps * per_warp;
-  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi1d_kernel), smem);
+  cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi1d_kernel<Sum64>), smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(reinterpret_cast<const void*>(xi1d_kernel<SumF64>), smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi1d_kernel, warps * 32, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xi1d_kernel<Sum64>, warps * 32, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+  unsigned* n_wide = reinterpret_cast<unsigned*>(counter + 1);
+  e = cudaMemsetAsync(counter, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   const int blocks =
       static_cast<int>(std::min<int64_t>(static_cast<int64_t>(dev.sms) * per_sm, (a.F.n + warps - 1) / warps));
-  LYA_COUNT(1), xi1d_kernel<<<blocks, warps * 32, smem, s>>>(a, pix, acc_bins, stage, per_warp, counter);
+  LYA_COUNT(1), xi1d_kernel<Sum64><<<blocks, warps * 32, smem, s>>>(a, pix, acc_bins, stage, per_warp, counter, n_wide);
+  e = cudaGetLastError();
+  // the forests left by it (the kernel ends at once where there are none)
+  if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  LYA_COUNT(1), xi1d_kernel<SumF64><<<blocks, warps * 32, smem, s>>>(a, pix, acc_bins, stage, per_warp, counter, n_wide);
   return cudaGetLastError();
 }
 

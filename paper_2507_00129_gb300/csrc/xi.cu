@@ -458,11 +458,6 @@ struct Walk64 {
   double cp64, sp64;
 };
 
-// Sums of N and W in FP64 (forest pairs beyond the integers).
-struct SumF64 {
-  double n, w;
-};
-
 template <class S>
 struct Run64 {
   S s;                       // the current run
@@ -470,19 +465,6 @@ struct Run64 {
   uint32_t cur, key;         // their bins
   bool in, on;               // the current bin lies in the grid; a run is held
 };
-
-__device__ __forceinline__ void add_bin64(const Sum64& s, uint32_t addr, int shift) {
-  const long long n = run_value(s.nh, s.nl, shift), w = run_value(s.wh, s.wl, shift);
-  asm volatile("{\n\tred.shared.add.u64 [%0], %1;\n\tred.shared.add.u64 [%0+8], %2;\n\t}" ::"r"(addr), "l"(n), "l"(w));
-}
-__device__ __forceinline__ void add_bin64(const SumF64& s, uint32_t addr, int) {
-  asm volatile("{\n\tred.shared.add.f64 [%0], %1;\n\tred.shared.add.f64 [%0+8], %2;\n\t}" ::"r"(addr), "d"(s.n), "d"(s.w));
-}
-
-__device__ __forceinline__ void add_products(SumF64& s, const int4& a, const int4& b) {
-  s.n = fma(__hiloint2double(a.y, a.x), __hiloint2double(b.y, b.x), s.n);
-  s.w = fma(__hiloint2double(a.w, a.z), __hiloint2double(b.w, b.z), s.w);
-}
 
 // Adds every lane's held run to its bin.
 template <class S>
@@ -557,8 +539,7 @@ __device__ void pair64(const Fp64Args& P, unsigned char* smem, int a, int b, int
   // a pixel's (w delta, w): integers, or the FP64 values
   auto value = [&](int64_t g, float w) {
     if (kExact) return P.v[g];
-    const double n = P.wd[g], d = w;
-    return make_int4(__double2loint(n), __double2hiint(n), __double2loint(d), __double2hiint(d));
+    return pack_f64(P.wd[g], w);
   };
   for (int ia = 0; ia < na; ia += tile) {
     const int ta = min(tile, na - ia);

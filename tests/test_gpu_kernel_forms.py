@@ -176,6 +176,30 @@ def test_bin_means_of_light_pixels(api, handle, factor, with_z):
             assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width), key
 
 
+@pytest.mark.parametrize("factor", [1.0, 30.0, 1e4, 1e8, 1e16])
+def test_xi1d_of_light_pixels(api, handle, factor):
+    """One pixel of `factor` times the others' weight, 60 Mpc/h beyond them: bins below 50 Mpc/h hold light pixels
+    only.  Tolerances as in test_fp64_sums_of_light_pixels."""
+    rng = np.random.default_rng(42)
+    forests = []
+    for k in range(40):
+        m = 48 + k % 2
+        d = 3000.0 + np.append(np.arange(m - 1), m + 60) + rng.uniform(0.0, 0.2, m)
+        w = rng.uniform(1, 4, m)
+        w[-1] *= factor if k % 3 else 1.0
+        forests.append((0.0, 0.0, d, np.log(3600.0) + 1e-4 * np.arange(m), rng.normal(0.05, 0.3, m), w))
+    cat = line_catalog(forests)
+    ref = oracle.xi1d.xi1d_sums(cat, 40, 200.0)
+    num, wsum, xi = api.lya_xi1d(handle, api.DeviceCatalog.from_host(cat), 40, 200.0)
+    api.lya_sync_status(handle)
+    n, w = num.cpu().numpy(), wsum.cpu().numpy()
+    assert np.all((w > 0) == (ref["wsum"] > 0))
+    assert np.all(np.abs(w - ref["wsum"]) <= 2.0 ** -35 * ref["wsum"])
+    light = ref["wsum"][:9]     # weights are at least 1: no more pixel pairs than this
+    wd = max(np.abs(f[5][:-1] * f[4][:-1]).max() for f in forests)
+    assert np.all(np.abs(n - ref["num"])[:9] <= 2.0 ** -35 * wd * wd * light)
+
+
 @pytest.mark.parametrize("lengths,step,n_bins,r_max,seed", [
     ((1, 2, 8, 9, 33, 34), 1.0, 20, 40.0, 21),           # below and above a block of rows and a group of lags
     ((255, 257, 264, 300), 0.5, 50, 200.0, 22),          # edges of a batch of 256 rows
