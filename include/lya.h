@@ -367,8 +367,8 @@ typedef struct {
  * forest_qso ([n_forests] device int64, may be NULL) gives the index of each
  * forest's quasar in qso (-1 = none).  num, wsum required, xi optional, each
  * [n_par*n_perp] float64.  FP32 separations (bin decisions within about
- * 6e-5 bin widths of an edge may differ from FP64 ones), exact per-run sums,
- * FP64 accumulation.  Builds the (forest, quasar) pair list each call
+ * 6e-5 bin widths of an edge may differ from FP64 ones), per-run sums to
+ * 2^-47 of themselves, FP64 accumulation.  Builds the (forest, quasar) pair list each call
  * (synchronises); refused during graph capture.  Limits: check of lya_bins,
  * and 16 bytes per bin of shared memory (n_par*n_perp <= 14,000 or so on
  * GB300; else LYA_ERR_TOO_LARGE). */

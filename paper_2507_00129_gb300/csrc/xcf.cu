@@ -24,6 +24,7 @@
 
 #include "dfloat.cuh"
 #include "exact.cuh"
+#include "fixed.cuh"
 
 namespace lya {
 namespace {
@@ -143,13 +144,22 @@ __device__ __forceinline__ int count_below_s(const float* a, int n, float v) {
   return lo;
 }
 
-// w S f as an unevaluated float pair (h, l): S = 2^27 H + L, |H| < 2^22, with f = 2^27 times the unit of S.
-__device__ __forceinline__ void run_times(long long S, float w, float f, float& h, float& l) {
-  const float H = static_cast<float>(static_cast<int>(S >> 27));
-  const float L = static_cast<float>(static_cast<int>(S) & 0x7FFFFFF) * 7.450580596923828125e-9f;   // 2^-27
-  const float p = H * w;
-  h = p * f;
-  l = (fmaf(H, w, -p) + L * w) * f;
+// Two sums times w as unevaluated float pairs (h, l), N and W side by side, to 2^-47 of themselves:
+// S = 2^24 H + L, |H| <= 2^24 and L in [-2^23, 2^23) exact in FP32, their products with their errors,
+// f = 2^24 times the units of the sums.
+__device__ __forceinline__ void run_times(const longlong2& S, float w, F2 f, float2& h, float2& l) {
+  const int hn = static_cast<int>((S.x + (1ll << 23)) >> 24), hw = static_cast<int>((S.y + (1ll << 23)) >> 24);
+  const int ln = static_cast<int>(static_cast<unsigned>(S.x) - (static_cast<unsigned>(hn) << 24));
+  const int lw = static_cast<int>(static_cast<unsigned>(S.y) - (static_cast<unsigned>(hw) << 24));
+  const F2 one = f2(1.f, 1.f), neg = f2(-1.f, -1.f), w1 = f2(w, w);
+  const float wl = w * 5.9604644775390625e-8f;   // w 2^-24, exact (w > 1e-27)
+  const F2 w2 = f2(wl, wl);
+  const F2 H = f2(static_cast<float>(hn), static_cast<float>(hw)), L = f2(static_cast<float>(ln), static_cast<float>(lw));
+  const F2 np = fma2(H, f2(-w, -w), 0ull), nq = fma2(L, f2(-wl, -wl), 0ull);   // minus the rounded products
+  const F2 ns = fma2(np, one, nq);                                             // minus their sum; |p| >= |q| or p = 0
+  const F2 err = fma2(fma2(np, neg, ns), one, fma2(nq, neg, 0ull));            // q - (s - p), exact
+  h = unf2(fma2(ns, fma2(f, neg, 0ull), 0ull));
+  l = unf2(fma2(fma2(err, one, fma2(fma2(H, w1, np), one, fma2(L, w2, nq))), f, 0ull));
 }
 
 // sqrt(q) to 2e-14 (one Newton step from FP32; exact FP64 roots and divisions
@@ -191,8 +201,10 @@ __device__ __forceinline__ XGeo pair_geo_s(const XcfArgs& A, int a, int q, const
 
 // One block per SM: teams of warps, each staging one forest at a time (atomic
 // counter) with integer prefix sums of its packed w delta and w on the forest's
-// own power-of-two scales (43 bits: 2^-44 of the largest value per pixel, exact
-// sums).  Warps take 32 of the forest's quasars at a time, one pair's geometry
+// own power-of-two scales (43 bits; the FP32 values are exact on them down to
+// 2^-19 of the largest, and so are the sums).  A forest with smaller weights than
+// that (or w delta of 32 neighbouring pixels below 2^-12), and scales out of FP32's
+// range, are summed pixel by pixel.  Warps take 32 of the forest's quasars at a time, one pair's geometry
 // per lane, then walk each pair's window together: bins ascend along the
 // window, so a run of equal bins [j0, j] sits in adjacent lanes, and its last
 // lane adds w_q (P[j + 1] - P[j0]) as a float pair to the block's double-float
@@ -204,7 +216,8 @@ __device__ __forceinline__ XGeo pair_geo_s(const XcfArgs& A, int a, int q, const
 // Measured (60,000 x 90,000, 100 x 50 bins): 27.5 ms with a compensated
 // segmented scan over the lanes per 32 pixels and FP64 square roots, divisions
 // and window ends per pair; 18 ms with the prefix sums in teams of eight warps,
-// 16 ms as it is.
+// 16 ms in as many teams as fit, 17.5 ms with the run sums' low halves and the
+// sums by pixel for forests that the integers do not hold.
 __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, int team_warps, unsigned long long* counter) {
   // [nb] (num hi, num lo, w hi, w lo) | per team: inclusive prefix sums (w delta, w) [cap] | per team: distances [cap]
   extern __shared__ float4 xs4[];
@@ -240,8 +253,19 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
     if (q1 <= q0 || n <= 0 || n > cap) continue;   // uniform over the team
     const Pix* fp = A.pix + A.F.off[f];
     const float mn = A.F.wdmax[f], mw = A.F.wmax[f];
-    // |value| 2^e < 2^43; values beyond FP32's range (their sums are infinite or NaN) are summed pixel by pixel
-    const bool plain = !(mn < 1e38f && mw < 1e38f);
+    // smallest w that is not 0, and smallest of the 32-pixel segments' largest |w delta| that is not 0 (not of less
+    // than 16 pixels at the forest's end), by the bits of the FP32 values
+    uint32_t low_w = 0xFFFFFFFFu, low_n = 0xFFFFFFFFu;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      const Pix P = (k0 + lane < n) ? fp[k0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const uint32_t top = __reduce_max_sync(kFull, __float_as_uint(fabsf(P.z)));
+      if (top && (n - k0 >= 16 || k0 == 0)) low_n = min(low_n, top);
+      if (P.y > 0.f) low_w = min(low_w, __float_as_uint(P.y));
+    }
+    low_w = __reduce_min_sync(kFull, low_w);
+    // |value| 2^e < 2^43
+    const bool plain = !(mn < 1e18f && mw < 1e18f && (mn == 0.f || (mn > 1e-24f && mn <= 4096.f * __uint_as_float(low_n))) &&
+                         (mw == 0.f || (mw > 1e-24f && mw <= 524288.f * __uint_as_float(low_w))));
     const int en = (mn > 0.f && !plain) ? 42 - ilogbf(mn) : 0, ew = (mw > 0.f && !plain) ? 42 - ilogbf(mw) : 0;
     for (int k = tt; k < n; k += team_warps * 32) xs[k] = fp[k].x;
     if (tw == 0 && !plain) {
@@ -271,8 +295,7 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
       }
     }
     sync();
-    // a run's integer sum S = 2^27 H + L as floats: H 2^27 2^-e and L 2^-e, the factor 2^(27 - e) applied last
-    const float fn = ldexpf(1.f, 27 - en), fw = ldexpf(1.f, 27 - ew);
+    const F2 unit = f2(ldexpf(1.f, 24 - en), ldexpf(1.f, 24 - ew));   // see run_times
     for (int64_t qb = q0 + static_cast<int64_t>(tw) * 32; qb < q1; qb += team_warps * 32) {
       XGeo g{0.f, 0.f, 0.f, 0.f, 0, 0};
       float wq = 0.f;
@@ -294,6 +317,7 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
         h.X0 = __shfl_sync(kFull, g.X0, t);
         h.Y0 = __shfl_sync(kFull, g.Y0, t);
         const float wqt = __shfl_sync(kFull, wq, t);
+        const bool by_pixel = plain || !(wqt < 1e27f && (wqt > 1e-27f || wqt == 0.f));
         for (int base = i0; base < i1; base += 32) {
           const int j = base + lane;
           const int bin = (j < i1) ? pixel_bin(h, xs[j], A.n_par, A.n_perp) : -1;
@@ -301,25 +325,29 @@ __global__ void __launch_bounds__(kXCW * 32, 1) xcf_kernel(XcfArgs A, int cap, i
           const unsigned heads = __ballot_sync(kFull, lane == 0 || prev != bin);
           if (bin >= 0 && (lane == 31 || nxt != bin)) {
             const int j0 = base + 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-            float hn, ln, hw, lw;
-            if (!plain) {
+            float2 hi = make_float2(0.f, 0.f), lo = hi;   // N, W
+            if (!by_pixel) {
               longlong2 S = pre[j];
               if (j0 > 0) {
                 const longlong2 p = pre[j0 - 1];
                 S.x -= p.x;
                 S.y -= p.y;
               }
-              run_times(S.x, wqt, fn, hn, ln);
-              run_times(S.y, wqt, fw, hw, lw);
+              run_times(S, wqt, unit, hi, lo);
             } else {
-              hn = ln = hw = lw = 0.f;
               for (int i = j0; i <= j; ++i) {
-                hn += wqt * fp[i].z;
-                hw += wqt * fp[i].y;
+                const float pn = wqt * fp[i].z, pw = wqt * fp[i].y;
+                float s, e;
+                two_sum(hi.x, pn, s, e);
+                hi.x = s;
+                lo.x += e + fmaf(wqt, fp[i].z, -pn);
+                two_sum(hi.y, pw, s, e);
+                hi.y = s;
+                lo.y += e + fmaf(wqt, fp[i].y, -pw);
               }
             }
-            df_atomic_add(reinterpret_cast<float2*>(&hist[bin]), hn, ln, A.err);
-            df_atomic_add(reinterpret_cast<float2*>(&hist[bin]) + 1, hw, lw, A.err);
+            df_atomic_add(reinterpret_cast<float2*>(&hist[bin]), hi.x, lo.x, A.err);
+            df_atomic_add(reinterpret_cast<float2*>(&hist[bin]) + 1, hi.y, lo.y, A.err);
           }
           __syncwarp();
         }

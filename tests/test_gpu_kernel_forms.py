@@ -327,6 +327,31 @@ def test_xcf_forms(api, handle, lengths, n_qso, bins, seed):
     assert np.all(np.abs(n - ref["num"]) <= 1e-6 * top * ref["wsum"] + ref["edge_n"] + 1e-300)
 
 
+@pytest.mark.parametrize("factor,forest,quasar", [
+    (30.0, 1.0, 1.0), (1e4, 1.0, 1.0), (1e8, 1.0, 1.0),
+    (4.0, 1e-12, 1e34), (4.0, 1e-30, 1e3), (4.0, 1e22, 1e-10),   # weights far from 1 whose products are not
+])
+def test_xcf_of_light_pixels(api, handle, factor, forest, quasar):
+    """Bins of light pixels beside heavy ones of the same forests.  The products of the FP32 weights are formed with
+    their errors and the sums are double-float: W to 2^-40 of the bin's own value off the bin edges; N is a sum of
+    FP32 w delta (2^-24 of each term)."""
+    cat = _light_and_heavy(factor)
+    rng = np.random.default_rng(7)
+    cat.weight *= np.float32(forest)
+    nq = 40
+    q = synth.Quasars(ra=rng.uniform(0, 2e-3, nq), dec=rng.uniform(0, 2e-3, nq), dist=rng.uniform(3000.0, 3040.0, nq),
+                      weight=(rng.uniform(0.5, 2.0, nq) * quasar).astype(np.float32), z=np.full(nq, 2.5))
+    b = synth.Bins(100, 5, 300.0, 25.0)
+    ref = oracle.xcf.xcf_sums(cat, q, b, eps_edge=6e-5)
+    num, wsum, _ = api.lya_xcf(handle, api.DeviceCatalog.from_host(cat), api.DeviceQuasars.from_host(q), b)
+    api.lya_sync_status(handle)
+    n, w = num.cpu().numpy(), wsum.cpu().numpy()
+    sure = (ref["count"] > 0) & (ref["edge_w"] == 0)
+    assert sure.sum() > 30
+    assert np.all(np.abs(w - ref["wsum"])[sure] <= 2.0 ** -40 * ref["wsum"][sure])
+    assert np.all(np.abs(n - ref["num"])[sure] <= 1e-6 * float(np.abs(cat.delta).max()) * ref["wsum"][sure])
+
+
 @pytest.mark.parametrize("lengths,n_qso,step,bins,p,seed", [
     ((1, 2, 31, 32, 33, 64), 12, 0.3, (10, 8, 60.0, 40.0), 1.0, 51),     # two batches of 32 pairs and a remainder
     ((32,), 32, 0.3, (10, 8, 60.0, 40.0), 1.0, 52),                      # exactly one batch
