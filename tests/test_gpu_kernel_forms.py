@@ -382,6 +382,25 @@ def test_xdmat_forms(api, handle, lengths, n_qso, step, bins, p, seed):
     assert np.all(np.abs(Wd.cpu().numpy() - W) <= 1e-6 * W + ref["edge_w"] + 1e-9)
 
 
+def test_dmat_rows_are_divided_by_their_weight(api, handle):
+    """With eta = I and whole-number weights every sum is exact, in any order, and D~_AA = W_A: the quotient of equal
+    numbers is 1 (times a rounded reciprocal it is not, for one W in seven)."""
+    rng = np.random.default_rng(61)
+    fs = [(*rng.uniform(0, 8e-3, 2), 3000.0 + 3.0 * rng.uniform(0, 1, 1) + 1.5 * np.arange(60), 8.2 + 1e-4 * np.arange(60),
+           rng.standard_normal(60), rng.integers(1, 8, 60)) for _ in range(12)]
+    cat = line_catalog(fs)
+    q = synth.Quasars(ra=rng.uniform(0, 8e-3, 30), dec=rng.uniform(0, 8e-3, 30), dist=rng.uniform(2950.0, 3150.0, 30),
+                      weight=rng.integers(1, 8, 30).astype(np.float32), z=np.full(30, 2.5))
+    b = synth.Bins(40, 12, 100.0, 60.0)
+    dc = api.DeviceCatalog.from_host(cat)
+    for D, w in (api.lya_dmat(handle, dc, b, 1.0, 3, eta="identity"),
+                 api.lya_xdmat(handle, dc, api.DeviceQuasars.from_host(q), b, 1.0, 3, eta="identity")):
+        D, w = D.cpu().numpy(), w.cpu().numpy()
+        on = w > 0
+        assert on.sum() > 100
+        np.testing.assert_array_equal(D[np.ix_(on, on)], np.eye(on.sum()))
+
+
 @pytest.mark.parametrize("n_r,n_alpha,n_theta,nf,factor", [
     (4, 5, 3, 14, 1.0),      # classes summed in shared memory
     (16, 1, 1, 14, 1.0),     # the most |r| bins
