@@ -17,10 +17,10 @@ namespace {
 constexpr int kTile = 64;     // output tile edge
 constexpr int kSt = 16;       // sub-samples per shared-memory stage
 
-// full sums, xi and 1 / W: 32 bins per block, 32 slices of the sub-samples
+// full sums and xi: 32 bins per block, 32 slices of the sub-samples
 // (one thread per bin walking all of them in turn took 0.23 ms for 768 x 2,500)
 __global__ void __launch_bounds__(1024) cov_totals_kernel(const double* num_s, const double* wsum_s, int n_sub, int nb,
-                                                          double* W, double* iW, double* xi) {
+                                                          double* W, double* xi) {
   __shared__ double sw[32][33], sn[32][33];
   const int t = threadIdx.x & 31, q = threadIdx.x >> 5;
   for (int A0 = blockIdx.x * 32; A0 < nb; A0 += gridDim.x * 32) {
@@ -39,7 +39,6 @@ __global__ void __launch_bounds__(1024) cov_totals_kernel(const double* num_s, c
     n = warp_sum_f64(sn[t][q]);
     if (t == 0 && A0 + q < nb) {
       W[A0 + q] = w;
-      iW[A0 + q] = (w != 0.0) ? 1.0 / w : 0.0;
       xi[A0 + q] = (w != 0.0) ? n / w : 0.0;
     }
     __syncthreads();
@@ -82,10 +81,10 @@ __global__ void __launch_bounds__(1024) cov_list_kernel(const int32_t* flag, int
 
 // C tile (64 x 64) per block of 16 x 16 threads, 4 x 4 outputs per thread;
 // tiles on and above the diagonal, written to both sides.  Bound by the FP64
-// pipe: an entry costs one multiply-add per sub-sample and three products
-// (dividing by W_A W_B cost more than the sum over 12 sub-samples).
+// pipe: an entry costs one multiply-add per sub-sample, and a division as much
+// as the sum over a dozen sub-samples.
 __global__ void __launch_bounds__(256) cov_kernel(const double* num_s, const double* wsum_s, int nb,
-                                                  const double* W, const double* iW, const double* xi,
+                                                  const double* W, const double* xi,
                                                   const int32_t* list, double* cov) {
   if (blockIdx.x < blockIdx.y) return;
   __shared__ double ar[kSt][kTile];
@@ -132,7 +131,8 @@ __global__ void __launch_bounds__(256) cov_kernel(const double* num_s, const dou
     for (int v = 0; v < 4; ++v) {
       const int B = c0 + tx * 4 + v;
       if (B >= nb) continue;
-      const double c = (W[A] * W[B] != 0.0) ? acc[u][v] * (iW[A] * iW[B]) : 0.0;   // (symmetric)
+      const double den = W[A] * W[B];
+      const double c = (den != 0.0) ? acc[u][v] / den : 0.0;   // (symmetric)
       cov[static_cast<int64_t>(A) * nb + B] = c;
       if (blockIdx.x != blockIdx.y) cov[static_cast<int64_t>(B) * nb + A] = c;
     }
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) cov_kernel(const double* num_s, const dou
 
 size_t covariance_scratch_bytes(int n_sub, int nb) {
   auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
-  return 3 * al(static_cast<size_t>(nb) * 8) + al((static_cast<size_t>(n_sub) + 1) * 4) + al(static_cast<size_t>(n_sub) * 4);
+  return 2 * al(static_cast<size_t>(nb) * 8) + al((static_cast<size_t>(n_sub) + 1) * 4) + al(static_cast<size_t>(n_sub) * 4);
 }
 
 cudaError_t launch_covariance(const double* num_s, const double* wsum_s, int n_sub, int nb, double* cov,
@@ -152,15 +152,14 @@ cudaError_t launch_covariance(const double* num_s, const double* wsum_s, int n_s
   auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
   char* sc = static_cast<char*>(scratch);
   double* W = reinterpret_cast<double*>(sc);
-  double* iW = reinterpret_cast<double*>(sc + al(static_cast<size_t>(nb) * 8));
-  double* xi = reinterpret_cast<double*>(sc + 2 * al(static_cast<size_t>(nb) * 8));
-  int32_t* list = reinterpret_cast<int32_t*>(sc + 3 * al(static_cast<size_t>(nb) * 8));
-  int32_t* flag = reinterpret_cast<int32_t*>(sc + 3 * al(static_cast<size_t>(nb) * 8) + al((static_cast<size_t>(n_sub) + 1) * 4));
-  LYA_COUNT(1), cov_totals_kernel<<<std::min((nb + 31) / 32, 2048), 1024, 0, s>>>(num_s, wsum_s, n_sub, nb, W, iW, xi);
+  double* xi = reinterpret_cast<double*>(sc + al(static_cast<size_t>(nb) * 8));
+  int32_t* list = reinterpret_cast<int32_t*>(sc + 2 * al(static_cast<size_t>(nb) * 8));
+  int32_t* flag = reinterpret_cast<int32_t*>(sc + 2 * al(static_cast<size_t>(nb) * 8) + al((static_cast<size_t>(n_sub) + 1) * 4));
+  LYA_COUNT(1), cov_totals_kernel<<<std::min((nb + 31) / 32, 2048), 1024, 0, s>>>(num_s, wsum_s, n_sub, nb, W, xi);
   LYA_COUNT(1), cov_flag_kernel<<<std::min(n_sub, 4096), 256, 0, s>>>(wsum_s, n_sub, nb, flag);
   LYA_COUNT(1), cov_list_kernel<<<1, 1024, 0, s>>>(flag, n_sub, list);
   const int nt = (nb + kTile - 1) / kTile;
-  LYA_COUNT(1), cov_kernel<<<dim3(nt, nt), 256, 0, s>>>(num_s, wsum_s, nb, W, iW, xi, list, cov);
+  LYA_COUNT(1), cov_kernel<<<dim3(nt, nt), 256, 0, s>>>(num_s, wsum_s, nb, W, xi, list, cov);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && xi_out) e = cudaMemcpyAsync(xi_out, xi, static_cast<size_t>(nb) * 8, cudaMemcpyDeviceToDevice, s);
   return e;

@@ -401,6 +401,21 @@ def test_dmat_rows_are_divided_by_their_weight(api, handle):
         np.testing.assert_array_equal(D[np.ix_(on, on)], np.eye(on.sum()))
 
 
+@pytest.mark.parametrize("n_sub,nb", [(2, 65), (33, 64), (1100, 130)])
+def test_covariance_of_whole_numbers(api, handle, n_sub, nb):
+    """Whole-number sums in two sub-samples (the first and the last) with N adding up to 0: every sum is exact, so an
+    entry is the correctly rounded quotient 2 n_A n_B / (W_A W_B)."""
+    rng = np.random.default_rng(n_sub)
+    n = rng.integers(-50, 51, nb).astype(np.float64)
+    num, w = np.zeros((n_sub, nb)), np.zeros((n_sub, nb))
+    num[0], num[-1] = n, -n
+    w[0], w[-1] = rng.integers(1, 60, nb), rng.integers(0, 60, nb)
+    cov, xi = api.lya_xi_covariance(handle, torch.from_numpy(num).cuda(), torch.from_numpy(w).cuda())
+    W = w.sum(axis=0)
+    np.testing.assert_array_equal(xi.cpu().numpy(), 0.0)
+    np.testing.assert_array_equal(cov.cpu().numpy(), 2.0 * np.outer(n, n) / np.outer(W, W))
+
+
 @pytest.mark.parametrize("n_r,n_alpha,n_theta,nf,factor", [
     (4, 5, 3, 14, 1.0),      # classes summed in shared memory
     (16, 1, 1, 14, 1.0),     # the most |r| bins
