@@ -162,13 +162,16 @@ __device__ __forceinline__ void run_times(const longlong2& S, float w, F2 f, flo
   l = unf2(fma2(fma2(err, one, fma2(fma2(H, w1, np), one, fma2(L, w2, nq))), f, 0ull));
 }
 
-// sqrt(q) to 2e-14 (one Newton step from FP32; exact FP64 roots and divisions
-// cost twenty FP64 operations each)
+// sqrt(q) to one unit in the last place: 1 / sqrt(q) to 2e-14 by a Newton step from
+// FP32, and the root corrected by its remainder, exact in a fused multiply-add
+// (a square root costs twice as many FP64 operations)
 __device__ __forceinline__ double root(double q) {
   const float qf = static_cast<float>(q);
   if (!(qf > 1e-30f)) return sqrt(q);
-  const double y = rsqrtf(qf);
-  return q * fma(0.5 * y, fma(-(q * y), y, 1.0), y);
+  const double y0 = rsqrtf(qf), h0 = 0.5 * y0;
+  const double h = fma(0.5 * h0, fma(-(q * y0), y0, 1.0), h0);   // 1 / (2 sqrt(q))
+  const double s = 2.0 * q * h;
+  return fma(fma(-s, s, q), h, s);
 }
 
 // Window geometry of one (forest, quasar) pair against the forest's staged
