@@ -137,11 +137,12 @@ struct X3Bin {
     const double dx = dj * A.F.ux[o] - x[0], dy = dj * A.F.uy[o] - x[1], dz = dj * A.F.uz[o] - x[2];
     const double r2 = dx * dx + dy * dy + dz * dz;
     if (!(r2 < rmax2 && r2 > 0.0)) return false;
-    // 1 / |r| to 2e-14: one Newton step from FP32 (an FP64 square root and division cost 20 times that)
+    // 1 / |r| to FP64 by two Newton steps from FP32 (a square root and a division cost five times that)
     const float r2f = static_cast<float>(r2);
     const float y0f = rsqrtf(r2f);
     const double y0 = y0f;
-    const double y = fma(0.5 * y0, fma(-(r2 * y0), y0, 1.0), y0);
+    const double y1 = fma(0.5 * y0, fma(-(r2 * y0), y0, 1.0), y0);
+    const double y = fma(0.5 * y1, fma(-(r2 * y1), y1, 1.0), y1);
     const double dot = dx * u[0] + dy * u[1] + dz * u[2];
     const float ctf = static_cast<float>(dot * y);
     const float fr = r2f * y0f * inv_dr_f, ft = acosf(fminf(1.f, fmaxf(-1.f, ctf))) * inv_dt_f;
