@@ -463,8 +463,10 @@ __device__ __forceinline__ Pair dm_load(const DmArgs& A, int item, const Sm& m, 
   const float Dc = (refa - refb) * P.cp, Ds = (refa + refb) * P.sp;
   // Histogram terms of the summed-over forest (w, w x) in fixed point, one
   // 32-bit word each: shared memory adds integers natively.  A (vector, bin)
-  // sum holds at most 2 / (cp hmin) + 2 pixels (two windows of width 1/cp).
-  const float runa = 2.f / (P.cp * A.F.hmin[a]) + 2.f, runb = 2.f / (P.cp * A.F.hmin[b]) + 2.f;
+  // sum holds at most 2 / (cp hmin) + 2 pixels (two windows of width 1/cp) of
+  // the forest's (one pixel has no gap: hmin is then next to 0).
+  const float runa = fminf(2.f / (P.cp * A.F.hmin[a]) + 2.f, static_cast<float>(P.na));
+  const float runb = fminf(2.f / (P.cp * A.F.hmin[b]) + 2.f, static_cast<float>(P.nb));
   const float sA0 = word_scale(runa * A.F.wmax[a]), sB0 = word_scale(runa * A.F.wmax[a] * A.F.xmax[a]);
   const float sA1 = word_scale(runb * A.F.wmax[b]), sB1 = word_scale(runb * A.F.wmax[b] * A.F.xmax[b]);
   const Pix* ga = A.pix + A.F.off[a];

@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(lya_catalog cat, int
       F.wmax[gf] = wmx;
       F.wdmax[gf] = wdmx;
       // packed distances of a sorted forest may repeat after rounding; a gap
-      // of 0 (or a single pixel) is recorded as a tiny positive number, which
-      // only makes the fixed-point bound more conservative
+      // of 0 (or a single pixel) is recorded as a tiny positive number; who
+      // bounds a run by it also bounds it by the forest's pixels
       F.hmin[gf] = (hmn > 1e-6f && hmn < INFINITY) ? hmn : 1e-6f;
       F.xmax[gf] = xmx;
       if (fp) {

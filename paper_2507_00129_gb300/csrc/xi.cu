@@ -270,7 +270,8 @@ __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, 
   const float fnpar = static_cast<float>(npar), fnperp = static_cast<float>(A.n_perp);
   // fixed-point scales: a run of in-grid pairs (fixed i, one bin) spans less
   // than 2 / cp in distance, so it holds at most 2 / (cp hmin_b) + 1 pixels of b
-  const float nrun = 2.f / (cp * A.F.hmin[bidx]) + 1.f;
+  // (one pixel has no gap: hmin is then next to 0)
+  const float nrun = fminf(2.f / (cp * A.F.hmin[bidx]) + 1.f, static_cast<float>(nb));
   const float scN = fixed_scale(A.F.wdmax[aidx] * A.F.wdmax[bidx] * nrun);
   const float scW = fixed_scale(A.F.wmax[aidx] * A.F.wmax[bidx] * nrun);
   const float inv_scN = 1.f / scN, inv_scW = 1.f / scW;

@@ -401,6 +401,30 @@ def test_dmat_rows_are_divided_by_their_weight(api, handle):
         np.testing.assert_array_equal(D[np.ix_(on, on)], np.eye(on.sum()))
 
 
+@pytest.mark.parametrize("lengths", [(1, 1, 1, 1, 30, 41), (1, 2, 3, 2, 1, 3)])
+def test_forests_of_few_pixels(api, handle, lengths):
+    """One pixel has no gap to its neighbour to bound a run by: W of xi and of D to 1e-6, D (whose entries are at most
+    1) to 1e-5, next to the edge allowances of test_dmat_on_a_grid_of_unequal_sides."""
+    cat = _catalog(lengths, 1.0, 71, patch=6e-3)
+    b = synth.Bins(13, 10, 65.0, 50.0)
+    pr = oracle.pairs.forest_pairs(cat, b)
+    fwd = oracle.xi.xi_sums(cat, b, pr, eps_edge=6e-5)
+    ref = oracle.dmat.dmat(cat, b, pr, processes=0, eps_edge=6e-5)
+    dc = api.DeviceCatalog.from_host(cat)
+    num, wsum, _ = api.lya_xi(handle, dc, b, "mixed")
+    D, w = api.lya_dmat(handle, dc, b, 1.0, 3)
+    api.lya_sync_status(handle)
+    W, E, R = fwd["wsum"], fwd["edge_w"], ref["dmat"]
+    assert np.count_nonzero(W) > 5
+    top = float(np.abs(cat.delta).max())
+    assert np.all(np.abs(wsum.cpu().numpy() - W) <= 1e-6 * W + E)
+    assert np.all(np.abs(num.cpu().numpy() - fwd["num"]) <= 1e-6 * top * top * W + fwd["edge_n"])
+    assert np.all(np.abs(w.cpu().numpy() - W) <= 1e-6 * W + E)
+    den = (W - E)[:, None]
+    edge = np.divide(ref["edge_d"] + np.abs(R) * E[:, None], den, out=np.zeros_like(R), where=den > 0)
+    assert np.all(np.abs(D.cpu().numpy() - R) <= 1e-5 + edge)
+
+
 @pytest.mark.parametrize("n_sub,nb", [(2, 65), (33, 64), (1100, 130)])
 def test_covariance_of_whole_numbers(api, handle, n_sub, nb):
     """Whole-number sums in two sub-samples (the first and the last) with N adding up to 0: every sum is exact, so an
