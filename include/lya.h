@@ -310,7 +310,8 @@ typedef struct {
  * during graph capture.  A main vertex with more neighbours within r_max
  * than one block holds (about 6,400 on GB300) is reported as
  * LYA_ERR_TOO_LARGE by the next synchronising call.  Limits: n_r, n_theta
- * <= 256, n_alpha <= 1024, at most 2^28 bins. */
+ * <= 256, n_alpha <= 1024, at most 2^28 bins.  Scratch: 16 bytes per bin, kept
+ * by the handle, where the device has room for it (slower without). */
 int lya_xi3(lya_handle* h, const lya_catalog* cat, const lya_bins3* bins, double* num, double* wsum,
             double* xi, void* stream);
 

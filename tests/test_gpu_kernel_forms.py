@@ -463,6 +463,33 @@ def test_xi3_grouped_vertices(api, handle, n_r, n_alpha, n_theta, nf, factor):
     np.testing.assert_array_equal(Wr, Wr.transpose(1, 0, 2, 4, 3))
 
 
+def test_xi3_without_room_for_scratch(api):
+    """A grid whose interleaved sums do not fit beside the caller's outputs on the device: the same result, summed in
+    the outputs.  A record's FP32 product is rounded twice in an order that follows the order in which its two
+    neighbours were found, so two calls differ by up to 2^-22 of each record."""
+    cat = synth.generate(synth.Spec(n_forests=14, seed=8, region="box", box_deg=0.3, grid="log10", delta_sigma=0.2))
+    g = oracle.xi3.Grid3(n_r=16, n_theta=64, n_alpha=64, r_max=15.0)   # 2^26 bins: 1.07 GB of sums, and a quarter
+    dc = api.DeviceCatalog.from_host(cat)
+    with api.Handle() as h:
+        n0, w0, x0 = api.lya_xi3(h, dc, g)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    block = torch.empty(free - 3 * 8 * n0.numel() - (700 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with api.Handle() as h:
+            out = api.lya_xi3(h, dc, g)
+            api.lya_sync_status(h)
+    finally:
+        del block
+        torch.cuda.empty_cache()
+    assert float(w0.sum()) > 0
+    assert bool(((out[1] - w0).abs() <= 2.0 ** -22 * w0).all())
+    top = float(np.abs(cat.delta).max()) ** 3
+    assert bool(((out[0] - n0).abs() <= 2.0 ** -22 * top * w0).all())
+    assert bool(((out[2] - x0).abs() <= 2.0 ** -21 * top).all())
+
+
 @pytest.mark.parametrize("factor", [30.0, 1e3, 1e6])
 def test_xi3_light_triplets_beside_a_heavy_forest(api, handle, factor):
     """One forest, 13.2 Mpc/h from the others, weighs `factor` times as much, so that its records fill bins of their
