@@ -56,6 +56,7 @@ cudaError_t grow(void** p, size_t* cap, size_t need) {
   size_t n = need + need / 4 + 256;
   cudaError_t e = cudaMalloc(p, n);
   if (e != cudaSuccess) {
+    cudaGetLastError();   // else the next launch of any call would report it
     *p = nullptr;
     return e;
   }
@@ -288,7 +289,7 @@ int ensure_workspace(lya_handle* h, int64_t nf, int64_t np) {
     const size_t bytes = static_cast<size_t>(cap) * (8 * 9 + 4 * 7) + 16 * 256;
     if (h->fbuf) { cudaDeviceSynchronize(); cudaFree(h->fbuf); h->fbuf = nullptr; }
     cudaError_t e = cudaMalloc(&h->fbuf, bytes);
-    if (e != cudaSuccess) { h->F_capacity = 0; return fail(h, LYA_ERR_NO_MEMORY, "forest workspace"); }
+    if (e != cudaSuccess) { cudaGetLastError(); h->F_capacity = 0; return fail(h, LYA_ERR_NO_MEMORY, "forest workspace"); }
     h->fbuf_cap = bytes;
     char* p = static_cast<char*>(h->fbuf);
     auto take = [&](size_t b) { char* q = p; p += (b + 255) & ~size_t(255); return q; };

@@ -937,10 +937,7 @@ cudaError_t run_xi3(const X3Args& a, const DevInfo& dev, void** scratch, size_t*
   // 204 ms on 5,000 SDSS-like forests)
   cudaError_t e = grow(scratch, scratch_cap, o_sums + static_cast<size_t>(nbins) * 16);
   const bool split = e == cudaErrorMemoryAllocation;
-  if (split) {
-    cudaGetLastError();
-    e = grow(scratch, scratch_cap, o_sums);
-  }
+  if (split) e = grow(scratch, scratch_cap, o_sums);
   LYA_TRY(e);
   char* sc = static_cast<char*>(*scratch);
   int32_t* deg = reinterpret_cast<int32_t*>(sc + o_deg);

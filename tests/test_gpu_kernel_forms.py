@@ -490,6 +490,31 @@ def test_xi3_without_room_for_scratch(api):
     assert bool(((out[2] - x0).abs() <= 2.0 ** -21 * top).all())
 
 
+def test_a_refused_allocation_does_not_reach_the_next_call(api):
+    """A call whose scratch does not fit is refused with LYA_ERR_NO_MEMORY (-4), and the next call runs."""
+    from paper_2507_00129_gb300._lib import LyaError
+    cat = synth.subset(synth.make(0), np.arange(40))
+    dc = api.DeviceCatalog.from_host(cat)
+    small, large = synth.bins_for(0), synth.Bins(150, 100, 100.0, 100.0)   # 1.8 GB of D, 2.25 GB of scratch
+    with api.Handle() as h:
+        n0, w0, _ = api.lya_xi(h, dc, small)
+        D = torch.empty((15000, 15000), dtype=torch.float64, device="cuda")
+        W = torch.empty(15000, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        block = torch.empty(torch.cuda.mem_get_info()[0] - (1 << 30), dtype=torch.uint8, device="cuda")
+        try:
+            with pytest.raises(LyaError) as e:
+                api.lya_dmat(h, dc, large, 1.0, 3, D=D, W=W)
+            assert e.value.code == -4
+        finally:
+            del block, D, W
+            torch.cuda.empty_cache()
+        n1, w1, _ = api.lya_xi(h, dc, small)
+        api.lya_sync_status(h)
+        assert bool(((w1 - w0).abs() <= 1e-11 * w0).all())
+
+
 @pytest.mark.parametrize("factor", [30.0, 1e3, 1e6])
 def test_xi3_light_triplets_beside_a_heavy_forest(api, handle, factor):
     """One forest, 13.2 Mpc/h from the others, weighs `factor` times as much, so that its records fill bins of their
