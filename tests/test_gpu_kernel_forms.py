@@ -425,6 +425,29 @@ def test_forests_of_few_pixels(api, handle, lengths):
     assert np.all(np.abs(D.cpu().numpy() - R) <= 1e-5 + edge)
 
 
+@pytest.mark.parametrize("lengths,step,bins,patch,seed", [
+    ((255, 256, 257, 258, 33), 0.3, (25, 25, 100.0, 100.0), 4e-3, 81),   # edges of a staged segment, all in the grid
+    ((512, 513, 31, 1, 32), 0.3, (40, 30, 60.0, 100.0), 4e-3, 82),       # ranges that end beside a segment's edge
+    ((300, 290, 64), 0.5, (30, 10, 45.0, 30.0), 8e-3, 83),               # clamps along both coordinates
+    ((96, 130, 257), 0.6, (25, 10, 50.0, 50.0), 0.0, 84),                # one line of sight: r_perp = 0
+])
+def test_gradient_forms(api, handle, lengths, step, bins, patch, seed):
+    """The gradient's staged segments of 256 pixels and their clamp-free ranges; allowance of
+    test_gpu_parity.test_backward_matches_oracle."""
+    cat = _catalog(lengths, step, seed, patch=patch)
+    b = synth.Bins(*bins)
+    pr = oracle.pairs.forest_pairs(cat, b)
+    c = np.random.default_rng(seed).normal(size=b.nbins)
+    fwd = oracle.xi.xi_sums(cat, b, pr)
+    gd_ref, gw_ref, info = oracle.adjoint.xi_grad(cat, b, c, pr, absolute=True, eps_edge=6e-5, fwd=fwd)
+    gd, gw = api.lya_xi_backward(handle, api.DeviceCatalog.from_host(cat), b, torch.from_numpy(c).cuda(),
+                                 torch.from_numpy(fwd["xi"]).cuda(), torch.from_numpy(fwd["wsum"]).cuda())
+    api.lya_sync_status(handle)
+    assert np.count_nonzero(gd_ref) > cat.n_pix // 2
+    assert np.all(np.abs(gd.cpu().numpy() - gd_ref) <= 1e-5 * info["grad_delta_abs"] + info["grad_delta_edge"] + 1e-12)
+    assert np.all(np.abs(gw.cpu().numpy() - gw_ref) <= 1e-5 * info["grad_weight_abs"] + info["grad_weight_edge"] + 1e-12)
+
+
 @pytest.mark.parametrize("n_sub,nb", [(2, 65), (33, 64), (1100, 130)])
 def test_covariance_of_whole_numbers(api, handle, n_sub, nb):
     """Whole-number sums in two sub-samples (the first and the last) with N adding up to 0: every sum is exact, so an
