@@ -49,7 +49,7 @@ FLOPS_PER_PAIR = 8  # 4 for the two scaled separations, 2 products, 2 accumulati
 # when they are resident) and its pair-list entry.
 XI_TRAFFIC = {
     # 5.4636 GB read + 26.1 MB written by one launch on a 20,000-forest catalogue of the DESI-Y5-like kind
-    # (5.8618e11 in-grid pixel pairs), profiles/hot_kernels_small_cases.md
+    # (5.8618e11 in-grid pixel pairs)
     "desi_y5_like": {"sha256": "749ca270012c674cd7c8cd503c0b988601a29d05c7d988f3cbb90ff125ddd696",
                      "bytes_per_pixel_pair": (5463552512 + 26142464) / 586182760646},
 }

@@ -32,25 +32,6 @@ namespace {
 constexpr int kAdjWarps = 8;
 constexpr int kAdjSeg = 256;   // staged pixels of a neighbour per warp
 
-__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float bp = s - hi;
-  const float e = (hi - (s - bp)) + (x - bp);
-  hi = s;
-  lo += e;
-}
-
-// Number of staged pixels whose key (the 32-bit word at `word` of each 16-byte
-// record, ascending) lies strictly below v (v NaN -> n).
-__device__ __forceinline__ int staged_below(const ulonglong2* a, int word, int n, float v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (reinterpret_cast<const float*>(a + mid)[word] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 // Constants of a visit: the table's address, the pair's factors and the clamps
 // into the guard row and column.
 struct Visit {

@@ -476,7 +476,7 @@ int run_xi(lya_handle* h, const lya_catalog* cats, int ncat, const lya_bins* b, 
     const bool tuned = h->tuned_for_npar == b->n_par;
     CK(plan_xi_mixed(h->dev, b->n_par, h->max_len, tuned ? h->tuned_grab : 4, &L), "plan xi");
     // a short list is dealt pair by pair: with four at a time the last teams
-    // finish alone (200 forests, 9 pairs per team: 267 against 259 us)
+    // finish alone (200 forests, 9 pairs per team: 267 against 246 us)
     if (!tuned && npairs < 64 * static_cast<int64_t>(L.blocks)) L.grab = 1;
     stage_begin(h, 0, s);
     CK(launch_xi_mixed(A, L, s), "xi kernel");
@@ -1093,8 +1093,8 @@ int lya_xi_bin_means_z(lya_handle* h, const lya_catalog* cat, const lya_bins* bi
   if ((st = ensure_pairs(h, cat, 1, bins, s))) return st;
   const int nb = bins->n_par * bins->n_perp;
   if (means_limit_bytes(nb, h->max_len, z_pix != nullptr) > h->dev.smem_optin)
-    return fail(h, LYA_ERR_TOO_LARGE, "bin means: 36 (44 with redshifts) bytes per bin + 8 (12) per pixel of the "
-                                      "longest forest above shared memory");
+    return fail(h, LYA_ERR_TOO_LARGE, "bin means: 36 (44 with redshifts) bytes per bin + 16 (24) per pixel of the longest "
+                                      "forest above the size of a block's shared memory");
   cudaError_t e = grow(&h->scratch2, &h->scratch2_cap, means_scratch_bytes(nb));
   if (e != cudaSuccess) return fail(h, LYA_ERR_NO_MEMORY, "bin-means scratch");
   MeansArgs A{};
@@ -1227,8 +1227,6 @@ XcfArgs xcf_args(lya_handle* h, const lya_catalog* cat, const lya_quasars* q, co
   A.F = h->F;
   A.Q = h->Q;
   A.wq = q->weight;
-  A.delta = cat->delta;
-  A.weight = cat->weight;
   A.n_par = b->n_par;
   A.n_perp = b->n_perp;
   A.r_par_max = b->r_par_max;
@@ -1258,7 +1256,7 @@ int lya_xcf(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, const
   int ml = 0;
   if ((st = build_xpairs(h, cat, qso, forest_qso, bins, &ml, s))) return st;
   if (xcf_limit_bytes(nb, ml) > h->dev.smem_optin)
-    return fail(h, LYA_ERR_TOO_LARGE, "cross-correlation: 16 bytes per bin + 20 per pixel of the longest forest above shared memory");
+    return fail(h, LYA_ERR_TOO_LARGE, "cross-correlation: 16 bytes per bin + 40 per pixel of the longest forest above the size of a block's shared memory");
   CK(cudaMemsetAsync(num, 0, static_cast<size_t>(nb) * 8, s), "zero num");
   CK(cudaMemsetAsync(wsum, 0, static_cast<size_t>(nb) * 8, s), "zero wsum");
   XcfArgs A = xcf_args(h, cat, qso, bins, ml);
@@ -1324,7 +1322,8 @@ int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max
   if ((st = read_flags(h, s, &flags))) return st;
   if ((st = flags_to_status(h, flags))) return st;
   if (xi1d_limit_bytes(n_bins, ml) > h->dev.smem_optin)
-    return fail(h, LYA_ERR_TOO_LARGE, "1D correlation: 16 bytes per bin + 24 per pixel of the longest forest above shared memory");
+    return fail(h, LYA_ERR_TOO_LARGE, "1D correlation: 16 bytes per bin + 28 per pixel of the longest forest above the size of a "
+                                      "block's shared memory");
   CK(cudaMemsetAsync(num, 0, static_cast<size_t>(n_bins) * 8, s), "zero num");
   CK(cudaMemsetAsync(wsum, 0, static_cast<size_t>(n_bins) * 8, s), "zero wsum");
   X1Args A{};

@@ -237,12 +237,14 @@ __device__ __forceinline__ bool bin_at(float rp, float rt, float fnpar, float fn
   return rp < fnpar && rt < fnperp;
 }
 
-// Tile q of 2 rows x W columns of the union support's upper triangle: acc = sum
+constexpr int kTileW = 4;   // columns of a tile
+
+// Tile q of 2 rows x kTileW columns of the union support's upper triangle: acc = sum
 // over the batch's vectors of a a^T + b b^T.  Tiles of one column block are
 // consecutive, so the lanes of a warp read consecutive 16-byte row pairs (4
-// shared-memory passes) and the same columns (W / 2 broadcasts).
-template <int W>
-__device__ __forceinline__ void dm_tile(const F2* V, int ldv, int q, int nv, float (&acc)[2][W], int* row, int* col) {
+// shared-memory passes) and the same columns (two broadcasts).
+__device__ __forceinline__ void dm_tile(const F2* V, int ldv, int q, int nv, float (&acc)[2][kTileW], int* row, int* col) {
+  constexpr int W = kTileW;
   // column block cb has W / 2 (cb + 1) row pairs
   int cb = static_cast<int>((sqrtf(16.f / W * q + 1.f) - 1.f) * 0.5f);
   while (W / 4 * cb * (cb + 1) > q) --cb;
@@ -354,9 +356,10 @@ __device__ void dm_tiles_tc(const float* V, int ldv, int ns, int cbn, const int3
 // Subtract a tile from the triangle, or from G with FP64 atomics for wide
 // pairs.  S is ascending, so positions r <= c of it are entries of the upper
 // triangle.
-template <bool GLOBAL, int W>
+template <bool GLOBAL>
 __device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t* S, int g0, int ns, int L, int nbins,
-                                              int row, int col, const float (&acc)[2][W]) {
+                                              int row, int col, const float (&acc)[2][kTileW]) {
+  constexpr int W = kTileW;
   int lc[W];
 #pragma unroll
   for (int v = 0; v < W; ++v) lc[v] = S[min(col + v, ns - 1)];
@@ -381,14 +384,15 @@ __device__ __forceinline__ void dm_tile_store(double* G, float* U, const int32_t
   }
 }
 
-template <bool GLOBAL, int W>
+template <bool GLOBAL>
 __device__ __forceinline__ void dm_tiles(const F2* V, int ldv, int nv, double* G, float* U, const int32_t* S, int g0,
                                          int ns, int L, int nbins) {
+  constexpr int W = kTileW;
   const int nc = (ns + W - 1) / W;
   for (int q = threadIdx.x; q < W / 4 * nc * (nc + 1); q += kDmThreads) {
     float acc[2][W];
     int row, col;
-    dm_tile<W>(V, ldv, q, nv, acc, &row, &col);
+    dm_tile(V, ldv, q, nv, acc, &row, &col);
     dm_tile_store<GLOBAL>(G, U, S, g0, ns, L, nbins, row, col, acc);
   }
 }
@@ -735,12 +739,12 @@ __device__ void dm_vectors(const DmArgs& A, const Pair& P, double* G, int t0, in
     }
     __syncthreads();
     // rank-1 updates of the batch: register tiles of S x S, one per thread,
-    // each adding its 16 entries to the triangle
+    // each adding its 8 entries to the triangle
     if (eta) {
       if (!GLOBAL && A.tensor_tiles) {
         dm_tiles_tc(reinterpret_cast<const float*>(m.V), ldv, ns, B.cbn, m.S, m.U, L, wid, nwarps, lane);
       } else {
-        dm_tiles<GLOBAL, 4>(m.V, ldv, B.cbn, G, m.U, m.S, g0, ns, L, nbins);
+        dm_tiles<GLOBAL>(m.V, ldv, B.cbn, G, m.U, m.S, g0, ns, L, nbins);
       }
     }
     dirty = ns;

@@ -49,6 +49,25 @@ __device__ __forceinline__ float fixed_scale(float B) {
   return __uint_as_float(static_cast<uint32_t>(min(max(ex, 1), 254)) << 23);
 }
 
+// Knuth's TwoSum: (hi, lo) += x with the rounding error of hi + x kept in lo.
+__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
+  const float s = hi + x;
+  const float bp = s - hi;
+  lo += (hi - (s - bp)) + (x - bp);
+  hi = s;
+}
+
+// Number of staged pixels whose key (the 32-bit word at `word` of each 16-byte
+// record, ascending) lies strictly below v (0 for a NaN).
+__device__ __forceinline__ int staged_below(const ulonglong2* a, int word, int n, float v) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (reinterpret_cast<const float*>(a + mid)[word] < v) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
 // e of a scale 2^e
 __device__ __forceinline__ int scale_exponent(float sc) {
   return static_cast<int>((__float_as_uint(sc) >> 23) & 0xFFu) - 127;

@@ -55,15 +55,6 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void red_add_f32_shared(uint32_t addr, float v) {
-  asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(addr), "f"(v));
-}
-
-template <int OFF>
-__device__ __forceinline__ void red_add_f32_shared_off(uint32_t addr, float v) {
-  asm volatile("red.shared.add.f32 [%0+%2], %1;" ::"r"(addr), "f"(v), "n"(OFF));
-}
-
 __device__ __forceinline__ void red_add_f64_global(double* p, double v) {
   asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
@@ -95,7 +86,7 @@ __device__ __forceinline__ bool keep_pair(int a, int b, uint64_t seed, uint64_t 
   return all || (splitmix64(seed ^ ((lo << 32) | hi)) < thr);
 }
 
-// Number of elements of the sorted array a[0..n) strictly below v (v NaN -> n).
+// Number of elements of the sorted array a[0..n) strictly below v (0 for a NaN).
 __device__ __forceinline__ int count_below(const Pix* a, int n, float v) {
   int lo = 0, hi = n;
   while (lo < hi) {
@@ -274,8 +265,6 @@ struct XcfArgs {
   const int2* pairs;     // (forest, quasar), grouped by forest
   const int64_t* qoff;   // [F.n + 1] forest f's pairs: qoff[f] .. qoff[f+1]
   int64_t n_pairs;
-  const float* delta;    // caller's pixel arrays (single catalogue: packed index = pixel index)
-  const float* weight;
   const Pix* pix;
   Forests F;
   Forests Q;

@@ -64,14 +64,6 @@ constexpr int kSmallTablesLen = 384;
 constexpr int kMaxPar64 = 256;   // largest n_par of the FP64 path
 constexpr int kMaxSeg = 1024;    // pixel buffer cap per warp
 
-// Knuth's TwoSum: (hi, lo) += x with the rounding error of hi + x kept in lo.
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float bp = s - hi;
-  lo += (hi - (s - bp)) + (x - bp);
-  hi = s;
-}
-
 // A lane's ended run, held in registers until the warp adds the held runs to
 // the chunk histogram.
 struct Held {
@@ -208,8 +200,8 @@ __device__ __forceinline__ void fold_chunk(const TeamSm& w, int nrows, int npar,
           const int a = r * npar + p;
           const float vn = fmaf(static_cast<float>(a2), 1.f / 65536.f, static_cast<float>(static_cast<int32_t>(a1))) * inv_scN;
           const float vw = fmaf(static_cast<float>(b2), 1.f / 65536.f, static_cast<float>(static_cast<int32_t>(b1))) * inv_scW;
-          two_sum(nhi[a], nlo[a], vn);
-          two_sum(whi[a], wlo[a], vw);
+          two_sum_add(nhi[a], nlo[a], vn);
+          two_sum_add(whi[a], wlo[a], vw);
         }
         nh[k] = 0u;
         nl[k] = 0u;
@@ -246,16 +238,6 @@ __device__ __forceinline__ void flush_acc(const TeamSm& w, const XiArgs& A, int 
     }
   }
   __syncthreads();
-}
-
-// Number of staged pixels with distance strictly below v (v NaN -> n).
-__device__ __forceinline__ int staged_below(const ulonglong2* buf, int n, float v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (*reinterpret_cast<const float*>(buf + mid) < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
 }
 
 // Bin rows t0 .. t0 + K - 1 of forest pair (a, b) into the chunk histogram
@@ -307,8 +289,8 @@ __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, 
         if (sp > 0.f) dhi = fminf(dhi, (fnperp - fmaf(xf, sp, Ds)) / sp);
         dlo -= fabsf(dlo) * 1e-5f + 1e-2f;
         dhi += fabsf(dhi) * 1e-5f + 1e-2f;
-        jlo = staged_below(w.buf, segn, dlo);
-        jhi = staged_below(w.buf, segn, dhi);
+        jlo = staged_below(w.buf, 0, segn, dlo);
+        jhi = staged_below(w.buf, 0, segn, dhi);
       }
       // two chunks with work at a time, one per warp, then a fold
       unsigned todo = __ballot_sync(0xffffffffu, jlo < jhi);
@@ -331,7 +313,7 @@ __device__ void pair_rows(const XiArgs& A, const TeamSm& w, int aidx, int bidx, 
   }
 }
 
-// HC words per chunk-histogram array, AC entries per accumulator array (see kTables)
+// HC words per chunk-histogram array, AC entries per accumulator array (see kHcapL)
 template <int HC, int AC>
 __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int kmax, int grab) {
   extern __shared__ __align__(16) unsigned char smem[];
