@@ -448,6 +448,59 @@ def test_gradient_forms(api, handle, lengths, step, bins, patch, seed):
     assert np.all(np.abs(gw.cpu().numpy() - gw_ref) <= 1e-5 * info["grad_weight_abs"] + info["grad_weight_edge"] + 1e-12)
 
 
+@pytest.mark.parametrize("lengths,step,bins,seed", [
+    ((1, 2, 7, 8, 9, 16, 33), 1.0, (25, 25, 100.0, 100.0), 91),   # below and above a block of rows
+    ((255, 256, 257, 300), 0.6, (50, 50, 200.0, 200.0), 92),      # edges of a tile
+    ((520, 90, 1), 0.25, (256, 4, 128.0, 16.0), 93),              # three tiles
+    ((40, 70, 110), 0.25, (1, 300, 60.0, 30.0), 94),              # bands of many rows
+])
+def test_weights_of_many_decades(api, handle, lengths, step, bins, seed):
+    """Weights over twelve decades within every forest: the sums that leave the integers.  FP64 path and 1D to the
+    order of their FP64 sums (n 2^-53 < 1e-12), bin means to their FP32 sums of 8 pairs (5e-7), cross-correlation to
+    2^-40 off the bin edges; N against W times the largest |delta|."""
+    cat = _catalog(lengths, step, seed)
+    rng = np.random.default_rng(seed)
+    cat.weight = (10.0 ** rng.uniform(-6.0, 6.0, cat.n_pix)).astype(np.float32)
+    top = float(np.abs(cat.delta).max())
+    b = synth.Bins(*bins)
+    dc = api.DeviceCatalog.from_host(cat)
+    cpu = lambda *t: [x.cpu().numpy() for x in t]   # noqa: E731
+
+    ref = oracle.xi.xi_sums(cat, b)
+    n, w, _ = cpu(*api.lya_xi(handle, dc, b, "fp64"))
+    assert np.all(np.abs(w - ref["wsum"]) <= 1e-12 * ref["wsum"])
+    assert np.all(np.abs(n - ref["num"]) <= 1e-12 * top * top * ref["wsum"])
+
+    ref = oracle.xi1d.xi1d_sums(cat, 37, 60.0)
+    n, w, _ = cpu(*api.lya_xi1d(handle, dc, 37, 60.0))
+    assert np.all(np.abs(w - ref["wsum"]) <= 1e-12 * ref["wsum"])
+    assert np.all(np.abs(n - ref["num"]) <= 1e-12 * top * top * ref["wsum"])
+
+    z = np.exp(cat.loglam) / 1215.67 - 1.0
+    ref = oracle.xi.bin_means(cat, b, eps_edge=6e-5, z=z)
+    got = api.lya_xi_bin_means(handle, dc, b, z_pix=torch.from_numpy(z).cuda())
+    W = ref["wsum"]
+    on = W > 4.0 * ref["edge_w"]
+    assert on.sum() > 0
+    assert np.all(np.abs(got["count"].cpu().numpy() - ref["count"]) <= ref["edge_c"])
+    assert np.all(np.abs(got["wsum"].cpu().numpy() - W) <= 1e-6 * W + ref["edge_w"])
+    frac = 2.0 * ref["edge_w"][on] / (W[on] - ref["edge_w"][on])
+    for key, width in (("rpar_mean", b.r_par_max / b.n_par), ("rperp_mean", b.r_perp_max / b.n_perp),
+                       ("dist_mean", float(cat.dist.max() - cat.dist.min())), ("z_mean", float(z.max() - z.min()))):
+        err = np.abs(got[key].cpu().numpy()[on] - ref[key][on])
+        assert np.all(err <= 1e-6 * np.abs(ref[key][on]) + frac * width), key
+
+    q = synth.Quasars(ra=rng.uniform(0, 2e-3, 30), dec=rng.uniform(0, 2e-3, 30), dist=rng.uniform(2950.0, 3200.0, 30),
+                      weight=(10.0 ** rng.uniform(-6.0, 6.0, 30)).astype(np.float32), z=np.full(30, 2.5))
+    ref = oracle.xcf.xcf_sums(cat, q, b, eps_edge=6e-5)
+    n, w, _ = cpu(*api.lya_xcf(handle, dc, api.DeviceQuasars.from_host(q), b))
+    sure = (ref["count"] > 0) & (ref["edge_w"] == 0)
+    assert sure.sum() > 0
+    assert np.all(np.abs(w - ref["wsum"])[sure] <= 2.0 ** -40 * ref["wsum"][sure])
+    assert np.all(np.abs(n - ref["num"])[sure] <= 1e-6 * top * ref["wsum"][sure])
+    api.lya_sync_status(handle)
+
+
 @pytest.mark.parametrize("n_sub,nb", [(2, 65), (33, 64), (1100, 130)])
 def test_covariance_of_whole_numbers(api, handle, n_sub, nb):
     """Whole-number sums in two sub-samples (the first and the last) with N adding up to 0: every sum is exact, so an
