@@ -306,7 +306,8 @@ typedef struct {
  * integers where the rounding to them (of the smallest W term and of a typical
  * N term of the integers' own bins) is no more than the products' own.  Builds (and caches) the forest-pair
  * list for r_par_max = r_perp_max = r_max.  Synchronises (a counting pass
- * sizes the kernel's neighbour capacity to the largest list); not allowed
+ * sizes the kernel's neighbour capacity to the longest chords of any vertex,
+ * 1e-2 Mpc/h wider than r_max); not allowed
  * during graph capture.  A main vertex with more neighbours within r_max
  * than one block holds (about 6,400 on GB300) is reported as
  * LYA_ERR_TOO_LARGE by the next synchronising call.  Limits: n_r, n_theta
@@ -327,8 +328,8 @@ int lya_xi3(lya_handle* h, const lya_catalog* cat, const lya_bins3* bins, double
  * mixed path of lya_xi; sums of up to 8 pixel pairs in FP32, then exact integers
  * (where these would round such a sum by more than 2^-21 of its smallest pair,
  * weights being too far apart: FP64) and FP64.  Builds the pair list if none is cached (synchronises); refused
- * during graph capture.  Limit: 36 bytes per bin + 8 per pixel of the longest
- * forest of shared memory. */
+ * during graph capture.  Limit: 36 bytes per bin + 16 per pixel of the longest
+ * forest within the size of a block's shared memory (227 KB). */
 int lya_xi_bin_means(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, double* wsum, double* rpar_mean,
                      double* rperp_mean, double* dist_mean, int64_t* npairs, void* stream);
 
@@ -339,8 +340,8 @@ int lya_xi_bin_means(lya_handle* h, const lya_catalog* cat, const lya_bins* bins
  * float64 device array of the catalogue's pixel redshifts, supplied by the
  * caller (the library holds no cosmology or rest-frame wavelength), read as
  * FP32 in the run sums.  z_pix and z_mean are both NULL (then this is
- * lya_xi_bin_means) or both given.  Limit: 44 bytes per bin + 12 per pixel of
- * the longest forest of shared memory. */
+ * lya_xi_bin_means) or both given.  Limit: 44 bytes per bin + 24 per pixel of
+ * the longest forest within 227 KB. */
 int lya_xi_bin_means_z(lya_handle* h, const lya_catalog* cat, const lya_bins* bins, const double* z_pix,
                        double* wsum, double* rpar_mean, double* rperp_mean, double* dist_mean, double* z_mean,
                        int64_t* npairs, void* stream);
@@ -398,7 +399,7 @@ int lya_xdmat(lya_handle* h, const lya_catalog* cat, const lya_quasars* qso, con
  * p < n_bins.  num, wsum required, xi optional, each [n_bins] float64.
  * Bins are the definition's in FP64; products and sums as with LYA_PREC_FP64.
  * Synchronises; refused during graph capture.  Limits: 1 <= n_bins <= 4096;
- * 16 bytes per bin + 24 per pixel of the longest forest of shared memory. */
+ * 16 bytes per bin + 28 per pixel of the longest forest within 227 KB. */
 int lya_xi1d(lya_handle* h, const lya_catalog* cat, int32_t n_bins, double r_max, double* num, double* wsum,
              double* xi, void* stream);
 

@@ -396,7 +396,8 @@ int grid_for(int64_t n, int threads) {
 size_t means_scratch_bytes(int nb) { return 6 * static_cast<size_t>(nb) * 8 + 8; }
 
 // The grids and forest lengths the entry point takes (36 or 44 bytes per bin
-// and 16 or 24 per pixel of the longest forest within a block's shared memory).
+// and 16 or 24 per pixel of the longest forest within the size of a block's shared
+// memory; the kernel itself needs less).
 int means_limit_bytes(int nb, int max_len, bool with_z) {
   const int base = 32 * nb + 4 * ((nb + 1) & ~1);
   return with_z ? base + 8 * nb + 2 * 12 * std::max(max_len, 1) : base + 2 * 8 * std::max(max_len, 1);
