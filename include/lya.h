@@ -303,13 +303,13 @@ typedef struct {
  * num, wsum (required), xi (optional): [n_r^2 n_alpha n_theta^2] float64.
  * The |r| and theta bins are those of FP64, cos alpha is FP32; products in
  * FP32 are added to FP64 bin sums, several vertices' together by way of exact
- * integers where the rounding to them (of the smallest W term and of a typical
- * N term of the integers' own bins) is no more than the products' own.  Builds (and caches) the forest-pair
- * list for r_par_max = r_perp_max = r_max.  Synchronises (a counting pass
+ * integers where these round the smallest W term by at most 2^-21 of itself and
+ * a typical N term by 2^-25.  Builds (and caches) the forest-pair list for
+ * r_par_max = r_perp_max = r_max.  Synchronises (a counting pass
  * sizes the kernel's neighbour capacity to the longest chords of any vertex,
  * 1e-2 Mpc/h wider than r_max); not allowed
  * during graph capture.  A main vertex with more neighbours within r_max
- * than one block holds (about 6,400 on GB300) is reported as
+ * than one block holds (about 7,200 on GB300) is reported as
  * LYA_ERR_TOO_LARGE by the next synchronising call.  Limits: n_r, n_theta
  * <= 256, n_alpha <= 1024, at most 2^28 bins.  Scratch: 16 bytes per bin, kept
  * by the handle, where the device has room for it (slower without). */

@@ -345,18 +345,19 @@ __global__ void __launch_bounds__(kX3Threads, 5) xi3_kernel(X3Args A, const int3
 //  * Sums are exact integers in two words, which shared memory adds natively: the
 //    high one in units of 2^eh as fine as the class's largest record (2^21 units)
 //    and the sum of all (2^30) allow, the low one with as many bits below as leave
-//    room for all records (xg_scale).  A record of a class is summed so only where
-//    the rounding is no more than that of its FP32 product (2^-24): of the
-//    smallest record for W, whose terms are positive, and of one of typical
-//    size for N, whose terms come arbitrarily close to 0.  Weights a few thousand times
-//    apart between neighbours are beyond that.  Such a class, one with few
+//    room for all records (xg_scale).  A class is summed so only where that rounds
+//    the smallest record of W, whose terms are positive, by at most 2^-21 of itself,
+//    and one of typical size of N, whose terms come arbitrarily close to 0, by at
+//    most 2^-25 (the FP32 product's own rounding is 2^-24; with 2^-24 for W as well
+//    the classes with many records, whose low words are short, go to L2: 2,000 forests
+//    on 5 x 4 x 8 bins 328 against 218 ms).  Such a class, one with few
 //    records (below kXGDirect a bin) and one whose products leave the FP32 range
 //    add their records to L2 as xi3_kernel does; with two blocks per SM the one's
 //    reductions in L2 run beside the other's in shared memory.
 // What bounds it: the shared-memory pipe (four reductions a record, 25 of 32
 // lanes on random bins) and L2's atomics.  Measured (5,000 SDSS-like forests,
 // r_max 40, 200,000 bins): xi3_kernel 204 ms,
-// this 157 ms; three words 227 ms, one block of 1,024 threads per SM 171 ms, no
+// this 161 ms; three words 227 ms, one block of 1,024 threads per SM 171 ms, no
 // direct classes 185 ms, kXGDirect 3, 12, 20: 160, 161, 186 ms; 64-bit words 449
 // ms (emulated).  Smaller grids gain more: 13 x 6^2 bins of 100 classes, 1,300
 // forests of a denser sky: 163 -> 54 ms.
@@ -704,7 +705,7 @@ __global__ void __launch_bounds__(kXGThreads, 2) xi3_group_kernel(X3Args A, cons
         if (!fn || !fw) continue;   // (sums that are infinite or not numbers among them)
         const int en = xg_scale(2.002f * bn, 1.01f * tn), ew = xg_scale(2.002f * bw, 1.01f * tw);
         const int k = min(21, __clz(recs));
-        if (tw != 0.f && !(lw >= pow2f(ew - k + 23))) continue;
+        if (tw != 0.f && !(lw >= pow2f(ew - k + 20))) continue;
         if (tn != 0.f && !(static_cast<float>(en - k + 24) <= s_typ)) continue;
         s_eh[c] = ((en + 256) << 16) | (ew + 256);
       }

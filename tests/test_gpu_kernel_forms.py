@@ -595,7 +595,7 @@ def test_a_refused_allocation_does_not_reach_the_next_call(api):
 def test_xi3_light_triplets_beside_a_heavy_forest(api, handle, factor):
     """One forest, 13.2 Mpc/h from the others, weighs `factor` times as much, so that its records fill bins of their
     own (the outermost |r| bin, theta near 90 degrees) and every other bin holds light ones only.  W to 1e-6 of each
-    bin's own value (FP32 products, and at most 2^-24 of a record in its rounding), N as in test_gpu_xi3."""
+    bin's own value (FP32 products, 2^-23, and at most 2^-21 of a record in its rounding), N as in test_gpu_xi3."""
     rng = np.random.default_rng(3)
     forests = []
     for k in range(8):
