@@ -48,10 +48,10 @@ FLOPS_PER_PAIR = 8  # 4 for the two scaled separations, 2 products, 2 accumulati
 # sources are unchanged.  Traffic grows with the pairs: every forest pair reads its two forests' pixels (from L2
 # when they are resident) and its pair-list entry.
 XI_TRAFFIC = {
-    # 5.4636 GB read + 26.1 MB written by one launch on a 20,000-forest catalogue of the DESI-Y5-like kind
+    # 5.4533 GB read + 23.9 MB written by one launch on a 20,000-forest catalogue of the DESI-Y5-like kind
     # (5.8618e11 in-grid pixel pairs)
-    "desi_y5_like": {"sha256": "749ca270012c674cd7c8cd503c0b988601a29d05c7d988f3cbb90ff125ddd696",
-                     "bytes_per_pixel_pair": (5463552512 + 26142464) / 586182760646},
+    "desi_y5_like": {"sha256": "c398d4bedfc0db60bd63dd78326eceda9ce5ab61d29eb0a937de489db3113d1d",
+                     "bytes_per_pixel_pair": (5453262848 + 23879168) / 586182760646},
 }
 
 
