@@ -319,7 +319,7 @@ __device__ void pair_means(const MeansArgs& A, const Acc& acc, unsigned char* sm
 // then added to the team's band histogram with native 32-bit reductions (runs
 // off the grid are dropped: all lanes' would go to one word).  The histogram is
 // added to the FP64 sums per tile.
-// What bounds it: issue (69%) of about 60 warp instructions per step, a third
+// What bounds it: issue (65%) of about 60 warp instructions per step, a third
 // of them at the ends of runs, which some lane has in every second step.
 // Eight teams per SM (26 KB each); more teams with smaller tables cost windows.
 // Measured (SDSS-like, 15,000 forests, 5.7e10 pixel pairs, with redshifts):
