@@ -50,7 +50,7 @@ FLOPS_PER_PAIR = 8  # 4 for the two scaled separations, 2 products, 2 accumulati
 XI_TRAFFIC = {
     # 5.4533 GB read + 23.9 MB written by one launch on a 20,000-forest catalogue of the DESI-Y5-like kind
     # (5.8618e11 in-grid pixel pairs)
-    "desi_y5_like": {"sha256": "c398d4bedfc0db60bd63dd78326eceda9ce5ab61d29eb0a937de489db3113d1d",
+    "desi_y5_like": {"sha256": "c36db96bd85760904331775a828e565ff3d3a8b3bac0e0bce6e8a22b8afa59ed",
                      "bytes_per_pixel_pair": (5453262848 + 23879168) / 586182760646},
 }
 

@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kXW * 32) xdm_kernel(XcfArgs A, int cap) {
 // FP32 packed distances when that value lies farther than `guard` from an
 // integer (the FP32 error is below guard / 2), else from the FP64 division of
 // the definition, so every bin is the definition's.
-// What bounds it: issue (73%), about 55 warp instructions per step of 32 pairs.
+// What bounds it: issue (71%), about 55 warp instructions per step of 32 pairs.
 // Measured (60,000 SDSS-like forests, 8.5e8 pairs): one warp per pixel with
 // FP64 prefix sums and two shared FP64 atomics per run of two pixels 25.1 ms,
 // this form 2.5 ms, and 0.05 ms for 21 forests of the second launch (0.13 ms with

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kTeam) xi_mixed_kernel(XiArgs A, int seg, int 
 // Rounding: 2^-54 of the forest's largest value per pixel, 2^-51 to 2^-45 of the
 // largest product per run (as the sums leave room), to nearest, none in the sums
 // below a tile; the run's is at most 2^-36 of the pair's smallest product w_i w_j.
-// What bounds it: issue (52%) and latencies of about 55 warp instructions per
+// What bounds it: issue (58%) and latencies of about 55 warp instructions per
 // step, of which the key and its edge test take 20, the six multiply-adds 6,
 // and the ends of runs (some lane in every second step) a quarter; a third of
 // the lanes' pairs lie off the grid at the ends of the diagonals.
